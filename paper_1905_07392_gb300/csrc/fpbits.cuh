@@ -3,7 +3,8 @@
 // FP64 pipe, which bounds the refinement residual kernels (measured: -8 % for
 // the cell-centred, -20 % for the nodal residual).  In kernels that are not
 // FP64-bound the 64-bit integer work costs more than it saves (the solution
-// update, the strain-rate kernel), so they keep the instructions.  Each
+// update, the strain-rate kernel), so they keep the instructions; the
+// widening (f32_to_f64) works on 32-bit words and pays there.  Each
 // function gives the same bits as the conversion it replaces (nearest, ties
 // to even; exact widening) and falls back to that conversion outside the
 // normal ranges.
@@ -51,6 +52,17 @@ __device__ inline float f64_to_f32_pow2(double x, double sc)
     if (E == 0 || E == 2047 || !u64_to_f32((b & 0xfffffffffffffull) | (1ull << 52), E - 1075 + k, f))
         return __double2float_rn(x * sc);
     return (b >> 63) ? -f : f;
+}
+
+// (double)x from the bit fields, on 32-bit words (five integer operations
+// instead of one FP64-pipe slot, which costs a warp sixteen cycles here);
+// subnormals, infinities and NaN take the conversion.
+__device__ inline double f32_to_f64(float x)
+{
+    const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)x;   // not a normal number
+    const unsigned hi = a ? (a >> 3) + 0x38000000u : 0u;                // exponent bias 127 -> 1023
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 
 }  // namespace ebv

@@ -23,10 +23,23 @@
 
 namespace ebv {
 
+// Device scalars of a solve (c->scal).  S_ALPHA = rz/pq and S_BETA = rz/rz_old
+// are formed once, by the reduction that completes their last operand
+// (kRedAlpha, kRedBeta), S_ISIG = 1/S_SIG where S_SIG is set: an FP64 division
+// costs about twenty FP64-pipe slots, and with 2 FP64 lanes per SM the vector
+// kernels spent most of their time on the same quotient in every thread
+// (k_cg_update32 on 64^3: 9.3 us with it, 1.8 us without; 256^3: 28.5 -> 26.4;
+// k_cg_pupdate32 on 64^3: 6.9 -> 1.8 us; FP64 k_cg_pupdate on 128^3: 10.8 -> 6.0).
+enum { S_BB = 0, S_RR = 1, S_RZ = 2, S_RZOLD = 3, S_PQ = 4, S_REL = 16, S_PREV = 17, S_T2 = 18, S_SIG = 19,
+       S_ISIG = 20, S_ALPHA = 21, S_BETA = 22 };
+
 // ===========================================================================
 // Reductions
 // ===========================================================================
 namespace {
+
+// What a reduction does with its sum besides storing it.
+enum { kRedSum = 0, kRedAlpha = 1, kRedBeta = 2 };
 
 template <int kThreads>
 __device__ inline double block_sum(double v)
@@ -98,7 +111,7 @@ __device__ inline double block_sum3_t(T v)
 // kRedCtas SMs.  The barrier is the hardware cluster barrier (no spin).
 constexpr int kRedCtas = 8, kRedThreads = 512;
 __global__ void __cluster_dims__(kRedCtas, 1, 1) __launch_bounds__(kRedThreads)
-    k_reduce_final(const double *part, int n, double *out)
+    k_reduce_final(const double *part, int n, double *out, double *scal, int post)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
@@ -114,6 +127,8 @@ __global__ void __cluster_dims__(kRedCtas, 1, 1) __launch_bounds__(kRedThreads)
         double t = 0.0;
         for (int r = 0; r < kRedCtas; r++) t += csum[r];
         *out = t;
+        if (post == kRedAlpha) scal[S_ALPHA] = scal[S_RZ] / t;   // t = p.q
+        if (post == kRedBeta) scal[S_BETA] = t / scal[S_RZOLD];  // t = r.z (unused by a first iteration)
     }
 }
 
@@ -131,8 +146,20 @@ __global__ void __launch_bounds__(256) k_dot(const double *__restrict__ a, const
 
 ebv_status reduce_sum(Ctx *c, const double *part, int nblocks, double *out_dev)
 {
-    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas), dim3(kRedThreads), 0, part, nblocks, out_dev);
+    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas), dim3(kRedThreads), 0, part, nblocks, out_dev, c->scal,
+               (int)kRedSum);
     return EBV_OK;
+}
+// r.z or p.q of a CG iteration, with the quotient it completes.
+static void reduce_rz(Ctx *c, int nblocks)
+{
+    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas), dim3(kRedThreads), 0, c->part, nblocks, c->scal + S_RZ, c->scal,
+               (int)kRedBeta);
+}
+static void reduce_pq(Ctx *c, int nblocks)
+{
+    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas), dim3(kRedThreads), 0, c->part, nblocks, c->scal + S_PQ, c->scal,
+               (int)kRedAlpha);
 }
 
 namespace {
@@ -2304,7 +2331,6 @@ __global__ void __launch_bounds__(kCoarseThreads) k_cc_coarse_vcycle(CoarseVC<T>
 // ===========================================================================
 // Krylov glue
 // ===========================================================================
-enum { S_BB = 0, S_RR = 1, S_RZ = 2, S_RZOLD = 3, S_PQ = 4, S_REL = 16, S_PREV = 17, S_T2 = 18, S_SIG = 19 };
 
 // Scale of the refinement solver's FP32 residuals: a power of two near 1/|b|
 // (1 when |b| is 0 or not finite), so that corrections of right-hand sides far
@@ -2318,6 +2344,7 @@ __global__ void k_set_sigma(double *scal, int x_zero)
     double sig = 1.0;
     if (bb > 0.0 && isfinite(bb)) sig = ldexp(1.0, -ilogb(sqrt(bb)));
     scal[S_SIG] = sig;
+    scal[S_ISIG] = 1.0 / sig;   // exact: a power of two
     scal[S_BB] = bb * sig * sig;
     if (x_zero) scal[S_RR] = scal[S_BB];
 }
@@ -2468,7 +2495,7 @@ __global__ void __launch_bounds__(256) k_cg_update(double *__restrict__ x, doubl
                                                    const double *__restrict__ p, const double *__restrict__ q,
                                                    const double *__restrict__ scal, int n, double *__restrict__ part)
 {
-    const double a = scal[S_RZ] / scal[S_PQ];
+    const double a = scal[S_ALPHA];
     double v = 0.0;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         x[s] += a * p[s];
@@ -2484,7 +2511,7 @@ __global__ void k_cg_pupdate(double *__restrict__ p, const double *__restrict__ 
                              int n, const int *__restrict__ ctl)
 {
     const int first = ctl[C_K] == 0;
-    const double beta = first ? 0.0 : scal[S_RZ] / scal[S_RZOLD];
+    const double beta = first ? 0.0 : scal[S_BETA];
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
         p[s] = first ? z[s] : z[s] + beta * p[s];
 }
@@ -2497,7 +2524,16 @@ __global__ void __launch_bounds__(256) k_dot32(const float *__restrict__ a, cons
                                                double *__restrict__ part)
 {
     float v = 0.0f;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) v += a[s] * b[s];
+    const int n4 = n >> 2, t0 = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
+    const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
+    for (int s = t0; s < n4; s += st) {
+        const float4 u = a4[s], w = b4[s];
+        v += u.x * w.x;
+        v += u.y * w.y;
+        v += u.z * w.z;
+        v += u.w * w.w;
+    }
+    for (int s = 4 * n4 + t0; s < n; s += st) v += a[s] * b[s];
     double dv = block_sum<256>((double)v);
     if (threadIdx.x == 0) part[blockIdx.x] = dv;
 }
@@ -2509,7 +2545,7 @@ __global__ void __launch_bounds__(256) k_cg_update32(float *__restrict__ r, cons
                                                      const double *__restrict__ scal, int n,
                                                      double *__restrict__ part)
 {
-    const float a = (float)(scal[S_RZ] / scal[S_PQ]);
+    const float a = (float)scal[S_ALPHA];
     float v = 0.0f;
     // 16-byte vectors (the arrays come from cudaMalloc), then the n % 4 tail:
     // four independent loads per thread keep enough bytes in flight
@@ -2545,8 +2581,8 @@ __global__ void k_cg_pupdate32(float *__restrict__ p, float *__restrict__ e, con
                                const double *__restrict__ scal, int n, const int *__restrict__ ctl)
 {
     const int k = ctl[C_K];
-    const float beta = k == 0 ? 0.0f : (float)(scal[S_RZ] / scal[S_RZOLD]);
-    const float a = k == 0 ? 0.0f : (float)(scal[S_RZOLD] / scal[S_PQ]);
+    const float beta = k == 0 ? 0.0f : (float)scal[S_BETA];
+    const float a = k == 0 ? 0.0f : (float)scal[S_ALPHA];   // of the iteration before
     // one element (each lane of a vector, and the tail)
     auto upd = [&](float &pv, float &ev, float zv) {
         if (k == 0) {
@@ -2592,23 +2628,43 @@ __global__ void k_add32to64(double *__restrict__ x, const float *__restrict__ e,
                             const double *__restrict__ scal, const int *__restrict__ ctl, int n)
 {
     const int k = ctl[C_K];
-    const float a = (float)(scal[S_RZOLD] / scal[S_PQ]);
-    const double isig = 1.0 / scal[S_SIG];   // exact: a power of two
+    const float a = (float)scal[S_ALPHA];
+    const double isig = scal[S_ISIG];
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
-        x[s] += (double)final_e(e, p, a, k, s) * isig;
+        x[s] += f32_to_f64(final_e(e, p, a, k, s)) * isig;
 }
 
-// k_add32to64 with e and p FP32 row-split vectors
-__global__ void k_add32to64_split(GridD g, double *__restrict__ x, const float *__restrict__ e,
-                                  const float *__restrict__ p, const double *__restrict__ scal,
-                                  const int *__restrict__ ctl)
+// k_add32to64 with e and p FP32 row-split vectors.  A thread owns one column
+// and kAddPz planes, all loads before the stores: no division by the row
+// length per cell, and one FP64 operation (the FMA; the widening is integer
+// work, f32_to_f64).  64^3: 9.8 -> 4.1 us; 256^3 83 us (81 before), 4.9 TB/s
+// of its 24 bytes per cell.
+constexpr int kAddPz = 4;
+inline dim3 add_grid(const GridD &g)
 {
-    const int n = ncell(g);
-    const int k = ctl[C_K];
-    const float a = (float)(scal[S_RZOLD] / scal[S_PQ]);
-    const double isig = 1.0 / scal[S_SIG];   // exact: a power of two
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
-        x[s] += (double)final_e(e, p, a, k, cix<float>(g, s % g.nx, (s / g.nx) % g.ny, s / (g.nx * g.ny))) * isig;
+    return dim3((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + kAddPz - 1) / kAddPz);
+}
+__global__ void __launch_bounds__(256) k_add32to64_split(GridD g, double *__restrict__ x, const float *__restrict__ e,
+                                                         const float *__restrict__ p,
+                                                         const double *__restrict__ scal,
+                                                         const int *__restrict__ ctl)
+{
+    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k0 = blockIdx.z * kAddPz;
+    if (i >= g.nx || j >= g.ny) return;
+    const int kit = ctl[C_K];
+    const float a = (float)scal[S_ALPHA];
+    const double isig = scal[S_ISIG];
+    double xv[kAddPz];
+    float ev[kAddPz];
+#pragma unroll
+    for (int q = 0; q < kAddPz; q++) {
+        if (k0 + q >= g.nz) continue;
+        xv[q] = x[cidx(g, i, j, k0 + q)];
+        ev[q] = final_e(e, p, a, kit, cix<float>(g, i, j, k0 + q));
+    }
+#pragma unroll
+    for (int q = 0; q < kAddPz; q++)
+        if (k0 + q < g.nz) x[cidx(g, i, j, k0 + q)] = xv[q] + f32_to_f64(ev[q]) * isig;
 }
 
 __global__ void k_fill(double *a, int n, double v)
@@ -3206,6 +3262,8 @@ struct Problem {
 };
 
 inline int vblocks(int n) { return std::min(kReduceBlocks, (n + 255) / 256); }
+// for the FP32 CG kernels, whose threads take four elements at a time
+inline int v4blocks(int n) { return std::min(kReduceBlocks, (n / 4 + 255) / 256 + 1); }
 
 // A loop whose condition is decided on the device.  Eager mode: next()
 // reads the condition word back (one synchronisation per pass).  Capture
@@ -3355,10 +3413,10 @@ ebv_status pcg(Ctx *c, Problem &P, const double *b, double *x, int *iters, doubl
         while (inner.next()) {
             P.precond(c, r, z);
             EBV_LAUNCH(c, k_dot, dim3(vblocks(n)), dim3(256), 0, r, z, n, c->part);
-            reduce_sum(c, c->part, vblocks(n), c->scal + S_RZ);
+            reduce_rz(c, vblocks(n));
             EBV_LAUNCH(c, k_cg_pupdate, dim3(vblocks(n)), dim3(256), 0, p, z, c->scal, n, c->ctl);
             P.apply_dot(c, p, q);
-            reduce_sum(c, c->part, P.apply_blocks(), c->scal + S_PQ);
+            reduce_pq(c, P.apply_blocks());
             EBV_LAUNCH(c, k_cg_update, dim3(vblocks(n)), dim3(256), 0, x, r, p, q, c->scal, n, c->part);
             EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, vblocks(n), c->scal, c->ctl, tol,
                        maxit, 0, inner.h, inner.use_h);
@@ -3412,13 +3470,13 @@ ebv_status pcg_refine(Ctx *c, Problem &P, const double *b, double *x, int *iters
         EBV_LAUNCH(c, k_set_cond, dim3(1), dim3(32), 0, c->ctl, C_COND_IN, 1, inner.h, inner.use_h);
         while (inner.next()) {
             const int nd = P.precond32_dot(c, r, z);
-            if (!nd) EBV_LAUNCH(c, k_dot32, dim3(vblocks(n)), dim3(256), 0, r, z, n, c->part);
-            reduce_sum(c, c->part, nd ? nd : vblocks(n), c->scal + S_RZ);
-            EBV_LAUNCH(c, k_cg_pupdate32, dim3(vblocks(n)), dim3(256), 0, p, e, z, c->scal, n, c->ctl);
+            if (!nd) EBV_LAUNCH(c, k_dot32, dim3(v4blocks(n)), dim3(256), 0, r, z, n, c->part);
+            reduce_rz(c, nd ? nd : v4blocks(n));
+            EBV_LAUNCH(c, k_cg_pupdate32, dim3(v4blocks(n)), dim3(256), 0, p, e, z, c->scal, n, c->ctl);
             P.apply_dot32(c, p, q);
-            reduce_sum(c, c->part, P.apply_blocks32(), c->scal + S_PQ);
-            EBV_LAUNCH(c, k_cg_update32, dim3(vblocks(n)), dim3(256), 0, r, q, c->scal, n, c->part);
-            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, vblocks(n), c->scal, c->ctl, tol,
+            reduce_pq(c, P.apply_blocks32());
+            EBV_LAUNCH(c, k_cg_update32, dim3(v4blocks(n)), dim3(256), 0, r, q, c->scal, n, c->part);
+            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, v4blocks(n), c->scal, c->ctl, tol,
                        maxit, 1, inner.h, inner.use_h);
         }
         inner_count = inner.body_launches();
@@ -3472,7 +3530,7 @@ struct CcProblem : Problem {
     }
     void add32(Ctx *c, double *x, const float *e, const float *p) override
     {
-        EBV_LAUNCH(c, k_add32to64_split, dim3(vblocks(n())), dim3(256), 0, H->lv[0].g, x, e, p, c->scal, c->ctl);
+        EBV_LAUNCH(c, k_add32to64_split, add_grid(H->lv[0].g), dim3(32, 8), 0, H->lv[0].g, x, e, p, c->scal, c->ctl);
     }
     void to32(Ctx *c, const double *b, float *r) override
     {

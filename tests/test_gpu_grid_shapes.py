@@ -1,0 +1,60 @@
+"""One step against the oracle on grids of many shapes (paper Algorithm 1): the
+solver kernels choose their form by the grid -- one level or several, levels
+within one block, odd and even row lengths, odd bottoms, sizes that are or are
+not multiples of 8 and 16 -- and every choice must give the oracle's step.
+The tolerance is that of the other parity tests: both sides solve to 1e-13,
+and a relative residual of 1e-13 bounds u and p to 1e-10.  The captured step
+(advance_graph) must give the eager step's result bit for bit.  The sphere's
+centre is off the grid's centre by another amount along each axis: with equal
+offsets the two largest components of the wall normal are equal in many cut
+cells, and which of them Eq. dudn then takes as its axis is decided by the last
+bit of the geometry.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+SHAPES = [(5, 3, 7),      # a single level, odd rows
+          (6, 4, 10),     # two levels, bottom 3 x 2 x 5
+          (14, 14, 14),   # bottom 7^3 = 343 unknowns, 512 nodes
+          (12, 10, 14),   # every level within one block
+          (16, 16, 16), (32, 32, 32),
+          (20, 12, 28),   # odd half-rows on level 1
+          (24, 20, 28),   # nx a multiple of 8 but not of 16
+          (48, 16, 32),   # a multiple of 16, flat
+          (40, 24, 56)]   # a multiple of 8, odd bottom
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n", SHAPES)
+def test_step_matches_oracle(n, precision):
+    from paper_1905_07392_gb300 import ebvisc as E
+    h = 1.0 / n[0]
+    c = tuple((0.5 * v + o) * h for v, o in zip(n, (0.013, 0.131, 0.272)))
+    r = 0.3 * min(n) * h
+    kw = dict(rho=1.0, mu=1.0, tau0=2.0, m=1e3, bi_cfl=0.5)
+    s = E.Solver(n, h, tol=1e-13, max_iters=5000, precision=precision, **kw)
+    s.build_sphere(c, r)
+    g = O.Grid(n=n, h=h)
+    geo = O.build_geometry(g, O.Shape(kind=O.SHAPE_SPHERE, p=c + (r,)))
+    P = O.Params(tol=1e-13, max_iters=200000, **kw)
+    rng = np.random.Generator(np.random.PCG64(n[0]))
+    u0 = rng.uniform(-1e-3, 1e-3, size=(3, g.ncell))
+    u0[2] += 1.0
+    u0 = (u0 * (geo.alpha > 0)).ravel()
+    uo, po, sto = O.advance(g, geo, P, u0, np.zeros(g.nnode))
+    u, p = torch.tensor(u0, device=DEV), torch.zeros(g.nnode, dtype=torch.float64, device=DEV)
+    st = s.advance(u, p)
+    assert st["dt"] == pytest.approx(sto["dt"], rel=1e-12)
+    assert np.linalg.norm(u.cpu().numpy() - uo) <= 1e-10 * np.linalg.norm(uo)
+    assert np.linalg.norm(p.cpu().numpy() - po) <= 1e-10 * np.linalg.norm(po)
+    ug, pg = torch.tensor(u0, device=DEV), torch.zeros(g.nnode, dtype=torch.float64, device=DEV)
+    sg = s.advance_graph(ug, pg, steps=1)
+    assert torch.equal(u, ug) and torch.equal(p, pg)
+    assert sg["iters"] == st["iters"]
+    s.close()
