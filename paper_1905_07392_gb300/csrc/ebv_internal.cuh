@@ -190,7 +190,7 @@ struct CcHier {
     int L = 0;                 // number of levels (level L-1 is the bottom)
     CcLevel lv[kMaxLevels];
     double *binv = nullptr;    // bottom inverse of the selected variant, nb x nb
-    double *bmat = nullptr;    // scratch for the bottom factorisations, nvar x nb x 2nb
+    double *bmat = nullptr;    // scratch of the bottom inverses
     int nb = 0;
     // Variants of one operator that differ only in which box faces enter the
     // diagonal (the three velocity components of the viscous solve: a slip

@@ -2015,80 +2015,201 @@ __global__ void k_nd_active(GridD g, const double *__restrict__ alpha, uint8_t *
 // Dense bottom solve
 // ===========================================================================
 
+// Edge of the padded bottom matrix: nb rounded up to whole pivot blocks, the
+// rows past nb those of the identity.
+constexpr int kGjB = 16;
+__host__ __device__ inline int gj_pad(int nb) { return (nb + kGjB - 1) / kGjB * kGjB; }
+// doubles of scratch per matrix: two copies and two pivot-block inverses
+inline size_t gj_scratch(int nb) { return 2 * (size_t)gj_pad(nb) * gj_pad(nb) + 2 * kGjB * kGjB; }
+
+// Bottom matrices of the variants of one operator (blockIdx.y; they differ in
+// the diagonal), one block per row: np x np, natural numbering.
 template <class T>
-__global__ void k_cc_bottom_assemble(VOp<T> A, double *__restrict__ M, int nb)
+struct BottomDiag {
+    const T *d[3];
+};
+template <class T>
+__global__ void __launch_bounds__(128) k_cc_bottom_assemble(VOp<T> A, BottomDiag<T> D, double *__restrict__ M, int nb,
+                                                            size_t mstride)
 {
     const GridD &g = A.g;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nb; r += gridDim.x * blockDim.x) {
-        double *row = M + (size_t)r * 2 * nb;
-        for (int s = 0; s < 2 * nb; s++) row[s] = 0.0;
-        row[nb + r] = 1.0;
-        int i = r % g.nx, j = (r / g.nx) % g.ny, k = r / (g.nx * g.ny);
-        double bxl = (double)T(A.bx[fidxT<T>(g, 0, i, j, k)]), bxh = (double)T(A.bx[fidxT<T>(g, 0, i + 1, j, k)]);
-        double byl = (double)T(A.by[fidxT<T>(g, 1, i, j, k)]), byh = (double)T(A.by[fidxT<T>(g, 1, i, j + 1, k)]);
-        double bzl = (double)T(A.bz[fidxT<T>(g, 2, i, j, k)]), bzh = (double)T(A.bz[fidxT<T>(g, 2, i, j, k + 1)]);
-        double diag = (double)A.diag[cix<T>(g, i, j, k)];
-        row[r] = diag > 0.0 ? diag : 1.0;
-        if (i > 0) row[r - 1] = -bxl;
-        if (i < g.nx - 1) row[r + 1] = -bxh;
-        if (j > 0) row[r - g.nx] = -byl;
-        if (j < g.ny - 1) row[r + g.nx] = -byh;
-        if (k > 0) row[r - g.nx * g.ny] = -bzl;
-        if (k < g.nz - 1) row[r + g.nx * g.ny] = -bzh;
-    }
+    const int r = blockIdx.x, np = gridDim.x;
+    double *row = M + blockIdx.y * mstride + (size_t)r * np;
+    for (int s = threadIdx.x; s < np; s += blockDim.x) row[s] = (s == r) ? 1.0 : 0.0;
+    __syncthreads();
+    if (threadIdx.x || r >= nb) return;
+    int i = r % g.nx, j = (r / g.nx) % g.ny, k = r / (g.nx * g.ny);
+    double bxl = (double)T(A.bx[fidxT<T>(g, 0, i, j, k)]), bxh = (double)T(A.bx[fidxT<T>(g, 0, i + 1, j, k)]);
+    double byl = (double)T(A.by[fidxT<T>(g, 1, i, j, k)]), byh = (double)T(A.by[fidxT<T>(g, 1, i, j + 1, k)]);
+    double bzl = (double)T(A.bz[fidxT<T>(g, 2, i, j, k)]), bzh = (double)T(A.bz[fidxT<T>(g, 2, i, j, k + 1)]);
+    double diag = (double)D.d[blockIdx.y][cix<T>(g, i, j, k)];
+    row[r] = diag > 0.0 ? diag : 1.0;
+    if (i > 0) row[r - 1] = -bxl;
+    if (i < g.nx - 1) row[r + 1] = -bxh;
+    if (j > 0) row[r - g.nx] = -byl;
+    if (j < g.ny - 1) row[r + g.nx] = -byh;
+    if (k > 0) row[r - g.nx * g.ny] = -bzl;
+    if (k < g.nz - 1) row[r + g.nx * g.ny] = -bzh;
 }
 
-__global__ void k_nd_bottom_assemble(GridD g, const double *__restrict__ alpha, const uint8_t *__restrict__ act,
-                                     double *__restrict__ M, int nb)
+__global__ void __launch_bounds__(128) k_nd_bottom_assemble(GridD g, const double *__restrict__ alpha,
+                                                            const uint8_t *__restrict__ act, double *__restrict__ M,
+                                                            int nb)
 {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nb; r += gridDim.x * blockDim.x) {
-        double *row = M + (size_t)r * 2 * nb;
-        for (int s = 0; s < 2 * nb; s++) row[s] = 0.0;
-        row[nb + r] = 1.0;
-        int i = r % (g.nx + 1), j = (r / (g.nx + 1)) % (g.ny + 1), k = r / ((g.nx + 1) * (g.ny + 1));
-        if (!act[r]) { row[r] = 1.0; continue; }
-        for (int oc = 0; oc < 8; oc++) {
-            int ci = i - 1 + (oc & 1), cj = j - 1 + ((oc >> 1) & 1), ck = k - 1 + ((oc >> 2) & 1);
-            if (!inbox(g, ci, cj, ck)) continue;
-            double al = alpha[cidx(g, ci, cj, ck)];
-            if (!(al > 0.0)) continue;
-            int oa = (i - ci) | ((j - cj) << 1) | ((k - ck) << 2);
-            for (int ob = 0; ob < 8; ob++) {
-                int n = nidx(g, ci + (ob & 1), cj + ((ob >> 1) & 1), ck + ((ob >> 2) & 1));
-                if (!act[n]) continue;
-                row[n] += g.h * al * kQ1[__popc(oa ^ ob)];
-            }
+    const int r = blockIdx.x, np = gridDim.x;
+    double *row = M + (size_t)r * np;
+    for (int s = threadIdx.x; s < np; s += blockDim.x) row[s] = 0.0;
+    __syncthreads();
+    if (threadIdx.x) return;
+    if (r >= nb || !act[r]) { row[r] = 1.0; return; }
+    int i = r % (g.nx + 1), j = (r / (g.nx + 1)) % (g.ny + 1), k = r / ((g.nx + 1) * (g.ny + 1));
+    for (int oc = 0; oc < 8; oc++) {
+        int ci = i - 1 + (oc & 1), cj = j - 1 + ((oc >> 1) & 1), ck = k - 1 + ((oc >> 2) & 1);
+        if (!inbox(g, ci, cj, ck)) continue;
+        double al = alpha[cidx(g, ci, cj, ck)];
+        if (!(al > 0.0)) continue;
+        int oa = (i - ci) | ((j - cj) << 1) | ((k - ck) << 2);
+        for (int ob = 0; ob < 8; ob++) {
+            int n = nidx(g, ci + (ob & 1), cj + ((ob >> 1) & 1), ck + ((ob >> 2) & 1));
+            if (!act[n]) continue;
+            row[n] += g.h * al * kQ1[__popc(oa ^ ob)];
         }
     }
 }
 
-// Gauss-Jordan elimination of [M | I] in one CTA (SPD: no pivoting needed);
-// the right half becomes the inverse, copied to inv.  CTA q of the grid
-// inverts matrix q of the nb x 2nb matrices stored one after another in M into
-// inv_q (up to three at once: the variants of one operator).
-__global__ void __launch_bounds__(1024) k_gauss_jordan(double *__restrict__ Mall, int nb, double *inv0,
-                                                       double *inv1, double *inv2)
+// Inverse of an SPD matrix in place by Gauss-Jordan elimination with pivot
+// blocks of kGjB rows (no pivoting needed), for up to three matrices of one
+// size at once.  With P = A_KK^-1, one step replaces
+//   A_KK by P, A_Kj by P A_Kj, A_iK by -A_iK P, A_ij by A_ij - A_iK P A_Kj.
+// One launch per step over tiles of TE x TE entries, from one copy of the
+// matrix into the other; the tile that forms the next step's diagonal block
+// also inverts it, and the last step writes the unpadded inverse.  The work
+// is nb^3 FP64 multiply-adds and one SM does two per cycle: one block per
+// matrix on the augmented [A | I] (the form before) took 0.23 ms for 64
+// unknowns, 0.84 ms for 105 and 6.0 ms for 210; over the tiles 50, 90 and 247 us
+// (about 10 us a step, two thirds of it the next block's inverse).  Tiles of 32
+// where 16 x 16 ones would make more than two waves (each tile forms
+// A_iK P itself, a third of the work at 32 and half of it at 16).
+struct GjArgs {
+    const double *src[3];
+    double *dst[3];
+    double *piv[3];      // two kGjB x kGjB inverses each: this step's and the next one's
+    int np, ldo, nout;   // padded size; leading dimension and size of the output
+    int K;               // pivot block
+};
+
+// a (kGjB x kGjB, shared) := its inverse; 256 threads, one entry each.
+__device__ inline void gj_invert_block(double (*a)[kGjB + 1], double *sc)
 {
-    __shared__ double fac[kBottomMax];
-    const int w = 2 * nb;
-    double *__restrict__ M = Mall + (size_t)blockIdx.x * nb * w;
-    double *__restrict__ inv = blockIdx.x == 0 ? inv0 : (blockIdx.x == 1 ? inv1 : inv2);
-    for (int col = 0; col < nb; col++) {
-        double piv = M[(size_t)col * w + col];
+    const int r = threadIdx.x / kGjB, c = threadIdx.x % kGjB;
+    for (int k = 0; k < kGjB; k++) {
         __syncthreads();
-        for (int s = threadIdx.x; s < w; s += blockDim.x) M[(size_t)col * w + s] /= piv;
+        if (threadIdx.x == 0) *sc = 1.0 / a[k][k];
         __syncthreads();
-        for (int r = threadIdx.x; r < nb; r += blockDim.x) fac[r] = (r == col) ? 0.0 : M[(size_t)r * w + col];
+        const double p = *sc, f = a[r][k], q = a[k][c], v = a[r][c];
         __syncthreads();
-        for (int e = threadIdx.x; e < nb * w; e += blockDim.x) {
-            int r = e / w, s = e - r * w;
-            if (r != col) M[e] -= fac[r] * M[(size_t)col * w + s];
-        }
-        __syncthreads();
+        if (r == k) a[r][c] = (c == k) ? p : q * p;
+        else a[r][c] = (c == k) ? -f * p : v - f * (q * p);
     }
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int r = e / nb, s = e - r * nb;
-        inv[e] = M[(size_t)r * w + nb + s];
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(256) k_gj_first(GjArgs a)
+{
+    __shared__ double d[kGjB][kGjB + 1];
+    __shared__ double sc;
+    const int r = threadIdx.x / kGjB, c = threadIdx.x % kGjB, q = blockIdx.x;
+    d[r][c] = a.src[q][(size_t)r * a.np + c];
+    gj_invert_block(d, &sc);
+    a.piv[q][threadIdx.x] = d[r][c];
+}
+
+template <int TE>
+__global__ void __launch_bounds__(256) k_gj_step(GjArgs a)
+{
+    constexpr int B = kGjB, NE = TE * TE / 256;
+    __shared__ double sl[TE][B + 1], sr[B][TE + 1], sp[B][B + 1], sc[TE][B + 1];
+    __shared__ double inv;
+    const int q = blockIdx.z, np = a.np, K0 = a.K * B;
+    const int I0 = blockIdx.y * TE, J0 = blockIdx.x * TE, tid = threadIdx.x;
+    const double *A = a.src[q];
+    for (int e = tid; e < TE * B; e += 256) {
+        const int r = e / B, c = e % B;
+        sl[r][c] = I0 + r < np ? A[(size_t)(I0 + r) * np + K0 + c] : 0.0;
+        const int r2 = e / TE, c2 = e % TE;
+        sr[r2][c2] = J0 + c2 < np ? A[(size_t)(K0 + r2) * np + J0 + c2] : 0.0;
+    }
+    const double *P = a.piv[q] + (a.K & 1) * B * B;
+    sp[tid / B][tid % B] = P[tid];
+    __syncthreads();
+    // the row factors: A_iK P, and -P for the pivot rows themselves
+    for (int e = tid; e < TE * B; e += 256) {
+        const int r = e / B, c = e % B, pr = I0 + r - K0;
+        double v = 0.0;
+        if (pr >= 0 && pr < B) {
+            v = -sp[pr][c];
+        } else {
+#pragma unroll
+            for (int k = 0; k < B; k++) v += sl[r][k] * sp[k][c];
+        }
+        sc[r][c] = v;
+    }
+    __syncthreads();
+    const int N1 = K0 + B;   // first row of the next pivot block
+    double out[NE];
+#pragma unroll
+    for (int u = 0; u < NE; u++) {
+        const int e = tid + 256 * u, r = e / TE, c = e % TE, i = I0 + r, j = J0 + c;
+        const bool pr = i >= K0 && i < K0 + B, pc = j >= K0 && j < K0 + B;
+        double v;
+        if (pc) {
+            v = -sc[r][j - K0];
+        } else {
+            v = (pr || i >= np || j >= np) ? 0.0 : A[(size_t)i * np + j];
+#pragma unroll
+            for (int k = 0; k < B; k++) v -= sc[r][k] * sr[k][c];
+        }
+        out[u] = v;
+        if (i < a.nout && j < a.nout) a.dst[q][(size_t)i * a.ldo + j] = v;
+    }
+    // the next step's diagonal block and its inverse
+    if (N1 < np && N1 >= I0 && N1 < I0 + TE && N1 >= J0 && N1 < J0 + TE) {
+#pragma unroll
+        for (int u = 0; u < NE; u++) {
+            const int e = tid + 256 * u, r = I0 + e / TE - N1, c = J0 + e % TE - N1;
+            if (r >= 0 && r < B && c >= 0 && c < B) sp[r][c] = out[u];
+        }
+        gj_invert_block(sp, &inv);
+        a.piv[q][((a.K + 1) & 1) * B * B + tid] = sp[tid / B][tid % B];
+    }
+}
+
+// inv_q := the inverse of matrix q (assembled in M + q gj_scratch(nb)).
+void bottom_invert(Ctx *c, double *M, int nb, int nmat, double *const *inv)
+{
+    const int np = gj_pad(nb), ns = np / kGjB;
+    GjArgs a;
+    a.np = np;
+    for (int q = 0; q < 3; q++) {
+        double *m = M + (size_t)std::min(q, nmat - 1) * gj_scratch(nb);
+        a.src[q] = m;
+        a.dst[q] = nullptr;
+        a.piv[q] = m + 2 * (size_t)np * np;
+    }
+    EBV_LAUNCH(c, k_gj_first, dim3(nmat), dim3(256), 0, a);
+    const bool big = (long long)ns * ns * nmat > 2 * 152;
+    for (int K = 0; K < ns; K++) {
+        const bool last = K + 1 == ns;
+        a.K = K;
+        a.ldo = last ? nb : np;
+        a.nout = last ? nb : np;
+        for (int q = 0; q < nmat; q++) {
+            double *m = M + (size_t)q * gj_scratch(nb);
+            a.src[q] = m + (size_t)(K & 1) * np * np;
+            a.dst[q] = last ? inv[q] : m + (size_t)((K + 1) & 1) * np * np;
+        }
+        if (big) EBV_LAUNCH(c, k_gj_step<32>, dim3((np + 31) / 32, (np + 31) / 32, nmat), dim3(256), 0, a);
+        else EBV_LAUNCH(c, k_gj_step<16>, dim3(ns, ns, nmat), dim3(256), 0, a);
     }
 }
 
@@ -3614,21 +3735,17 @@ ebv_status cc_finish_hierarchy(Ctx *c, CcHier &H, bool fp32)
         }
     }
     const int lb = H.L - 1;
-    const size_t msz = (size_t)H.nb * 2 * H.nb;
-    for (int q = 0; q < H.nvar; q++) {
-        if (fp32) {
-            VOp<float> A = vop<float>(H.lv[lb]);
-            A.diag = H.vdiag_f[q][lb];
-            EBV_LAUNCH(c, k_cc_bottom_assemble<float>, dim3((H.nb + 127) / 128), dim3(128), 0, A, H.bmat + q * msz,
-                       H.nb);
-        } else {
-            VOp<double> A = vop<double>(H.lv[lb]);
-            A.diag = H.vdiag_d[q][lb];
-            EBV_LAUNCH(c, k_cc_bottom_assemble<double>, dim3((H.nb + 127) / 128), dim3(128), 0, A, H.bmat + q * msz,
-                       H.nb);
-        }
+    const dim3 ga(gj_pad(H.nb), H.nvar);
+    if (fp32) {
+        BottomDiag<float> D = {{H.vdiag_f[0][lb], H.vdiag_f[1][lb], H.vdiag_f[2][lb]}};
+        EBV_LAUNCH(c, k_cc_bottom_assemble<float>, ga, dim3(128), 0, vop<float>(H.lv[lb]), D, H.bmat, H.nb,
+                   gj_scratch(H.nb));
+    } else {
+        BottomDiag<double> D = {{H.vdiag_d[0][lb], H.vdiag_d[1][lb], H.vdiag_d[2][lb]}};
+        EBV_LAUNCH(c, k_cc_bottom_assemble<double>, ga, dim3(128), 0, vop<double>(H.lv[lb]), D, H.bmat, H.nb,
+                   gj_scratch(H.nb));
     }
-    EBV_LAUNCH(c, k_gauss_jordan, dim3(H.nvar), dim3(1024), 0, H.bmat, H.nb, H.vbinv[0], H.vbinv[1], H.vbinv[2]);
+    bottom_invert(c, H.bmat, H.nb, H.nvar, H.vbinv);
     select_variant(H, 0);
     return EBV_OK;
 }
@@ -3721,7 +3838,7 @@ ebv_status setup_solvers(Ctx *c)
             else Lv.cov = c->mac.lv[l].cov;
         }
         for (int q = 0; q < H->nvar; q++) H->vbinv[q] = dalloc<double>((size_t)nbc * nbc, e);
-        H->bmat = dalloc<double>((size_t)H->nvar * nbc * 2 * nbc, e);
+        H->bmat = dalloc<double>((size_t)H->nvar * gj_scratch((int)nbc), e);
         select_variant(*H, 0);
     }
     // nodal hierarchy
@@ -3744,7 +3861,7 @@ ebv_status setup_solvers(Ctx *c)
         Lv.lam_max = 2.0;
     }
     c->nd.binv = dalloc<double>((size_t)nbn * nbn, e);
-    c->nd.bmat = dalloc<double>((size_t)nbn * 2 * nbn, e);
+    c->nd.bmat = dalloc<double>(gj_scratch((int)nbn), e);
     // level vectors: large enough for nodes of that level (>= cells)
     int Lmax = std::max(L, Ln);
     for (int l = 0; l < Lmax; l++) {
@@ -3820,9 +3937,8 @@ ebv_status setup_geometry_solvers(Ctx *c)
         }
     }
     const NdLevel &B = N.lv[N.L - 1];
-    EBV_LAUNCH(c, k_nd_bottom_assemble, dim3((N.nb + 127) / 128), dim3(128), 0, B.g, B.alpha_d, B.act, N.bmat, N.nb);
-    EBV_LAUNCH(c, k_gauss_jordan, dim3(1), dim3(1024), 0, N.bmat, N.nb, N.binv, (double *)nullptr,
-               (double *)nullptr);
+    EBV_LAUNCH(c, k_nd_bottom_assemble, dim3(gj_pad(N.nb)), dim3(128), 0, B.g, B.alpha_d, B.act, N.bmat, N.nb);
+    bottom_invert(c, N.bmat, N.nb, 1, &N.binv);
     EBV_CUDA_TRY(c, cudaGetLastError());
     return autotune_shapes(c);
 }
