@@ -926,7 +926,7 @@ void ebv_destroy(ebv_ctx *c)
             CcLevel &L = H->lv[l];
             cudaFree(L.extra_d); cudaFree(L.extra_f);
             for (int q = 0; q < H->nvar; q++) {
-                cudaFree(H->vdiag_d[q][l]); cudaFree(H->vdiag_f[q][l]); cudaFree(H->vdinv_f[q][l]);
+                cudaFree(H->vdiag_d[q][l]); cudaFree(H->vdiag_f[q][l]);   // (vdinv_f lies in the same block)
             }
             for (int d = 0; d < 3; d++) { cudaFree(L.bf_d[d]); cudaFree(L.bf_f[d]); cudaFree(L.bf_h[d]); }
             cudaFree(L.bxp);

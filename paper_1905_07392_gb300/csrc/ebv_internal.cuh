@@ -172,7 +172,10 @@ struct CcLevel {
     // rounded from bf_f) and the diagonal diag_f formed from those rounded
     // faces; the level-0 Krylov operator keeps the FP32 faces with diag_a.
     float *diag_f = nullptr, *diag_a = nullptr;
-    float *dinv_f = nullptr;   // 1/diag_f (0 where diag_f <= 0), the smoother's multiplier
+    // 1/diag_f (0 where diag_f <= 0), the smoother's multiplier: the second
+    // half of diag_f's block.  In EBV_FP64 that block holds the FP64 inverse
+    // diagonal instead (the FP32 pair is not used then).
+    float *dinv_f = nullptr;
     __nv_bfloat16 *bf_h[3] = {nullptr, nullptr, nullptr};
     uint8_t *cov = nullptr;  // 1 where the cell is covered (identity row)
     void *bxp = nullptr;     // padded x faces of the fused sweep (V-cycle face type), or none

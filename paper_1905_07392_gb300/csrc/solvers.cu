@@ -178,7 +178,7 @@ struct CcOp {
     GridD g;
     const T *diag;
     const F *bx, *by, *bz;
-    const T *dinv = nullptr;   // FP32 V-cycle: 1/diag (0 where diag <= 0)
+    const T *dinv = nullptr;   // V-cycle operator: 1/diag (0 where diag <= 0)
 };
 // The V-cycle's operator: in FP32 its faces are stored in BF16 (half the
 // bytes of the face arrays every colour pass reads whole); the Krylov
@@ -295,8 +295,10 @@ __device__ inline void cc_row(const CcOp<T, F> &A, int i, int j, int k, const T 
 constexpr int GS_PZ = 2;
 
 // The Gauss-Seidel value of cell (i,j,k): (b + sum beta x_nb) / diag, 0 on
-// cells with no diagonal (see k_cc_gs for kCorr and zero_start); FP32 levels
-// multiply by the stored inverse diagonal instead of dividing.
+// cells with no diagonal (see k_cc_gs for kCorr and zero_start), formed with
+// the stored inverse diagonal: an FP64 division is about twenty FP64-pipe
+// operations, three times the rest of the cell (a 128^3 FP64 colour pass took
+// 33.7 us with it, 16.8 without).
 template <class T, bool kCorr>
 __device__ inline T gs_cell(const VOp<T> &A, const T *__restrict__ x, const T *__restrict__ b, int i, int j,
                             int k, int zero_start, const T *__restrict__ xc, const GridD &gc)
@@ -305,7 +307,7 @@ __device__ inline T gs_cell(const VOp<T> &A, const T *__restrict__ x, const T *_
     const int sy = g.nx, sz = g.nx * g.ny;
     const CellPos p = cell_pos<T>(g, i, j, k);
     const int c = p.c;
-    const T diag = sizeof(T) == 4 ? T(0) : A.diag[c], bc = b[c];
+    const T di = A.dinv[c], bc = b[c];
     T off = 0;
     if (!zero_start) {
         const T bxl = T(A.bx[p.fx0]), bxh = T(A.bx[p.fx1]);
@@ -327,8 +329,7 @@ __device__ inline T gs_cell(const VOp<T> &A, const T *__restrict__ x, const T *_
         if (k > 0) off += bzl * xd;
         if (k < g.nz - 1) off += bzh * xu;
     }
-    if constexpr (sizeof(T) == 4) return (bc + off) * A.dinv[c];
-    return diag > T(0) ? (bc + off) / diag : T(0);
+    return (bc + off) * di;
 }
 
 // kDot (the last pass of a V-cycle on the finest level): also block partials
@@ -1274,13 +1275,19 @@ __global__ void k_cc_make_diag(GridD g, const T *__restrict__ extra, const T *__
                        j == g.ny - 1 ? 3 : -1, k == 0 ? 4 : -1, k == g.nz - 1 ? 5 : -1};
     T *out[3] = {d0, d1, d2};
     T *inv[3] = {i0, i1, i2};
+    // away from the box sides the variants agree: one sum (and one quotient)
+    const bool side = i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1;
+    T s = e, si = T(0);
     for (int q = 0; q < nvar; q++) {
-        const unsigned m = masks >> (6 * q);
-        T s = e;
+        if (q == 0 || side) {
+            const unsigned m = masks >> (6 * q);
+            s = e;
 #pragma unroll
-        for (int t = 0; t < 6; t++) s += (sd[t] < 0 || ((m >> sd[t]) & 1u)) ? f[t] : T(0);
+            for (int t = 0; t < 6; t++) s += (sd[t] < 0 || ((m >> sd[t]) & 1u)) ? f[t] : T(0);
+            if (inv[q]) si = s > T(0) ? T(1) / s : T(0);
+        }
         out[q][c] = s;
-        if (inv[q]) inv[q][c] = s > T(0) ? T(1) / s : T(0);
+        if (inv[q]) inv[q][c] = si;
     }
 }
 
@@ -2825,6 +2832,7 @@ VOp<T> vop(const CcLevel &L)
     A.g = L.g;
     if constexpr (sizeof(T) == 8) {
         A.diag = (const T *)L.diag_d; A.bx = (const T *)L.bf_d[0]; A.by = (const T *)L.bf_d[1]; A.bz = (const T *)L.bf_d[2];
+        A.dinv = (const T *)L.diag_f;   // (the block of diag_f and dinv_f: see CcLevel)
     } else {
         A.diag = (const T *)L.diag_f;
         if constexpr (kVcycleBf16) {
@@ -2841,15 +2849,18 @@ VOp<T> vop(const CcLevel &L)
 
 // diagonals of every variant of level l from its extra and faces, in precision
 // T (FP32: the V-cycle's, from the faces rounded as it stores them).
+// inv (FP64): also the inverse diagonals, which the FP64 V-cycle reads.
 template <class T>
-void cc_make_diag(Ctx *c, CcHier &H, int l)
+void cc_make_diag(Ctx *c, CcHier &H, int l, bool inv = false)
 {
     const CcLevel &L = H.lv[l];
     unsigned masks = 0;
     for (int q = 0; q < H.nvar; q++) masks |= (H.side_mask[q] & 0x3fu) << (6 * q);
     if constexpr (sizeof(T) == 8)
         EBV_LAUNCH(c, k_cc_make_diag<double>, cgrid(L.g), block3(), 0, L.g, L.extra_d, L.bf_d[0], L.bf_d[1],
-                   L.bf_d[2], H.nvar, masks, H.vdiag_d[0][l], H.vdiag_d[1][l], H.vdiag_d[2][l]);
+                   L.bf_d[2], H.nvar, masks, H.vdiag_d[0][l], H.vdiag_d[1][l], H.vdiag_d[2][l],
+                   inv ? (double *)H.vdiag_f[0][l] : nullptr, inv ? (double *)H.vdiag_f[1][l] : nullptr,
+                   inv ? (double *)H.vdiag_f[2][l] : nullptr);
     else
         EBV_LAUNCH(c, (k_cc_make_diag<float, kVcycleBf16>), cgrid(L.g), block3(), 0, L.g, L.extra_f, L.bf_f[0], L.bf_f[1],
                    L.bf_f[2], H.nvar, masks, H.vdiag_f[0][l], H.vdiag_f[1][l], H.vdiag_f[2][l], H.vdinv_f[0][l],
@@ -3707,7 +3718,7 @@ ebv_status solve(Ctx *c, Problem &P, const double *b, double *x, int *iters, dou
 ebv_status cc_finish_hierarchy(Ctx *c, CcHier &H, bool fp32)
 {
     CcLevel &L0 = H.lv[0];
-    cc_make_diag<double>(c, H, 0);
+    cc_make_diag<double>(c, H, 0, !fp32);
     if (fp32) {
         // level 0 in FP32: the Krylov operator (the FP64 diagonal rounded),
         // then the V-cycle's BF16 faces and the diagonal formed from them
@@ -3731,7 +3742,7 @@ ebv_status cc_finish_hierarchy(Ctx *c, CcHier &H, bool fp32)
         } else {
             EBV_LAUNCH(c, k_cc_coarsen<double>, gr, block3(), 0, F.g, F.extra_d, F.bf_d[0], F.bf_d[1], F.bf_d[2],
                        F.cov, Cc.g, Cc.cov, Cc.extra_d, Cc.bf_d[0], Cc.bf_d[1], Cc.bf_d[2]);
-            cc_make_diag<double>(c, H, l + 1);
+            cc_make_diag<double>(c, H, l + 1, true);
         }
     }
     const int lb = H.L - 1;
@@ -3822,8 +3833,9 @@ ebv_status setup_solvers(Ctx *c)
             Lv.extra_f = dalloc<float>(nc, e);
             for (int q = 0; q < H->nvar; q++) {
                 H->vdiag_d[q][l] = dalloc<double>(nc, e);
-                H->vdiag_f[q][l] = dalloc<float>(nc, e);
-                H->vdinv_f[q][l] = dalloc<float>(nc, e);
+                const size_t np = (nc + 31) / 32 * 32;   // (keeps dinv_f 128-byte aligned)
+                H->vdiag_f[q][l] = dalloc<float>(2 * np, e);
+                H->vdinv_f[q][l] = H->vdiag_f[q][l] ? H->vdiag_f[q][l] + np : nullptr;
                 if (l == 0) H->vdiag_a[q] = dalloc<float>(nc, e);
             }
             for (int d = 0; d < 3; d++) {
