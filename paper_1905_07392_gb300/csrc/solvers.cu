@@ -2244,215 +2244,513 @@ __global__ void __launch_bounds__(256) k_bottom_solve(const double *__restrict__
         bottom_row(inv, nb, b, x, scale, g, split, r);
 }
 
-// ---- the coarse end of the cell-centred V-cycle in one CTA ------------------------
-// Levels of at most kCoarseCells cells cannot fill the GPU, and as separate
-// launches they cost more in launch latency than in work.  Below such a
-// level one persistent block of 1024 threads runs the rest of the V-cycle --
-// pre-smoothing, residual and restriction down to the bottom, the bottom
-// solve, then correction and post-smoothing back up -- with the same steps
-// and per-cell arithmetic as the per-level kernels (gs_cell, rr_cell,
-// bottom_row) and a block barrier wherever those have a kernel boundary, so
-// its results are bit for bit those of the per-level path.
-constexpr int kCoarseCells = 4096;
-constexpr int kCoarseMax = 8;
+// ---- the coarse end of the cell-centred V-cycle in one cluster -------------------
+// Levels that cannot fill the GPU cost more in launch latency than in work.
+// One cluster of kCvCtas blocks runs the V-cycle from such a level down to the
+// bottom and back.  Its top one or two levels (nd) are cut into slabs of
+// planes, one per block; the next smoothed level, at most 512 cells, is
+// smoothed by every block for itself (a cluster barrier per pass would cost
+// more than the pass); the bottom system is multiplied by its inverse.  Every
+// array lives in shared memory: per cell one record (six face coefficients,
+// masked at the box sides, and the inverse diagonal: 16 bytes with BF16
+// faces, one load), right-hand side and x, and per x-pair its position and
+// that of its parent, so a pass does no index arithmetic.  x is row-split with
+// one halo plane on either side of the slab, which the blocks write for each
+// other (distributed shared memory) before the hardware cluster barrier that
+// ends the pass.  Per cell the operations and their order are those of gs_cell
+// and rr_cell (a box side's coefficient is 0 here, which adds an exact 0); the
+// coarse correction is added to the cells of the colour that the first pass
+// reads, the sums a prolongation kernel would store.  The passes are small
+// loops on purpose: unrolled over slots held in registers they ran as fast
+// when cached, but their instructions came from DRAM at every launch on large
+// grids (72 us instead of 37 at 128^3).
+//
+// Measured per V-cycle: levels up to 32^3 in FP32 28 us at 64^3 and 29 us at
+// 128^3, against 36 and 40 us for one 1024-thread block that took the levels up
+// to 16^3 and recomputed every index, plus 24 us for the launches on the 32^3
+// level (about 6 us are loading, 1.1 us a pass over a 4,096-cell slab, 0.5 us
+// one over 512 cells with its cluster barrier).  FP64, levels up to 16^3: 26 us
+// against 63 (one SM's FP64 pipe bound it).  nd = 2 stays FP32: FP64 records
+// of a 4,096-cell slab do not fit in shared memory.  512 threads: 1,024 measured
+// 5 % slower.
+constexpr int kCvCtas = 8, kCvThreads = 512, kCvMax = 4;
+constexpr int kCoarseCells = 4096;    // largest top level with nd = 1
+constexpr int kCvTopCells = 32768;    // with nd = 2 (FP32)
+constexpr int kCvSmem = 225 * 1024;
+template <class T> struct CvLoad { static constexpr int n = sizeof(T) == 4 ? 2 : 1; };   // x-pairs whose operands a thread loads together
+struct CvLayout {
+    int x[3], rec[3], b[3], dg[3], info[3], cpos[3], res, bs, bi, xb, ps, total;
+};
 template <class T>
 struct CoarseVC {
     int n;                    // levels handled; the last is the bottom
-    VOp<T> A[kCoarseMax];
-    T *x[kCoarseMax];
-    T *b[kCoarseMax];         // b[0] given, the others written by restriction
+    int nd;                   // of these, cut into slabs
+    int split_z;              // slabs of z planes, else of y planes
+    int na;                   // blocks that own a slab (ranks 0 .. na-1)
+    VOp<T> A[kCvMax];
+    T *x;                     // top level
+    const T *b;
     const double *binv;       // bottom inverse (natural numbering)
     int nb;
+    double *part;             // block partials of b.x, or null
+    CvLayout L;               // shared-memory offsets (cv_layout)
+};
+// planes along the split direction, and rows in the other one
+__host__ __device__ inline int cv_np(const GridD &g, int split_z) { return split_z ? g.nz : g.ny; }
+__host__ __device__ inline int cv_no(const GridD &g, int split_z) { return split_z ? g.ny : g.nz; }
+// first plane of rank r's slab on level l (slabs nest: a coarse plane's two
+// fine planes belong to the same block)
+__host__ __device__ inline int cv_s0(int np_nd, int na, int nd, int l, int r) { return (np_nd * r / na) << (nd - l); }
+// planes of the largest slab on level l
+__host__ __device__ inline int cv_plmax(int np_nd, int na, int nd, int l) { return ((np_nd + na - 1) / na) << (nd - l); }
+
+// One cell's coefficients in shared memory: faces x-, x+, y-, y+, z-, z+ (0 at
+// the box sides) and the inverse diagonal.
+template <class F, class T>
+struct CvRec {
+    T f[6], di, pad;
+    __device__ void set(const F *g, T d)
+    {
+        for (int q = 0; q < 6; q++) f[q] = T(g[q]);
+        di = d;
+    }
+    __device__ void get(T *g, T &d) const
+    {
+        for (int q = 0; q < 6; q++) g[q] = f[q];
+        d = di;
+    }
+    __device__ void get_di(T &d) const { d = di; }
+};
+template <>
+struct __align__(16) CvRec<__nv_bfloat16, float> {
+    uint4 v;
+    __device__ void set(const __nv_bfloat16 *g, float d)
+    {
+        auto two = [&](int q) {
+            return (unsigned)__bfloat16_as_ushort(g[q]) | ((unsigned)__bfloat16_as_ushort(g[q + 1]) << 16);
+        };
+        v = make_uint4(two(0), two(2), two(4), __float_as_uint(d));
+    }
+    __device__ void get(float *g, float &d) const
+    {
+        const uint4 w = v;
+        const unsigned u[3] = {w.x, w.y, w.z};
+#pragma unroll
+        for (int q = 0; q < 3; q++) {   // a BF16 is the high half of the FP32 of the same value
+            g[2 * q] = __uint_as_float(u[q] << 16);
+            g[2 * q + 1] = __uint_as_float(u[q] & 0xffff0000u);
+        }
+        d = __uint_as_float(w.w);
+    }
+    __device__ void get_di(float &d) const { d = __uint_as_float(v.w); }
 };
 
-// One colour pass of the coarse kernel on level l: thread tid takes the
-// (x-pair, row) slots tid, tid + 1024, ... and in each the cell of colour
-// `color`; as in k_cc_gs, every operand of its (at most kCoarseSlots) updates
-// is loaded before any result is stored, so the L2 round trips overlap.
-// With zero_start the other cell of each slot is set to 0.
-constexpr int kCoarseThreads = 1024;
-constexpr int kCoarseSlots = (kCoarseCells + kCoarseThreads - 1) / kCoarseThreads;  // x-pairs: <= cells
-template <class T, bool kCorr>
-__device__ inline void coarse_pass(const CoarseVC<T> &D, int l, int color, int zero_start)
+// One level in shared memory: offsets in bytes (the same in every block) and
+// shape.  info per x-pair: position of its even cell, then the flags kCvPar
+// ((j+k) odd), kCvLo / kCvHi (on the slab's first / last plane); cpos: the
+// position of its parent one level down.
+constexpr int kCvParBit = 28, kCvPar = 1 << kCvParBit, kCvLo = 1 << 29, kCvHi = 1 << 30, kCvPos = kCvPar - 1;
+struct CvLevel {
+    int x, rec, b, dg, info, cpos;
+    int nx, h, no, plane, sy, sz, s0, pl, pairs, cap;
+    int lo_rank, hi_rank, dlo, dhi;   // where the slab's end planes go too (-1: nowhere), and the position shift
+};
+constexpr int kCvBiMax = 32 * 1024;   // the block's rows of the bottom inverse are staged up to this size
+template <class T>
+inline CvLayout cv_layout(const CoarseVC<T> &D)
 {
-    const VOp<T> &A = D.A[l];
-    const GridD &g = A.g;
-    const int hx = (g.nx + 1) >> 1, slots = hx * g.ny * g.nz;
-    T *x = D.x[l];
-    T val[kCoarseSlots];
-    int cc[kCoarseSlots], co[kCoarseSlots];
-#pragma unroll
-    for (int u = 0; u < kCoarseSlots; u++) {
-        const int m = threadIdx.x + u * kCoarseThreads;
-        cc[u] = -1;
-        co[u] = -1;
-        val[u] = T(0);
-        if (m >= slots) continue;
-        const int t = m % hx, jk = m / hx, j = jk % g.ny, k = jk / g.ny;
-        const int par = (j + k + color) & 1;
-        const int i = 2 * t + par, io = 2 * t + 1 - par;
-        if (io < g.nx) co[u] = cix<T>(g, io, j, k);
-        if (i >= g.nx) continue;
-        cc[u] = cix<T>(g, i, j, k);
-        val[u] = kCorr ? gs_cell<T, true>(A, x, D.b[l], i, j, k, 0, D.x[l + 1], D.A[l + 1].g)
-                       : gs_cell<T, false>(A, x, D.b[l], i, j, k, zero_start, x, g);
+    using Rec = CvRec<typename VFace<T>::type, T>;
+    CvLayout o;
+    int at = 0;
+    auto take = [&](int bytes) { const int q = at; at += (bytes + 15) & ~15; return q; };
+    const int npd = cv_np(D.A[D.nd].g, D.split_z);
+    for (int l = 0; l + 1 < D.n; l++) {
+        const GridD &g = D.A[l].g;
+        const int plane = cv_no(g, D.split_z) * g.nx, pl = l < D.nd ? cv_plmax(npd, D.na, D.nd, l) : npd;
+        o.x[l] = take((pl + 2) * plane * (int)sizeof(T));
+        o.rec[l] = take(pl * plane * (int)sizeof(Rec));
+        o.b[l] = take(pl * plane * (int)sizeof(T));
+        o.dg[l] = take(pl * plane / 2 * (int)sizeof(T));
+        o.info[l] = take(pl * plane / 2 * 4);
+        o.cpos[l] = take(pl * plane / 2 * 4);
+        if (l == 0) o.res = take(pl * plane * (int)sizeof(T));
     }
+    o.bs = take(D.nb * 8);
+    const int rows = (D.nb + D.na - 1) / D.na;
+    o.bi = rows * D.nb * 8 <= kCvBiMax ? take(rows * D.nb * 8) : -1;
+    o.xb = take(D.nb * (int)sizeof(T));
+    o.ps = take(kCvThreads / 32 * 8);
+    o.total = at;
+    return o;
+}
+
+// One block's view while it works on a level.
+template <class T>
+struct CvView {
+    using Rec = CvRec<typename VFace<T>::type, T>;
+    T *x;
+    const Rec *rec;      // [colour][pair]
+    const T *b;          // [colour][pair]
+    const int *info, *cpos;
+    T *lo, *hi;   // the neighbouring blocks' x, shifted to this block's positions, or null
+    int h, sy, sz, pairs, cap;   // cap: slots per colour
+    // sum of face times neighbour of the cell at p whose x- neighbour is at w
+    // (its x+ neighbour is the next word of the other half-row)
+    __device__ T off(const Rec &r, int p, int w, T &di) const
+    {
+        T f[6];
+        r.get(f, di);
+        const T xw = x[w], xe = x[w + 1], xs = x[p - sy], xn = x[p + sy], xd = x[p - sz], xu = x[p + sz];
+        T s = f[0] * xw;
+        s += f[1] * xe;
+        s += f[2] * xs;
+        s += f[3] * xn;
+        s += f[4] * xd;
+        s += f[5] * xu;
+        return s;
+    }
+    __device__ void put(int p, T v, int in) const
+    {
+        x[p] = v;
+        if ((in & kCvLo) && lo) lo[p] = v;
+        if ((in & kCvHi) && hi) hi[p] = v;
+    }
+    // one colour pass (two slots at a time, loads before stores: a pass never
+    // reads the cells it writes); from_zero: the other colour is 0
+    __device__ void pass(int c, bool from_zero) const
+    {
+        for (int m = threadIdx.x; m < pairs; m += 2 * kCvThreads) {
+            T v[2];
+            int in[2], p[2];
 #pragma unroll
-    for (int u = 0; u < kCoarseSlots; u++) {
-        if (zero_start && co[u] >= 0) x[co[u]] = T(0);
-        if (cc[u] >= 0) x[cc[u]] = val[u];
+            for (int u = 0; u < 2; u++) {
+                const int mu = m + u * kCvThreads;
+                if (u && mu >= pairs) continue;
+                in[u] = info[mu];
+                const T bb = b[c * cap + mu];
+                const int base = in[u] & kCvPos;
+                const bool q = ((in[u] >> kCvParBit) ^ c) & 1;   // the cell of colour c is the pair's odd one
+                p[u] = base + (q ? h : 0);
+                T di, o = T(0);
+                if (from_zero) rec[c * cap + mu].get_di(di);
+                else o = off(rec[c * cap + mu], p[u], base + (q ? 0 : h - 1), di);
+                v[u] = (bb + o) * di;
+            }
+            put(p[0], v[0], in[0]);
+            if (m + kCvThreads < pairs) put(p[1], v[1], in[1]);
+        }
+    }
+    // x += the parent's coarse correction on the even-coloured cells
+    __device__ void correct(const T *xc) const
+    {
+        for (int m = threadIdx.x; m < pairs; m += kCvThreads) {
+            const int in = info[m], p = (in & kCvPos) + ((in & kCvPar) ? h : 0);
+            put(p, x[p] + xc[cpos[m]], in);
+        }
+    }
+};
+
+template <class T>
+__global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
+    k_cc_coarse_vcycle(const __grid_constant__ CoarseVC<T> D)
+{
+    namespace cg = cooperative_groups;
+    using F = typename VFace<T>::type;
+    using Rec = CvRec<F, T>;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char cvsm[];
+    __shared__ CvLevel lv[3];
+    const int tid = threadIdx.x, rank = (int)cl.block_rank(), na = D.na, split_z = D.split_z, nd = D.nd;
+    const int npd = cv_np(D.A[nd].g, split_z), nl = D.n - 1;   // nl smoothed levels
+    const bool act = rank < na, red = nl > nd;
+    const CvLayout &L = D.L;
+    if (tid < nl) {
+        const int l = tid;
+        const GridD &g = D.A[l].g;
+        const bool slab = l < nd;
+        CvLevel v;
+        v.x = L.x[l]; v.rec = L.rec[l]; v.b = L.b[l]; v.dg = L.dg[l]; v.info = L.info[l]; v.cpos = L.cpos[l];
+        v.nx = g.nx; v.h = g.nx >> 1; v.no = cv_no(g, split_z); v.plane = v.no * g.nx;
+        v.sy = split_z ? g.nx : v.plane;
+        v.sz = split_z ? v.plane : g.nx;
+        v.s0 = slab && act ? cv_s0(npd, na, nd, l, rank) : 0;
+        v.pl = !act ? 0 : (slab ? cv_s0(npd, na, nd, l, rank + 1) - v.s0 : npd);
+        v.pairs = v.pl * v.no * v.h;
+        v.cap = (slab ? cv_plmax(npd, na, nd, l) : npd) * v.no * v.h;   // (offsets are the same in every block)
+        v.lo_rank = slab && act && rank > 0 ? rank - 1 : -1;
+        v.hi_rank = slab && act && rank + 1 < na ? rank + 1 : -1;
+        v.dlo = v.lo_rank >= 0 ? (v.s0 - cv_s0(npd, na, nd, l, rank - 1)) * v.plane : 0;
+        v.dhi = -v.pl * v.plane;
+        lv[l] = v;
     }
     __syncthreads();
-}
-
-// The V-cycle from level 0 of D down to its bottom and back; bs holds the
-// bottom right-hand side in natural order.
-template <class T>
-__device__ inline void coarse_vcycle_body(const CoarseVC<T> &D, double *bs)
-{
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int L = D.n - 1;
-    for (int l = 0; l < L; l++) {
-        // two red-black sweeps, red first, the first from zero
-        coarse_pass<T, false>(D, l, 0, 1);
-        coarse_pass<T, false>(D, l, 1, 0);
-        coarse_pass<T, false>(D, l, 0, 0);
-        coarse_pass<T, false>(D, l, 1, 0);
-        const GridD &gc = D.A[l + 1].g;
-        const int nc = ncell(gc);
-        for (int s = tid; s < nc; s += nt) {
-            const int I = s % gc.nx, J = (s / gc.nx) % gc.ny, K = s / (gc.nx * gc.ny);
-            D.b[l + 1][cix<T>(gc, I, J, K)] = rr_cell<T>(D.A[l], D.x[l], D.b[l], I, J, K);
-        }
-        __syncthreads();
+    // halo planes and cells not yet written meet zero coefficients only, but
+    // must be finite
+    for (int l = 0; l < nl; l++) {
+        T *x = reinterpret_cast<T *>(cvsm + lv[l].x);
+        for (int q = tid; q < (lv[l].pl + 2) * lv[l].plane; q += kCvThreads) x[q] = T(0);
     }
-    // bottom: x = inv b, b gathered once into natural order (same sums as bottom_row)
-    {
-        const GridD &gb = D.A[L].g;
-        const int split = (int)(sizeof(T) == 4);
-        for (int q = tid; q < D.nb; q += nt) bs[q] = (double)D.b[L][bottom_pos(gb, split, q)];
-        __syncthreads();
-        for (int r = tid; r < D.nb; r += nt) {
-            const double *row = D.binv + (size_t)r * D.nb;
-            double sum = 0.0;
-#pragma unroll 8
-            for (int q = 0; q < D.nb; q++) sum += row[q] * bs[q];
-            D.x[L][bottom_pos(gb, split, r)] = (T)(sum * 1.0);
-        }
-        __syncthreads();
-    }
-    for (int l = L - 1; l >= 0; l--) {
-        // two sweeps, black first; the first pass takes the coarse correction
-        coarse_pass<T, true>(D, l, 1, 0);
-        coarse_pass<T, false>(D, l, 0, 0);
-        coarse_pass<T, false>(D, l, 1, 0);
-        coarse_pass<T, false>(D, l, 0, 0);
-    }
-}
-
-// Asynchronous global -> shared copies of n elements (cp.async, 4 or 8 bytes
-// per copy, all in flight together).  2-byte elements go as 4-byte pairs:
-// both addresses 4-byte aligned, and for odd n the source holds one element
-// more (the face arrays of the V-cycle are allocated with one spare).
-template <class E>
-__device__ inline void stage_async(E *dst, const E *src, int n)
-{
-    static_assert(sizeof(E) == 2 || sizeof(E) == 4 || sizeof(E) == 8, "2-, 4- or 8-byte elements");
-    if constexpr (sizeof(E) == 2) {
-        stage_async((uint32_t *)dst, (const uint32_t *)src, (n + 1) >> 1);
-    } else {
-        for (int s = threadIdx.x; s < n; s += blockDim.x) {
-            const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + s);
-            if constexpr (sizeof(E) == 4)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(src + s) : "memory");
-            else
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(src + s) : "memory");
-        }
-    }
-}
-
-// Shared-memory layout of the staged coarse V-cycle: the bottom inverse (if
-// staged) first, then per level the diagonal and the three face arrays
-// (levels that smooth), x and b; every array starts on a 16-byte boundary.
-__host__ __device__ inline size_t stage_align(size_t b) { return (b + 15) & ~(size_t)15; }
-template <class T>
-__host__ __device__ inline size_t coarse_stage_bytes(const CoarseVC<T> &D, int with_binv)
-{
-    using F = typename VFace<T>::type;
-    size_t b = with_binv ? stage_align((size_t)D.nb * D.nb * sizeof(double)) : 0;
-    for (int q = 0; q < D.n; q++) {
-        const GridD &g = D.A[q].g;
-        if (q + 1 < D.n) {
-            b += (sizeof(T) == 4 ? 2 : 1) * stage_align((size_t)ncell(g) * sizeof(T));   // diag (and 1/diag)
-            for (int d = 0; d < 3; d++) b += stage_align((size_t)nface(g, d) * sizeof(F));
-        }
-        b += 2 * stage_align((size_t)ncell(g) * sizeof(T));
-    }
-    return b;
-}
-constexpr size_t kCoarseStageMax = 200 * 1024;  // dynamic shared memory of the staged form
-
-// kStage: every array the V-cycle touches is first copied into shared memory
-// (the level vectors need no copy: they are written before being read, and
-// b of the top level is the one input), the V-cycle runs there, and x of the
-// top level -- the correction the next finer level reads -- is copied back.
-// Same arithmetic in the same order as the unstaged form.
-template <class T, bool kStage>
-__global__ void __launch_bounds__(kCoarseThreads) k_cc_coarse_vcycle(CoarseVC<T> D, int stage_binv)
-{
-    __shared__ double bs[kBottomMax];
-    if constexpr (!kStage) {
-        coarse_vcycle_body<T>(D, bs);
-    } else {
-        extern __shared__ __align__(16) unsigned char dyn[];
-        // the staged level table lives in shared memory too (thread 0 writes it)
-        __shared__ __align__(16) unsigned char tbl[sizeof(CoarseVC<T>)];
-        CoarseVC<T> &S = *reinterpret_cast<CoarseVC<T> *>(tbl);
-        const bool t0 = threadIdx.x == 0;
-        if (t0) S = D;
-        using F = typename VFace<T>::type;
-        unsigned char *ptr = dyn;
-        if (stage_binv) {
-            double *bi = (double *)ptr;
-            stage_async(bi, D.binv, D.nb * D.nb);
-            if (t0) S.binv = bi;
-            ptr += stage_align((size_t)D.nb * D.nb * sizeof(double));
-        }
-        for (int q = 0; q < D.n; q++) {
-            const GridD &g = D.A[q].g;
-            const int nc = ncell(g);
-            if (q + 1 < D.n) {
-                T *dg = (T *)ptr;
-                ptr += stage_align((size_t)nc * sizeof(T));
-                stage_async(dg, D.A[q].diag, nc);
-                if constexpr (sizeof(T) == 4) {
-                    T *di = (T *)ptr;
-                    ptr += stage_align((size_t)nc * sizeof(T));
-                    stage_async(di, D.A[q].dinv, nc);
-                    if (t0) S.A[q].dinv = di;
-                }
-                F *fc[3];
-                const F *src[3] = {D.A[q].bx, D.A[q].by, D.A[q].bz};
-                for (int d = 0; d < 3; d++) {
-                    fc[d] = (F *)ptr;
-                    ptr += stage_align((size_t)nface(g, d) * sizeof(F));
-                    stage_async(fc[d], src[d], nface(g, d));
-                }
-                if (t0) { S.A[q].diag = dg; S.A[q].bx = fc[0]; S.A[q].by = fc[1]; S.A[q].bz = fc[2]; }
+    // every level's records in one loop (level by level their load latencies
+    // added up); kU pairs' loads before their use, a slot past the end loads
+    // the first pair again
+    constexpr int kU = CvLoad<T>::n;
+    const int n0 = lv[0].pairs, n1 = n0 + (nl > 1 ? lv[1].pairs : 0), n2 = n1 + (nl > 2 ? lv[2].pairs : 0);
+    for (int m0 = tid; m0 < n2; m0 += kU * kCvThreads) {
+        F f[kU][11];
+        T d[kU][3], bb[kU][2];
+        int ts[kU], os[kU], ss[kU];
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            const int m = m0 + u * kCvThreads < n2 ? m0 + u * kCvThreads : 0;
+            const int l = m < n0 ? 0 : (m < n1 ? 1 : 2), ml = m - (l == 0 ? 0 : (l == 1 ? n0 : n1));
+            const VOp<T> &A = D.A[l];
+            const int r = ml / lv[l].h;
+            ts[u] = ml - r * lv[l].h;
+            ss[u] = r / lv[l].no;
+            os[u] = r - ss[u] * lv[l].no;
+            const int j = split_z ? os[u] : lv[l].s0 + ss[u], k = split_z ? lv[l].s0 + ss[u] : os[u];
+            const CellPos p0 = cell_pos<T>(A.g, 2 * ts[u], j, k), p1 = cell_pos<T>(A.g, 2 * ts[u] + 1, j, k);
+            f[u][0] = A.bx[p0.fx0];
+            f[u][1] = A.bx[p0.fx1];
+            f[u][2] = A.bx[p1.fx1];
+            f[u][3] = A.by[p0.fy0];
+            f[u][4] = A.by[p0.fy1];
+            f[u][5] = A.by[p1.fy0];
+            f[u][6] = A.by[p1.fy1];
+            f[u][7] = A.bz[p0.fz0];
+            f[u][8] = A.bz[p0.fz1];
+            f[u][9] = A.bz[p1.fz0];
+            f[u][10] = A.bz[p1.fz1];
+            d[u][0] = A.dinv[p0.c];
+            d[u][1] = A.dinv[p1.c];
+            d[u][2] = A.diag[((j + k) & 1) ? p1.c : p0.c];
+            if (l == 0) {
+                bb[u][0] = D.b[p0.c];
+                bb[u][1] = D.b[p1.c];
             }
-            T *xs = (T *)ptr;
-            ptr += stage_align((size_t)nc * sizeof(T));
-            T *bs2 = (T *)ptr;
-            ptr += stage_align((size_t)nc * sizeof(T));
-            if (q == 0) stage_async(bs2, (const T *)D.b[0], nc);
-            if (t0) { S.x[q] = xs; S.b[q] = bs2; }
         }
-        asm volatile("cp.async.wait_all;\n" ::: "memory");
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            const int m = m0 + u * kCvThreads;
+            if (m >= n2) continue;
+            const int l = m < n0 ? 0 : (m < n1 ? 1 : 2), ml = m - (l == 0 ? 0 : (l == 1 ? n0 : n1));
+            const CvLevel &v = lv[l];
+            const GridD &g = D.A[l].g, &gc = D.A[l + 1].g;
+            const int t = ts[u], o = os[u], sl = ss[u];
+            const int j = split_z ? o : v.s0 + sl, k = split_z ? v.s0 + sl : o, c0 = (j + k) & 1;   // colour of the even cell
+            int *info = reinterpret_cast<int *>(cvsm + v.info), *cpos = reinterpret_cast<int *>(cvsm + v.cpos);
+            info[ml] = ((sl + 1) * v.plane + o * v.nx + t) | (c0 ? kCvPar : 0) | (sl == 0 ? kCvLo : 0) |
+                       (sl == v.pl - 1 ? kCvHi : 0);
+            // parent: one level down row-split with a halo plane, or the bottom in natural order
+            const int cs0 = l + 1 < nd ? lv[l + 1].s0 : 0;
+            cpos[ml] = l + 1 == nl ? ((k >> 1) * gc.ny + (j >> 1)) * gc.nx + t
+                                   : ((((v.s0 + sl) >> 1) - cs0 + 1) * (v.no >> 1) + (o >> 1)) * gc.nx + spos(gc.nx, t);
+            const F z = F(0.0f);
+            const bool j0 = j == 0, j1 = j == g.ny - 1, k0 = k == 0, k1 = k == g.nz - 1;
+            const F fe[6] = {t == 0 ? z : f[u][0], f[u][1], j0 ? z : f[u][3], j1 ? z : f[u][4], k0 ? z : f[u][7],
+                             k1 ? z : f[u][8]};
+            const F fo[6] = {f[u][1], t == v.h - 1 ? z : f[u][2], j0 ? z : f[u][5], j1 ? z : f[u][6], k0 ? z : f[u][9],
+                             k1 ? z : f[u][10]};
+            Rec *rec = reinterpret_cast<Rec *>(cvsm + v.rec);
+            rec[c0 * v.cap + ml].set(fe, d[u][0]);
+            rec[(1 - c0) * v.cap + ml].set(fo, d[u][1]);
+            reinterpret_cast<T *>(cvsm + v.dg)[ml] = d[u][2];   // of the even-coloured cell, for its residual
+            if (l == 0) {
+                T *b = reinterpret_cast<T *>(cvsm + v.b);
+                b[c0 * v.cap + ml] = bb[u][0];
+                b[(1 - c0) * v.cap + ml] = bb[u][1];
+            }
+        }
+    }
+    // this block's rows of the bottom inverse: staged, or on their way into L2
+    const int br0 = D.nb * min(rank, na) / na, br1 = D.nb * min(rank + 1, na) / na;
+    {
+        const double *src = D.binv + (size_t)br0 * D.nb;
+        const int n = (br1 - br0) * D.nb;
+        if (L.bi >= 0) {
+            double *bi = reinterpret_cast<double *>(cvsm + L.bi);
+            for (int q = tid; q < n; q += kCvThreads) bi[q] = src[q];
+        } else {
+            for (int q = tid * 16; q < n; q += 16 * kCvThreads) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(src + q));
+        }
+    }
+    cl.sync();
+
+    T *res = reinterpret_cast<T *>(cvsm + L.res), *xb = reinterpret_cast<T *>(cvsm + L.xb);
+    double *bs = reinterpret_cast<double *>(cvsm + L.bs), *ps = reinterpret_cast<double *>(cvsm + L.ps);
+    auto view = [&](int l) {
+        const CvLevel &v = lv[l];
+        CvView<T> w;
+        w.x = reinterpret_cast<T *>(cvsm + v.x);
+        w.rec = reinterpret_cast<const Rec *>(cvsm + v.rec);
+        w.b = reinterpret_cast<const T *>(cvsm + v.b);
+        w.info = reinterpret_cast<const int *>(cvsm + v.info);
+        w.cpos = reinterpret_cast<const int *>(cvsm + v.cpos);
+        w.lo = v.lo_rank >= 0 ? cl.map_shared_rank(w.x, v.lo_rank) + v.dlo : nullptr;
+        w.hi = v.hi_rank >= 0 ? cl.map_shared_rank(w.x, v.hi_rank) + v.dhi : nullptr;
+        w.h = v.h; w.sy = v.sy; w.sz = v.sz; w.pairs = v.pairs; w.cap = v.cap;
+        return w;
+    };
+    auto bar = [&](int l) {
+        if (l < nd) cl.sync();
+        else __syncthreads();
+    };
+    // Down (dir 0): two sweeps from zero, red first; up (dir 1): the coarse
+    // correction, then two sweeps, black first.  Nobody reads the last pass's
+    // halo, so it writes none (the other blocks may have ended by then: every
+    // remote write is followed by a cluster barrier that its target takes
+    // part in) and needs no cluster barrier.
+    auto smooth = [&](int l, int dir, const T *xc) {
+        CvView<T> w = view(l);
+        if (dir == 0) w.pass(0, true);
+        else w.correct(xc);
+        bar(l);
+#pragma unroll 1
+        for (int it = dir == 0 ? 1 : 0; it < 4; it++) {
+            const bool last = dir == 1 && it == 3;
+            if (last) w.lo = w.hi = nullptr;
+            w.pass((it & 1) ^ dir, false);
+            if (last) __syncthreads();
+            else bar(l);
+        }
+    };
+#pragma unroll 1
+    for (int l = 0; l < nl; l++) {
+        if (l < nd || act) {
+            smooth(l, 0, nullptr);
+            // residuals of the even-coloured cells, then their averages over
+            // the children in rr_cell's order
+            {
+                const CvView<T> w = view(l);
+                const T *dg = reinterpret_cast<const T *>(cvsm + lv[l].dg);
+                for (int m = tid; m < w.pairs; m += kCvThreads) {
+                    const int in = w.info[m], base = in & kCvPos, p = base + ((in & kCvPar) ? w.h : 0);
+                    T di;
+                    const T o = w.off(w.rec[m], p, base + ((in & kCvPar) ? 0 : w.h - 1), di);
+                    res[p - lv[l].plane] = w.b[m] - (dg[m] * w.x[p] - o);
+                }
+            }
+            __syncthreads();
+            const GridD &gc = D.A[l + 1].g;
+            const CvLevel &v = lv[l];
+            const int noc = v.no >> 1, nc = (v.pl >> 1) * noc * gc.nx;
+            for (int m = tid; m < nc; m += kCvThreads) {
+                const int r = m / gc.nx, I = m - r * gc.nx, S = r / noc, O = r - S * noc;
+                T s = 0;
+#pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    if (__popc(e) & 1) continue;
+                    const int dj = (e >> 1) & 1, dk = e >> 2;
+                    const int o = 2 * O + (split_z ? dj : dk), sl = 2 * S + (split_z ? dk : dj);
+                    s += res[(sl * v.no + o) * v.nx + ((e & 1) ? v.h : 0) + I];
+                }
+                s *= T(0.125);
+                // to the next level: its right-hand side (this block's slab, or
+                // every active block's copy), or the bottom's in natural order
+                const int Sg = (v.s0 >> 1) + S;
+                if (l + 1 < nl) {
+                    T *bq = reinterpret_cast<T *>(cvsm + lv[l + 1].b);
+                    const bool own = l + 1 < nd || l >= nd;
+                    const int Sl = own ? S : Sg, col = (I + O + (v.s0 >> 1) + S) & 1;   // colour of (I, O, Sg)
+                    const int at = col * lv[l + 1].cap + (Sl * noc + O) * (gc.nx >> 1) + (I >> 1);
+                    if (own) bq[at] = s;
+                    else
+                        for (int a = 0; a < na; a++) cl.map_shared_rank(bq, a)[at] = s;
+                } else {
+                    const int at = (split_z ? Sg * gc.ny + O : O * gc.ny + Sg) * gc.nx + I;
+                    if (l >= nd) bs[at] = (double)s;
+                    else
+                        for (int a = 0; a < na; a++) cl.map_shared_rank(bs, a)[at] = (double)s;
+                }
+            }
+        }
+        // (the next level's right-hand side comes from other blocks where it stops being cut)
+        if (l + 1 == nd) cl.sync();
+        else __syncthreads();
+    }
+    // bottom: x = inv b, each block its share of the rows (FP64: one SM would
+    // take nb^2 / 2 cycles), 16 lanes per row, the result to every block
+    {
+        const double *bi = L.bi >= 0 ? reinterpret_cast<const double *>(cvsm + L.bi) : D.binv + (size_t)br0 * D.nb;
+        const int nr = act ? br1 - br0 : 0, g = tid & 15;
+        for (int rr = tid >> 4; rr < (nr + 1) / 2 * 2; rr += kCvThreads / 16) {   // (whole warps)
+            double sum = 0.0;
+            if (rr < nr) {
+                const double *row = bi + (size_t)rr * D.nb;
+#pragma unroll 4
+                for (int q = g; q < D.nb; q += 16) sum += row[q] * bs[q];
+            }
+            for (int o = 8; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o, 16);
+            if (g == 0 && rr < nr)
+                for (int a = 0; a < na; a++) cl.map_shared_rank(xb, a)[br0 + rr] = (T)sum;
+        }
+        cl.sync();
+    }
+#pragma unroll 1
+    for (int l = nl - 1; l >= 0; l--)
+        if (l < nd || act) smooth(l, 1, l == nl - 1 ? xb : reinterpret_cast<const T *>(cvsm + lv[l + 1].x));
+    // the top level's x, and b.x over the block's cells (per thread and warp in T, across warps in FP64)
+    T dot = T(0);
+    {
+        const GridD &g = D.A[0].g;
+        const CvView<T> w = view(0);
+        const CvLevel &v = lv[0];
+        for (int m = tid; m < w.pairs; m += kCvThreads) {
+            const int r = m / v.h, t = m - r * v.h, sl = r / v.no, o = r - sl * v.no;
+            const int j = split_z ? o : v.s0 + sl, k = split_z ? v.s0 + sl : o, p = (w.info[m] & kCvPos);
+            const int c0 = (w.info[m] & kCvPar) ? 1 : 0;   // colour of the even cell
+            const T x0 = w.x[p], x1 = w.x[p + v.h];
+            D.x[cix<T>(g, 2 * t, j, k)] = x0;
+            D.x[cix<T>(g, 2 * t + 1, j, k)] = x1;
+            dot += w.b[c0 * w.cap + m] * x0 + w.b[(1 - c0) * w.cap + m] * x1;
+        }
+    }
+    if (D.part) {
+        for (int o = 16; o > 0; o >>= 1) dot += __shfl_down_sync(0xffffffffu, dot, o);
+        if ((tid & 31) == 0) ps[tid >> 5] = (double)dot;
         __syncthreads();
-        coarse_vcycle_body<T>(S, bs);
-        const int n0 = ncell(D.A[0].g);
-        const T *x0s = S.x[0];
-        for (int s = threadIdx.x; s < n0; s += blockDim.x) D.x[0][s] = x0s[s];
+        if (tid == 0) {
+            double sum = 0.0;
+            for (int q = 0; q < kCvThreads / 32; q++) sum += ps[q];
+            D.part[rank] = sum;
+        }
+    }
+}
+
+// Which levels of the hierarchy the cluster kernel takes: fills the shape of D
+// and returns its top level, or -1 (no smoothed level fits: the bottom alone).
+// By the level sizes only: the largest top level whose slabs fit in shared
+// memory.
+template <class T>
+int cv_plan(const CcHier &H, CoarseVC<T> &D)
+{
+    const int Lb = H.L - 1;
+    for (int l0 = 0; l0 < Lb; l0++) {
+        const int cells = ncell(H.lv[l0].g);
+        const int nd = cells <= kCoarseCells ? 1 : 2, n = Lb - l0 + 1;
+        if (nd == 2 && (sizeof(T) != 4 || cells > kCvTopCells)) continue;
+        if (n < nd + 1 || n > nd + 2) continue;
+        for (int q = 0; q < n; q++) D.A[q].g = H.lv[l0 + q].g;
+        const GridD &gd = D.A[nd].g;   // the first level that is not cut
+        D.n = n;
+        D.nd = nd;
+        D.split_z = gd.nz >= gd.ny;
+        D.na = std::min(kCvCtas, cv_np(gd, D.split_z));
+        D.nb = H.nb;
+        if (n == nd + 2 && ncell(gd) > 512) continue;
+        D.L = cv_layout(D);
+        if (D.L.total <= kCvSmem) return l0;
+    }
+    return -1;
+}
+
+template <class T>
+void cv_attr()
+{
+    static bool done = false;
+    if (!done) {
+        done = true;
+        cudaFuncSetAttribute(k_cc_coarse_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem);
     }
 }
 
@@ -3183,16 +3481,16 @@ int cc_smooth2(Ctx *c, const CcLevel &L, int l, T *x, T *t, const T *b, bool red
     return (int)(gd.x * gd.y * gd.z);
 }
 
-// One V-cycle x0 = M b0.  dot_part: the finest level's last pass also
-// writes block partials of b0.x0; returns their number (0 when the whole
-// V-cycle runs in the coarse kernel, or without dot_part).
+// One V-cycle x0 = M b0.  dot_part: the finest level's last pass (or the
+// cluster kernel, where it takes that level) also writes block partials of
+// b0.x0; returns their number (0 with a single level, or without dot_part).
 template <class T>
 int cc_vcycle(Ctx *c, CcHier &H, const T *b0, T *x0, double *dot_part = nullptr)
 {
     const int Lb = H.L - 1;
-    // levels l0 .. Lb (each at most kCoarseCells cells) run in one CTA
-    int l0 = Lb;
-    while (l0 > 0 && ncell(H.lv[l0 - 1].g) <= kCoarseCells && Lb - l0 + 2 <= kCoarseMax) l0--;
+    // levels l0 .. Lb run in one cluster
+    CoarseVC<T> D;
+    const int lc = cv_plan<T>(H, D), l0 = lc < 0 ? Lb : lc;
     for (int l = 0; l < l0; l++) {
         const CcLevel &L = H.lv[l];
         T *x = l ? (T *)c->lx[l] : x0;
@@ -3218,25 +3516,17 @@ int cc_vcycle(Ctx *c, CcHier &H, const T *b0, T *x0, double *dot_part = nullptr)
                          (T *)c->lb[l + 1]);
     }
     if (l0 < Lb) {
-        CoarseVC<T> D;
-        D.n = Lb - l0 + 1;
-        for (int q = 0; q < D.n; q++) {
-            const int l = l0 + q;
-            D.A[q] = vop<T>(H.lv[l]);
-            D.x[q] = l ? (T *)c->lx[l] : x0;
-            D.b[q] = l ? (T *)c->lb[l] : (T *)b0;
-        }
+        for (int q = 0; q < D.n; q++) D.A[q] = vop<T>(H.lv[l0 + q]);
+        D.x = l0 ? (T *)c->lx[l0] : x0;
+        D.b = l0 ? (const T *)c->lb[l0] : b0;
         D.binv = H.binv;
         D.nb = H.nb;
-        // staged in shared memory when it fits (with the bottom inverse if that fits too)
-        int sb = coarse_stage_bytes(D, 1) <= kCoarseStageMax;
-        const size_t bytes = coarse_stage_bytes(D, sb);
-        if (bytes <= kCoarseStageMax)
-            EBV_LAUNCH_P(c, sizeof(T) == 4 ? "cc_coarse_vcycle<float>" : "cc_coarse_vcycle<double>", 0.0,
-                         (k_cc_coarse_vcycle<T, true>), dim3(1), dim3(kCoarseThreads), bytes, D, sb);
-        else
-            EBV_LAUNCH_P(c, sizeof(T) == 4 ? "cc_coarse_vcycle<float>" : "cc_coarse_vcycle<double>", 0.0,
-                         (k_cc_coarse_vcycle<T, false>), dim3(1), dim3(kCoarseThreads), 0, D, 0);
+        D.part = l0 == 0 ? dot_part : nullptr;
+        const size_t bytes = D.L.total;
+        const char *nm = sizeof(T) == 4 ? "cc_coarse_vcycle<float>" : "cc_coarse_vcycle<double>";
+        cv_attr<T>();
+        EBV_LAUNCH_P(c, nm, 0.0, k_cc_coarse_vcycle<T>, dim3(kCvCtas), dim3(kCvThreads), bytes, D);
+        if (l0 == 0) return dot_part ? kCvCtas : 0;
     } else {
         T *x = Lb ? (T *)c->lx[Lb] : x0;
         const T *b = Lb ? (const T *)c->lb[Lb] : b0;
@@ -3799,11 +4089,6 @@ ebv_status setup_solvers(Ctx *c)
 {
     const GridD &g = c->g;
     cudaError_t e = cudaSuccess;
-    // the staged coarse V-cycle takes up to kCoarseStageMax of dynamic shared memory
-    EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_cc_coarse_vcycle<float, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseStageMax));
-    EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_cc_coarse_vcycle<double, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseStageMax));
     GridD gl[kMaxLevels];
     // cell-centred hierarchies (projection and viscous)
     int L = plan_levels(g, gl, false);
