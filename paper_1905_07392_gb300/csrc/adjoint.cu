@@ -909,8 +909,10 @@ __global__ void k_mask_scale(int N3, int ncomp, const uint8_t *__restrict__ flag
 }
 
 // a = alpha lam on fluid cells (the adjoint of alpha psi)
+// (a may be lam)
 __global__ void k_alpha_times(int N3, const uint8_t *__restrict__ flag, const double *__restrict__ alpha,
-                              const double *__restrict__ lam, double *__restrict__ a)
+                              const double *lam, double *a)
+
 {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N3; c += gridDim.x * blockDim.x)
         a[c] = flag[c] ? alpha[c] * lam[c] : 0.0;

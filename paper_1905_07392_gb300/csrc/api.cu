@@ -167,13 +167,11 @@ ebv_status viscous_update(Ctx *c, const double *eta, const double *psi, double *
     EBV_LAUNCH(c, k_init_guess, dim3(kReduceBlocks), dim3(256), 0, N3, c->flag, psi, c->prm.rho, 1.0 / c->prm.rho,
                pow2 ? 1 : 0, ut);
     TRY(visc_build(c, eta));
-    for (int q = 0; q < 3; q++) {
-        int it = 0;
-        double res = 0.0;
-        c->cur_slot = slot + q;
-        TRY(visc_solve(c, psi + (size_t)q * N3, q, ut + (size_t)q * N3, &it, &res));
-        if (st) { st->iters[slot + q] = it; st->res[slot + q] = res; }
-    }
+    int it[3] = {0, 0, 0};
+    double res[3] = {0.0, 0.0, 0.0};
+    c->cur_slot = slot;
+    TRY(visc_solve(c, psi, ut, it, res));
+    for (int q = 0; q < 3 && st; q++) { st->iters[slot + q] = it[q]; st->res[slot + q] = res[q]; }
     return EBV_OK;
 }
 
@@ -561,10 +559,10 @@ ebv_status ebv_create(const ebv_grid *grid, const ebv_params *params, void *stre
     ok &= alloc(&c->kr, V, as) && alloc(&c->kz, V, as) && alloc(&c->kp, V, as) && alloc(&c->kq, V, as);
     ok &= alloc(&c->kr32, V, as) && alloc(&c->kz32, V, as) && alloc(&c->kp32, V, as) && alloc(&c->kq32, V, as) &&
           alloc(&c->ke32, V, as);
-    ok &= alloc(&c->part, (size_t)1 << 20, as) && alloc(&c->scal, 32, as);
+    ok &= alloc(&c->part, (size_t)1 << 20, as) && alloc(&c->scal, 3 * 32, as);
     ok &= cudaMallocHost(&c->scal_host, 32 * sizeof(double)) == cudaSuccess;
-    ok &= alloc(&c->ctl, C_LEN, as) && alloc(&c->sstat, kSstatLen, as);
-    ok &= cudaMallocHost(&c->ctl_host, C_LEN * sizeof(int)) == cudaSuccess;
+    ok &= alloc(&c->ctl, 4 * C_LEN, as) && alloc(&c->sstat, kSstatLen, as);
+    ok &= cudaMallocHost(&c->ctl_host, 4 * C_LEN * sizeof(int)) == cudaSuccess;
     ok &= cudaMallocHost(&c->sstat_host, kSstatLen * sizeof(double)) == cudaSuccess;
     c->vec_len = V;
     if (!ok) {
@@ -577,8 +575,8 @@ ebv_status ebv_create(const ebv_grid *grid, const ebv_params *params, void *stre
         cudaGetLastError();
         return st == EBV_ERR_OOM ? EBV_ERR_OOM : EBV_ERR_INVALID;
     }
-    cudaMemsetAsync(c->scal, 0, 32 * sizeof(double), c->stream);
-    cudaMemsetAsync(c->ctl, 0, C_LEN * sizeof(int), c->stream);
+    cudaMemsetAsync(c->scal, 0, 3 * 32 * sizeof(double), c->stream);
+    cudaMemsetAsync(c->ctl, 0, 4 * C_LEN * sizeof(int), c->stream);
     cudaMemsetAsync(c->sstat, 0, kSstatLen * sizeof(double), c->stream);
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) {
         ebv_destroy(c);
@@ -1057,13 +1055,12 @@ ebv_status visc_adjoint(Ctx *c, AdjBufs &B, const double *eta, const double *x, 
 {
     const size_t N3 = ncell(c->g);
     TRY(visc_build(c, eta));
+    // (slots 13..15: a joint solve takes three)
+    c->cur_slot = 13;
+    TRY(visc_solve_rhs(c, xb, psib, nullptr, nullptr));   // psib holds the lambdas
     for (int q = 0; q < 3; q++) {
-        int it = 0;
-        double res = 0.0;
-        c->cur_slot = 12;
-        TRY(visc_solve_rhs(c, q, xb + q * N3, B.lam, &it, &res));
-        TRY(adj_alpha_times(c, B.lam, psib + q * N3));
-        TRY(adj_visc_eta(c, q, B.lam, x + q * N3, etab));
+        TRY(adj_visc_eta(c, q, psib + q * N3, x + q * N3, etab));
+        TRY(adj_alpha_times(c, psib + q * N3, psib + q * N3));
     }
     return EBV_OK;
 }
@@ -1090,7 +1087,7 @@ ebv_status adjoint_step_impl(Ctx *c, const double *u, const double *p, double dt
         TRY(launch_mac_rhs(c, uF, c->rhs_c));
         int it = 0;
         double res = 0.0;
-        c->cur_slot = 10;   // the reverse pass's solves use slots 10..13
+        c->cur_slot = 10;   // the reverse pass's solves use slots 10..15
         TRY(mac_solve(c, c->rhs_c, c->phi, &it, &res));
         TRY(launch_mac_correct(c, uF, c->phi));
         TRY(launch_convective(c, w, uF, C));

@@ -308,6 +308,12 @@ struct Ctx {
     double *scal = nullptr;      // device scalars
     double *scal_host = nullptr; // pinned mirror
     size_t vec_len = 0;
+    // vectors of velocity components 1 and 2 in a joint viscous solve, carved
+    // from scratch (carve_components): level corrections, right-hand sides and
+    // sweep targets by level, Krylov vectors by number
+    enum { CV_X, CV_B, CV_T, CV_K, CV_KINDS };
+    void *cvec[2][CV_KINDS][kMaxLevels] = {};
+    bool joint = false;
 
     // Solver loop control lives on the device: the convergence tests run in
     // one-thread kernels that write a condition word (read back by the host
@@ -481,12 +487,13 @@ ebv_status mac_solve(Ctx *c, const double *b, double *x, int *iters, double *res
 // operators A_q(eta) of the three viscous solves (q = velocity component):
 // shared coefficients, per-component diagonals and bottom inverses
 ebv_status visc_build(Ctx *c, const double *eta);
-// A_q x = alpha psi_q + boundary terms, after visc_build
-ebv_status visc_solve(Ctx *c, const double *psi_comp, int comp, double *x, int *iters, double *res);
+// A_q x_q = alpha psi_q + boundary terms, q = 0..2, after visc_build (psi, x:
+// 3 x cells; iters, res: 3 entries)
+ebv_status visc_solve(Ctx *c, const double *psi, double *x, int *iters, double *res);
 ebv_status nodal_solve(Ctx *c, const double *b, double *x, int *iters, double *res);
-// A_q x = rhs (the viscous operator with the given right-hand side instead of
-// alpha psi + boundary terms), from x = 0, after visc_build
-ebv_status visc_solve_rhs(Ctx *c, int comp, const double *rhs, double *x, int *iters, double *res);
+// A_q x_q = rhs_q (the given right-hand sides instead of alpha psi + boundary
+// terms), from x = 0, after visc_build
+ebv_status visc_solve_rhs(Ctx *c, const double *rhs, double *x, int *iters, double *res);
 // reductions (solvers.cu)
 ebv_status reduce_sum(Ctx *c, const double *part, int nblocks, double *out_dev);
 

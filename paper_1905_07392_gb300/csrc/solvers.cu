@@ -58,6 +58,49 @@ __device__ inline double block_sum(double v)
 }
 
 __device__ inline int block_linear() { return (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x; }
+
+// The solvers run one system, or the three velocity components' viscous
+// systems side by side: same grid and faces, own diagonals, vectors, scalars
+// and loop control.  Launches on a component axis do the work of three (the
+// levels that cannot fill the GPU cost launches and latency, not work: two
+// steps at 64^3 21.3 ms with the components one after another, 17.1 ms
+// together; viscous solves on 192 x 160 x 224 14.8 and 11.6 ms); each
+// component's operations, and so its results, are those of a solve alone, and
+// a component that has converged is frozen while the others go on.  3-D
+// kernels carry the component in blockIdx.z (component-major), the others in
+// blockIdx.y.
+constexpr int kMaxComp = 3;
+template <class T>
+struct V3 {
+    T *p[kMaxComp] = {};
+    V3() = default;
+    __host__ __device__ V3(T *a, T *b, T *c) : p{a, b, c} {}
+    template <class U>
+    __host__ __device__ V3(const V3<U> &o) : p{o.p[0], o.p[1], o.p[2]} {}
+};
+template <class T>
+inline V3<T> one(T *p)
+{
+    return V3<T>(p, nullptr, nullptr);
+}
+// component and plane-block of a 3-D launch of nzb blocks per component
+struct CompZ {
+    int comp, z;
+    __device__ explicit CompZ(int nzb)
+    {
+        comp = (int)blockIdx.z >= nzb ? ((int)blockIdx.z >= 2 * nzb ? 2 : 1) : 0;
+        z = (int)blockIdx.z - comp * nzb;
+    }
+    __device__ int linear() const { return (z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x; }
+};
+// act: the loop condition word of component 0 (the others C_LEN apart), or
+// null where every component runs
+__device__ inline bool comp_off(const int *act, int comp) { return act && act[comp * C_LEN] == 0; }
+constexpr int kScalLen = 32;                        // device scalars per component
+constexpr size_t kPartLen = (size_t)1 << 20;        // doubles in c->part
+constexpr size_t kPartComp = kPartLen / kMaxComp;   // of these per component when three run together
+// joint control words, behind the components' own
+enum { J_OUT = kMaxComp * C_LEN, J_IN, J_IT, J_NOUT };
 __device__ inline int thread_linear() { return (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x; }
 
 // 3-D blocks of 256 threads: block sum keyed on the linear thread index.
@@ -111,19 +154,26 @@ __device__ inline double block_sum3_t(T v)
 // kRedCtas SMs.  The barrier is the hardware cluster barrier (no spin).
 constexpr int kRedCtas = 8, kRedThreads = 512;
 __global__ void __cluster_dims__(kRedCtas, 1, 1) __launch_bounds__(kRedThreads)
-    k_reduce_final(const double *part, int n, double *out, double *scal, int post)
+    k_reduce_final(const double *part, int n, double *out, double *scal, int post, const int *act)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ double csum[kRedCtas];
+    cl.barrier_arrive();   // (no block's shared memory is written before that block runs)
+    const int comp = blockIdx.y;
+    part += comp * kPartComp;
+    out += comp * kScalLen;
+    scal += comp * kScalLen;
+    const bool off = comp_off(act, comp);
     const int q = (int)cl.block_rank();
     const int lo = (int)((long long)n * q / kRedCtas), hi = (int)((long long)n * (q + 1) / kRedCtas);
     double v = 0.0;
     for (int s = lo + threadIdx.x; s < hi; s += kRedThreads) v += part[s];
     v = block_sum<kRedThreads>(v);
+    cl.barrier_wait();
     if (threadIdx.x == 0) *cl.map_shared_rank(&csum[q], 0) = v;
     cl.sync();
-    if (q == 0 && threadIdx.x == 0) {
+    if (q == 0 && threadIdx.x == 0 && !off) {
         double t = 0.0;
         for (int r = 0; r < kRedCtas; r++) t += csum[r];
         *out = t;
@@ -132,9 +182,11 @@ __global__ void __cluster_dims__(kRedCtas, 1, 1) __launch_bounds__(kRedThreads)
     }
 }
 
-__global__ void __launch_bounds__(256) k_dot(const double *__restrict__ a, const double *__restrict__ b,
-                                             int n, double *__restrict__ part)
+__global__ void __launch_bounds__(256) k_dot(V3<const double> av, V3<const double> bv, int n,
+                                             double *__restrict__ part)
 {
+    const double *__restrict__ a = av.p[blockIdx.y], *__restrict__ b = bv.p[blockIdx.y];
+    part += blockIdx.y * kPartComp;
     double v = 0.0;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
         v += a[s] * b[s];
@@ -147,19 +199,16 @@ __global__ void __launch_bounds__(256) k_dot(const double *__restrict__ a, const
 ebv_status reduce_sum(Ctx *c, const double *part, int nblocks, double *out_dev)
 {
     EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas), dim3(kRedThreads), 0, part, nblocks, out_dev, c->scal,
-               (int)kRedSum);
+               (int)kRedSum, (const int *)nullptr);
     return EBV_OK;
 }
-// r.z or p.q of a CG iteration, with the quotient it completes.
-static void reduce_rz(Ctx *c, int nblocks)
+// A sum of every component's partials into its scalar S; r.z and p.q of a CG
+// iteration with the quotient they complete.
+static void reduce_comp(Ctx *c, int nc, int nblocks, int S, int post = kRedSum, const int *act = nullptr,
+                        const double *part = nullptr)
 {
-    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas), dim3(kRedThreads), 0, c->part, nblocks, c->scal + S_RZ, c->scal,
-               (int)kRedBeta);
-}
-static void reduce_pq(Ctx *c, int nblocks)
-{
-    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas), dim3(kRedThreads), 0, c->part, nblocks, c->scal + S_PQ, c->scal,
-               (int)kRedAlpha);
+    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas, nc), dim3(kRedThreads), 0, part ? part : c->part, nblocks,
+               c->scal + S, c->scal, post, act);
 }
 
 namespace {
@@ -180,6 +229,19 @@ struct CcOp {
     const F *bx, *by, *bz;
     const T *dinv = nullptr;   // V-cycle operator: 1/diag (0 where diag <= 0)
 };
+// The operators of the components: one set of faces, their own diagonals.
+template <class T, class F = T>
+struct CcOp3 {
+    CcOp<T, F> A;
+    const T *diag[kMaxComp], *dinv[kMaxComp];
+    __device__ CcOp<T, F> op(int comp) const
+    {
+        CcOp<T, F> B = A;
+        B.diag = diag[comp];
+        B.dinv = dinv[comp];
+        return B;
+    }
+};
 // The V-cycle's operator: in FP32 its faces are stored in BF16 (half the
 // bytes of the face arrays every colour pass reads whole); the Krylov
 // operator it preconditions keeps FP32 faces (CcOp<T>).  Built with
@@ -195,6 +257,7 @@ template <> struct VFace<float> { using type = __nv_bfloat16; };
 constexpr bool kVcycleBf16 = true;
 #endif
 template <class T> using VOp = CcOp<T, typename VFace<T>::type>;
+template <class T> using VOp3 = CcOp3<T, typename VFace<T>::type>;
 
 // Array layout of the cell-centred multigrid, by precision.  FP64 arrays are
 // in the natural order (x fastest).  FP32 arrays -- the coefficients of every
@@ -337,16 +400,21 @@ __device__ inline T gs_cell(const VOp<T> &A, const T *__restrict__ x, const T *_
 // the other colour, which this pass does not change -- i.e. r.z of the
 // preconditioned CG, without a separate pass over both vectors.
 template <class T, bool kCorr = false, bool kDot = false>
-__global__ void __launch_bounds__(256) k_cc_gs(VOp<T> A, T *__restrict__ x, const T *__restrict__ b,
-                                               int color, int zero_start, const T *__restrict__ xc = nullptr,
+__global__ void __launch_bounds__(256) k_cc_gs(VOp3<T> A3, V3<T> xv, V3<const T> bv, int nzb, const int *act,
+                                               int color, int zero_start, V3<const T> xcv = V3<const T>(),
                                                GridD gc = GridD(), double *__restrict__ part = nullptr)
 {
+    const CompZ cz(nzb);
+    if (comp_off(act, cz.comp)) return;
+    const VOp<T> A = A3.op(cz.comp);
+    T *__restrict__ x = xv.p[cz.comp];
+    const T *__restrict__ b = bv.p[cz.comp], *__restrict__ xc = xcv.p[cz.comp];
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int kk = blockIdx.z * blockDim.z + threadIdx.z;
+    const int kk = cz.z * blockDim.z + threadIdx.z;
     const GridD &g = A.g;
-    const bool act = 2 * t < g.nx && j < g.ny;
-    if (!kDot && !act) return;   // (with kDot every thread reaches the block sum)
+    const bool own = 2 * t < g.nx && j < g.ny;
+    if (!kDot && !own) return;   // (with kDot every thread reaches the block sum)
     T val[GS_PZ];
     int cc[GS_PZ];
 #pragma unroll
@@ -355,7 +423,7 @@ __global__ void __launch_bounds__(256) k_cc_gs(VOp<T> A, T *__restrict__ x, cons
         const int i = 2 * t + ((j + k + color) & 1);
         cc[h] = -1;
         val[h] = T(0);
-        if (!act || k >= g.nz || i >= g.nx) continue;
+        if (!own || k >= g.nz || i >= g.nx) continue;
         cc[h] = cix<T>(g, i, j, k);
         val[h] = gs_cell<T, kCorr>(A, x, b, i, j, k, zero_start, xc, gc);
     }
@@ -372,7 +440,7 @@ __global__ void __launch_bounds__(256) k_cc_gs(VOp<T> A, T *__restrict__ x, cons
             const int k = GS_PZ * kk + h;
             const int io = 2 * t + 1 - ((j + k + color) & 1);
             if (cc[h] >= 0) dot += b[cc[h]] * val[h];
-            if (act && k < g.nz && io < g.nx) {
+            if (own && k < g.nz && io < g.nx) {
                 const int co = cix<T>(g, io, j, k);
                 dot += b[co] * x[co];
             }
@@ -380,7 +448,7 @@ __global__ void __launch_bounds__(256) k_cc_gs(VOp<T> A, T *__restrict__ x, cons
     }
     if constexpr (kDot) {
         const double sdot = block_sum3_t<T>(dot);
-        if (thread_linear() == 0) part[block_linear()] = sdot;
+        if (thread_linear() == 0) part[cz.comp * kPartComp + cz.linear()] = sdot;
     }
 }
 
@@ -413,17 +481,22 @@ __device__ inline void load4(const F *p, float v[4])
 // neighbour value plus its parent's coarse correction xc, level gc); its
 // coarse rows in registers ask for 3 resident blocks per SM.
 template <int kPz, bool kCorr = false>
-__global__ void __launch_bounds__(256, kCorr ? 3 : (kPz == 1 ? 5 : 4)) k_cc_gs4(VOp<float> A, float *__restrict__ x,
-                                                                 const float *__restrict__ b, int color,
-                                                                 int zero_start, const float *__restrict__ xc = nullptr,
+__global__ void __launch_bounds__(256, kCorr ? 3 : (kPz == 1 ? 5 : 4)) k_cc_gs4(VOp3<float> A3, V3<float> xv,
+                                                                 V3<const float> bv, int nzb, const int *act, int color,
+                                                                 int zero_start, V3<const float> xcv = V3<const float>(),
                                                                  GridD gc = GridD())
 {
     using F = typename VFace<float>::type;
+    const CompZ cz(nzb);
+    if (comp_off(act, cz.comp)) return;
+    const VOp<float> A = A3.op(cz.comp);
+    float *__restrict__ x = xv.p[cz.comp];
+    const float *__restrict__ b = bv.p[cz.comp], *__restrict__ xc = xcv.p[cz.comp];
     const GridD &g = A.g;
     const int hx = g.nx >> 1;
     const int t0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int kb = (blockIdx.z * blockDim.z + threadIdx.z) * kPz;
+    const int kb = (cz.z * blockDim.z + threadIdx.z) * kPz;
     if (t0 >= hx || j >= g.ny) return;
     const int sy = g.nx, sz = g.nx * g.ny;
     float val[kPz][4];
@@ -521,11 +594,14 @@ inline dim3 gs4_grid(const GridD &g, dim3 bk, int pz)
     const int nq = (g.nx >> 1) / 4, nzg = (g.nz + pz - 1) / pz;
     return dim3((nq + bk.x - 1) / bk.x, (g.ny + bk.y - 1) / bk.y, (nzg + bk.z - 1) / bk.z);
 }
-inline void launch_gs4(cudaStream_t st, dim3 bk, int pz, const VOp<float> &A, float *x, const float *b, int color,
+// a 3-D grid for nc components
+inline dim3 comp_grid(dim3 g, int nc) { return dim3(g.x, g.y, g.z * nc); }
+inline void launch_gs4(cudaStream_t st, dim3 bk, int pz, const VOp3<float> &A, V3<float> x, V3<const float> b, int color,
                        int zs)
 {
-    if (pz == 1) k_cc_gs4<1><<<gs4_grid(A.g, bk, 1), bk, 0, st>>>(A, x, b, color, zs);
-    else k_cc_gs4<2><<<gs4_grid(A.g, bk, 2), bk, 0, st>>>(A, x, b, color, zs);
+    const dim3 gr = gs4_grid(A.A.g, bk, pz);
+    if (pz == 1) k_cc_gs4<1><<<gr, bk, 0, st>>>(A, x, b, gr.z, nullptr, color, zs);
+    else k_cc_gs4<2><<<gr, bk, 0, st>>>(A, x, b, gr.z, nullptr, color, zs);
 }
 
 // ---------------------------------------------------------------------------
@@ -606,15 +682,21 @@ struct RbSmem {
 template <class F>
 struct RbArgs {
     GridD g;                // this level
-    float *xout;
+    V3<float> xout;
     double *part;           // kDot partials
     int *ctl;
+    const int *act;
+    int nzb;                // chunks per component
     int c0, kz;             // first colour, planes per chunk
     long long spin;         // bound of one wait, clock64 cycles
 };
 
 struct RbMaps {
-    CUtensorMap x, b, d, fx, fy, fz, xc;   // xc: the coarse correction (kCorr)
+    struct Comp {
+        CUtensorMap x, b, d, xc;   // xc: the coarse correction (kCorr)
+    };
+    CUtensorMap fx, fy, fz;
+    Comp v[kMaxComp];
 };
 
 // Coarse planes step q loads (kCorr): step m needs coarse planes (m-1)/2 ..
@@ -625,7 +707,7 @@ __device__ inline int rb_coarse_count(int q, int m) { return q == 0 ? 2 : (((m +
 
 template <class F>
 __device__ inline void rb_issue(unsigned char *sm, uint64_t *bar, int q, int m0, int p0, int y0, bool zero,
-                                bool corr, const RbMaps &tm)
+                                bool corr, const RbMaps &tm, const RbMaps::Comp &tc)
 {
     using S = RbSmem<F>;
     const int m = m0 + q;
@@ -639,19 +721,19 @@ __device__ inline void rb_issue(unsigned char *sm, uint64_t *bar, int q, int m0,
         const int nk = rb_coarse_count(q, m), cfirst = q == 0 ? ((m - 1) >> 1) : ((m + 1) >> 1);
         for (int t = 0; t < nk; t++) {
             const int C = cfirst + t;
-            tma_load_4d(sm + S::oK + ((C + 3) % 3) * S::kK, &tm.xc, p0 / 2 - 4, 0, y0 / 2 - 1, C, b);
+            tma_load_4d(sm + S::oK + ((C + 3) % 3) * S::kK, &tc.xc, p0 / 2 - 4, 0, y0 / 2 - 1, C, b);
         }
     }
     if (!zero) {
         if (q == 0) {
-            tma_load_4d(sm + S::oX + ((m - 1 + 8) & 3) * S::kX, &tm.x, p0 - 4, 0, y0 - 2, m - 1, b);
-            tma_load_4d(sm + S::oX + ((m + 8) & 3) * S::kX, &tm.x, p0 - 4, 0, y0 - 2, m, b);
+            tma_load_4d(sm + S::oX + ((m - 1 + 8) & 3) * S::kX, &tc.x, p0 - 4, 0, y0 - 2, m - 1, b);
+            tma_load_4d(sm + S::oX + ((m + 8) & 3) * S::kX, &tc.x, p0 - 4, 0, y0 - 2, m, b);
         }
-        tma_load_4d(sm + S::oX + ((m + 1 + 8) & 3) * S::kX, &tm.x, p0 - 4, 0, y0 - 2, m + 1, b);
+        tma_load_4d(sm + S::oX + ((m + 1 + 8) & 3) * S::kX, &tc.x, p0 - 4, 0, y0 - 2, m + 1, b);
     }
     const int sb = (m + 3) % 3;
-    tma_load_4d(sm + S::oB + sb * S::kC, &tm.b, p0 - 4, 0, y0 - 1, m, b);
-    tma_load_4d(sm + S::oD + sb * S::kC, &tm.d, p0 - 4, 0, y0 - 1, m, b);
+    tma_load_4d(sm + S::oB + sb * S::kC, &tc.b, p0 - 4, 0, y0 - 1, m, b);
+    tma_load_4d(sm + S::oD + sb * S::kC, &tc.d, p0 - 4, 0, y0 - 1, m, b);
     tma_load_4d(sm + S::oY + sb * S::kY, &tm.fy, p0 - 8, 0, y0 - 1, m, b);
     tma_load_4d(sm + S::oXF + sb * S::kZ, &tm.fx, p0 - 8, 0, y0 - 1, m, b);
     if (q == 0) tma_load_4d(sm + S::oZ + ((m + 8) & 3) * S::kZ, &tm.fz, p0 - 8, 0, y0 - 1, m, b);
@@ -679,8 +761,12 @@ __global__ void __launch_bounds__(RB_THREADS, 2)
     const GridD &g = a.g;
     const int hx = g.nx >> 1;
     const int p0 = blockIdx.x * RB_HW, y0 = blockIdx.y * RB_TY;
-    const int z0 = blockIdx.z * a.kz, z1 = min(g.nz, z0 + a.kz);
-    if (z0 >= z1) return;
+    const CompZ cz(a.nzb);
+    const int z0 = cz.z * a.kz, z1 = min(g.nz, z0 + a.kz);
+    if (z0 >= z1 || comp_off(a.act, cz.comp)) return;
+    const RbMaps::Comp &tc = tm.v[cz.comp];
+    int *const ctl = a.ctl + cz.comp * C_LEN;
+    float *const xout = a.xout.p[cz.comp];
     const int tid = threadIdx.x, c1 = 1 - a.c0;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + S::oBar);
     int *flag = reinterpret_cast<int *>(sm + S::oMisc);
@@ -700,7 +786,7 @@ __global__ void __launch_bounds__(RB_THREADS, 2)
     auto cor_row = [&](int J) { return (J - (y0 / 2 - 1)) * 2 * RB_KW; };
     auto cor_col = [&](int I) { return (I & 1) * RB_KW + (I >> 1) - (p0 / 2 - 4); };
     if (smem_u32(sm) & 127) {   // tile destinations must be 128-byte aligned: report, load nothing
-        if (tid == 0) atomicCAS(a.ctl + C_ERR, 0, E_SMEM);
+        if (tid == 0) atomicCAS(ctl + C_ERR, 0, E_SMEM);
         return;
     }
     if (tid == 0) {
@@ -710,8 +796,8 @@ __global__ void __launch_bounds__(RB_THREADS, 2)
     }
     __syncthreads();
     if (tid == 0) {
-        rb_issue<F>(sm, bar, 0, m0, p0, y0, kZero, kCorr, tm);
-        rb_issue<F>(sm, bar, 1, m0, p0, y0, kZero, kCorr, tm);
+        rb_issue<F>(sm, bar, 0, m0, p0, y0, kZero, kCorr, tm, tc);
+        rb_issue<F>(sm, bar, 1, m0, p0, y0, kZero, kCorr, tm, tc);
     }
     // second colour and output: thread -> positions pq, pq+1 of both halves of tile row r
     const int r = tid >> 4, pq = p0 + 2 * (tid & 15);
@@ -872,7 +958,7 @@ __global__ void __launch_bounds__(RB_THREADS, 2)
             // a load did not arrive in time: record it, let the loads in
             // flight land (bounded) and stop this block
             if (tid == 0) {
-                atomicCAS(a.ctl + C_ERR, 0, E_TIMEOUT);
+                atomicCAS(ctl + C_ERR, 0, E_TIMEOUT);
                 for (int s = q; s < min(nstep, q + 2); s++)
                     mbar_wait_bounded(bar + s % RB_NBAR, (s / RB_NBAR) & 1, kRbDrainCycles);
             }
@@ -936,7 +1022,7 @@ __global__ void __launch_bounds__(RB_THREADS, 2)
                     v[0][e] = h2 ? s1[e] : s2[e];
                     v[1][e] = h2 ? s2[e] : s1[e];
                 }
-                float *o = a.xout + (size_t)(mm * g.ny + j2) * g.nx + pq;
+                float *o = xout + (size_t)(mm * g.ny + j2) * g.nx + pq;
                 *reinterpret_cast<float2 *>(o) = make_float2(v[0][0], v[0][1]);
                 *reinterpret_cast<float2 *>(o + hx) = make_float2(v[1][0], v[1][1]);
                 if constexpr (kDot) {
@@ -959,11 +1045,11 @@ __global__ void __launch_bounds__(RB_THREADS, 2)
         if (kDot && q >= 2 && tid == 32) {
             double s = 0.0;
             for (int w = 0; w < RB_THREADS / 32; w++) s += wsum[w];
-            a.part[(size_t)mm * (gridDim.x * gridDim.y) + blockIdx.y * gridDim.x + blockIdx.x] = s;
+            a.part[cz.comp * kPartComp + (size_t)mm * (gridDim.x * gridDim.y) + blockIdx.y * gridDim.x + blockIdx.x] = s;
         }
         if (tid == 0 && q + 2 < nstep) {
             fence_proxy_async();
-            rb_issue<F>(sm, bar, q + 2, m0, p0, y0, kZero, kCorr, tm);
+            rb_issue<F>(sm, bar, q + 2, m0, p0, y0, kZero, kCorr, tm, tc);
         }
     }
 }
@@ -1003,10 +1089,15 @@ using RbF = typename VFace<float>::type;
 // together), each plane's partial reduced on its own.  Grid (tiles x,
 // tiles y, ceil(nz / kGs2Planes)).
 constexpr int kGs2Planes = 4;
-__global__ void __launch_bounds__(RB_THREADS) k_cc_gs2_dot(VOp<float> A, float *__restrict__ x,
-                                                            const float *__restrict__ b, int c1,
-                                                            double *__restrict__ part)
+__global__ void __launch_bounds__(RB_THREADS) k_cc_gs2_dot(VOp3<float> A3, V3<float> xv, V3<const float> bv, int nzb,
+                                                            const int *act, int c1, double *__restrict__ part)
 {
+    const CompZ cz(nzb);
+    if (comp_off(act, cz.comp)) return;
+    const VOp<float> A = A3.op(cz.comp);
+    float *__restrict__ x = xv.p[cz.comp];
+    const float *__restrict__ b = bv.p[cz.comp];
+    part += cz.comp * kPartComp;
     __shared__ double wsum[kGs2Planes][RB_THREADS / 32];
     const GridD &g = A.g;
     const int tid = threadIdx.x, hx = g.nx >> 1, hf = (g.nx + 2) >> 1;
@@ -1016,7 +1107,7 @@ __global__ void __launch_bounds__(RB_THREADS) k_cc_gs2_dot(VOp<float> A, float *
     float dsum[kGs2Planes];
 #pragma unroll
     for (int pl = 0; pl < kGs2Planes; pl++) {
-        const int k = blockIdx.z * kGs2Planes + pl;
+        const int k = cz.z * kGs2Planes + pl;
         dsum[pl] = 0.f;
         if (j >= g.ny || pq >= hx || k >= g.nz) continue;
         const int h2 = (c1 + j + k) & 1;
@@ -1075,7 +1166,7 @@ __global__ void __launch_bounds__(RB_THREADS) k_cc_gs2_dot(VOp<float> A, float *
     }
     __syncthreads();
     if (tid < kGs2Planes) {
-        const int k = blockIdx.z * kGs2Planes + tid;
+        const int k = cz.z * kGs2Planes + tid;
         if (k < g.nz) {
             double s = 0.0;
             for (int w = 0; w < RB_THREADS / 32; w++) s += wsum[tid][w];
@@ -1119,15 +1210,15 @@ __device__ inline T rr_cell(const VOp<T> &A, const T *__restrict__ x, const T *_
 
 // Residual of the 8 children, averaged into the coarse right-hand side.
 template <class T>
-__global__ void __launch_bounds__(256) k_cc_resid_restrict(VOp<T> A, const T *__restrict__ x,
-                                                           const T *__restrict__ b, GridD gc,
-                                                           T *__restrict__ bc)
+__global__ void __launch_bounds__(256) k_cc_resid_restrict(VOp3<T> A3, V3<const T> x, V3<const T> b, GridD gc,
+                                                           V3<T> bc, int nzb, const int *act)
 {
+    const CompZ cz(nzb);
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = blockIdx.y * blockDim.y + threadIdx.y;
-    const int K = blockIdx.z * blockDim.z + threadIdx.z;
-    if (I >= gc.nx || J >= gc.ny || K >= gc.nz) return;
-    bc[cix<T>(gc, I, J, K)] = rr_cell<T>(A, x, b, I, J, K);
+    const int K = cz.z * blockDim.z + threadIdx.z;
+    if (I >= gc.nx || J >= gc.ny || K >= gc.nz || comp_off(act, cz.comp)) return;
+    bc.p[cz.comp][cix<T>(gc, I, J, K)] = rr_cell<T>(A3.op(cz.comp), x.p[cz.comp], b.p[cz.comp], I, J, K);
 }
 
 // k_cc_resid_restrict for FP32 levels with nx a multiple of 8: a thread
@@ -1141,14 +1232,19 @@ __global__ void __launch_bounds__(256) k_cc_resid_restrict(VOp<T> A, const T *__
 // odd coarse cells are the two halves of the coarse row).  Bound by load
 // latency: capped at 64 registers (from 75) for four blocks per SM, 16 %
 // faster at 256^3.
-__global__ void __launch_bounds__(256, 4) k_cc_rr4(VOp<float> A, const float *__restrict__ x,
-                                               const float *__restrict__ b, GridD gc, float *__restrict__ bc)
+__global__ void __launch_bounds__(256, 4) k_cc_rr4(VOp3<float> A3, V3<const float> xv, V3<const float> bv, GridD gc,
+                                               V3<float> bcv, int nzb, const int *act)
 {
+    const CompZ cz(nzb);
+    if (comp_off(act, cz.comp)) return;
+    const VOp<float> A = A3.op(cz.comp);
+    const float *__restrict__ x = xv.p[cz.comp], *__restrict__ b = bv.p[cz.comp];
+    float *__restrict__ bc = bcv.p[cz.comp];
     const GridD &g = A.g;
     const int hx = g.nx >> 1, hf = (g.nx + 2) >> 1;
     const int I0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int J = blockIdx.y * blockDim.y + threadIdx.y;
-    const int K = blockIdx.z * blockDim.z + threadIdx.z;
+    const int K = cz.z * blockDim.z + threadIdx.z;
     if (I0 >= gc.nx || J >= gc.ny || K >= gc.nz) return;
     const int sy = g.nx, sz = g.nx * g.ny;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1435,35 +1531,38 @@ __global__ void k_visc_coeffs(GridD g, GeomD geo, ParamsD p, const double *__res
     extra[c] = e;
 }
 
-// Right-hand side of the viscous solve of component comp: alpha psi plus, for
-// each box face of the cell on a Dirichlet side of comp, its coefficient
-// (k_visc_coeffs) times the boundary value.
-__global__ void k_visc_rhs(GridD g, GeomD geo, int comp, const double *__restrict__ psi,
-                           const double *__restrict__ bx, const double *__restrict__ by,
-                           const double *__restrict__ bz, double *__restrict__ b)
+// Right-hand sides of the three viscous solves: alpha psi plus, for each box
+// face of the cell on a Dirichlet side of the component, its coefficient
+// (k_visc_coeffs) times the boundary value; faces are read at the box sides only.
+__global__ void k_visc_rhs(GridD g, GeomD geo, const double *__restrict__ psi, const double *__restrict__ bx,
+                           const double *__restrict__ by, const double *__restrict__ bz, double *__restrict__ b)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = blockIdx.z * blockDim.z + threadIdx.z;
     if (i >= g.nx || j >= g.ny || k >= g.nz) return;
-    const int c = cidx(g, i, j, k);
+    const int c = cidx(g, i, j, k), N3 = geo.ncell;
     if (geo.flag[c] == 0) {
-        b[c] = 0.0;
+        for (int q = 0; q < 3; q++) b[q * N3 + c] = 0.0;
         return;
     }
+    const bool side = i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1;
+    const double al = geo.alpha[c];
     const double *B[3] = {bx, by, bz};
     const int id[3] = {i, j, k};
-    double rb = 0.0;
-    for (int d = 0; d < 3; d++)
-        for (int hs = 0; hs < 2; hs++) {
-            int pos = id[d] + hs;
-            if (pos != 0 && pos != dimn(g, d)) continue;
-            int fi[3] = {i, j, k};
-            fi[d] += hs;
-            double val;
-            if (side_dirichlet(g, 2 * d + hs, comp, &val)) rb += B[d][fidx(g, d, fi[0], fi[1], fi[2])] * val;
-        }
-    b[c] = geo.alpha[c] * psi[c] + rb;
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        double rb = 0.0, val;
+        if (side)
+            for (int d = 0; d < 3; d++)
+                for (int hs = 0; hs < 2; hs++) {
+                    if (id[d] != (hs ? dimn(g, d) - 1 : 0)) continue;
+                    int fi[3] = {i, j, k};
+                    fi[d] += hs;
+                    if (side_dirichlet(g, 2 * d + hs, q, &val)) rb += B[d][fidx(g, d, fi[0], fi[1], fi[2])] * val;
+                }
+        b[q * N3 + c] = al * psi[q * N3 + c] + rb;
+    }
 }
 
 // q = A p (level 0) and block partials of p.q in FP64 (per thread and warp
@@ -1473,15 +1572,20 @@ __global__ void k_visc_rhs(GridD g, GeomD geo, int comp, const double *__restric
 // solver's true residual in one pass; |r|^2 only decides convergence, so it
 // is summed from the stored FP32 values, per thread and warp in FP32).
 template <class T, bool kRes = false>
-__global__ void __launch_bounds__(256) k_cc_apply_dot(CcOp<T> A, const T *__restrict__ p, T *__restrict__ q,
-                                                      double *__restrict__ part, const T *__restrict__ b = nullptr,
-                                                      float *__restrict__ r32 = nullptr,
-                                                      const double *__restrict__ sig = nullptr)
+__global__ void __launch_bounds__(256) k_cc_apply_dot(CcOp3<T> A3, V3<const T> pv, V3<T> qv, double *__restrict__ part,
+                                                      int nzb, const int *act, V3<const T> bv = V3<const T>(),
+                                                      V3<float> rv = V3<float>(), const double *__restrict__ sig = nullptr)
 {
-    const double sc = (kRes && sig) ? *sig : 1.0;
+    const CompZ cz(nzb);
+    if (comp_off(act, cz.comp)) return;
+    const CcOp<T> A = A3.op(cz.comp);
+    const T *__restrict__ p = pv.p[cz.comp], *__restrict__ b = bv.p[cz.comp];
+    T *__restrict__ q = qv.p[cz.comp];
+    float *__restrict__ r32 = rv.p[cz.comp];
+    const double sc = (kRes && sig) ? sig[cz.comp * kScalLen] : 1.0;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int kk = blockIdx.z * blockDim.z + threadIdx.z;
+    const int kk = cz.z * blockDim.z + threadIdx.z;
     T v = 0;
     float vr = 0.0f;
     if (i < A.g.nx && j < A.g.ny) {
@@ -1511,7 +1615,7 @@ __global__ void __launch_bounds__(256) k_cc_apply_dot(CcOp<T> A, const T *__rest
             }
     }
     const double vs = kRes ? block_sum3_t<float>(vr) : block_sum3_t<T>(v);
-    if (thread_linear() == 0) part[block_linear()] = vs;
+    if (thread_linear() == 0) part[cz.comp * kPartComp + cz.linear()] = vs;
 }
 
 // k_cc_apply_dot<float> for levels with nx a multiple of 8: a thread forms
@@ -1525,14 +1629,19 @@ constexpr int kApply4X = 16, kApply4Y = 8, kApply4Z = 2;
 // The vectorised apply and restriction serve grids where they launch at least
 // this many blocks (two per SM of 152); smaller grids keep one cell per thread.
 constexpr long long kVecMinBlocks = 304;
-__global__ void __launch_bounds__(256) k_cc_apply4(CcOp<float> A, const float *__restrict__ p, float *__restrict__ q,
-                                                  double *__restrict__ part)
+__global__ void __launch_bounds__(256) k_cc_apply4(CcOp3<float> A3, V3<const float> pv, V3<float> qv,
+                                                  double *__restrict__ part, int nzb, const int *act)
 {
+    const CompZ cz(nzb);
+    if (comp_off(act, cz.comp)) return;
+    const CcOp<float> A = A3.op(cz.comp);
+    const float *__restrict__ p = pv.p[cz.comp];
+    float *__restrict__ q = qv.p[cz.comp];
     const GridD &g = A.g;
     const int hx = g.nx >> 1, hf = (g.nx + 2) >> 1, nq = hx >> 2;
     const int tx = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int kk = blockIdx.z * blockDim.z + threadIdx.z;
+    const int kk = cz.z * blockDim.z + threadIdx.z;
     const int sy = g.nx, sz = g.nx * g.ny;
     float v = 0.f;
     if (tx < 2 * nq && j < g.ny) {
@@ -1578,7 +1687,7 @@ __global__ void __launch_bounds__(256) k_cc_apply4(CcOp<float> A, const float *_
         }
     }
     const double vs = block_sum3_t<float>(v);
-    if (thread_linear() == 0) part[block_linear()] = vs;
+    if (thread_linear() == 0) part[cz.comp * kPartComp + cz.linear()] = vs;
 }
 inline dim3 apply4_grid(const GridD &g)
 {
@@ -2236,12 +2345,12 @@ __device__ inline void bottom_row(const double *__restrict__ inv, int nb, const 
     x[bottom_pos(g, split, r)] = (T)(s * scale);
 }
 template <class T>
-__global__ void __launch_bounds__(256) k_bottom_solve(const double *__restrict__ inv, int nb,
-                                                      const T *__restrict__ b, T *__restrict__ x,
+__global__ void __launch_bounds__(256) k_bottom_solve(V3<const double> inv, int nb, V3<const T> b, V3<T> x,
                                                       double scale, GridD g, int split)
 {
+    const int q = blockIdx.y;
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nb; r += gridDim.x * blockDim.x)
-        bottom_row(inv, nb, b, x, scale, g, split, r);
+        bottom_row(inv.p[q], nb, b.p[q], x.p[q], scale, g, split, r);
 }
 
 // ---- the coarse end of the cell-centred V-cycle in one cluster -------------------
@@ -2287,10 +2396,10 @@ struct CoarseVC {
     int nd;                   // of these, cut into slabs
     int split_z;              // slabs of z planes, else of y planes
     int na;                   // blocks that own a slab (ranks 0 .. na-1)
-    VOp<T> A[kCvMax];
-    T *x;                     // top level
-    const T *b;
-    const double *binv;       // bottom inverse (natural numbering)
+    VOp3<T> A3[kCvMax];
+    V3<T> x;                  // top level
+    V3<const T> b;
+    V3<const double> binv;    // bottom inverses (natural numbering)
     int nb;
     double *part;             // block partials of b.x, or null
     CvLayout L;               // shared-memory offsets (cv_layout)
@@ -2363,9 +2472,9 @@ inline CvLayout cv_layout(const CoarseVC<T> &D)
     CvLayout o;
     int at = 0;
     auto take = [&](int bytes) { const int q = at; at += (bytes + 15) & ~15; return q; };
-    const int npd = cv_np(D.A[D.nd].g, D.split_z);
+    const int npd = cv_np(D.A3[D.nd].A.g, D.split_z);
     for (int l = 0; l + 1 < D.n; l++) {
-        const GridD &g = D.A[l].g;
+        const GridD &g = D.A3[l].A.g;
         const int plane = cv_no(g, D.split_z) * g.nx, pl = l < D.nd ? cv_plmax(npd, D.na, D.nd, l) : npd;
         o.x[l] = take((pl + 2) * plane * (int)sizeof(T));
         o.rec[l] = take(pl * plane * (int)sizeof(Rec));
@@ -2460,13 +2569,13 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char cvsm[];
     __shared__ CvLevel lv[3];
-    const int tid = threadIdx.x, rank = (int)cl.block_rank(), na = D.na, split_z = D.split_z, nd = D.nd;
-    const int npd = cv_np(D.A[nd].g, split_z), nl = D.n - 1;   // nl smoothed levels
+    const int comp = blockIdx.y, tid = threadIdx.x, rank = (int)cl.block_rank(), na = D.na, split_z = D.split_z, nd = D.nd;
+    const int npd = cv_np(D.A3[nd].A.g, split_z), nl = D.n - 1;   // nl smoothed levels
     const bool act = rank < na, red = nl > nd;
     const CvLayout &L = D.L;
     if (tid < nl) {
         const int l = tid;
-        const GridD &g = D.A[l].g;
+        const GridD &g = D.A3[l].A.g;
         const bool slab = l < nd;
         CvLevel v;
         v.x = L.x[l]; v.rec = L.rec[l]; v.b = L.b[l]; v.dg = L.dg[l]; v.info = L.info[l]; v.cpos = L.cpos[l];
@@ -2503,7 +2612,7 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
         for (int u = 0; u < kU; u++) {
             const int m = m0 + u * kCvThreads < n2 ? m0 + u * kCvThreads : 0;
             const int l = m < n0 ? 0 : (m < n1 ? 1 : 2), ml = m - (l == 0 ? 0 : (l == 1 ? n0 : n1));
-            const VOp<T> &A = D.A[l];
+            const VOp<T> &A = D.A3[l].A;
             const int r = ml / lv[l].h;
             ts[u] = ml - r * lv[l].h;
             ss[u] = r / lv[l].no;
@@ -2521,12 +2630,12 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
             f[u][8] = A.bz[p0.fz1];
             f[u][9] = A.bz[p1.fz0];
             f[u][10] = A.bz[p1.fz1];
-            d[u][0] = A.dinv[p0.c];
-            d[u][1] = A.dinv[p1.c];
-            d[u][2] = A.diag[((j + k) & 1) ? p1.c : p0.c];
+            d[u][0] = D.A3[l].dinv[comp][p0.c];
+            d[u][1] = D.A3[l].dinv[comp][p1.c];
+            d[u][2] = D.A3[l].diag[comp][((j + k) & 1) ? p1.c : p0.c];
             if (l == 0) {
-                bb[u][0] = D.b[p0.c];
-                bb[u][1] = D.b[p1.c];
+                bb[u][0] = D.b.p[comp][p0.c];
+                bb[u][1] = D.b.p[comp][p1.c];
             }
         }
 #pragma unroll
@@ -2535,7 +2644,7 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
             if (m >= n2) continue;
             const int l = m < n0 ? 0 : (m < n1 ? 1 : 2), ml = m - (l == 0 ? 0 : (l == 1 ? n0 : n1));
             const CvLevel &v = lv[l];
-            const GridD &g = D.A[l].g, &gc = D.A[l + 1].g;
+            const GridD &g = D.A3[l].A.g, &gc = D.A3[l + 1].A.g;
             const int t = ts[u], o = os[u], sl = ss[u];
             const int j = split_z ? o : v.s0 + sl, k = split_z ? v.s0 + sl : o, c0 = (j + k) & 1;   // colour of the even cell
             int *info = reinterpret_cast<int *>(cvsm + v.info), *cpos = reinterpret_cast<int *>(cvsm + v.cpos);
@@ -2565,7 +2674,7 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
     // this block's rows of the bottom inverse: staged, or on their way into L2
     const int br0 = D.nb * min(rank, na) / na, br1 = D.nb * min(rank + 1, na) / na;
     {
-        const double *src = D.binv + (size_t)br0 * D.nb;
+        const double *src = D.binv.p[comp] + (size_t)br0 * D.nb;
         const int n = (br1 - br0) * D.nb;
         if (L.bi >= 0) {
             double *bi = reinterpret_cast<double *>(cvsm + L.bi);
@@ -2631,7 +2740,7 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
                 }
             }
             __syncthreads();
-            const GridD &gc = D.A[l + 1].g;
+            const GridD &gc = D.A3[l + 1].A.g;
             const CvLevel &v = lv[l];
             const int noc = v.no >> 1, nc = (v.pl >> 1) * noc * gc.nx;
             for (int m = tid; m < nc; m += kCvThreads) {
@@ -2671,7 +2780,7 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
     // bottom: x = inv b, each block its share of the rows (FP64: one SM would
     // take nb^2 / 2 cycles), 16 lanes per row, the result to every block
     {
-        const double *bi = L.bi >= 0 ? reinterpret_cast<const double *>(cvsm + L.bi) : D.binv + (size_t)br0 * D.nb;
+        const double *bi = L.bi >= 0 ? reinterpret_cast<const double *>(cvsm + L.bi) : D.binv.p[comp] + (size_t)br0 * D.nb;
         const int nr = act ? br1 - br0 : 0, g = tid & 15;
         for (int rr = tid >> 4; rr < (nr + 1) / 2 * 2; rr += kCvThreads / 16) {   // (whole warps)
             double sum = 0.0;
@@ -2692,7 +2801,7 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
     // the top level's x, and b.x over the block's cells (per thread and warp in T, across warps in FP64)
     T dot = T(0);
     {
-        const GridD &g = D.A[0].g;
+        const GridD &g = D.A3[0].A.g;
         const CvView<T> w = view(0);
         const CvLevel &v = lv[0];
         for (int m = tid; m < w.pairs; m += kCvThreads) {
@@ -2700,8 +2809,8 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
             const int j = split_z ? o : v.s0 + sl, k = split_z ? v.s0 + sl : o, p = (w.info[m] & kCvPos);
             const int c0 = (w.info[m] & kCvPar) ? 1 : 0;   // colour of the even cell
             const T x0 = w.x[p], x1 = w.x[p + v.h];
-            D.x[cix<T>(g, 2 * t, j, k)] = x0;
-            D.x[cix<T>(g, 2 * t + 1, j, k)] = x1;
+            D.x.p[comp][cix<T>(g, 2 * t, j, k)] = x0;
+            D.x.p[comp][cix<T>(g, 2 * t + 1, j, k)] = x1;
             dot += w.b[c0 * w.cap + m] * x0 + w.b[(1 - c0) * w.cap + m] * x1;
         }
     }
@@ -2712,7 +2821,7 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
         if (tid == 0) {
             double sum = 0.0;
             for (int q = 0; q < kCvThreads / 32; q++) sum += ps[q];
-            D.part[rank] = sum;
+            D.part[comp * kPartComp + rank] = sum;
         }
     }
 }
@@ -2720,7 +2829,9 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
 // Which levels of the hierarchy the cluster kernel takes: fills the shape of D
 // and returns its top level, or -1 (no smoothed level fits: the bottom alone).
 // By the level sizes only: the largest top level whose slabs fit in shared
-// memory.
+// memory.  The finest level of a grid above 16^3 keeps its own kernels: its
+// last sweep forms r.z, and the whole GPU's sweeps of 32^3 cells (4.3 us each)
+// take about as long as eight blocks'.
 template <class T>
 int cv_plan(const CcHier &H, CoarseVC<T> &D)
 {
@@ -2728,10 +2839,10 @@ int cv_plan(const CcHier &H, CoarseVC<T> &D)
     for (int l0 = 0; l0 < Lb; l0++) {
         const int cells = ncell(H.lv[l0].g);
         const int nd = cells <= kCoarseCells ? 1 : 2, n = Lb - l0 + 1;
-        if (nd == 2 && (sizeof(T) != 4 || cells > kCvTopCells)) continue;
+        if (nd == 2 && (l0 == 0 || sizeof(T) != 4 || cells > kCvTopCells)) continue;
         if (n < nd + 1 || n > nd + 2) continue;
-        for (int q = 0; q < n; q++) D.A[q].g = H.lv[l0 + q].g;
-        const GridD &gd = D.A[nd].g;   // the first level that is not cut
+        for (int q = 0; q < n; q++) D.A3[q].A.g = H.lv[l0 + q].g;
+        const GridD &gd = D.A3[nd].A.g;   // the first level that is not cut
         D.n = n;
         D.nd = nd;
         D.split_z = gd.nz >= gd.ny;
@@ -2763,9 +2874,10 @@ void cv_attr()
 // below 1 (down to round-off) do not underflow in FP32.  Multiplying by a
 // power of two is exact, so in the usual range every FP32 operation gives
 // the same bits as without it.  The FP64 norms are scaled alike.
-__global__ void k_set_sigma(double *scal, int x_zero)
+__global__ void k_set_sigma(double *scal, int nc, int x_zero)
 {
-    if (threadIdx.x) return;
+    if ((int)threadIdx.x >= nc) return;
+    scal += threadIdx.x * kScalLen;
     const double bb = scal[S_BB];
     double sig = 1.0;
     if (bb > 0.0 && isfinite(bb)) sig = ldexp(1.0, -ilogb(sqrt(bb)));
@@ -2783,16 +2895,24 @@ __device__ inline void set_cond(int *ctl, int slot, int v, cudaGraphConditionalH
     if (use_h) cudaGraphSetConditional(h, v ? 1u : 0u);
 }
 
-__global__ void k_set_cond(int *ctl, int slot, int v, cudaGraphConditionalHandle h, int use_h)
+// Opens the CG loop of the coming pass: of the components whose pass runs.
+__global__ void k_inner_begin(int *ctl, int nc, cudaGraphConditionalHandle h, int use_h)
 {
-    if (threadIdx.x == 0) set_cond(ctl, slot, v, h, use_h);
+    if (threadIdx.x) return;
+    for (int q = 0; q < nc; q++) ctl[q * C_LEN + C_COND_IN] = ctl[q * C_LEN + C_COND_OUT];
+    set_cond(ctl, J_IN, 1, h, use_h);
 }
 
-__global__ void k_solve_begin(int *ctl)
+__global__ void k_solve_begin(int *ctl, int nc)
 {
-    if (threadIdx.x == 0) {
-        ctl[C_IT] = 0; ctl[C_K] = 0; ctl[C_NOUT] = 0; ctl[C_STALL] = 0; ctl[C_ERR] = 0; ctl[C_ZERO] = 0;
+    if (threadIdx.x) return;
+    for (int q = 0; q < nc; q++) {
+        int *c = ctl + q * C_LEN;
+        c[C_IT] = 0; c[C_K] = 0; c[C_NOUT] = 0; c[C_STALL] = 0; c[C_ERR] = 0; c[C_ZERO] = 0;
+        c[C_COND_OUT] = 1;
     }
+    ctl[J_IT] = 0;
+    ctl[J_NOUT] = 0;
 }
 
 // After a true residual (S_RR = |b - A x|^2, S_BB = |b|^2): record the
@@ -2801,41 +2921,49 @@ __global__ void k_solve_begin(int *ctl)
 // at max_pass, iterations at maxit; a non-finite norm stops with E_NAN; b = 0
 // flags x for zeroing.  For refinement, the inner target and stall state of
 // the coming correction solve are set here.
-__global__ void k_outer_check(double *scal, int *ctl, double tol, int maxit, int max_pass, int refine,
+__global__ void k_outer_check(double *scal0, int *ctl0, int nc, double tol, int maxit, int max_pass, int refine,
                               double inner_drop, cudaGraphConditionalHandle h, int use_h)
 {
     if (threadIdx.x) return;
-    const double bb = scal[S_BB], rr = scal[S_RR];
-    int go = 0;
-    if (ctl[C_ERR] == 0) {
-        if (!isfinite(rr) || !isfinite(bb)) {
-            ctl[C_ERR] = E_NAN;
-        } else if (bb == 0.0) {
-            ctl[C_ZERO] = 1;
-            scal[S_REL] = 0.0;
-        } else {
-            const double rel = sqrt(rr / bb);
-            scal[S_REL] = rel;
-            go = rel > tol && ctl[C_IT] < maxit && ctl[C_NOUT] < max_pass;
-            if (go && refine) {
-                const double f = fmax(inner_drop, 0.5 * tol / rel);
-                scal[S_T2] = rr * f * f;
-                scal[S_PREV] = rr;
-                ctl[C_STALL] = 0;
+    int any = 0;
+    for (int q = 0; q < nc; q++) {
+        double *scal = scal0 + q * kScalLen;
+        int *ctl = ctl0 + q * C_LEN;
+        if (!ctl[C_COND_OUT]) continue;   // (this component's solve has ended)
+        const double bb = scal[S_BB], rr = scal[S_RR];
+        int go = 0;
+        if (ctl[C_ERR] == 0) {
+            if (!isfinite(rr) || !isfinite(bb)) {
+                ctl[C_ERR] = E_NAN;
+            } else if (bb == 0.0) {
+                ctl[C_ZERO] = 1;
+                scal[S_REL] = 0.0;
+            } else {
+                const double rel = sqrt(rr / bb);
+                scal[S_REL] = rel;
+                go = rel > tol && ctl[C_IT] < maxit && ctl[C_NOUT] < max_pass;
+                if (go && refine) {
+                    const double f = fmax(inner_drop, 0.5 * tol / rel);
+                    scal[S_T2] = rr * f * f;
+                    scal[S_PREV] = rr;
+                    ctl[C_STALL] = 0;
+                }
             }
         }
+        ctl[C_NOUT]++;
+        ctl[C_K] = 0;
+        ctl[C_COND_OUT] = go;
+        any |= go;
     }
-    ctl[C_NOUT]++;
-    ctl[C_K] = 0;
-    set_cond(ctl, C_COND_OUT, go, h, use_h);
+    ctl0[J_NOUT]++;
+    set_cond(ctl0, J_OUT, any, h, use_h);
 }
 
 // After one CG iteration (S_RR = recursive residual norm^2).  FP64 path:
 // continue while |r|/|b| > tol/2.  Refinement path: continue until the
 // correction's residual is below its target, or it has stalled (three
 // iterations in a row that do not cut |r|^2 by 4: the FP32 round-off floor).
-__device__ inline void inner_check(double *scal, int *ctl, double tol, int maxit, int refine,
-                                   cudaGraphConditionalHandle h, int use_h)
+__device__ inline int inner_check(double *scal, int *ctl, double tol, int maxit, int refine)
 {
     scal[S_RZOLD] = scal[S_RZ];
     ctl[C_IT]++;
@@ -2858,50 +2986,88 @@ __device__ inline void inner_check(double *scal, int *ctl, double tol, int maxit
         scal[S_PREV] = rr;
     }
     if (ctl[C_IT] >= maxit || ctl[C_ERR]) go = 0;   // (an error word set by a kernel ends the solve)
-    set_cond(ctl, C_COND_IN, go, h, use_h);
+    ctl[C_COND_IN] = go;
+    return go;
 }
 
 // S_RR = the sum of the update's n block partials, then the same decision
-// (one launch instead of a reduction and a check).
-__global__ void __launch_bounds__(1024) k_reduce_inner_check(const double *part, int n, double *scal, int *ctl,
+// (one launch instead of a reduction and a check), per component; the loop goes
+// on while one does.
+__global__ void __launch_bounds__(1024) k_reduce_inner_check(const double *part, int n, double *scal, int *ctl, int nc,
                                                              double tol, int maxit, int refine,
                                                              cudaGraphConditionalHandle h, int use_h)
 {
-    double v = 0.0;
-    for (int s = threadIdx.x; s < n; s += 1024) v += part[s];
-    v = block_sum<1024>(v);
+    __shared__ double sm[kMaxComp][32];
+    double v[kMaxComp];
+    int on[kMaxComp];
+#pragma unroll
+    for (int q = 0; q < kMaxComp; q++) {
+        v[q] = 0.0;
+        on[q] = q < nc ? ctl[q * C_LEN + C_COND_IN] : 0;
+    }
+    for (int q = 0; q < nc; q++)
+        for (int s = threadIdx.x; s < n; s += 1024) v[q] += part[q * kPartComp + s];
+    // (as block_sum<1024>, the components' warp sums behind one barrier)
+    for (int q = 0; q < nc; q++) {
+        double w = v[q];
+        for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(0xffffffffu, w, o);
+        if ((threadIdx.x & 31) == 0) sm[q][threadIdx.x >> 5] = w;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    int any = 0;
+    for (int q = 0; q < nc; q++) {
+        double w = sm[q][threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(0xffffffffu, w, o);
+        if (threadIdx.x == 0 && on[q]) {
+            scal[q * kScalLen + S_RR] = w;
+            any |= inner_check(scal + q * kScalLen, ctl + q * C_LEN, tol, maxit, refine);
+        }
+    }
     if (threadIdx.x == 0) {
-        scal[S_RR] = v;
-        inner_check(scal, ctl, tol, maxit, refine, h, use_h);
+        ctl[J_IT]++;
+        set_cond(ctl, J_IN, any, h, use_h);
     }
 }
 
 // End of a solve: per-slot statistics, and the step's first failure
 // (100 x error + slot) kept in C_STEPERR.
-__global__ void k_solve_end(const double *scal, int *ctl, double tol, double *sstat, int slot)
+// The launch accounting of the joint loops goes to the first component's slot.
+__global__ void k_solve_end(const double *scal0, int *ctl0, int nc, double tol, double *sstat, int slot0)
 {
     if (threadIdx.x) return;
-    const double rel = scal[S_REL];
-    sstat[3 * slot] = ctl[C_IT];
-    sstat[3 * slot + 1] = rel;
-    sstat[3 * slot + 2] = ctl[C_NOUT];
-    int e = ctl[C_ERR];
-    if (e == 0 && !(rel <= tol)) e = E_NOTCONV;
-    if (e) ctl[C_ERR] = e;
-    if (e && ctl[C_STEPERR] == 0) ctl[C_STEPERR] = 100 * e + slot;
-    sstat[kSstatAcc + 2 * slot] += ctl[C_IT];
-    sstat[kSstatAcc + 2 * slot + 1] += ctl[C_NOUT] - 1;
+    for (int q = 0; q < nc; q++) {
+        const double *scal = scal0 + q * kScalLen;
+        int *ctl = ctl0 + q * C_LEN;
+        const int slot = slot0 + q;
+        const double rel = scal[S_REL];
+        sstat[3 * slot] = ctl[C_IT];
+        sstat[3 * slot + 1] = rel;
+        sstat[3 * slot + 2] = ctl[C_NOUT];
+        int e = ctl[C_ERR];
+        if (e == 0 && !(rel <= tol)) e = E_NOTCONV;
+        if (e) ctl[C_ERR] = e;
+        if (e && ctl0[C_STEPERR] == 0) ctl0[C_STEPERR] = 100 * e + slot;
+    }
+    sstat[kSstatAcc + 2 * slot0] += ctl0[J_IT];
+    sstat[kSstatAcc + 2 * slot0 + 1] += ctl0[J_NOUT] - 1;
 }
 
-__global__ void k_zero_if(double *x, int n, const int *ctl)
+__global__ void k_zero_if(V3<double> xv, int n, const int *ctl)
 {
-    if (!ctl[C_ZERO]) return;
+    if (!ctl[blockIdx.y * C_LEN + C_ZERO]) return;
+    double *x = xv.p[blockIdx.y];
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) x[s] = 0.0;
 }
 
-__global__ void __launch_bounds__(256) k_resid_init(const double *__restrict__ b, const double *__restrict__ q,
-                                                    double *__restrict__ r, int n, double *__restrict__ part)
+__global__ void __launch_bounds__(256) k_resid_init(V3<const double> bv, V3<const double> qv, V3<double> rv, int n,
+                                                    double *__restrict__ part, const int *act)
 {
+    const int comp = blockIdx.y;
+    if (comp_off(act, comp)) return;
+    const double *__restrict__ b = bv.p[comp], *__restrict__ q = qv.p[comp];
+    double *__restrict__ r = rv.p[comp];
+    part += comp * kPartComp;
     double v = 0.0, w = 0.0;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         double rs = b[s] - q[s];
@@ -2917,10 +3083,16 @@ __global__ void __launch_bounds__(256) k_resid_init(const double *__restrict__ b
     }
 }
 
-__global__ void __launch_bounds__(256) k_cg_update(double *__restrict__ x, double *__restrict__ r,
-                                                   const double *__restrict__ p, const double *__restrict__ q,
-                                                   const double *__restrict__ scal, int n, double *__restrict__ part)
+__global__ void __launch_bounds__(256) k_cg_update(V3<double> xv, V3<double> rv, V3<const double> pv,
+                                                   V3<const double> qv, const double *__restrict__ scal, int n,
+                                                   double *__restrict__ part, const int *act)
 {
+    const int comp = blockIdx.y;
+    if (comp_off(act, comp)) return;
+    double *__restrict__ x = xv.p[comp], *__restrict__ r = rv.p[comp];
+    const double *__restrict__ p = pv.p[comp], *__restrict__ q = qv.p[comp];
+    scal += comp * kScalLen;
+    part += comp * kPartComp;
     const double a = scal[S_ALPHA];
     double v = 0.0;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
@@ -2933,9 +3105,15 @@ __global__ void __launch_bounds__(256) k_cg_update(double *__restrict__ x, doubl
     if (threadIdx.x == 0) part[blockIdx.x] = v;
 }
 
-__global__ void k_cg_pupdate(double *__restrict__ p, const double *__restrict__ z, const double *__restrict__ scal,
-                             int n, const int *__restrict__ ctl)
+__global__ void k_cg_pupdate(V3<double> pv, V3<const double> zv, const double *__restrict__ scal, int n,
+                             const int *__restrict__ ctl, const int *act)
 {
+    const int comp = blockIdx.y;
+    if (comp_off(act, comp)) return;
+    double *__restrict__ p = pv.p[comp];
+    const double *__restrict__ z = zv.p[comp];
+    scal += comp * kScalLen;
+    ctl += comp * C_LEN;
     const int first = ctl[C_K] == 0;
     const double beta = first ? 0.0 : scal[S_BETA];
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
@@ -2946,9 +3124,10 @@ __global__ void k_cg_pupdate(double *__restrict__ p, const double *__restrict__ 
 // Per-thread sums of the FP32 kernels stay FP32 (a few dozen terms), block and
 // final sums are FP64.
 
-__global__ void __launch_bounds__(256) k_dot32(const float *__restrict__ a, const float *__restrict__ b, int n,
-                                               double *__restrict__ part)
+__global__ void __launch_bounds__(256) k_dot32(V3<const float> av, V3<const float> bv, int n, double *__restrict__ part)
 {
+    const float *__restrict__ a = av.p[blockIdx.y], *__restrict__ b = bv.p[blockIdx.y];
+    part += blockIdx.y * kPartComp;
     float v = 0.0f;
     const int n4 = n >> 2, t0 = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
     const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
@@ -2967,10 +3146,16 @@ __global__ void __launch_bounds__(256) k_dot32(const float *__restrict__ a, cons
 // r -= a q with a = rz/pq, partials of r.r.  (The solution update e += a p
 // of the same iteration is deferred to the next k_cg_pupdate32, which reads
 // p anyway, and after the last iteration to k_add32to64*.)
-__global__ void __launch_bounds__(256) k_cg_update32(float *__restrict__ r, const float *__restrict__ q,
+__global__ void __launch_bounds__(256) k_cg_update32(V3<float> rv, V3<const float> qv,
                                                      const double *__restrict__ scal, int n,
-                                                     double *__restrict__ part)
+                                                     double *__restrict__ part, const int *act)
 {
+    const int comp = blockIdx.y;
+    if (comp_off(act, comp)) return;
+    float *__restrict__ r = rv.p[comp];
+    const float *__restrict__ q = qv.p[comp];
+    scal += comp * kScalLen;
+    part += comp * kPartComp;
     const float a = (float)scal[S_ALPHA];
     float v = 0.0f;
     // 16-byte vectors (the arrays come from cudaMalloc), then the n % 4 tail:
@@ -3003,9 +3188,15 @@ __global__ void __launch_bounds__(256) k_cg_update32(float *__restrict__ r, cons
 // Iteration k of the FP32 CG: p = z (k = 0) or z + beta p, beta = rz/rz_old;
 // for k >= 1 first the previous iteration's solution update with the old p,
 // e = a p (k = 1) or e + a p, a = rz_old/pq (that iteration's step).
-__global__ void k_cg_pupdate32(float *__restrict__ p, float *__restrict__ e, const float *__restrict__ z,
-                               const double *__restrict__ scal, int n, const int *__restrict__ ctl)
+__global__ void k_cg_pupdate32(V3<float> pv3, V3<float> ev3, V3<const float> zv3, const double *__restrict__ scal, int n,
+                               const int *__restrict__ ctl, const int *act)
 {
+    const int comp = blockIdx.y;
+    if (comp_off(act, comp)) return;
+    float *__restrict__ p = pv3.p[comp], *__restrict__ e = ev3.p[comp];
+    const float *__restrict__ z = zv3.p[comp];
+    scal += comp * kScalLen;
+    ctl += comp * C_LEN;
     const int k = ctl[C_K];
     const float beta = k == 0 ? 0.0f : (float)scal[S_BETA];
     const float a = k == 0 ? 0.0f : (float)scal[S_ALPHA];   // of the iteration before
@@ -3070,13 +3261,17 @@ inline dim3 add_grid(const GridD &g)
 {
     return dim3((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + kAddPz - 1) / kAddPz);
 }
-__global__ void __launch_bounds__(256) k_add32to64_split(GridD g, double *__restrict__ x, const float *__restrict__ e,
-                                                         const float *__restrict__ p,
-                                                         const double *__restrict__ scal,
-                                                         const int *__restrict__ ctl)
+__global__ void __launch_bounds__(256) k_add32to64_split(GridD g, V3<double> xv3, V3<const float> ev3,
+                                                         V3<const float> pv3, const double *__restrict__ scal,
+                                                         const int *__restrict__ ctl, int nzb, const int *act)
 {
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k0 = blockIdx.z * kAddPz;
-    if (i >= g.nx || j >= g.ny) return;
+    const CompZ cz(nzb);
+    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k0 = cz.z * kAddPz;
+    if (i >= g.nx || j >= g.ny || comp_off(act, cz.comp)) return;
+    double *__restrict__ x = xv3.p[cz.comp];
+    const float *__restrict__ e = ev3.p[cz.comp], *__restrict__ p = pv3.p[cz.comp];
+    scal += cz.comp * kScalLen;
+    ctl += cz.comp * C_LEN;
     const int kit = ctl[C_K];
     const float a = (float)scal[S_ALPHA];
     const double isig = scal[S_ISIG];
@@ -3143,6 +3338,48 @@ VOp<T> vop(const CcLevel &L)
         A.dinv = (const T *)L.dinv_f;
     }
     return A;
+}
+
+// The operators of level l for nc components: the selected variant, or all
+// three (component q takes variant q).
+template <class T>
+CcOp3<T> ccop3(const CcHier &H, int nc)
+{
+    CcOp3<T> O;
+    O.A = ccop<T>(H.lv[0]);
+    for (int q = 0; q < kMaxComp; q++) {
+        O.dinv[q] = nullptr;
+        if (nc == 1) O.diag[q] = O.A.diag;
+        else if constexpr (sizeof(T) == 8) O.diag[q] = (const T *)H.vdiag_d[q][0];
+        else O.diag[q] = (const T *)H.vdiag_a[q];
+    }
+    return O;
+}
+template <class T>
+VOp3<T> vop3(const CcHier &H, int l, int nc)
+{
+    VOp3<T> O;
+    O.A = vop<T>(H.lv[l]);
+    for (int q = 0; q < kMaxComp; q++) {
+        O.diag[q] = O.A.diag;
+        O.dinv[q] = O.A.dinv;
+        if (nc == 1) continue;
+        if constexpr (sizeof(T) == 8) {
+            O.diag[q] = (const T *)H.vdiag_d[q][l];
+            O.dinv[q] = (const T *)H.vdiag_f[q][l];
+        } else {
+            O.diag[q] = (const T *)H.vdiag_f[q][l];
+            O.dinv[q] = (const T *)H.vdinv_f[q][l];
+        }
+    }
+    return O;
+}
+// vector of every component: the first has its own arrays, the others theirs in
+// the carved scratch (carve_components)
+template <class T>
+V3<T> comp_vec(Ctx *c, void *first, int kind, int l)
+{
+    return V3<T>((T *)first, (T *)c->cvec[0][kind][l], (T *)c->cvec[1][kind][l]);
 }
 
 // diagonals of every variant of level l from its extra and faces, in precision
@@ -3235,7 +3472,6 @@ inline dim3 ch_grid(const GridD &g, dim3 bk)
 
 // ---- the fused sweep on the host: where it applies, tensor maps, shape -----
 enum { RB_ZERO = 0, RB_PLAIN = 1, RB_CORR = 2, RB_DOT = 3 };
-constexpr size_t kPartLen = (size_t)1 << 20;   // doubles in c->part
 
 inline int rb_ntiles(const GridD &g) { return ((g.nx / 2 + RB_HW - 1) / RB_HW) * ((g.ny + RB_TY - 1) / RB_TY); }
 
@@ -3310,9 +3546,9 @@ int rb_resident()
 
 // Planes per chunk of a block: the fewest waves of resident blocks times the
 // steps of one block (its planes and the two of the chunk's start).
-int rb_kz(const GridD &g)
+int rb_kz(const GridD &g, int nc = 1)
 {
-    const long long nt = rb_ntiles(g), res = rb_resident();
+    const long long nt = (long long)nc * rb_ntiles(g), res = rb_resident();
     long long best = -1;
     int bkz = g.nz;
     for (int nc = 1; nc <= g.nz; nc++) {
@@ -3327,21 +3563,23 @@ int rb_kz(const GridD &g)
 }
 
 // One fused sweep (maps already encoded by rb_maps).
-void rb_launch(Ctx *c, const char *name, const GridD &g, const RbMaps &tm, float *xout, int c0, int mode,
-               double *part, int kz = 0)
+void rb_launch(Ctx *c, const char *name, const GridD &g, const RbMaps &tm, V3<float> xout, int c0, int mode,
+               double *part, int kz = 0, int nc = 1, const int *act = nullptr)
 {
     RbArgs<RbF> a;
     a.g = g;
     a.xout = xout;
     a.part = part;
     a.ctl = c->ctl;
+    a.act = act;
     a.c0 = c0;
-    a.kz = kz > 0 ? kz : rb_kz(g);
+    a.kz = kz > 0 ? kz : rb_kz(g, nc);
+    a.nzb = (g.nz + a.kz - 1) / a.kz;
     a.spin = spin_limit();
-    const dim3 gr((g.nx / 2 + RB_HW - 1) / RB_HW, (g.ny + RB_TY - 1) / RB_TY, (g.nz + a.kz - 1) / a.kz);
+    const dim3 gr((g.nx / 2 + RB_HW - 1) / RB_HW, (g.ny + RB_TY - 1) / RB_TY, a.nzb * nc);
     // algorithmic bytes: x written, x read (not from zero), b, 1/diag, three
     // faces, the coarse correction (1/8 word per cell)
-    const double nb = (double)ncell(g) * (4.0 + (mode == RB_ZERO ? 0.0 : 4.0) + 8.0 + 3.0 * sizeof(RbF) +
+    const double nb = (double)nc * ncell(g) * (4.0 + (mode == RB_ZERO ? 0.0 : 4.0) + 8.0 + 3.0 * sizeof(RbF) +
                                           (mode == RB_CORR ? 0.5 : 0.0));
     const int sb = RbSmem<RbF>::bytes;
     switch (mode) {
@@ -3378,12 +3616,14 @@ const char *const kRbName[8] = {"cc_rb_sweep<float> L0", "cc_rb_sweep<float> L1"
 // for bit: ebv_set_fused_sweep picks the passes (0), the faster of the two as
 // timed when the solvers are set up (1, the default) or the fused pass (2).
 template <class T>
-int cc_smooth2(Ctx *c, const CcLevel &L, int l, T *x, T *t, const T *b, bool red_first, bool zero_start,
-               const T *xc = nullptr, const GridD *gc = nullptr, double *dot_part = nullptr)
+int cc_smooth2(Ctx *c, const CcHier &H, int l, int nc, const int *act, V3<T> x, V3<T> t, V3<const T> b, bool red_first,
+               bool zero_start, V3<const T> xc = V3<const T>(), const GridD *gc = nullptr, double *dot_part = nullptr)
 {
-    VOp<T> A = vop<T>(L);
+    const CcLevel &L = H.lv[l];
+    const VOp3<T> A = vop3<T>(H, l, nc);
     const int c0 = red_first ? 0 : 1;
     const GridD &g = L.g;
+    const bool corr = gc != nullptr;
     bool tiles = false;   // r.z partials per (plane, tile)
     if constexpr (sizeof(T) == 4) {
         if (rb_fusable(g)) {
@@ -3392,36 +3632,39 @@ int cc_smooth2(Ctx *c, const CcLevel &L, int l, T *x, T *t, const T *b, bool red
             // each kind of sweep (from zero, plain, after the coarse correction,
             // with r.z) was timed on its own against its colour passes
             const int mode = fused_sweep_mode();
-            const int k1 = zero_start ? RB_ZERO : (xc ? RB_CORR : RB_PLAIN), k2 = dot_part ? RB_DOT : RB_PLAIN;
+            const int k1 = zero_start ? RB_ZERO : (corr ? RB_CORR : RB_PLAIN), k2 = dot_part ? RB_DOT : RB_PLAIN;
             // (the pair runs x -> t -> x fused, or in place as passes: one form for both)
             const bool faster = L.rb_ms[k1][0] + L.rb_ms[k2][0] < L.rb_ms[k1][1] + L.rb_ms[k2][1];
-            bool use = (mode == 2 || (mode == 1 && faster)) && rb_map(c, x, 0, g, &m1.x) &&
-                       rb_map(c, t, 0, g, &m2.x) && rb_map(c, b, 1, g, &m1.b) && rb_map(c, A.dinv, 1, g, &m1.d) &&
-                       rb_map(c, L.bxp, 4, g, &m1.fx) && rb_map(c, A.by, 2, g, &m1.fy) &&
-                       rb_map(c, A.bz, 3, g, &m1.fz);
-            if (use) {
-                m2.b = m1.b;
-                m2.d = m1.d;
-                m2.fx = m1.fx;
-                m2.fy = m1.fy;
-                m2.fz = m1.fz;
-                m1.xc = m2.xc = m1.b;   // (read by the correction sweep only)
-                if (k1 == RB_CORR) use = rb_map(c, xc, 5, *gc, &m1.xc);
+            bool use = (mode == 2 || (mode == 1 && faster)) && rb_map(c, L.bxp, 4, g, &m1.fx) &&
+                       rb_map(c, A.A.by, 2, g, &m1.fy) && rb_map(c, A.A.bz, 3, g, &m1.fz);
+            m2.fx = m1.fx;
+            m2.fy = m1.fy;
+            m2.fz = m1.fz;
+            for (int q = 0; q < nc && use; q++) {
+                RbMaps::Comp &v1 = m1.v[q], &v2 = m2.v[q];
+                use = rb_map(c, x.p[q], 0, g, &v1.x) && rb_map(c, t.p[q], 0, g, &v2.x) &&
+                      rb_map(c, b.p[q], 1, g, &v1.b) && rb_map(c, A.dinv[q], 1, g, &v1.d);
+                v2.b = v1.b;
+                v2.d = v1.d;
+                v1.xc = v2.xc = v1.b;   // (read by the correction sweep only)
+                if (use && k1 == RB_CORR) use = rb_map(c, xc.p[q], 5, *gc, &v1.xc);
             }
             if (use) {
                 const char *nm = kRbName[l < 7 ? l : 7];
-                rb_launch(c, nm, g, m1, t, c0, k1, nullptr, L.rb_kz);
-                rb_launch(c, nm, g, m2, x, c0, k2, dot_part, L.rb_kz);
+                const int kz = nc == 1 ? L.rb_kz : 0;   // (the timed chunking is that of one component)
+                rb_launch(c, nm, g, m1, t, c0, k1, nullptr, kz, nc, act);
+                rb_launch(c, nm, g, m2, x, c0, k2, dot_part, kz, nc, act);
                 return dot_part ? rb_ntiles(g) * g.nz : 0;
             }
         }
     }
     // algorithmic bytes of one colour pass: half of one sweep's x read and
     // write, b, diagonal and 3 face coefficients (in their storage type)
-    const double nb = 0.5 * ((4.0 * sizeof(T) + 3.0 * sizeof(typename VFace<T>::type)) * (double)ncell(g));
+    const double nb = nc * 0.5 * ((4.0 * sizeof(T) + 3.0 * sizeof(typename VFace<T>::type)) * (double)ncell(g));
     // threads: x-pairs x rows x groups of GS_PZ planes, in the level's block shape
     const dim3 bk = L.gs_blk, gr = gs_grid(g, bk);
     const char *name = kGsName[sizeof(T) == 4][l < 7 ? l : 7];
+    const V3<const T> none = V3<const T>();
     for (int s = 0; s < 2; s++) {
         const int z = (s == 0 && zero_start) ? 1 : 0;
         // the plain passes of FP32 levels with half-rows of a multiple of 4
@@ -3429,33 +3672,38 @@ int cc_smooth2(Ctx *c, const CcLevel &L, int l, T *x, T *t, const T *b, bool red
         auto plain = [&](int color, int zs) {
             if constexpr (sizeof(T) == 4) {
                 if (gs4_ok(g)) {
+                    const dim3 g4 = gs4_grid(g, L.gs4_blk, L.gs4_pz);
                     if (L.gs4_pz == 1)
-                        EBV_LAUNCH_P(c, name, nb, (k_cc_gs4<1>), gs4_grid(g, L.gs4_blk, 1), L.gs4_blk, 0, A, x, b,
+                        EBV_LAUNCH_P(c, name, nb, (k_cc_gs4<1>), comp_grid(g4, nc), L.gs4_blk, 0, A, x, b, g4.z, act,
                                      color, zs);
                     else
-                        EBV_LAUNCH_P(c, name, nb, (k_cc_gs4<2>), gs4_grid(g, L.gs4_blk, 2), L.gs4_blk, 0, A, x, b,
+                        EBV_LAUNCH_P(c, name, nb, (k_cc_gs4<2>), comp_grid(g4, nc), L.gs4_blk, 0, A, x, b, g4.z, act,
                                      color, zs);
                     return;
                 }
             }
-            EBV_LAUNCH_P(c, name, nb, (k_cc_gs<T, false>), gr, bk, 0, A, x, b, color, zs, nullptr, GridD());
+            EBV_LAUNCH_P(c, name, nb, (k_cc_gs<T, false>), comp_grid(gr, nc), bk, 0, A, x, b, gr.z, act, color, zs, none,
+                         GridD());
         };
-        if (s == 0 && xc) {  // the first pass after the coarse-grid correction (+ the coarse array)
+        if (s == 0 && corr) {  // the first pass after the coarse-grid correction (+ the coarse array)
             const char *nmc = kGsCorrName[sizeof(T) == 4][l < 7 ? l : 7];
-            const double nbc = nb + 0.125 * sizeof(T) * (double)ncell(g);
+            const double nbc = nb + nc * 0.125 * sizeof(T) * (double)ncell(g);
             bool done = false;
             if constexpr (sizeof(T) == 4) {
                 if (gs4_ok(g)) {   // vectorised, same results
+                    const dim3 g4 = gs4_grid(g, L.gs4_blk, L.gs4_pz);
                     if (L.gs4_pz == 1)
-                        EBV_LAUNCH_P(c, nmc, nbc, (k_cc_gs4<1, true>), gs4_grid(g, L.gs4_blk, 1), L.gs4_blk, 0, A, x, b,
-                                     c0, z, xc, *gc);
+                        EBV_LAUNCH_P(c, nmc, nbc, (k_cc_gs4<1, true>), comp_grid(g4, nc), L.gs4_blk, 0, A, x, b, g4.z,
+                                     act, c0, z, xc, *gc);
                     else
-                        EBV_LAUNCH_P(c, nmc, nbc, (k_cc_gs4<2, true>), gs4_grid(g, L.gs4_blk, 2), L.gs4_blk, 0, A, x, b,
-                                     c0, z, xc, *gc);
+                        EBV_LAUNCH_P(c, nmc, nbc, (k_cc_gs4<2, true>), comp_grid(g4, nc), L.gs4_blk, 0, A, x, b, g4.z,
+                                     act, c0, z, xc, *gc);
                     done = true;
                 }
             }
-            if (!done) EBV_LAUNCH_P(c, nmc, nbc, (k_cc_gs<T, true>), gr, bk, 0, A, x, b, c0, z, xc, *gc);
+            if (!done)
+                EBV_LAUNCH_P(c, nmc, nbc, (k_cc_gs<T, true>), comp_grid(gr, nc), bk, 0, A, x, b, gr.z, act, c0, z, xc,
+                             *gc);
         }
         else
             plain(c0, z);
@@ -3464,14 +3712,16 @@ int cc_smooth2(Ctx *c, const CcLevel &L, int l, T *x, T *t, const T *b, bool red
             if constexpr (sizeof(T) == 4) {
                 const dim3 gt((g.nx / 2 + RB_HW - 1) / RB_HW, (g.ny + RB_TY - 1) / RB_TY,
                               (g.nz + kGs2Planes - 1) / kGs2Planes);
-                EBV_LAUNCH_P(c, kGsDotName[1], nb, k_cc_gs2_dot, gt, dim3(RB_THREADS), 0, A, x, b, 1 - c0, dot_part);
+                EBV_LAUNCH_P(c, kGsDotName[1], nb, k_cc_gs2_dot, comp_grid(gt, nc), dim3(RB_THREADS), 0, A, x, b, gt.z,
+                             act, 1 - c0, dot_part);
                 return rb_ntiles(g) * g.nz;
             }
         } else if (s == 1 && dot_part) {
             // fixed block shape: the grouping of its partial sums must not
             // follow the autotuned shape, or results would depend on timing
-            EBV_LAUNCH_P(c, kGsDotName[sizeof(T) == 4], nb, (k_cc_gs<T, false, true>), gs_grid(g, block3()), block3(),
-                         0, A, x, b, 1 - c0, 0, nullptr, GridD(), dot_part);
+            const dim3 gd = gs_grid(g, block3());
+            EBV_LAUNCH_P(c, kGsDotName[sizeof(T) == 4], nb, (k_cc_gs<T, false, true>), comp_grid(gd, nc), block3(), 0, A,
+                         x, b, gd.z, act, 1 - c0, 0, none, GridD(), dot_part);
         } else {
             plain(1 - c0, 0);
         }
@@ -3485,20 +3735,22 @@ int cc_smooth2(Ctx *c, const CcLevel &L, int l, T *x, T *t, const T *b, bool red
 // cluster kernel, where it takes that level) also writes block partials of
 // b0.x0; returns their number (0 with a single level, or without dot_part).
 template <class T>
-int cc_vcycle(Ctx *c, CcHier &H, const T *b0, T *x0, double *dot_part = nullptr)
+int cc_vcycle(Ctx *c, CcHier &H, int nc, const int *act, V3<const T> b0, V3<T> x0, double *dot_part = nullptr)
 {
     const int Lb = H.L - 1;
     // levels l0 .. Lb run in one cluster
     CoarseVC<T> D;
     const int lc = cv_plan<T>(H, D), l0 = lc < 0 ? Lb : lc;
+    auto X = [&](int l) { return l ? comp_vec<T>(c, c->lx[l], Ctx::CV_X, l) : x0; };
+    auto B = [&](int l) { return l ? V3<const T>(comp_vec<T>(c, c->lb[l], Ctx::CV_B, l)) : b0; };
+    auto Tv = [&](int l) { return comp_vec<T>(c, c->lt[l], Ctx::CV_T, l); };
     for (int l = 0; l < l0; l++) {
         const CcLevel &L = H.lv[l];
-        T *x = l ? (T *)c->lx[l] : x0;
-        const T *b = l ? (const T *)c->lb[l] : b0;
-        cc_smooth2<T>(c, L, l, x, (T *)c->lt[l], b, true, true);
+        cc_smooth2<T>(c, H, l, nc, act, X(l), Tv(l), B(l), true, true);
         const CcLevel &Lc = H.lv[l + 1];
+        const V3<T> bc = comp_vec<T>(c, c->lb[l + 1], Ctx::CV_B, l + 1);
         // x, b, diagonal, 3 faces (storage type) read, 1/8 word written
-        const double nbr = ((3.0 + 1.0 / 8.0) * sizeof(T) + 3.0 * sizeof(typename VFace<T>::type)) * (double)ncell(L.g);
+        const double nbr = nc * ((3.0 + 1.0 / 8.0) * sizeof(T) + 3.0 * sizeof(typename VFace<T>::type)) * (double)ncell(L.g);
         const char *nmr = kRrName[sizeof(T) == 4][l < 3 ? l : 3];
         bool vec = false;
         if constexpr (sizeof(T) == 4) {
@@ -3506,40 +3758,41 @@ int cc_vcycle(Ctx *c, CcHier &H, const T *b0, T *x0, double *dot_part = nullptr)
                                         (Lc.g.nz + bk.z - 1) / bk.z);
             // four coarse cells per thread, vector loads (same results), where
             // that still gives two blocks per SM (small levels keep the scalar kernel)
-            if (gs4_ok(L.g) && (long long)gr.x * gr.y * gr.z >= kVecMinBlocks) {
-                EBV_LAUNCH_P(c, nmr, nbr, k_cc_rr4, gr, bk, 0, vop<float>(L), x, b, Lc.g, (float *)c->lb[l + 1]);
+            if (gs4_ok(L.g) && (long long)gr.x * gr.y * gr.z * nc >= kVecMinBlocks) {
+                EBV_LAUNCH_P(c, nmr, nbr, k_cc_rr4, comp_grid(gr, nc), bk, 0, vop3<float>(H, l, nc), X(l), B(l), Lc.g, bc,
+                             gr.z, act);
                 vec = true;
             }
         }
-        if (!vec)
-            EBV_LAUNCH_P(c, nmr, nbr, k_cc_resid_restrict<T>, cgrid(Lc.g), block3(), 0, vop<T>(L), x, b, Lc.g,
-                         (T *)c->lb[l + 1]);
+        if (!vec) {
+            const dim3 gr = cgrid(Lc.g);
+            EBV_LAUNCH_P(c, nmr, nbr, k_cc_resid_restrict<T>, comp_grid(gr, nc), block3(), 0, vop3<T>(H, l, nc), X(l),
+                         B(l), Lc.g, bc, gr.z, act);
+        }
     }
+    V3<const double> binv = one<const double>(H.binv);
+    if (nc > 1)
+        for (int q = 0; q < nc; q++) binv.p[q] = H.vbinv[q];
     if (l0 < Lb) {
-        for (int q = 0; q < D.n; q++) D.A[q] = vop<T>(H.lv[l0 + q]);
-        D.x = l0 ? (T *)c->lx[l0] : x0;
-        D.b = l0 ? (const T *)c->lb[l0] : b0;
-        D.binv = H.binv;
+        for (int q = 0; q < D.n; q++) D.A3[q] = vop3<T>(H, l0 + q, nc);
+        D.x = X(l0);
+        D.b = B(l0);
+        D.binv = binv;
         D.nb = H.nb;
         D.part = l0 == 0 ? dot_part : nullptr;
         const size_t bytes = D.L.total;
         const char *nm = sizeof(T) == 4 ? "cc_coarse_vcycle<float>" : "cc_coarse_vcycle<double>";
         cv_attr<T>();
-        EBV_LAUNCH_P(c, nm, 0.0, k_cc_coarse_vcycle<T>, dim3(kCvCtas), dim3(kCvThreads), bytes, D);
+        EBV_LAUNCH_P(c, nm, 0.0, k_cc_coarse_vcycle<T>, dim3(kCvCtas, nc), dim3(kCvThreads), bytes, D);
         if (l0 == 0) return dot_part ? kCvCtas : 0;
     } else {
-        T *x = Lb ? (T *)c->lx[Lb] : x0;
-        const T *b = Lb ? (const T *)c->lb[Lb] : b0;
-        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 255) / 256), dim3(256), 0, H.binv, H.nb, b, x, 1.0,
+        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 255) / 256, nc), dim3(256), 0, binv, H.nb, B(Lb), X(Lb), 1.0,
                    H.lv[Lb].g, (int)(sizeof(T) == 4));
     }
     for (int l = l0 - 1; l >= 0; l--) {
-        const CcLevel &L = H.lv[l];
-        T *x = l ? (T *)c->lx[l] : x0;
-        const T *b = l ? (const T *)c->lb[l] : b0;
         // prolongation folded into the first colour pass of the post-smoothing
-        const int nd = cc_smooth2<T>(c, L, l, x, (T *)c->lt[l], b, false, false, (const T *)c->lx[l + 1],
-                                     &H.lv[l + 1].g, l == 0 ? dot_part : nullptr);
+        const int nd = cc_smooth2<T>(c, H, l, nc, act, X(l), Tv(l), B(l), false, false, X(l + 1), &H.lv[l + 1].g,
+                                     l == 0 ? dot_part : nullptr);
         if (l == 0) return nd;
     }
     return 0;
@@ -3637,8 +3890,8 @@ void nd_vcycle(Ctx *c, NdHier &H, const T *b0, T *x0)
     {
         T *x = Lb ? (T *)c->lx[Lb] : x0;
         const T *b = Lb ? (const T *)c->lb[Lb] : b0;
-        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 255) / 256), dim3(256), 0, H.binv, H.nb, b, x, 1.0,
-                   H.lv[Lb].g, 0);
+        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 255) / 256), dim3(256), 0, one<const double>(H.binv), H.nb,
+                   one<const T>(b), one(x), 1.0, H.lv[Lb].g, 0);
     }
     for (int l = Lb - 1; l >= 0; l--) {
         const NdLevel &L = H.lv[l];
@@ -3655,32 +3908,29 @@ void nd_vcycle(Ctx *c, NdHier &H, const T *b0, T *x0)
 // Preconditioned conjugate gradients
 // ---------------------------------------------------------------------------
 
+// act: the loop condition words that gate a kernel's components (see comp_off),
+// given where skipping an ended component saves more than the word's load costs
 struct Problem {
+    int nc = 1;                                // components solved together
     virtual ~Problem() {}
     virtual int n() const = 0;
     virtual int apply_blocks() const = 0;      // partial sums written by apply_dot
     virtual int apply_blocks32() const { return apply_blocks(); }   // by apply_dot32
     virtual int resid_blocks() const { return apply_blocks(); }     // by resid32
     // q = A p with block partials of p.q in c->part, in FP64 or FP32
-    virtual void apply_dot(Ctx *c, const double *p, double *q) = 0;
-    virtual void apply_dot32(Ctx *c, const float *p, float *q) = 0;
-    // z = one V-cycle applied to r, in FP64 or FP32
-    virtual void precond(Ctx *c, const double *r, double *z) = 0;
-    virtual void precond32(Ctx *c, const float *r, float *z) = 0;
-    // precond32 that may also leave block partials of r.z in c->part:
-    // returns their number, 0 if it did not
-    virtual int precond32_dot(Ctx *c, const float *r, float *z)
-    {
-        precond32(c, r, z);
-        return 0;
-    }
+    virtual void apply_dot(Ctx *c, V3<const double> p, V3<double> q, const int *act) = 0;
+    virtual void apply_dot32(Ctx *c, V3<const float> p, V3<float> q, const int *act) = 0;
+    // z = one V-cycle applied to r, in FP64, or in FP32 possibly leaving block
+    // partials of r.z in c->part: returns their number, 0 if it did not
+    virtual void precond(Ctx *c, V3<const double> r, V3<double> z, const int *act) = 0;
+    virtual int precond32_dot(Ctx *c, V3<const float> r, V3<float> z, const int *act) = 0;
     // FP64 <-> FP32 vectors of the refinement solver (the FP32 side in the
     // layout of the problem's FP32 multigrid): r = b - A x in FP64 with
     // resid_blocks() block partials of |r|^2 in c->part; x += e
-    virtual void resid32(Ctx *c, const double *b, const double *x, float *r) = 0;
-    virtual void to32(Ctx *c, const double *b, float *r) = 0;   // r = b in the FP32 layout
+    virtual void resid32(Ctx *c, V3<const double> b, V3<const double> x, V3<float> r, const int *act) = 0;
+    virtual void to32(Ctx *c, V3<const double> b, V3<float> r) = 0;   // r = b in the FP32 layout
     // x += e + the deferred last step of the correction solve (search direction p)
-    virtual void add32(Ctx *c, double *x, const float *e, const float *p) = 0;
+    virtual void add32(Ctx *c, V3<double> x, V3<const float> e, V3<const float> p, const int *act) = 0;
 };
 
 inline int vblocks(int n) { return std::min(kReduceBlocks, (n + 255) / 256); }
@@ -3776,82 +4026,97 @@ struct DevLoop {
 
 // Issues the end-of-solve kernels and, in eager mode, reads the solve's
 // statistics and status back.
-ebv_status finish_solve(Ctx *c, double *x, int n, int *iters, double *res)
+ebv_status finish_solve(Ctx *c, int nc, V3<double> x, int n, int *iters, double *res)
 {
-    EBV_LAUNCH(c, k_zero_if, dim3(vblocks(n)), dim3(256), 0, x, n, c->ctl);
-    EBV_LAUNCH(c, k_solve_end, dim3(1), dim3(32), 0, c->scal, c->ctl, c->prm.tol, c->sstat, c->cur_slot);
+    EBV_LAUNCH(c, k_zero_if, dim3(vblocks(n), nc), dim3(256), 0, x, n, c->ctl);
+    EBV_LAUNCH(c, k_solve_end, dim3(1), dim3(32), 0, c->scal, c->ctl, nc, c->prm.tol, c->sstat, c->cur_slot);
     if (c->capturing) {
-        if (iters) *iters = 0;
-        if (res) *res = 0.0;
+        for (int q = 0; q < nc; q++) {
+            if (iters) iters[q] = 0;
+            if (res) res[q] = 0.0;
+        }
         return EBV_OK;
     }
-    const int s = c->cur_slot;
-    EBV_CUDA_TRY(c, cudaMemcpyAsync(c->sstat_host + 3 * s, c->sstat + 3 * s, 3 * sizeof(double),
+    const int s0 = c->cur_slot;
+    EBV_CUDA_TRY(c, cudaMemcpyAsync(c->sstat_host + 3 * s0, c->sstat + 3 * s0, 3 * nc * sizeof(double),
                                     cudaMemcpyDeviceToHost, c->stream));
-    EBV_CUDA_TRY(c, cudaMemcpyAsync(c->ctl_host + C_ERR, c->ctl + C_ERR, sizeof(int), cudaMemcpyDeviceToHost,
-                                    c->stream));
+    EBV_CUDA_TRY(c, cudaMemcpyAsync(c->ctl_host, c->ctl, nc * C_LEN * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     EBV_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    if (iters) *iters = (int)c->sstat_host[3 * s];
-    if (res) *res = c->sstat_host[3 * s + 1];
-    if (c->ctl_host[C_ERR] == E_NAN)
-        return c->fail(EBV_ERR_NAN, "non-finite residual (solve slot " + std::to_string(s) + ")");
-    if (c->ctl_host[C_ERR] == E_SMEM)
-        return c->fail(EBV_ERR_CUDA, "shared memory of the fused sweep not 128-byte aligned (solve slot " +
-                                         std::to_string(s) + ")");
-    if (c->ctl_host[C_ERR] == E_TIMEOUT)
-        return c->fail(EBV_ERR_TIMEOUT, "a bounded wait in the smoother gave up (solve slot " + std::to_string(s) + ")");
-    if (c->ctl_host[C_ERR] == E_NOTCONV)
-        return c->fail(EBV_ERR_NOT_CONVERGED, "linear solve did not reach the tolerance (solve slot " +
-                                                  std::to_string(s) + ", relative residual " +
-                                                  std::to_string(c->sstat_host[3 * s + 1]) + ", " +
-                                                  std::to_string((int)c->sstat_host[3 * s]) + " iterations)");
+    for (int q = 0; q < nc; q++) {
+        if (iters) iters[q] = (int)c->sstat_host[3 * (s0 + q)];
+        if (res) res[q] = c->sstat_host[3 * (s0 + q) + 1];
+    }
+    for (int q = 0; q < nc; q++) {
+        const int e = c->ctl_host[q * C_LEN + C_ERR], s = s0 + q;
+        if (e == E_NAN) return c->fail(EBV_ERR_NAN, "non-finite residual (solve slot " + std::to_string(s) + ")");
+        if (e == E_SMEM)
+            return c->fail(EBV_ERR_CUDA, "shared memory of the fused sweep not 128-byte aligned (solve slot " +
+                                             std::to_string(s) + ")");
+        if (e == E_TIMEOUT)
+            return c->fail(EBV_ERR_TIMEOUT, "a bounded wait in the smoother gave up (solve slot " + std::to_string(s) + ")");
+        if (e == E_NOTCONV)
+            return c->fail(EBV_ERR_NOT_CONVERGED, "linear solve did not reach the tolerance (solve slot " +
+                                                      std::to_string(s) + ", relative residual " +
+                                                      std::to_string(c->sstat_host[3 * s + 1]) + ", " +
+                                                      std::to_string((int)c->sstat_host[3 * s]) + " iterations)");
+    }
     return EBV_OK;
 }
+
+// Grids of at least this many cells skip the ended components of a joint solve
+// in every kernel; on smaller ones the condition word's load (half a
+// microsecond before each kernel's first) costs more than the redundant work,
+// which only rewrites scratch vectors.
+constexpr int kGateCells = 1 << 20;
 
 // Preconditioned CG in FP64, restarted from the true residual whenever the
 // recursive one has dropped below tol/2 but the true one is still above tol
 // (at most 20 passes).
-ebv_status pcg(Ctx *c, Problem &P, const double *b, double *x, int *iters, double *res)
+ebv_status pcg(Ctx *c, Problem &P, V3<const double> b, V3<double> x, int *iters, double *res)
 {
-    const int n = P.n();
+    const int n = P.n(), nc = P.nc;
     const double tol = c->prm.tol;
     const int maxit = c->prm.max_iters;
-    double *r = c->kr, *z = c->kz, *p = c->kp, *q = c->kq;
+    const V3<double> r = comp_vec<double>(c, c->kr, Ctx::CV_K, 0), z = comp_vec<double>(c, c->kz, Ctx::CV_K, 1),
+                     p = comp_vec<double>(c, c->kp, Ctx::CV_K, 2), q = comp_vec<double>(c, c->kq, Ctx::CV_K, 3);
+    const int *in = nc > 1 ? c->ctl + C_COND_IN : nullptr, *out = nc > 1 ? c->ctl + C_COND_OUT : nullptr;
+    const int *gin = n >= kGateCells ? in : nullptr;
+    const dim3 gv(vblocks(n), nc);
     auto true_residual = [&]() {
-        P.apply_dot(c, x, q);
-        EBV_LAUNCH(c, k_resid_init, dim3(vblocks(n)), dim3(256), 0, b, q, r, n, c->part);
-        reduce_sum(c, c->part, vblocks(n), c->scal + S_RR);
-        reduce_sum(c, c->part + vblocks(n), vblocks(n), c->scal + S_BB);
+        P.apply_dot(c, x, q, out);
+        EBV_LAUNCH(c, k_resid_init, gv, dim3(256), 0, b, q, r, n, c->part, out);
+        reduce_comp(c, nc, vblocks(n), S_RR, kRedSum, out);
+        reduce_comp(c, nc, vblocks(n), S_BB, kRedSum, out, c->part + vblocks(n));
     };
-    EBV_LAUNCH(c, k_solve_begin, dim3(1), dim3(32), 0, c->ctl);
-    DevLoop outer(c, C_COND_OUT);
+    EBV_LAUNCH(c, k_solve_begin, dim3(1), dim3(32), 0, c->ctl, nc);
+    DevLoop outer(c, J_OUT);
     true_residual();
-    EBV_LAUNCH(c, k_outer_check, dim3(1), dim3(32), 0, c->scal, c->ctl, tol, maxit, 20, 0, 0.0, outer.h,
+    EBV_LAUNCH(c, k_outer_check, dim3(1), dim3(32), 0, c->scal, c->ctl, nc, tol, maxit, 20, 0, 0.0, outer.h,
                outer.use_h);
     int inner_count = 0;
     while (outer.next()) {
-        DevLoop inner(c, C_COND_IN);
-        EBV_LAUNCH(c, k_set_cond, dim3(1), dim3(32), 0, c->ctl, C_COND_IN, 1, inner.h, inner.use_h);
+        DevLoop inner(c, J_IN);
+        EBV_LAUNCH(c, k_inner_begin, dim3(1), dim3(32), 0, c->ctl, nc, inner.h, inner.use_h);
         while (inner.next()) {
-            P.precond(c, r, z);
-            EBV_LAUNCH(c, k_dot, dim3(vblocks(n)), dim3(256), 0, r, z, n, c->part);
-            reduce_rz(c, vblocks(n));
-            EBV_LAUNCH(c, k_cg_pupdate, dim3(vblocks(n)), dim3(256), 0, p, z, c->scal, n, c->ctl);
-            P.apply_dot(c, p, q);
-            reduce_pq(c, P.apply_blocks());
-            EBV_LAUNCH(c, k_cg_update, dim3(vblocks(n)), dim3(256), 0, x, r, p, q, c->scal, n, c->part);
-            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, vblocks(n), c->scal, c->ctl, tol,
+            P.precond(c, r, z, gin);
+            EBV_LAUNCH(c, k_dot, gv, dim3(256), 0, r, z, n, c->part);
+            reduce_comp(c, nc, vblocks(n), S_RZ, kRedBeta, in);
+            EBV_LAUNCH(c, k_cg_pupdate, gv, dim3(256), 0, p, z, c->scal, n, c->ctl, in);
+            P.apply_dot(c, p, q, gin);
+            reduce_comp(c, nc, P.apply_blocks(), S_PQ, kRedAlpha, in);
+            EBV_LAUNCH(c, k_cg_update, gv, dim3(256), 0, x, r, p, q, c->scal, n, c->part, in);
+            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, vblocks(n), c->scal, c->ctl, nc, tol,
                        maxit, 0, inner.h, inner.use_h);
         }
         inner_count = inner.body_launches();
         true_residual();
-        EBV_LAUNCH(c, k_outer_check, dim3(1), dim3(32), 0, c->scal, c->ctl, tol, maxit, 20, 0, 0.0, outer.h,
+        EBV_LAUNCH(c, k_outer_check, dim3(1), dim3(32), 0, c->scal, c->ctl, nc, tol, maxit, 20, 0, 0.0, outer.h,
                    outer.use_h);
     }
     if (c->capturing)
         c->loop_recs.push_back({c->cur_slot, outer.body_launches() - inner_count, inner_count});
     if (!c->cap_err.empty() && c->capturing) return c->fail(EBV_ERR_CUDA, "graph capture: " + c->cap_err);
-    return finish_solve(c, x, n, iters, res);
+    return finish_solve(c, nc, x, n, iters, res);
 }
 
 // Iterative refinement for the FP32 path: the residual r = b - A x and the
@@ -3860,13 +4125,18 @@ ebv_status pcg(Ctx *c, Problem &P, const double *b, double *x, int *iters, doubl
 // coefficients, V-cycle) until its residual drops by `inner_drop` (or it
 // stalls), so FP64 arithmetic is spent once per refinement step instead of in
 // every Krylov iteration.  At most 60 corrections.
-ebv_status pcg_refine(Ctx *c, Problem &P, const double *b, double *x, int *iters, double *res, bool x_zero)
+ebv_status pcg_refine(Ctx *c, Problem &P, V3<const double> b, V3<double> x, int *iters, double *res, bool x_zero)
 {
-    const int n = P.n();
+    const int n = P.n(), nc = P.nc;
     const double tol = c->prm.tol;
     const int maxit = c->prm.max_iters;
     const double inner_drop = refine_inner_drop();
-    float *r = c->kr32, *z = c->kz32, *p = c->kp32, *q = c->kq32, *e = c->ke32;
+    const V3<float> r = comp_vec<float>(c, c->kr32, Ctx::CV_K, 0), z = comp_vec<float>(c, c->kz32, Ctx::CV_K, 1),
+                    p = comp_vec<float>(c, c->kp32, Ctx::CV_K, 2), q = comp_vec<float>(c, c->kq32, Ctx::CV_K, 3),
+                    e = comp_vec<float>(c, c->ke32, Ctx::CV_K, 4);
+    const int *in = nc > 1 ? c->ctl + C_COND_IN : nullptr, *out = nc > 1 ? c->ctl + C_COND_OUT : nullptr;
+    const int *gin = n >= kGateCells ? in : nullptr;
+    const dim3 gv(vblocks(n), nc), g4(v4blocks(n), nc);
     // x_zero: the first residual is b itself (its norm is |b|^2, reduced below)
     bool first_is_b = x_zero;
     auto true_residual = [&]() {
@@ -3875,42 +4145,42 @@ ebv_status pcg_refine(Ctx *c, Problem &P, const double *b, double *x, int *iters
             P.to32(c, b, r);
             return;
         }
-        P.resid32(c, b, x, r);
-        reduce_sum(c, c->part, P.resid_blocks(), c->scal + S_RR);
+        P.resid32(c, b, x, r, out);
+        reduce_comp(c, nc, P.resid_blocks(), S_RR, kRedSum, out);
     };
-    EBV_LAUNCH(c, k_solve_begin, dim3(1), dim3(32), 0, c->ctl);
-    EBV_LAUNCH(c, k_dot, dim3(vblocks(n)), dim3(256), 0, b, b, n, c->part);
-    reduce_sum(c, c->part, vblocks(n), c->scal + S_BB);
-    EBV_LAUNCH(c, k_set_sigma, dim3(1), dim3(32), 0, c->scal, x_zero ? 1 : 0);
-    DevLoop outer(c, C_COND_OUT);
+    EBV_LAUNCH(c, k_solve_begin, dim3(1), dim3(32), 0, c->ctl, nc);
+    EBV_LAUNCH(c, k_dot, gv, dim3(256), 0, b, b, n, c->part);
+    reduce_comp(c, nc, vblocks(n), S_BB);
+    EBV_LAUNCH(c, k_set_sigma, dim3(1), dim3(32), 0, c->scal, nc, x_zero ? 1 : 0);
+    DevLoop outer(c, J_OUT);
     true_residual();
-    EBV_LAUNCH(c, k_outer_check, dim3(1), dim3(32), 0, c->scal, c->ctl, tol, maxit, 60, 1, inner_drop, outer.h,
+    EBV_LAUNCH(c, k_outer_check, dim3(1), dim3(32), 0, c->scal, c->ctl, nc, tol, maxit, 60, 1, inner_drop, outer.h,
                outer.use_h);
     int inner_count = 0;
     while (outer.next()) {
-        DevLoop inner(c, C_COND_IN);
-        EBV_LAUNCH(c, k_set_cond, dim3(1), dim3(32), 0, c->ctl, C_COND_IN, 1, inner.h, inner.use_h);
+        DevLoop inner(c, J_IN);
+        EBV_LAUNCH(c, k_inner_begin, dim3(1), dim3(32), 0, c->ctl, nc, inner.h, inner.use_h);
         while (inner.next()) {
-            const int nd = P.precond32_dot(c, r, z);
-            if (!nd) EBV_LAUNCH(c, k_dot32, dim3(v4blocks(n)), dim3(256), 0, r, z, n, c->part);
-            reduce_rz(c, nd ? nd : v4blocks(n));
-            EBV_LAUNCH(c, k_cg_pupdate32, dim3(v4blocks(n)), dim3(256), 0, p, e, z, c->scal, n, c->ctl);
-            P.apply_dot32(c, p, q);
-            reduce_pq(c, P.apply_blocks32());
-            EBV_LAUNCH(c, k_cg_update32, dim3(v4blocks(n)), dim3(256), 0, r, q, c->scal, n, c->part);
-            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, v4blocks(n), c->scal, c->ctl, tol,
+            const int nd = P.precond32_dot(c, r, z, gin);
+            if (!nd) EBV_LAUNCH(c, k_dot32, g4, dim3(256), 0, r, z, n, c->part);
+            reduce_comp(c, nc, nd ? nd : v4blocks(n), S_RZ, kRedBeta, in);
+            EBV_LAUNCH(c, k_cg_pupdate32, g4, dim3(256), 0, p, e, z, c->scal, n, c->ctl, in);
+            P.apply_dot32(c, p, q, gin);
+            reduce_comp(c, nc, P.apply_blocks32(), S_PQ, kRedAlpha, in);
+            EBV_LAUNCH(c, k_cg_update32, g4, dim3(256), 0, r, q, c->scal, n, c->part, in);
+            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, v4blocks(n), c->scal, c->ctl, nc, tol,
                        maxit, 1, inner.h, inner.use_h);
         }
         inner_count = inner.body_launches();
-        P.add32(c, x, e, p);
+        P.add32(c, x, e, p, out);
         true_residual();
-        EBV_LAUNCH(c, k_outer_check, dim3(1), dim3(32), 0, c->scal, c->ctl, tol, maxit, 60, 1, inner_drop,
+        EBV_LAUNCH(c, k_outer_check, dim3(1), dim3(32), 0, c->scal, c->ctl, nc, tol, maxit, 60, 1, inner_drop,
                    outer.h, outer.use_h);
     }
     if (c->capturing)
         c->loop_recs.push_back({c->cur_slot, outer.body_launches() - inner_count, inner_count});
     if (!c->cap_err.empty() && c->capturing) return c->fail(EBV_ERR_CUDA, "graph capture: " + c->cap_err);
-    return finish_solve(c, x, n, iters, res);
+    return finish_solve(c, nc, x, n, iters, res);
 }
 
 struct CcProblem : Problem {
@@ -3919,44 +4189,56 @@ struct CcProblem : Problem {
     // two planes per thread
     dim3 agrid() const { const GridD &g = H->lv[0].g; return grid3(g.nx, g.ny, (g.nz + 1) / 2); }
     int apply_blocks() const override { return nblocks3(agrid()); }
-    void apply_dot(Ctx *c, const double *p, double *q) override
+    void apply_dot(Ctx *c, V3<const double> p, V3<double> q, const int *act) override
     {
         // p, diagonal, 3 faces, q: 6 words per cell
-        EBV_LAUNCH_P(c, "cc_apply_fp64", 48.0 * n(), k_cc_apply_dot<double>, agrid(), block3(), 0,
-                     ccop<double>(H->lv[0]), p, q, c->part);
+        const dim3 gr = agrid();
+        EBV_LAUNCH_P(c, "cc_apply_fp64", nc * 48.0 * n(), k_cc_apply_dot<double>, comp_grid(gr, nc), block3(), 0,
+                     ccop3<double>(*H, nc), p, q, c->part, gr.z, act);
     }
     // FP32 levels with nx a multiple of 8 large enough for two blocks per SM:
     // the vectorised apply (its own partials; the choice follows the grid only)
     bool vec32() const
     {
-        return gs4_ok(H->lv[0].g) && nblocks3(apply4_grid(H->lv[0].g)) >= kVecMinBlocks;
+        return gs4_ok(H->lv[0].g) && nc * nblocks3(apply4_grid(H->lv[0].g)) >= kVecMinBlocks;
     }
     int apply_blocks32() const override { return vec32() ? nblocks3(apply4_grid(H->lv[0].g)) : apply_blocks(); }
-    void apply_dot32(Ctx *c, const float *p, float *q) override
+    void apply_dot32(Ctx *c, V3<const float> p, V3<float> q, const int *act) override
     {
+        const dim3 g4 = apply4_grid(H->lv[0].g), gr = agrid();
         if (vec32())
-            EBV_LAUNCH_P(c, "cc_apply_fp32", 24.0 * n(), k_cc_apply4, apply4_grid(H->lv[0].g),
-                         dim3(kApply4X, kApply4Y, kApply4Z), 0, ccop<float>(H->lv[0]), p, q, c->part);
+            EBV_LAUNCH_P(c, "cc_apply_fp32", nc * 24.0 * n(), k_cc_apply4, comp_grid(g4, nc),
+                         dim3(kApply4X, kApply4Y, kApply4Z), 0, ccop3<float>(*H, nc), p, q, c->part, g4.z, act);
         else
-            EBV_LAUNCH_P(c, "cc_apply_fp32", 24.0 * n(), k_cc_apply_dot<float>, agrid(), block3(), 0,
-                         ccop<float>(H->lv[0]), p, q, c->part);
+            EBV_LAUNCH_P(c, "cc_apply_fp32", nc * 24.0 * n(), k_cc_apply_dot<float>, comp_grid(gr, nc), block3(), 0,
+                         ccop3<float>(*H, nc), p, q, c->part, gr.z, act);
     }
-    void precond(Ctx *c, const double *r, double *z) override { cc_vcycle<double>(c, *H, r, z); }
-    void precond32(Ctx *c, const float *r, float *z) override { cc_vcycle<float>(c, *H, r, z); }
-    int precond32_dot(Ctx *c, const float *r, float *z) override { return cc_vcycle<float>(c, *H, r, z, c->part); }
-    void resid32(Ctx *c, const double *b, const double *x, float *r) override
+    void precond(Ctx *c, V3<const double> r, V3<double> z, const int *act) override
+    {
+        cc_vcycle<double>(c, *H, nc, act, r, z);
+    }
+    int precond32_dot(Ctx *c, V3<const float> r, V3<float> z, const int *act) override
+    {
+        return cc_vcycle<float>(c, *H, nc, act, r, z, c->part);
+    }
+    void resid32(Ctx *c, V3<const double> b, V3<const double> x, V3<float> r, const int *act) override
     {
         // x, diagonal, 3 faces, b read, r (FP32) written: 6.5 words per cell
-        EBV_LAUNCH_P(c, "cc_resid_fp64", 52.0 * n(), (k_cc_apply_dot<double, true>), agrid(), block3(), 0,
-                     ccop<double>(H->lv[0]), x, (double *)nullptr, c->part, b, r, c->scal + S_SIG);
+        const dim3 gr = agrid();
+        EBV_LAUNCH_P(c, "cc_resid_fp64", nc * 52.0 * n(), (k_cc_apply_dot<double, true>), comp_grid(gr, nc), block3(), 0,
+                     ccop3<double>(*H, nc), x, V3<double>(), c->part, gr.z, act, b, r, c->scal + S_SIG);
     }
-    void add32(Ctx *c, double *x, const float *e, const float *p) override
+    void add32(Ctx *c, V3<double> x, V3<const float> e, V3<const float> p, const int *act) override
     {
-        EBV_LAUNCH(c, k_add32to64_split, add_grid(H->lv[0].g), dim3(32, 8), 0, H->lv[0].g, x, e, p, c->scal, c->ctl);
+        const dim3 gr = add_grid(H->lv[0].g);
+        EBV_LAUNCH(c, k_add32to64_split, comp_grid(gr, nc), dim3(32, 8), 0, H->lv[0].g, x, e, p, c->scal, c->ctl, gr.z,
+                   act);
     }
-    void to32(Ctx *c, const double *b, float *r) override
+    void to32(Ctx *c, V3<const double> b, V3<float> r) override
     {
-        EBV_LAUNCH(c, k_to_split, dim3(vblocks(n())), dim3(256), 0, H->lv[0].g, -1, b, r, c->scal + S_SIG);
+        for (int q = 0; q < nc; q++)
+            EBV_LAUNCH(c, k_to_split, dim3(vblocks(n())), dim3(256), 0, H->lv[0].g, -1, b.p[q], r.p[q],
+                       c->scal + q * kScalLen + S_SIG);
     }
 };
 
@@ -3964,41 +4246,91 @@ struct NdProblem : Problem {
     NdHier *H;
     int n() const override { return nnode(H->lv[0].g); }
     int apply_blocks() const override { return nd_tile_parts(H->lv[0]); }
-    void apply_dot(Ctx *c, const double *p, double *q) override
+    void apply_dot(Ctx *c, V3<const double> p, V3<double> q, const int *) override
     {
         // p read, q written, act and reg flags: 2.25 words per node
-        nd_tile_pass<double, ND_APPLY>(c, H->lv[0], "nodal_apply_fp64", 18.0 * n(), p, q, nullptr, nullptr, 0.0, 0.0,
-                                       c->part);
+        nd_tile_pass<double, ND_APPLY>(c, H->lv[0], "nodal_apply_fp64", 18.0 * n(), p.p[0], q.p[0], nullptr, nullptr, 0.0,
+                                       0.0, c->part);
     }
-    void apply_dot32(Ctx *c, const float *p, float *q) override
+    void apply_dot32(Ctx *c, V3<const float> p, V3<float> q, const int *) override
     {
-        nd_tile_pass<float, ND_APPLY>(c, H->lv[0], "nodal_apply_fp32", 12.0 * n(), p, q, nullptr, nullptr, 0.0f,
+        nd_tile_pass<float, ND_APPLY>(c, H->lv[0], "nodal_apply_fp32", 12.0 * n(), p.p[0], q.p[0], nullptr, nullptr, 0.0f,
                                     0.0f, c->part);
     }
-    void precond(Ctx *c, const double *r, double *z) override { nd_vcycle<double>(c, *H, r, z); }
-    void precond32(Ctx *c, const float *r, float *z) override { nd_vcycle<float>(c, *H, r, z); }
-    void resid32(Ctx *c, const double *b, const double *x, float *r) override
+    void precond(Ctx *c, V3<const double> r, V3<double> z, const int *) override
+    {
+        nd_vcycle<double>(c, *H, r.p[0], z.p[0]);
+    }
+    int precond32_dot(Ctx *c, V3<const float> r, V3<float> z, const int *) override
+    {
+        nd_vcycle<float>(c, *H, r.p[0], z.p[0]);
+        return 0;
+    }
+    void resid32(Ctx *c, V3<const double> b, V3<const double> x, V3<float> r, const int *) override
     {
         // x, b read, r (FP32) written, act and reg flags: 5.25 words per node
-        nd_tile_pass<double, ND_RES32>(c, H->lv[0], "nodal_resid_fp64", 22.0 * n(), x, nullptr, nullptr, b, 0.0,
-                                       0.0, c->part, r, c->scal + S_SIG);
+        nd_tile_pass<double, ND_RES32>(c, H->lv[0], "nodal_resid_fp64", 22.0 * n(), x.p[0], nullptr, nullptr, b.p[0], 0.0,
+                                       0.0, c->part, r.p[0], c->scal + S_SIG);
     }
-    void add32(Ctx *c, double *x, const float *e, const float *p) override
+    void add32(Ctx *c, V3<double> x, V3<const float> e, V3<const float> p, const int *) override
     {
-        EBV_LAUNCH(c, k_add32to64, dim3(vblocks(n())), dim3(256), 0, x, e, p, c->scal, c->ctl, n());
+        EBV_LAUNCH(c, k_add32to64, dim3(vblocks(n())), dim3(256), 0, x.p[0], e.p[0], p.p[0], c->scal, c->ctl, n());
     }
-    void to32(Ctx *c, const double *b, float *r) override
+    void to32(Ctx *c, V3<const double> b, V3<float> r) override
     {
-        EBV_LAUNCH(c, k_to32_scaled, dim3(vblocks(n())), dim3(256), 0, b, r, n(), c->scal + S_SIG);
+        EBV_LAUNCH(c, k_to32_scaled, dim3(vblocks(n())), dim3(256), 0, b.p[0], r.p[0], n(), c->scal + S_SIG);
     }
 };
 
 // x_zero: x holds zeros on entry (lets the refinement solver skip its first
 // operator application)
-ebv_status solve(Ctx *c, Problem &P, const double *b, double *x, int *iters, double *res, bool x_zero = false)
+ebv_status solve(Ctx *c, Problem &P, V3<const double> b, V3<double> x, int *iters, double *res, bool x_zero = false)
 {
     if (c->prm.precision != EBV_FP64) return pcg_refine(c, P, b, x, iters, res, x_zero);
     return pcg(c, P, b, x, iters, res);
+}
+
+// The level and Krylov vectors of components 1 and 2 in precision T, carved
+// from the cell gradients c->G and the face fluxes c->ff: explicit-term scratch
+// that nothing reads during a solve (9 and more than 9 cell fields; about 8.6
+// of each size are needed).  Sets c->joint: whether three components fit, and
+// their partial sums in c->part.
+template <class T>
+void carve_components(Ctx *c)
+{
+    const CcHier &H = c->visc;
+    const size_t N3 = ncell(c->g);
+    char *base[2] = {(char *)c->G, (char *)c->ff};
+    const size_t len[2] = {9 * N3 * 8, 3 * (size_t)(nface(c->g, 0) + nface(c->g, 1) + nface(c->g, 2)) * 8};
+    bool ok = true;
+    for (int q = 0; q < 2; q++) {
+        size_t at = 0;
+        auto take = [&](size_t n) -> void * {
+            void *p = base[q] + at;
+            at += (n * sizeof(T) + 255) / 256 * 256;
+            if (at > len[q]) ok = false;
+            return p;
+        };
+        for (int kind = 0; kind < Ctx::CV_KINDS; kind++)
+            for (int l = 0; l < kMaxLevels; l++) c->cvec[q][kind][l] = nullptr;
+        for (int k = 0; k < 5; k++) c->cvec[q][Ctx::CV_K][k] = take(N3);
+        for (int l = 0; l < H.L; l++) {
+            const size_t n = ncell(H.lv[l].g);
+            c->cvec[q][Ctx::CV_T][l] = take(n);
+            if (l == 0) continue;
+            c->cvec[q][Ctx::CV_X][l] = take(n);
+            c->cvec[q][Ctx::CV_B][l] = take(n);
+        }
+    }
+    CcProblem P;
+    P.H = &c->visc;
+    P.nc = kMaxComp;
+    const GridD &g = c->g;
+    const dim3 gd = gs_grid(g, block3());
+    const size_t tiles = rb_fusable(g) ? (size_t)rb_ntiles(g) * g.nz : 0;
+    const size_t parts = std::max<size_t>(std::max(std::max(P.apply_blocks(), P.apply_blocks32()), nblocks3(gd)),
+                                          std::max<size_t>(2 * kReduceBlocks, tiles));
+    c->joint = ok && parts <= kPartComp;
 }
 
 // Coarse levels of a cell-centred hierarchy whose level-0 FP64 coefficients
@@ -4237,6 +4569,8 @@ ebv_status setup_geometry_solvers(Ctx *c)
     EBV_LAUNCH(c, k_nd_bottom_assemble, dim3(gj_pad(N.nb)), dim3(128), 0, B.g, B.alpha_d, B.act, N.bmat, N.nb);
     bottom_invert(c, N.bmat, N.nb, 1, &N.binv);
     EBV_CUDA_TRY(c, cudaGetLastError());
+    if (c->prm.precision != EBV_FP64) carve_components<float>(c);
+    else carve_components<double>(c);
     return autotune_shapes(c);
 }
 
@@ -4273,11 +4607,15 @@ ebv_status autotune_shapes_t(Ctx *c)
     };
     for (int l = 0; l < c->mac.L; l++) {
         CcLevel &L = c->mac.lv[l];
-        VOp<T> A = vop<T>(L);
+        const VOp3<T> A = vop3<T>(c->mac, l, 1);
+        const V3<T> xv = one(x);
+        const V3<const T> bv = one<const T>(b), dv = one<const T>(d);
         float best = 1e30f;
         for (int q = 0; q < nc; q++) {
             const dim3 bk = cand[q], gr = gs_grid(L.g, bk);
-            float ms = time_it([&]() { k_cc_gs<T, false><<<gr, bk, 0, c->stream>>>(A, x, b, 0, 0, nullptr, GridD()); });
+            float ms = time_it([&]() {
+                k_cc_gs<T, false><<<gr, bk, 0, c->stream>>>(A, xv, bv, gr.z, nullptr, 0, 0, V3<const T>(), GridD());
+            });
             if (ms < best) { best = ms; L.gs_blk = bk; }
         }
         c->visc.lv[l].gs_blk = L.gs_blk;
@@ -4291,7 +4629,7 @@ ebv_status autotune_shapes_t(Ctx *c)
                 for (int pz = 1; pz <= 2; pz++)
                     for (const dim3 &bk : c4) {
                         if (bk.x > 2 * (unsigned)((L.g.nx >> 3) + 1)) continue;   // no block wider than twice a row
-                        float ms = time_it([&]() { launch_gs4(c->stream, bk, pz, A, x, b, 0, 0); });
+                        float ms = time_it([&]() { launch_gs4(c->stream, bk, pz, A, xv, bv, 0, 0); });
                         if (ms < best4) { best4 = ms; L.gs4_blk = bk; L.gs4_pz = pz; }
                     }
                 c->visc.lv[l].gs4_blk = L.gs4_blk;
@@ -4301,19 +4639,20 @@ ebv_status autotune_shapes_t(Ctx *c)
             // results), per kind of sweep: the faster serves it in switch mode 1
             RbMaps m;
             for (int q = 0; q < 4; q++) L.rb_ms[q][0] = 1e30f, L.rb_ms[q][1] = 0.f;
-            if (!c->batched && rb_fusable(L.g) && gs4_ok(L.g) && rb_map(c, x, 0, L.g, &m.x) && rb_map(c, b, 1, L.g, &m.b) &&
-                rb_map(c, A.dinv, 1, L.g, &m.d) && rb_map(c, L.bxp, 4, L.g, &m.fx) && rb_map(c, A.by, 2, L.g, &m.fy) &&
-                rb_map(c, A.bz, 3, L.g, &m.fz)) {
+            if (!c->batched && rb_fusable(L.g) && gs4_ok(L.g) && rb_map(c, x, 0, L.g, &m.v[0].x) &&
+                rb_map(c, b, 1, L.g, &m.v[0].b) && rb_map(c, A.dinv[0], 1, L.g, &m.v[0].d) &&
+                rb_map(c, L.bxp, 4, L.g, &m.fx) && rb_map(c, A.A.by, 2, L.g, &m.fy) &&
+                rb_map(c, A.A.bz, 3, L.g, &m.fz)) {
                 const long long nl = c->launches;
                 // planes per block: the model's choice, the most planes that
                 // still fill one wave, and half that (results do not depend on it)
                 const int nt = rb_ntiles(L.g), res = rb_resident(), nz = L.g.nz;
-                const int one = std::max(1, res / std::max(1, nt));   // chunks per wave
-                const int kzc[3] = {rb_kz(L.g), (nz + one - 1) / one, (nz + 2 * one - 1) / (2 * one)};
+                const int wave = std::max(1, res / std::max(1, nt));   // chunks per wave
+                const int kzc[3] = {rb_kz(L.g), (nz + wave - 1) / wave, (nz + 2 * wave - 1) / (2 * wave)};
                 float best = 1e30f;
                 for (int kz : kzc) {
                     const float ms = time_it(
-                        [&]() { rb_launch(c, "autotune", L.g, m, y, 0, RB_PLAIN, nullptr, kz); });
+                        [&]() { rb_launch(c, "autotune", L.g, m, one(y), 0, RB_PLAIN, nullptr, kz); });
                     if (ms < best) { best = ms; L.rb_kz = kz; }
                 }
                 // the correction sweep reads a coarse array: a zeroed vector with the next level's dims
@@ -4325,22 +4664,24 @@ ebv_status autotune_shapes_t(Ctx *c)
                 for (int kind = 0; kind < 4; kind++) {
                     if (kind == RB_CORR && !has_c) continue;   // (no correction sweep on the last level)
                     RbMaps mk = m;
-                    mk.xc = m.b;
-                    if (kind == RB_CORR && !rb_map(c, d, 5, gc, &mk.xc)) continue;
+                    mk.v[0].xc = m.v[0].b;
+                    if (kind == RB_CORR && !rb_map(c, d, 5, gc, &mk.v[0].xc)) continue;
                     const float ms_f = time_it([&]() {
-                        rb_launch(c, "autotune", L.g, mk, y, 0, kind, kind == RB_DOT ? c->part : nullptr, L.rb_kz);
+                        rb_launch(c, "autotune", L.g, mk, one(y), 0, kind, kind == RB_DOT ? c->part : nullptr, L.rb_kz);
                     });
                     const float ms_p = time_it([&]() {
                         if (kind == RB_CORR) {
+                            const dim3 g4 = gs4_grid(L.g, L.gs4_blk, L.gs4_pz);
                             if (L.gs4_pz == 1)
-                                k_cc_gs4<1, true><<<gs4_grid(L.g, L.gs4_blk, 1), L.gs4_blk, 0, c->stream>>>(A, x, b, 0, 0, d, gc);
+                                k_cc_gs4<1, true><<<g4, L.gs4_blk, 0, c->stream>>>(A, xv, bv, g4.z, nullptr, 0, 0, dv, gc);
                             else
-                                k_cc_gs4<2, true><<<gs4_grid(L.g, L.gs4_blk, 2), L.gs4_blk, 0, c->stream>>>(A, x, b, 0, 0, d, gc);
+                                k_cc_gs4<2, true><<<g4, L.gs4_blk, 0, c->stream>>>(A, xv, bv, g4.z, nullptr, 0, 0, dv, gc);
                         }
                         else
-                            launch_gs4(c->stream, L.gs4_blk, L.gs4_pz, A, x, b, 0, kind == RB_ZERO ? 1 : 0);
-                        if (kind == RB_DOT) k_cc_gs2_dot<<<gt, RB_THREADS, 0, c->stream>>>(A, x, b, 1, c->part);
-                        else launch_gs4(c->stream, L.gs4_blk, L.gs4_pz, A, x, b, 1, 0);
+                            launch_gs4(c->stream, L.gs4_blk, L.gs4_pz, A, xv, bv, 0, kind == RB_ZERO ? 1 : 0);
+                        if (kind == RB_DOT)
+                            k_cc_gs2_dot<<<gt, RB_THREADS, 0, c->stream>>>(A, xv, bv, gt.z, nullptr, 1, c->part);
+                        else launch_gs4(c->stream, L.gs4_blk, L.gs4_pz, A, xv, bv, 1, 0);
                     });
                     L.rb_ms[kind][0] = ms_f;
                     L.rb_ms[kind][1] = ms_p;
@@ -4380,7 +4721,7 @@ ebv_status mac_solve(Ctx *c, const double *b, double *x, int *iters, double *res
     CcProblem P;
     P.H = &c->mac;
     EBV_LAUNCH(c, k_fill, dim3(vblocks(ncell(c->g))), dim3(256), 0, x, ncell(c->g), 0.0);
-    return solve(c, P, b, x, iters, res, true);
+    return solve(c, P, one<const double>(b), one(x), iters, res, true);
 }
 
 ebv_status visc_build(Ctx *c, const double *eta)
@@ -4392,27 +4733,45 @@ ebv_status visc_build(Ctx *c, const double *eta)
     return cc_finish_hierarchy(c, c->visc, c->prm.precision != EBV_FP64);
 }
 
-ebv_status visc_solve(Ctx *c, const double *psi_comp, int comp, double *x, int *iters, double *res)
+namespace {
+// The three viscous systems with right-hand sides b (3 x cells): together where
+// the other components' vectors and partial sums fit (c->joint), else one
+// after another.
+ebv_status visc_solve_all(Ctx *c, const double *b, double *x, int *iters, double *res, bool x_zero)
+{
+    const int N3 = ncell(c->g), slot = c->cur_slot;
+    CcProblem P;
+    P.H = &c->visc;
+    if (c->joint) {
+        P.nc = kMaxComp;
+        return solve(c, P, V3<const double>(b, b + N3, b + 2 * (size_t)N3), V3<double>(x, x + N3, x + 2 * (size_t)N3),
+                     iters, res, x_zero);
+    }
+    for (int q = 0; q < kMaxComp; q++) {
+        select_variant(c->visc, q);
+        c->cur_slot = slot + q;
+        ebv_status st = solve(c, P, one<const double>(b + q * (size_t)N3), one(x + q * (size_t)N3),
+                              iters ? iters + q : nullptr, res ? res + q : nullptr, x_zero);
+        if (st != EBV_OK) return st;
+    }
+    return EBV_OK;
+}
+}  // namespace
+
+ebv_status visc_solve(Ctx *c, const double *psi, double *x, int *iters, double *res)
 {
     const GridD &g = c->g;
     CcLevel &V0 = c->visc.lv[0];
-    EBV_LAUNCH(c, k_visc_rhs, cgrid(g), block3(), 0, g, geomd(c), comp, psi_comp, V0.bf_d[0], V0.bf_d[1],
-               V0.bf_d[2], c->rhs_c);
-    select_variant(c->visc, comp);
-    CcProblem P;
-    P.H = &c->visc;
-    return solve(c, P, c->rhs_c, x, iters, res);
+    // (c->DC: scratch of the explicit terms, 3 x cells)
+    EBV_LAUNCH(c, k_visc_rhs, cgrid(g), block3(), 0, g, geomd(c), psi, V0.bf_d[0], V0.bf_d[1], V0.bf_d[2], c->DC);
+    return visc_solve_all(c, c->DC, x, iters, res, false);
 }
 
-ebv_status visc_solve_rhs(Ctx *c, int comp, const double *rhs, double *x, int *iters, double *res)
+ebv_status visc_solve_rhs(Ctx *c, const double *rhs, double *x, int *iters, double *res)
 {
-    const int n = ncell(c->g);
-    EBV_CUDA_TRY(c, cudaMemcpyAsync(c->rhs_c, rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-    select_variant(c->visc, comp);
+    const int n = 3 * ncell(c->g);
     EBV_LAUNCH(c, k_fill, dim3(vblocks(n)), dim3(256), 0, x, n, 0.0);
-    CcProblem P;
-    P.H = &c->visc;
-    return solve(c, P, c->rhs_c, x, iters, res, true);
+    return visc_solve_all(c, rhs, x, iters, res, true);
 }
 
 ebv_status nodal_solve(Ctx *c, const double *b, double *x, int *iters, double *res)
@@ -4421,7 +4780,7 @@ ebv_status nodal_solve(Ctx *c, const double *b, double *x, int *iters, double *r
     EBV_LAUNCH(c, k_zero_inactive, dim3(vblocks(nn)), dim3(256), 0, nn, c->nd.lv[0].act, x);
     NdProblem P;
     P.H = &c->nd;
-    return solve(c, P, b, x, iters, res);
+    return solve(c, P, one<const double>(b), one(x), iters, res);
 }
 
 
