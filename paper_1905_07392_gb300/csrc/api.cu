@@ -938,7 +938,7 @@ void ebv_destroy(ebv_ctx *c)
         if (l) cudaFree(L.alpha_d);
         cudaFree(L.alpha_f);
         cudaFree(L.act);
-        cudaFree(L.reg);
+        cudaFree(L.kind);
         cudaFree(L.irr);
     }
     cudaFree(c->nd.binv);

@@ -1702,6 +1702,8 @@ inline dim3 apply4_grid(const GridD &g)
 // coordinates.
 // ===========================================================================
 
+// node kinds: inactive, active with all 8 cells full (so interior), other active
+enum { ND_OFF = 0, ND_REG = 1, ND_IRR = 2 };
 __constant__ double kQ1[4] = {1.0 / 3.0, 0.0, -1.0 / 12.0, -1.0 / 12.0};
 
 template <class T>
@@ -1710,7 +1712,7 @@ struct NdOp {
     T h;                   // g.h in the operator's precision
     const T *alpha;        // cells
     const uint8_t *act;    // nodes
-    const uint8_t *reg;    // nodes whose 8 cells are full (level 0), else nullptr
+    const uint8_t *kind;   // per node: ND_OFF, ND_REG (all 8 cells full) or ND_IRR; null on small levels
 };
 
 // Row of the nodal operator at node (i,j,k), assembled in stencil form.  With
@@ -1738,7 +1740,7 @@ __device__ inline void nd_row(const NdOp<T> &A, int i, int j, int k, const T *__
 {
     const GridD &g = A.g;
     const int NXn = g.nx + 1, NYn = g.ny + 1;
-    if (A.reg && A.reg[nidx(g, i, j, k)]) {
+    if (A.kind && A.kind[nidx(g, i, j, k)] == ND_REG) {
         // all 8 cells full (so the node is interior): the constant stencil
         // 8/3 at the centre, -1/6 on the 12 face diagonals, -1/12 on the 8
         // body diagonals (times h)
@@ -1841,103 +1843,144 @@ __global__ void __launch_bounds__(256) k_nd_cheb(NdOp<T> A, const T *__restrict_
     xout[n] = xn + dn;
 }
 
-// ---- nodal passes in plane-sum form (levels with regular-node flags) ------------
-// With E_x, E_y, E_z the sums of the two neighbours along one axis, the
-// regular stencil's face-diagonal sum is (E_x E_y + E_x E_z + E_y E_z) x and
-// its body-diagonal sum E_x E_y E_z x.  Per plane k let A_k = the four axis
-// neighbours within the plane and B_k = its four in-plane diagonals; then
-//   face diagonals of node k = B_k + A_{k-1} + A_{k+1},
-//   body diagonals of node k = B_{k-1} + B_{k+1}.
-// A block of NT_X x NT_Y threads owns as many node columns and marches NT_Z
+// ---- nodal passes in plane-sum form (levels with node kinds) ------------------------
+// On a regular node the row is 8/3 x - (2 fd + bd) / 12 with fd, bd the sums of
+// the 12 face- and 8 body-diagonal neighbours.  Per plane let A = the four axis
+// neighbours within the plane, B = its four diagonals and C = 2 A + B; then
+//   2 fd + bd = 2 B_k + C_{k-1} + C_{k+1}.
+// A block of NT_X x NT_Y threads owns as many node columns and marches kz
 // planes: each plane of x (with its one-node halo) is staged in shared memory
 // while the next plane's loads are in flight (two buffers: the one written at
 // plane kk was last read at plane kk - 2, before every thread passed plane
-// kk - 1's barrier), A and B of three planes stay in registers, and the node
-// operands are fetched one plane ahead.  The tile kernel takes the regular
-// and the inactive nodes; the active nodes that are not regular (box faces,
-// cut cells: a few per cent) are listed once and take nd_row in k_nd_irr, so
-// no warp of the march diverges into the general row.  Modes:
+// kk - 1's barrier), B and C stay in registers, and the node operands are
+// fetched one plane ahead.  Interior nodes only (1 .. n-1: with the box faces
+// the tiles of a 2^q grid would be almost empty in their last row and column);
+// the box faces and the interior nodes that are active but not regular (cut
+// cells) are listed once per geometry and take the general row nd_row in the
+// first blocks of the same launch, so no warp of the march diverges into it.
+// kz is the largest of 16, 8, 4, 2 that still gives four blocks per SM.  (A
+// form without shared memory -- a warp per 32 columns x 4 rows, x neighbours by
+// shuffle -- was as fast on small grids and half as fast on 256^3: 169 us for
+// 89, its loads per plane bound by their latency at 16 warps per SM.)  Modes:
 //   ND_CHEB   one Chebyshev step, as k_nd_cheb (out = x_out, d updated);
 //   ND_RESID  out = b - A x, as k_nd_resid;
 //   ND_APPLY  out = A x (x on inactive nodes) with block partials of x.out;
 //   ND_RES32  r = b - A x (b - x on inactive nodes) in T, stored to the FP32
 //             vector out32, with block partials of |r|^2 (the refinement
 //             solver's true residual; T = double).
-// The sums are associated differently from the one-node kernels.
+// The sums are associated differently from the one-node kernels.  Measured per
+// Chebyshev step, against 16 planes per block at every size, box faces
+// included, and the listed nodes in a launch of their own: FP64 32^3 25.3 + 6.2
+// -> 6.1 us, 128^3 106 + 14.4 -> 86.7 us (FP64-pipe bound: 14 operations per
+// node, of 17), its 64^3 level (one node per thread before) 18.7 -> 10 us; FP32
+// 64^3 8.0 + 2.9 -> 4.2 us, 256^3 89 + 10.4 -> 89.7 us (HBM).
 enum { ND_CHEB = 0, ND_RESID = 1, ND_APPLY = 2, ND_RES32 = 3 };
-constexpr int NT_X = 32, NT_Y = 8, NT_Z = 16;
-constexpr long long kTileNodes = 1 << 20;   // coarse levels with at least this many nodes march too
+constexpr int NT_X = 32, NT_Y = 8, NT_T = NT_X * NT_Y;
 constexpr int NT_W = NT_X + 2, NT_H = NT_Y + 2, NT_N = NT_W * NT_H;
-constexpr int NT_SLOTS = (NT_N + NT_X * NT_Y - 1) / (NT_X * NT_Y);
+constexpr int NT_SLOTS = (NT_N + NT_T - 1) / NT_T;
+constexpr int kKindNodes = 4096;   // coarse levels with at least this many nodes take the march too
 
-inline dim3 nd_tile_grid(const GridD &g)
+// Launch of a pass: blocks of listed nodes first, then of tiles.
+struct NdShape {
+    int ntx, nty, kz, nlb, blocks;
+};
+inline NdShape nd_shape(const GridD &g, int nlist)
 {
-    return dim3((g.nx + 1 + NT_X - 1) / NT_X, (g.ny + 1 + NT_Y - 1) / NT_Y, (g.nz + 1 + NT_Z - 1) / NT_Z);
+    NdShape s;
+    const int mz = g.nz - 1;   // interior nodes along z
+    s.ntx = (g.nx - 1 + NT_X - 1) / NT_X;
+    s.nty = (g.ny - 1 + NT_Y - 1) / NT_Y;
+    s.kz = 16;
+    while (s.kz > 2 && (long long)s.ntx * s.nty * ((mz + s.kz - 1) / s.kz) < 4 * 152) s.kz /= 2;
+    s.nlb = (nlist + NT_T - 1) / NT_T;
+    s.blocks = s.nlb + s.ntx * s.nty * ((mz + s.kz - 1) / s.kz);
+    return s;
 }
 
 template <class T, int kMode>
-__global__ void __launch_bounds__(NT_X * NT_Y) k_nd_tile(NdOp<T> A, const T *__restrict__ xin, T *__restrict__ out,
-                                                       T *__restrict__ dvec, const T *__restrict__ b, T cd, T cr,
-                                                       double *__restrict__ part, float *__restrict__ out32,
-                                                       const double *__restrict__ sig)
+__global__ void __launch_bounds__(NT_T) k_nd_pass(NdOp<T> A, NdShape sh, const int *__restrict__ list, int nlist,
+                                                          const T *__restrict__ xin, T *__restrict__ out,
+                                                          T *__restrict__ dvec, const T *__restrict__ b, T cd, T cr,
+                                                          double *__restrict__ part, float *__restrict__ out32,
+                                                          const double *__restrict__ sig)
 {
     const double sc = (kMode == ND_RES32 && sig) ? *sig : 1.0;
-    __shared__ T sx[2][NT_H][NT_W];
     const GridD &g = A.g;
-    const int NX = g.nx + 1, NY = g.ny + 1, NZ = g.nz + 1;
-    const int sy = NX, sz = NX * NY;
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * NT_X + tx;
-    const int i0 = blockIdx.x * NT_X, j0 = blockIdx.y * NT_Y, k0 = blockIdx.z * NT_Z;
-    const int i = i0 + tx, j = j0 + ty;
-    const bool col = i < NX && j < NY;
-    const int kend = min(k0 + NT_Z, NZ);   // nodes k0 .. kend-1; planes k0-1 .. kend
-    // halo-tile slots of this thread: offset within a plane, -1 outside the box
-    int soff[NT_SLOTS];
-#pragma unroll
-    for (int u = 0; u < NT_SLOTS; u++) {
-        const int sl = tid + u * NT_X * NT_Y;
-        const int rr = sl / NT_W, qq = sl - rr * NT_W;
-        const int gi = i0 - 1 + qq, gj = j0 - 1 + rr;
-        soff[u] = (sl < NT_N && gi >= 0 && gi < NX && gj >= 0 && gj < NY) ? gj * sy + gi : -1;
-    }
-    T pre[NT_SLOTS];
-    auto fetch = [&](int kk) {
-#pragma unroll
-        for (int u = 0; u < NT_SLOTS; u++)
-            pre[u] = (soff[u] >= 0 && kk >= 0 && kk < NZ) ? xin[kk * sz + soff[u]] : T(0);
-    };
-    const T dreg = A.h * T(8.0 / 3.0), h12 = A.h * T(1.0 / 12.0);
-    const T crd = cr / dreg;   // regular nodes: cr / diag
-    T Am = 0, Bm = 0, A0 = 0, B0 = 0, X0 = 0;
-    uint8_t on_c = 0, rg_c = 0, on_n = 0, rg_n = 0;
-    T b_c = 0, d_c = 0, b_n = 0, d_n = 0;
+    const int NX = g.nx + 1, NY = g.ny + 1, tid = threadIdx.x;
     T v = 0;          // ND_APPLY: this thread's part of x.out
     float vr = 0.0f;  // ND_RES32: its part of |r|^2, from the stored FP32 values
-    fetch(k0 - 1);
-    for (int kk = k0 - 1; kk <= kend; kk++) {
-        T(*S)[NT_W] = sx[kk & 1];
+    if ((int)blockIdx.x < sh.nlb) {
+        const int t = blockIdx.x * NT_T + tid;
+        if (t < nlist) {
+            const int n = list[t];
+            const int i = n % NX, j = (n / NX) % NY, k = n / (NX * NY);
+            const bool on = A.act[n] != 0;
+            const T x0 = xin[n], bn = kMode != ND_APPLY ? b[n] : T(0);
+            T diag = T(1), ax = x0;
+            if (on) nd_row(A, i, j, k, xin, diag, ax);
+            if (kMode == ND_CHEB) {
+                const T dn = on ? (cd != T(0) ? cd * dvec[n] : T(0)) + cr * (bn - ax) / diag : T(0);
+                dvec[n] = dn;
+                out[n] = on ? x0 + dn : T(0);
+            }
+            if (kMode == ND_RESID) out[n] = on ? bn - ax : T(0);
+            if (kMode == ND_APPLY) { out[n] = ax; v = x0 * ax; }
+            if (kMode == ND_RES32) {
+                const float r = f64_to_f32_pow2(bn - ax, sc);
+                out32[n] = r;
+                vr = r * r;
+            }
+        }
+    } else {
+        __shared__ T sx[2][NT_H][NT_W];
+        const int tile = (int)blockIdx.x - sh.nlb, bx = tile % sh.ntx, tq = tile / sh.ntx, by = tq % sh.nty, bz = tq / sh.nty;
+        const int sy = NX, sz = NX * NY, tx = tid & 31, ty = tid >> 5;
+        const int i0 = 1 + bx * NT_X, j0 = 1 + by * NT_Y, k0 = 1 + bz * sh.kz;
+        const int i = i0 + tx, j = j0 + ty;
+        const bool col = i < g.nx && j < g.ny;
+        const int kend = min(k0 + sh.kz, g.nz);   // nodes k0 .. kend-1; planes k0-1 .. kend
+        // halo-tile slots of this thread: offset within a plane, -1 outside the box
+        int soff[NT_SLOTS];
 #pragma unroll
         for (int u = 0; u < NT_SLOTS; u++) {
-            const int sl = tid + u * NT_X * NT_Y;
-            if (sl < NT_N) (&S[0][0])[sl] = pre[u];
+            const int sl = tid + u * NT_T;
+            const int rr = sl / NT_W, qq = sl - rr * NT_W;
+            const int gi = i0 - 1 + qq, gj = j0 - 1 + rr;
+            soff[u] = (sl < NT_N && gi < NX && gj < NY) ? gj * sy + gi : -1;
         }
-        if (kk < kend) fetch(kk + 1);
-        // operands of node kk, finalised at the next plane
-        if (col && kk >= k0 && kk < kend) {
-            const int n = kk * sz + j * sy + i;
-            on_n = A.act[n];
-            rg_n = A.reg[n];
-            if (kMode != ND_APPLY) b_n = b[n];
-            if (kMode == ND_CHEB) d_n = dvec[n];
-        }
-        __syncthreads();
-        const T xc = S[ty + 1][tx + 1];
-        const T An = (S[ty + 1][tx] + S[ty + 1][tx + 2]) + (S[ty][tx + 1] + S[ty + 2][tx + 1]);
-        const T Bn = (S[ty][tx] + S[ty][tx + 2]) + (S[ty + 2][tx] + S[ty + 2][tx + 2]);
-        const int k = kk - 1;
-        if (col && k >= k0 && k < kend) {
-            const int n = k * sz + j * sy + i;
-            if (!on_c) {
+        T pre[NT_SLOTS];
+        auto fetch = [&](int kk) {
+#pragma unroll
+            for (int u = 0; u < NT_SLOTS; u++) pre[u] = soff[u] >= 0 ? xin[kk * sz + soff[u]] : T(0);
+        };
+        const T dreg = A.h * T(8.0 / 3.0), h12 = A.h * T(1.0 / 12.0);
+        const T crd = cr / dreg, c0 = crd * dreg, c1 = crd * h12;   // regular nodes: cr / diag
+        T Cm = 0, C0 = 0, B0 = 0, X0 = 0, b_c = 0, d_c = 0, b_n = 0, d_n = 0;
+        int kd_c = -1, kd_n = -1;   // node kind, -1: no node of this block
+        fetch(k0 - 1);
+        for (int kk = k0 - 1; kk <= kend; kk++) {
+            T(*S)[NT_W] = sx[kk & 1];
+#pragma unroll
+            for (int u = 0; u < NT_SLOTS; u++) {
+                const int sl = tid + u * NT_T;
+                if (sl < NT_N) (&S[0][0])[sl] = pre[u];
+            }
+            if (kk < kend) fetch(kk + 1);
+            // operands of node kk, finalised at the next plane
+            kd_n = -1;
+            if (col && kk >= k0 && kk < kend) {
+                const int n = kk * sz + j * sy + i;
+                kd_n = A.kind[n];
+                if (kMode != ND_APPLY) b_n = b[n];
+                if (kMode == ND_CHEB) d_n = dvec[n];
+            }
+            __syncthreads();
+            const T xc = S[ty + 1][tx + 1];
+            const T An = (S[ty + 1][tx] + S[ty + 1][tx + 2]) + (S[ty][tx + 1] + S[ty + 2][tx + 1]);
+            const T Bn = (S[ty][tx] + S[ty][tx + 2]) + (S[ty + 2][tx] + S[ty + 2][tx + 2]);
+            const T Cn = T(2) * An + Bn;
+            const int n = (kk - 1) * sz + j * sy + i;
+            if (kd_c == ND_OFF) {
                 if (kMode == ND_CHEB) { out[n] = T(0); dvec[n] = T(0); }
                 if (kMode == ND_RESID) out[n] = T(0);
                 if (kMode == ND_APPLY) { out[n] = X0; v += X0 * X0; }
@@ -1946,65 +1989,30 @@ __global__ void __launch_bounds__(NT_X * NT_Y) k_nd_tile(NdOp<T> A, const T *__r
                     out32[n] = r;
                     vr += r * r;
                 }
-            } else if (rg_c) {
-                const T ax = dreg * X0 - h12 * (T(2) * (B0 + Am + An) + (Bm + Bn));
+            } else if (kd_c == ND_REG) {
+                const T t = T(2) * B0 + (Cm + Cn);   // 2 fd + bd
                 if (kMode == ND_CHEB) {
-                    const T dn = (cd != T(0) ? cd * d_c : T(0)) + crd * (b_c - ax);
+                    const T dn = (cd != T(0) ? cd * d_c : T(0)) + crd * b_c - c0 * X0 + c1 * t;
                     dvec[n] = dn;
                     out[n] = X0 + dn;
-                }
-                if (kMode == ND_RESID) out[n] = b_c - ax;
-                if (kMode == ND_APPLY) { out[n] = ax; v += X0 * ax; }
-                if (kMode == ND_RES32) {
-                    const float r = f64_to_f32_pow2(b_c - ax, sc);
-                    out32[n] = r;
-                    vr += r * r;
+                } else {
+                    const T ax = dreg * X0 - h12 * t;
+                    if (kMode == ND_RESID) out[n] = b_c - ax;
+                    if (kMode == ND_APPLY) { out[n] = ax; v += X0 * ax; }
+                    if (kMode == ND_RES32) {
+                        const float r = f64_to_f32_pow2(b_c - ax, sc);
+                        out32[n] = r;
+                        vr += r * r;
+                    }
                 }
             }
+            Cm = C0; C0 = Cn; B0 = Bn; X0 = xc;
+            kd_c = kd_n; b_c = b_n; d_c = d_n;
         }
-        Am = A0; Bm = B0; A0 = An; B0 = Bn; X0 = xc;
-        on_c = on_n; rg_c = rg_n; b_c = b_n; d_c = d_n;
     }
     if constexpr (kMode == ND_APPLY || kMode == ND_RES32) {
         const double vs = kMode == ND_RES32 ? block_sum3_t<float>(vr) : block_sum3_t<T>(v);
-        if (thread_linear() == 0) part[block_linear()] = vs;
-    }
-}
-
-// The listed nodes (active, not regular) of a level-0 pass: nd_row per node,
-// the same outputs as k_nd_tile's mode; ND_APPLY partials per block.
-template <class T, int kMode>
-__global__ void __launch_bounds__(256) k_nd_irr(NdOp<T> A, const int *__restrict__ list, int nlist,
-                                                const T *__restrict__ xin, T *__restrict__ out, T *__restrict__ dvec,
-                                                const T *__restrict__ b, T cd, T cr, double *__restrict__ part,
-                                                float *__restrict__ out32, const double *__restrict__ sig)
-{
-    const double sc = (kMode == ND_RES32 && sig) ? *sig : 1.0;
-    const GridD &g = A.g;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    T v = 0;
-    if (t < nlist) {
-        const int n = list[t];
-        const int NX = g.nx + 1, NY = g.ny + 1;
-        const int i = n % NX, j = (n / NX) % NY, k = n / (NX * NY);
-        T diag, ax;
-        nd_row(A, i, j, k, xin, diag, ax);
-        if (kMode == ND_CHEB) {
-            const T dn = (cd != T(0) ? cd * dvec[n] : T(0)) + cr * (b[n] - ax) / diag;
-            dvec[n] = dn;
-            out[n] = xin[n] + dn;
-        }
-        if (kMode == ND_RESID) out[n] = b[n] - ax;
-        if (kMode == ND_APPLY) { out[n] = ax; v = xin[n] * ax; }
-        if (kMode == ND_RES32) {
-            const float r = f64_to_f32_pow2(b[n] - ax, sc);
-            out32[n] = r;
-            v = T(r) * T(r);
-        }
-    }
-    if constexpr (kMode == ND_APPLY || kMode == ND_RES32) {
-        const double vs = block_sum3_t<T>(v);
-        if (threadIdx.x == 0) part[blockIdx.x] = vs;
+        if (tid == 0) part[blockIdx.x] = vs;
     }
 }
 
@@ -2093,7 +2101,8 @@ __global__ void k_nd_alpha_coarsen(GridD gf, const double *__restrict__ af, Grid
     ac[cidx(gc, I, J, K)] = 0.125 * s;
 }
 
-__global__ void k_nd_regular(GridD g, const double *__restrict__ alpha, uint8_t *__restrict__ reg)
+__global__ void k_nd_kind(GridD g, const double *__restrict__ alpha, const uint8_t *__restrict__ act,
+                          uint8_t *__restrict__ kind)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -2104,7 +2113,8 @@ __global__ void k_nd_regular(GridD g, const double *__restrict__ alpha, uint8_t 
         int ci = i - 1 + (oc & 1), cj = j - 1 + ((oc >> 1) & 1), ck = k - 1 + ((oc >> 2) & 1);
         if (!inbox(g, ci, cj, ck) || alpha[cidx(g, ci, cj, ck)] != 1.0) all = false;
     }
-    reg[nidx(g, i, j, k)] = all ? 1 : 0;
+    const int n = nidx(g, i, j, k);
+    kind[n] = !act[n] ? ND_OFF : (all ? ND_REG : ND_IRR);
 }
 
 __global__ void k_nd_active(GridD g, const double *__restrict__ alpha, uint8_t *__restrict__ act)
@@ -2329,28 +2339,27 @@ void bottom_invert(Ctx *c, double *M, int nb, int nmat, double *const *inv)
     }
 }
 
-// x = scale inv b; the dense system is numbered in the natural order, the
+// x = inv b; the dense system is numbered in the natural order, the
 // vectors of a row-split (FP32 cell-centred) level are mapped through g.
 __device__ inline int bottom_pos(const GridD &g, int split, int r)
 {
     if (!split) return r;
     return cix<float>(g, r % g.nx, (r / g.nx) % g.ny, r / (g.nx * g.ny));
 }
+// One warp per row, eight rows per block: a row's products are FP64-pipe work
+// and a serial chain for one thread (125 unknowns: 13-25 us for one block with
+// a thread per row, 2-4 us so).
 template <class T>
-__device__ inline void bottom_row(const double *__restrict__ inv, int nb, const T *__restrict__ b,
-                                  T *__restrict__ x, double scale, const GridD &g, int split, int r)
+__global__ void __launch_bounds__(256) k_bottom_solve(V3<const double> inv, int nb, V3<const T> b, V3<T> x, GridD g,
+                                                      int split)
 {
+    const int c = blockIdx.y, r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (r >= nb) return;
+    const double *row = inv.p[c] + (size_t)r * nb;
     double s = 0.0;
-    for (int q = 0; q < nb; q++) s += inv[(size_t)r * nb + q] * (double)b[bottom_pos(g, split, q)];
-    x[bottom_pos(g, split, r)] = (T)(s * scale);
-}
-template <class T>
-__global__ void __launch_bounds__(256) k_bottom_solve(V3<const double> inv, int nb, V3<const T> b, V3<T> x,
-                                                      double scale, GridD g, int split)
-{
-    const int q = blockIdx.y;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nb; r += gridDim.x * blockDim.x)
-        bottom_row(inv.p[q], nb, b.p[q], x.p[q], scale, g, split, r);
+    for (int q = lane; q < nb; q += 32) s += row[q] * (double)b.p[c][bottom_pos(g, split, q)];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) x.p[c][bottom_pos(g, split, r)] = (T)s;
 }
 
 // ---- the coarse end of the cell-centred V-cycle in one cluster -------------------
@@ -3424,7 +3433,7 @@ NdOp<T> ndop(const NdLevel &L)
     if constexpr (sizeof(T) == 8) A.alpha = (const T *)L.alpha_d;
     else A.alpha = (const T *)L.alpha_f;
     A.act = L.act;
-    A.reg = L.reg;
+    A.kind = L.kind;
     return A;
 }
 
@@ -3786,8 +3795,8 @@ int cc_vcycle(Ctx *c, CcHier &H, int nc, const int *act, V3<const T> b0, V3<T> x
         EBV_LAUNCH_P(c, nm, 0.0, k_cc_coarse_vcycle<T>, dim3(kCvCtas, nc), dim3(kCvThreads), bytes, D);
         if (l0 == 0) return dot_part ? kCvCtas : 0;
     } else {
-        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 255) / 256, nc), dim3(256), 0, binv, H.nb, B(Lb), X(Lb), 1.0,
-                   H.lv[Lb].g, (int)(sizeof(T) == 4));
+        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 7) / 8, nc), dim3(256), 0, binv, H.nb, B(Lb), X(Lb), H.lv[Lb].g,
+                   (int)(sizeof(T) == 4));
     }
     for (int l = l0 - 1; l >= 0; l--) {
         // prolongation folded into the first colour pass of the post-smoothing
@@ -3819,29 +3828,18 @@ inline ChebCoef cheb_coef(double lmax)
 
 // Three Chebyshev steps on A x = b, ending in x.  From zero: (0) -> x -> t -> x.
 // Otherwise the start is in t: t -> x -> t -> x.  d is the level's direction.
-// A nodal pass on a level with regular-node flags: the plane march over the
-// regular and inactive nodes, then the listed nodes (their ND_APPLY partials
-// follow the march's).
-inline int nd_tile_blocks(const GridD &g)
-{
-    const dim3 gr = nd_tile_grid(g);
-    return (int)(gr.x * gr.y * gr.z);
-}
+// A nodal pass on a level with node kinds: one launch for the listed nodes and
+// the march; block partials per block of the launch.
 template <class T, int kMode>
-void nd_tile_pass(Ctx *c, const NdLevel &L, const char *name, double nbytes, const T *xin, T *out, T *d,
-                const T *b, T cd, T cr, double *part, float *out32 = nullptr, const double *sig = nullptr)
+void nd_pass(Ctx *c, const NdLevel &L, const char *name, double nbytes, const T *xin, T *out, T *d, const T *b, T cd, T cr,
+             double *part, float *out32 = nullptr, const double *sig = nullptr)
 {
-    const NdOp<T> A = ndop<T>(L);
-    EBV_LAUNCH_P(c, name, nbytes, (k_nd_tile<T, kMode>), nd_tile_grid(L.g), dim3(NT_X, NT_Y), 0, A, xin, out, d, b,
-                 cd, cr, part, out32, sig);
-    static const char *const kIrrName[4] = {"nodal_listed_nodes chebyshev", "nodal_listed_nodes residual",
-                                            "nodal_listed_nodes apply", "nodal_listed_nodes refinement residual"};
-    if (L.nirr)
-        EBV_LAUNCH_P(c, kIrrName[kMode], 0.0, (k_nd_irr<T, kMode>), dim3((L.nirr + 255) / 256), dim3(256), 0, A, L.irr,
-                     L.nirr, xin, out, d, b, cd, cr, part ? part + nd_tile_blocks(L.g) : nullptr, out32, sig);
+    const NdShape sh = nd_shape(L.g, L.nirr);
+    EBV_LAUNCH_P(c, name, nbytes, (k_nd_pass<T, kMode>), dim3(sh.blocks), dim3(NT_T), 0, ndop<T>(L), sh, L.irr,
+                 L.nirr, xin, out, d, b, cd, cr, part, out32, sig);
 }
-// partial sums written by nd_tile_pass on level L
-inline int nd_tile_parts(const NdLevel &L) { return nd_tile_blocks(L.g) + (L.nirr ? (L.nirr + 255) / 256 : 0); }
+// partial sums written by nd_pass on level L
+inline int nd_pass_parts(const NdLevel &L) { return nd_shape(L.g, L.nirr).blocks; }
 
 template <class T>
 void nd_smooth(Ctx *c, const NdLevel &L, int l, T *x, T *t, const T *b, bool zero_start)
@@ -3855,8 +3853,8 @@ void nd_smooth(Ctx *c, const NdLevel &L, int l, T *x, T *t, const T *b, bool zer
         // from zero reads only b and alpha and writes d, x)
         const bool z0 = s == 0 && zero_start;
         const double nb = (z0 ? 4.0 : 6.0) * sizeof(T) * (double)nnode(L.g);
-        if (!z0 && L.reg)   // levels with regular-node flags: plane-sum form
-            nd_tile_pass<T, ND_CHEB>(c, L,
+        if (!z0 && L.kind)   // levels with node kinds: plane-sum form
+            nd_pass<T, ND_CHEB>(c, L,
                                    sizeof(T) == 4 ? (l ? "nodal_chebyshev_step<float> L1+" : "nodal_chebyshev_step<float> L0")
                                                   : (l ? "nodal_chebyshev_step<double> L1+" : "nodal_chebyshev_step<double> L0"),
                                    nb, src, dst, d, b, (T)k.cd[s], (T)k.cr[s], nullptr);
@@ -3878,9 +3876,9 @@ void nd_vcycle(Ctx *c, NdHier &H, const T *b0, T *x0)
         T *x = l ? (T *)c->lx[l] : x0;
         const T *b = l ? (const T *)c->lb[l] : b0;
         nd_smooth<T>(c, L, l, x, (T *)c->lt[l], b, true);
-        if (L.reg)
-            nd_tile_pass<T, ND_RESID>(c, L, l ? "k_nd_resid<T> tiled L1+" : "k_nd_resid<T> tiled L0", 0.0, x, (T *)c->lr[l], nullptr, b, T(0), T(0),
-                                    nullptr);
+        if (L.kind)
+            nd_pass<T, ND_RESID>(c, L, l ? "nodal_residual L1+" : "nodal_residual L0", 0.0, x, (T *)c->lr[l], nullptr, b,
+                                 T(0), T(0), nullptr);
         else
             EBV_LAUNCH(c, k_nd_resid<T>, ngrid(L.g), block3(), 0, ndop<T>(L), x, b, (T *)c->lr[l]);
         const NdLevel &Lc = H.lv[l + 1];
@@ -3890,8 +3888,8 @@ void nd_vcycle(Ctx *c, NdHier &H, const T *b0, T *x0)
     {
         T *x = Lb ? (T *)c->lx[Lb] : x0;
         const T *b = Lb ? (const T *)c->lb[Lb] : b0;
-        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 255) / 256), dim3(256), 0, one<const double>(H.binv), H.nb,
-                   one<const T>(b), one(x), 1.0, H.lv[Lb].g, 0);
+        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 7) / 8), dim3(256), 0, one<const double>(H.binv), H.nb,
+                   one<const T>(b), one(x), H.lv[Lb].g, 0);
     }
     for (int l = Lb - 1; l >= 0; l--) {
         const NdLevel &L = H.lv[l];
@@ -4245,16 +4243,16 @@ struct CcProblem : Problem {
 struct NdProblem : Problem {
     NdHier *H;
     int n() const override { return nnode(H->lv[0].g); }
-    int apply_blocks() const override { return nd_tile_parts(H->lv[0]); }
+    int apply_blocks() const override { return nd_pass_parts(H->lv[0]); }
     void apply_dot(Ctx *c, V3<const double> p, V3<double> q, const int *) override
     {
         // p read, q written, act and reg flags: 2.25 words per node
-        nd_tile_pass<double, ND_APPLY>(c, H->lv[0], "nodal_apply_fp64", 18.0 * n(), p.p[0], q.p[0], nullptr, nullptr, 0.0,
+        nd_pass<double, ND_APPLY>(c, H->lv[0], "nodal_apply_fp64", 18.0 * n(), p.p[0], q.p[0], nullptr, nullptr, 0.0,
                                        0.0, c->part);
     }
     void apply_dot32(Ctx *c, V3<const float> p, V3<float> q, const int *) override
     {
-        nd_tile_pass<float, ND_APPLY>(c, H->lv[0], "nodal_apply_fp32", 12.0 * n(), p.p[0], q.p[0], nullptr, nullptr, 0.0f,
+        nd_pass<float, ND_APPLY>(c, H->lv[0], "nodal_apply_fp32", 12.0 * n(), p.p[0], q.p[0], nullptr, nullptr, 0.0f,
                                     0.0f, c->part);
     }
     void precond(Ctx *c, V3<const double> r, V3<double> z, const int *) override
@@ -4269,7 +4267,7 @@ struct NdProblem : Problem {
     void resid32(Ctx *c, V3<const double> b, V3<const double> x, V3<float> r, const int *) override
     {
         // x, b read, r (FP32) written, act and reg flags: 5.25 words per node
-        nd_tile_pass<double, ND_RES32>(c, H->lv[0], "nodal_resid_fp64", 22.0 * n(), x.p[0], nullptr, nullptr, b.p[0], 0.0,
+        nd_pass<double, ND_RES32>(c, H->lv[0], "nodal_resid_fp64", 22.0 * n(), x.p[0], nullptr, nullptr, b.p[0], 0.0,
                                        0.0, c->part, r.p[0], c->scal + S_SIG);
     }
     void add32(Ctx *c, V3<double> x, V3<const float> e, V3<const float> p, const int *) override
@@ -4484,9 +4482,9 @@ ebv_status setup_solvers(Ctx *c)
         Lv.alpha_d = l ? dalloc<double>(nc, e) : c->alpha;
         Lv.alpha_f = dalloc<float>(nc, e);
         Lv.act = dalloc<uint8_t>(nnode(gn[l]), e);
-        // regular-node flags (and the plane march) where the level is large
-        // enough to fill the GPU with marching blocks
-        Lv.reg = (l == 0 || nnode(gn[l]) >= kTileNodes) ? dalloc<uint8_t>(nnode(gn[l]), e) : nullptr;
+        // node kinds (and with them the plane march): the finest level, and
+        // the coarse ones large enough that it is the faster form
+        Lv.kind = (l == 0 || nnode(gn[l]) >= kKindNodes) ? dalloc<uint8_t>(nnode(gn[l]), e) : nullptr;
         Lv.lam_max = 2.0;
     }
     c->nd.binv = dalloc<double>((size_t)nbn * nbn, e);
@@ -4542,21 +4540,26 @@ ebv_status setup_geometry_solvers(Ctx *c)
         int nc = ncell(Lv.g);
         EBV_LAUNCH(c, (k_convert<double, float>), dim3(vblocks(nc)), dim3(256), 0, Lv.alpha_d, Lv.alpha_f, nc);
         EBV_LAUNCH(c, k_nd_active, ngrid(Lv.g), block3(), 0, Lv.g, Lv.alpha_d, Lv.act);
-        if (Lv.reg) EBV_LAUNCH(c, k_nd_regular, ngrid(Lv.g), block3(), 0, Lv.g, Lv.alpha_d, Lv.reg);
+        if (Lv.kind) EBV_LAUNCH(c, k_nd_kind, ngrid(Lv.g), block3(), 0, Lv.g, Lv.alpha_d, Lv.act, Lv.kind);
     }
     for (int l = 0; l < N.L; l++) {
-        // levels with regular-node flags: the active nodes that are not
-        // regular, in ascending order, for the listed half of their passes
+        // levels with node kinds: the nodes that take the general row, in
+        // ascending order -- the box faces, and inside the active nodes that
+        // are not regular
         NdLevel &Lv = N.lv[l];
-        if (!Lv.reg) continue;
-        const int nn = nnode(Lv.g);
-        std::vector<uint8_t> act(nn), reg(nn);
-        EBV_CUDA_TRY(c, cudaMemcpyAsync(act.data(), Lv.act, nn, cudaMemcpyDeviceToHost, c->stream));
-        EBV_CUDA_TRY(c, cudaMemcpyAsync(reg.data(), Lv.reg, nn, cudaMemcpyDeviceToHost, c->stream));
+        if (!Lv.kind) continue;
+        const GridD &gl = Lv.g;
+        const int nn = nnode(gl);
+        std::vector<uint8_t> kind(nn);
+        EBV_CUDA_TRY(c, cudaMemcpyAsync(kind.data(), Lv.kind, nn, cudaMemcpyDeviceToHost, c->stream));
         EBV_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
         std::vector<int> irr;
-        for (int n = 0; n < nn; n++)
-            if (act[n] && !reg[n]) irr.push_back(n);
+        for (int k = 0, n = 0; k <= gl.nz; k++)
+            for (int j = 0; j <= gl.ny; j++) {
+                const bool row = k == 0 || k == gl.nz || j == 0 || j == gl.ny;
+                for (int i = 0; i <= gl.nx; i++, n++)
+                    if (row || i == 0 || i == gl.nx || kind[n] == ND_IRR) irr.push_back(n);
+            }
         if (Lv.irr) cudaFree(Lv.irr);
         Lv.irr = nullptr;
         Lv.nirr = (int)irr.size();

@@ -83,3 +83,28 @@ def test_vcycle_contracts(n, precision):
     assert max(it[:4] + it[5:9]) <= 26, it   # (slots 4 and 9 are the nodal solves)
     assert max(st["res"]) <= 1e-12
     s.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n", [(2, 2, 2), (4, 2, 6), (36, 20, 28), (64, 16, 32), (32, 8, 8)])
+def test_nodal_projection_matches_oracle(n, precision):
+    """The nodal passes march tiles of 32 x 8 interior nodes and list the rest: no interior, one
+    node, partial tiles, exactly full ones.  Both sides solve to 1e-13 (see above for the bound)."""
+    from paper_1905_07392_gb300 import ebvisc as E
+    h = 1.0 / n[0]
+    c, r = tuple((0.5 * v + 0.1) * h for v in n), 0.3 * min(n) * h
+    s = E.Solver(n, h, tol=1e-13, max_iters=5000, precision=precision)
+    s.build_sphere(c, r)
+    g = O.Grid(n=n, h=h)
+    geo = O.build_geometry(g, O.Shape(kind=O.SHAPE_SPHERE, p=c + (r,)))
+    P = O.Params(tol=1e-13, max_iters=200000)
+    rng = np.random.Generator(np.random.PCG64(n[0] + n[1]))
+    ut0 = (rng.uniform(-0.1, 0.1, size=(3, g.ncell)) * (geo.alpha > 0)).ravel()
+    p0 = rng.uniform(-1.0, 1.0, size=g.nnode)
+    dt = 0.01
+    uo, po = O.nodal_project(g, geo, P, dt, ut0.copy(), p0.copy())[:2]
+    u, p = torch.tensor(ut0, device=DEV), torch.tensor(p0, device=DEV)
+    s.solve_projection(u, p, dt)
+    assert np.linalg.norm(u.cpu().numpy() - uo) <= 1e-10 * np.linalg.norm(uo)
+    assert np.linalg.norm(p.cpu().numpy() - po) <= 1e-10 * np.linalg.norm(po)
+    s.close()
