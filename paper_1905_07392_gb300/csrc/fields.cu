@@ -57,34 +57,29 @@ __device__ inline double upwind_normal(double uL, double uR)
     return 0.0;
 }
 
-// Robust cell-centred derivative along d (paper Sec. "Strain rate tensor and
-// apparent viscosity"): central, one-sided quadratic next to a covered cell,
-// first order with a single neighbour, zero without one.
-__device__ inline double d_robust(const GridD &g, const uint8_t *flag, const double *f, int i,
-                                  int j, int k, int d, double ih)
+// 2 h times the robust cell-centred derivative along d (paper Sec. "Strain rate
+// tensor and apparent viscosity"): central, one-sided quadratic next to a
+// covered cell, first order with a single neighbour, zero without one.  The
+// scaling is left to the caller: the strain rate needs it once, not nine times.
+__device__ inline double d2h_robust(const GridD &g, const uint8_t *flag, const double *f, int i,
+                                    int j, int k, int d)
 {
     int3 e = unit(d);
     bool ip = avail(g, flag, i + e.x, j + e.y, k + e.z);
     bool im = avail(g, flag, i - e.x, j - e.y, k - e.z);
+    if (ip && im) return f[cidx(g, i + e.x, j + e.y, k + e.z)] - f[cidx(g, i - e.x, j - e.y, k - e.z)];
     double f0 = f[cidx(g, i, j, k)];
-    if (ip && im)
-        return (f[cidx(g, i + e.x, j + e.y, k + e.z)] - f[cidx(g, i - e.x, j - e.y, k - e.z)]) *
-               (0.5 * ih);
     if (im) {
         double f1 = f[cidx(g, i - e.x, j - e.y, k - e.z)];
-        if (avail(g, flag, i - 2 * e.x, j - 2 * e.y, k - 2 * e.z)) {
-            double f2 = f[cidx(g, i - 2 * e.x, j - 2 * e.y, k - 2 * e.z)];
-            return (0.5 * f2 - 2.0 * f1 + 1.5 * f0) * ih;
-        }
-        return (f0 - f1) * ih;
+        if (avail(g, flag, i - 2 * e.x, j - 2 * e.y, k - 2 * e.z))
+            return f[cidx(g, i - 2 * e.x, j - 2 * e.y, k - 2 * e.z)] - 4.0 * f1 + 3.0 * f0;
+        return 2.0 * (f0 - f1);
     }
     if (ip) {
         double f1 = f[cidx(g, i + e.x, j + e.y, k + e.z)];
-        if (avail(g, flag, i + 2 * e.x, j + 2 * e.y, k + 2 * e.z)) {
-            double f2 = f[cidx(g, i + 2 * e.x, j + 2 * e.y, k + 2 * e.z)];
-            return (-1.5 * f0 + 2.0 * f1 - 0.5 * f2) * ih;
-        }
-        return (f1 - f0) * ih;
+        if (avail(g, flag, i + 2 * e.x, j + 2 * e.y, k + 2 * e.z))
+            return -3.0 * f0 + 4.0 * f1 - f[cidx(g, i + 2 * e.x, j + 2 * e.y, k + 2 * e.z)];
+        return 2.0 * (f1 - f0);
     }
     return 0.0;
 }
@@ -171,18 +166,18 @@ __global__ void __launch_bounds__(256) k_strain_eta(GridD g, const uint8_t *__re
             return;
         }
     }
-    double Gm[3][3];
-    const double ih = g.ih;
+    double Gm[3][3];   // 2 h times the gradient
+    const double hh = 0.5 * g.ih;
 #pragma unroll
     for (int d = 0; d < 3; d++)
 #pragma unroll
-        for (int q = 0; q < 3; q++) Gm[d][q] = d_robust(g, flag, u + q * N3, i, j, k, d, ih);
+        for (int q = 0; q < 3; q++) Gm[d][q] = d2h_robust(g, flag, u + q * N3, i, j, k, d);
     // sr^2 = |G + G^T|^2 / 2 = 2 (G_00^2 + G_11^2 + G_22^2) + the squares of
     // the three off-diagonal sums; sr and 1/sr from one reciprocal square root
     const double xy = Gm[0][1] + Gm[1][0], xz = Gm[0][2] + Gm[2][0], yz = Gm[1][2] + Gm[2][1];
-    const double s = 2.0 * (Gm[0][0] * Gm[0][0] + Gm[1][1] * Gm[1][1] + Gm[2][2] * Gm[2][2]) +
-                     (xy * xy + xz * xz + yz * yz);
-    const double rsr = s > 0.0 ? rsqrt(s) : 0.0;
+    const double s = (2.0 * (Gm[0][0] * Gm[0][0] + Gm[1][1] * Gm[1][1] + Gm[2][2] * Gm[2][2]) +
+                      (xy * xy + xz * xz + yz * yz)) * (hh * hh);
+    const double rsr = gt_nonneg(s, 0.0) ? rsqrt(s) : 0.0;
     const double sr = s * rsr;
     eta[c] = eta_of(p, sr, rsr);
     if (srate) srate[c] = sr;
@@ -190,7 +185,7 @@ __global__ void __launch_bounds__(256) k_strain_eta(GridD g, const uint8_t *__re
 #pragma unroll
         for (int d = 0; d < 3; d++)
 #pragma unroll
-            for (int q = 0; q < 3; q++) G[(3 * d + q) * N3 + c] = Gm[d][q];
+            for (int q = 0; q < 3; q++) G[(3 * d + q) * N3 + c] = Gm[d][q] * hh;
 }
 
 // ---- flow diagnostics (Sec. "Cylinder moving through Bingham fluid") ------
@@ -208,21 +203,23 @@ __global__ void __launch_bounds__(256) k_flow_diag(GridD g, const uint8_t *__res
         sdev[c] = 0.0;
         return;
     }
-    double Gm[3][3];
-    const double ih = g.ih;
+    double Gm[3][3];   // 2 h times the gradient (Lambda is a ratio)
+    const double hh = 0.5 * g.ih;
 #pragma unroll
     for (int d = 0; d < 3; d++)
 #pragma unroll
-        for (int q = 0; q < 3; q++) Gm[d][q] = d_robust(g, flag, u + q * N3, i, j, k, d, ih);
+        for (int q = 0; q < 3; q++) Gm[d][q] = d2h_robust(g, flag, u + q * N3, i, j, k, d);
     const double xy = Gm[0][1] + Gm[1][0], xz = Gm[0][2] + Gm[2][0], yz = Gm[1][2] + Gm[2][1];
     const double s = 2.0 * (Gm[0][0] * Gm[0][0] + Gm[1][1] * Gm[1][1] + Gm[2][2] * Gm[2][2]) +
-                     (xy * xy + xz * xz + yz * yz);   // ||g||^2
+                     (xy * xy + xz * xz + yz * yz);   // (2 h)^2 ||g||^2
     const double wx = Gm[1][2] - Gm[2][1], wy = Gm[2][0] - Gm[0][2], wz = Gm[0][1] - Gm[1][0];
     const double w2 = wx * wx + wy * wy + wz * wz;
-    lam[c] = (s + w2) > 0.0 ? (s - w2) / (s + w2) : 0.0;
-    const double rsr = s > 0.0 ? rsqrt(s) : 0.0;
-    const double sr = s * rsr;
-    sdev[c] = p.tau0 > 0.0 ? eta_of(p, sr, rsr) * sr / p.tau0 - 1.0 : 0.0;
+    const double sw = s + w2, sh = s * (hh * hh);
+    lam[c] = gt_nonneg(sw, 0.0) ? (s - w2) / sw : 0.0;
+    const double rsr = gt_nonneg(sh, 0.0) ? rsqrt(sh) : 0.0;
+    const double sr = sh * rsr;
+    // (one rounding with the subtraction, in place of the division's)
+    sdev[c] = p.tau0 > 0.0 ? fma(eta_of(p, sr, rsr) * sr, p.inv_tau0, -1.0) : 0.0;
 }
 
 // ---- normal face velocities (slopes, extrapolation, upwinding) ------------
