@@ -254,9 +254,9 @@ struct NdLevel {
     double *alpha_d = nullptr;   // cell volume fractions at this level
     float *alpha_f = nullptr;
     uint8_t *act = nullptr;      // 1 for active nodes
-    uint8_t *kind = nullptr;     // node kinds (ND_OFF, ND_REG, ND_IRR) on the levels that take the
-                                 // plane march, else null
-    int *irr = nullptr;          // with kind: the nodes that take the general row, ascending
+    uint8_t *kind = nullptr;     // node kinds (ND_OFF, ND_REG, ND_IRR)
+    bool march = false;          // takes the plane march; then
+    int *irr = nullptr;          // the nodes that take the general row, ascending
     int nirr = 0;
     double lam_max = 2.0;        // bound of the spectrum of D^-1 A
     dim3 ch_blk = dim3(32, 4, 2);  // Chebyshev-step block shape (autotuned per level)

@@ -1712,7 +1712,7 @@ struct NdOp {
     T h;                   // g.h in the operator's precision
     const T *alpha;        // cells
     const uint8_t *act;    // nodes
-    const uint8_t *kind;   // per node: ND_OFF, ND_REG (all 8 cells full) or ND_IRR; null on small levels
+    const uint8_t *kind;   // per node: ND_OFF, ND_REG (all 8 cells full) or ND_IRR
 };
 
 // Row of the nodal operator at node (i,j,k), assembled in stencil form.  With
@@ -1740,7 +1740,7 @@ __device__ inline void nd_row(const NdOp<T> &A, int i, int j, int k, const T *__
 {
     const GridD &g = A.g;
     const int NXn = g.nx + 1, NYn = g.ny + 1;
-    if (A.kind && A.kind[nidx(g, i, j, k)] == ND_REG) {
+    if (A.kind[nidx(g, i, j, k)] == ND_REG) {
         // all 8 cells full (so the node is interior): the constant stencil
         // 8/3 at the centre, -1/6 on the 12 face diagonals, -1/12 on the 8
         // body diagonals (times h)
@@ -2874,6 +2874,359 @@ void cv_attr()
     }
 }
 
+// ---- the coarse end of the nodal V-cycle in one cluster --------------------------
+// Below a level of at most kNcNodes nodes a nodal V-cycle is ten launches per
+// level of two to four microseconds each.  One cluster of kNcCtas blocks runs
+// that level and all below it: every smoothed level in slabs of node planes
+// (nested: a coarse plane K belongs to the block of fine plane 2K), the vectors,
+// cell fractions and node records in shared memory, the planes at a slab's ends
+// written to the neighbouring blocks before the cluster barrier that ends a
+// step, and the bottom rows shared out.  Steps and per-node operations are those
+// of k_nd_cheb, k_nd_resid, k_nd_restrict and k_nd_prolong.  Every remote write
+// is followed by a cluster barrier that its target takes part in.
+// kNcNodes: FP32 a 16^3-cell level; FP64 an 8^3-cell one (of a 17^3-node level
+// the FP64 operations alone take eight SMs 5 us a step, a launch over the whole
+// GPU 4).  Per V-cycle 31 us in FP32 for 19 launches of 2.2-3.8 us and their
+// gaps (two steps at 64^3 15.1 -> 14.6 ms), 25 us in FP64 for ten of 2-5 us
+// (64^3 gradient, 12-instance sweep: 3.5 and 2.8 % faster).  A step over 600
+// nodes of the 17^3 level takes 1.5 us, half of it instruction issue.
+constexpr int kNcCtas = 8, kNcThreads = 512, kNcMax = 4, kNcSmem = 200 * 1024;
+template <class T> struct NcNodes { static constexpr int n = sizeof(T) == 4 ? 8192 : 1024; };
+struct NcLayout {
+    int x[kNcMax], t[kNcMax], d[kNcMax], b[kNcMax], dg[kNcMax], di[kNcMax], al[kNcMax], rec[kNcMax], bs, xb, total;
+};
+template <class T>
+struct NdCoarse {
+    int n;                 // levels; the last is the bottom
+    int na;                // blocks that own a slab
+    NdOp<T> A[kNcMax];
+    T *x;
+    const T *b;
+    const double *binv;
+    int nb;
+    T cd[3], cr[3];
+    NcLayout L;
+};
+// first node plane of rank r's slab on smoothed level l of ns (npb: planes of
+// the last smoothed level)
+__host__ __device__ inline int nc_s0(int npb, int na, int ns, int l, int np, int r)
+{
+    return r >= na ? np : (npb * r / na) << (ns - 1 - l);
+}
+template <class T>
+inline NcLayout nc_layout(const NdCoarse<T> &D)
+{
+    NcLayout o;
+    int at = 0;
+    auto take = [&](size_t bytes) { const int q = at; at += (int)((bytes + 15) & ~(size_t)15); return q; };
+    const int ns = D.n - 1, npb = D.A[ns - 1].g.nz + 1;
+    for (int l = 0; l < ns; l++) {
+        const GridD &g = D.A[l].g;
+        const int P = (g.nx + 1) * (g.ny + 1), np = g.nz + 1;
+        int pl = 0;
+        for (int r = 0; r < D.na; r++)
+            pl = std::max(pl, nc_s0(npb, D.na, ns, l, np, r + 1) - nc_s0(npb, D.na, ns, l, np, r));
+        o.x[l] = take((size_t)(pl + 2) * P * sizeof(T));
+        o.t[l] = take((size_t)(pl + 2) * P * sizeof(T));
+        o.d[l] = take((size_t)pl * P * sizeof(T));
+        o.b[l] = take((size_t)pl * P * sizeof(T));
+        o.dg[l] = take((size_t)pl * P * sizeof(T));
+        o.di[l] = take((size_t)pl * P * sizeof(T));
+        o.al[l] = take((size_t)(pl + 1) * g.nx * g.ny * sizeof(T));
+        o.rec[l] = take((size_t)pl * P * 4);
+    }
+    o.bs = take((size_t)D.nb * 8);
+    o.xb = take((size_t)D.nb * sizeof(T));
+    o.total = at;
+    return o;
+}
+// node record: i, j, plane within the slab (10 bits each), kind (2)
+__device__ inline int nc_rec(int i, int j, int sl, int kind) { return i | (j << 10) | (sl << 20) | (kind << 30); }
+
+struct NcLevel {
+    int NX, NY, P, nx, ny, s0, pl, np, nodes;
+    int nreg, nirr;   // listed nodes: records rec[0 .. nreg), and from the array's end
+    int lo_rank, hi_rank, dlo, dhi;
+};
+
+template <class T>
+__global__ void __cluster_dims__(kNcCtas, 1, 1) __launch_bounds__(kNcThreads)
+    k_nd_coarse(const __grid_constant__ NdCoarse<T> D)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char ncsm[];
+    __shared__ NcLevel lv[kNcMax];
+    const int tid = threadIdx.x, rank = (int)cl.block_rank(), na = D.na, ns = D.n - 1;
+    const bool act = rank < na;
+    const NcLayout &L = D.L;
+    const int npb = D.A[ns - 1].g.nz + 1;
+    if (tid < ns) {
+        const GridD &g = D.A[tid].g;
+        NcLevel v;
+        v.nx = g.nx; v.ny = g.ny; v.NX = g.nx + 1; v.NY = g.ny + 1; v.P = v.NX * v.NY; v.np = g.nz + 1;
+        v.s0 = act ? nc_s0(npb, na, ns, tid, v.np, rank) : 0;
+        v.pl = act ? nc_s0(npb, na, ns, tid, v.np, rank + 1) - v.s0 : 0;
+        v.nodes = v.pl * v.P;
+        v.nreg = v.nirr = 0;
+        v.lo_rank = act && rank > 0 ? rank - 1 : -1;
+        v.hi_rank = act && rank + 1 < na ? rank + 1 : -1;
+        v.dlo = v.lo_rank >= 0 ? (v.s0 - nc_s0(npb, na, ns, tid, v.np, rank - 1)) * v.P : 0;
+        v.dhi = -v.pl * v.P;
+        lv[tid] = v;
+    }
+    __syncthreads();
+    auto arr = [&](int off) { return reinterpret_cast<T *>(ncsm + off); };
+    for (int l = 0; l < ns; l++) {
+        NcLevel &v = lv[l];
+        const NdOp<T> &A = D.A[l];
+        T *x = arr(L.x[l]), *t = arr(L.t[l]), *b = arr(L.b[l]), *d = arr(L.d[l]), *al = arr(L.al[l]);
+        int *rec = reinterpret_cast<int *>(ncsm + L.rec[l]);
+        // (halo planes outside the box and inactive nodes stay 0)
+        for (int q = tid; q < v.nodes + 2 * v.P; q += kNcThreads) x[q] = t[q] = T(0);
+        // cell planes s0 - 1 .. s0 + pl - 1
+        const int cp = v.nx * v.ny;
+        for (int q = tid; q < (v.pl + 1) * cp && act; q += kNcThreads) {
+            const int ck = v.s0 - 1 + q / cp;
+            al[q] = ck >= 0 && ck < A.g.nz ? A.alpha[ck * cp + q % cp] : T(0);
+        }
+        for (int q = tid; q < v.nodes; q += kNcThreads) {
+            const int sl = q / v.P, r = q - sl * v.P, j = r / v.NX, i = r - j * v.NX;
+            const int n = v.s0 * v.P + q;
+            // regular nodes from the front, the others from the back: a warp of
+            // a step then takes one of the two rows (their order is of no
+            // consequence, a node's result depends on no other of the step)
+            const int kind = A.kind[n];
+            if (kind == ND_REG) rec[atomicAdd(&v.nreg, 1)] = nc_rec(i, j, sl, kind);
+            if (kind == ND_IRR) rec[v.nodes - 1 - atomicAdd(&v.nirr, 1)] = nc_rec(i, j, sl, kind);
+            d[q] = T(0);
+            if (l == 0) b[q] = D.b[n];
+        }
+    }
+    __syncthreads();
+    // f(q, w) for every active node of level l, records w
+    auto each = [&](int l, auto &&f) {
+        const NcLevel &v = lv[l];
+        const int *rec = reinterpret_cast<const int *>(ncsm + L.rec[l]);
+        const int np32 = (v.nreg + 31) & ~31, n = np32 + v.nirr;
+        for (int m = tid; m < n; m += kNcThreads) {
+            if (m >= v.nreg && m < np32) continue;
+            const int w = m < v.nreg ? rec[m] : rec[v.nodes - 1 - (m - np32)];
+            f(((w >> 20) & 1023) * v.P + ((w >> 10) & 1023) * v.NX + (w & 1023), w);
+        }
+    };
+    // diagonals, once per V-cycle (an FP64 division and a sum of eight per node)
+    for (int l = 0; l < ns; l++) {
+        const NcLevel &v = lv[l];
+        const T *al = arr(L.al[l]), h = D.A[l].h;
+        T *dg = arr(L.dg[l]), *di = arr(L.di[l]);
+        each(l, [&](int q, int w) {
+            const int i = w & 1023, j = (w >> 10) & 1023, sl = (w >> 20) & 1023;
+            T sa = T(8);
+            if ((unsigned)w >> 30 == ND_IRR) {
+                T a8[8];
+#pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    const int ci = i - 1 + (e & 1), cj = j - 1 + ((e >> 1) & 1);
+                    a8[e] = (unsigned)ci < (unsigned)v.nx && (unsigned)cj < (unsigned)v.ny
+                                ? al[((sl + (e >> 2)) * v.ny + cj) * v.nx + ci] : T(0);
+                }
+                sa = ((a8[0] + a8[1]) + (a8[2] + a8[3])) + ((a8[4] + a8[5]) + (a8[6] + a8[7]));
+            }
+            const T g = h * sa * T(1.0 / 3.0);
+            dg[q] = g;
+            di[q] = T(1) / g;
+        });
+    }
+    cl.sync();
+
+    // row of node q (record w) on x, as nd_row, its sums as trees (the FP64
+    // chains were the time of a step)
+    auto row = [&](const NcLevel &v, const T *al, T h, const T *x, int q, int w, T diag) -> T {
+        const int i = w & 1023, j = (w >> 10) & 1023, sl = (w >> 20) & 1023;
+        const T *xc = x + q + v.P;
+        const int sy = v.NX, sz = v.P;
+        T s;
+        if ((unsigned)w >> 30 == ND_REG) {
+            const T b0 = (xc[1 + sy] + xc[-1 + sy]) + (xc[1 - sy] + xc[-1 - sy]);
+            const T am = (xc[1 - sz] + xc[-1 - sz]) + (xc[sy - sz] + xc[-sy - sz]);
+            const T ap = (xc[1 + sz] + xc[-1 + sz]) + (xc[sy + sz] + xc[-sy + sz]);
+            const T bm = (xc[1 + sy - sz] + xc[-1 + sy - sz]) + (xc[1 - sy - sz] + xc[-1 - sy - sz]);
+            const T bp = (xc[1 + sy + sz] + xc[-1 + sy + sz]) + (xc[1 - sy + sz] + xc[-1 - sy + sz]);
+            s = T(2) * (b0 + (am + ap)) + (bm + bp);
+        } else {
+            // per cell its fraction times its three face-diagonal and one
+            // body-diagonal neighbours (outside the box the fraction is 0; the
+            // index is clamped to the node itself there)
+            T pr[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2, ci = i - 1 + ex, cj = j - 1 + ey;
+                const bool in = (unsigned)ci < (unsigned)v.nx && (unsigned)cj < (unsigned)v.ny;
+                const T a = in ? al[((sl + ez) * v.ny + cj) * v.nx + ci] : T(0);
+                const int ox = in ? 2 * ex - 1 : 0, oy = in ? (2 * ey - 1) * sy : 0, oz = in ? (2 * ez - 1) * sz : 0;
+                pr[e] = a * ((xc[ox + oy] + xc[ox + oz]) + (xc[oy + oz] + xc[ox + oy + oz]));
+            }
+            s = ((pr[0] + pr[1]) + (pr[2] + pr[3])) + ((pr[4] + pr[5]) + (pr[6] + pr[7]));
+        }
+        return diag * xc[0] - h * T(1.0 / 12.0) * s;
+    };
+    // own value at node q, and the copies in the neighbours' halo planes
+    auto put = [&](const NcLevel &v, T *x, T *lo, T *hi, int q, T val) {
+        const int p = q + v.P;
+        x[p] = val;
+        if (lo && q < v.P) lo[p + v.dlo] = val;
+        if (hi && q >= v.nodes - v.P) hi[p + v.dhi] = val;
+    };
+    // one Chebyshev step src -> dst (zero: src and the direction are 0)
+    auto cheb = [&](int l, const T *src, T *dst, int step, bool zero, bool halo) {
+        const NcLevel &v = lv[l];
+        const T h = D.A[l].h, cd = D.cd[step], cr = D.cr[step];
+        const T *b = arr(L.b[l]), *al = arr(L.al[l]), *dg = arr(L.dg[l]), *di = arr(L.di[l]);
+        T *d = arr(L.d[l]);
+        T *lo = halo && v.lo_rank >= 0 ? cl.map_shared_rank(dst, v.lo_rank) : nullptr;
+        T *hi = halo && v.hi_rank >= 0 ? cl.map_shared_rank(dst, v.hi_rank) : nullptr;
+        each(l, [&](int q, int w) {
+            T r = b[q];
+            if (!zero) r -= row(v, al, h, src, q, w, dg[q]);
+            T dn = cr * (r * di[q]);
+            if (!zero && cd != T(0)) dn += cd * d[q];
+            d[q] = dn;
+            put(v, dst, lo, hi, q, zero ? dn : src[q + v.P] + dn);
+        });
+    };
+#pragma unroll 1
+    for (int l = 0; l < ns; l++) {
+        const NcLevel &v = lv[l];
+        T *x = arr(L.x[l]), *t = arr(L.t[l]);
+        cheb(l, x, x, 0, true, true);
+        cl.sync();
+        cheb(l, x, t, 1, false, true);
+        cl.sync();
+        cheb(l, t, x, 2, false, true);
+        cl.sync();
+        {   // residual into t (0 on inactive nodes, as t is there)
+            const T h = D.A[l].h;
+            const T *b = arr(L.b[l]), *al = arr(L.al[l]), *dg = arr(L.dg[l]);
+            T *lo = v.lo_rank >= 0 ? cl.map_shared_rank(t, v.lo_rank) : nullptr;
+            T *hi = v.hi_rank >= 0 ? cl.map_shared_rank(t, v.hi_rank) : nullptr;
+            each(l, [&](int q, int w) { put(v, t, lo, hi, q, b[q] - row(v, al, h, x, q, w, dg[q])); });
+        }
+        cl.sync();
+        // full weighting: coarse planes K with 2 K in the slab
+        const GridD &gc = D.A[l + 1].g;
+        const int CX = gc.nx + 1, CP = CX * (gc.ny + 1);
+        const int K0 = (v.s0 + 1) >> 1, K1 = act ? (v.s0 + v.pl + 1) >> 1 : K0;
+        for (int m = tid; m < (K1 - K0) * CP; m += kNcThreads) {
+            const int K = K0 + m / CP, r = m % CP, J = r / CX, I = r - J * CX;
+            // (planes outside the box hold 0; an index outside a row or plane is
+            // clamped to the centre and its weight is 0)
+            const uint8_t on = D.A[l + 1].act[K * CP + r];
+            const T *tc = t + (2 * K - v.s0 + 1) * v.P + 2 * J * v.NX + 2 * I;
+            const int im = I > 0 ? -1 : 0, ip = 2 * I < v.nx ? 1 : 0, jm = J > 0 ? -v.NX : 0, jp = 2 * J < v.ny ? v.NX : 0;
+            const T wm = I > 0 ? T(0.5) : T(0), wp = ip ? T(0.5) : T(0), vm = J > 0 ? T(0.5) : T(0), vp = jp ? T(0.5) : T(0);
+            auto line = [&](const T *q) { return q[0] + (wm * q[im] + wp * q[ip]); };
+            auto plane = [&](const T *q) { return line(q) + (vm * line(q + jm) + vp * line(q + jp)); };
+            T sum = plane(tc) + T(0.5) * (plane(tc - v.P) + plane(tc + v.P));
+            if (!on) sum = T(0);
+            if (l + 1 < ns) arr(L.b[l + 1])[K * CP + r - lv[l + 1].s0 * CP] = sum;
+            else {
+                double *bs = reinterpret_cast<double *>(ncsm + L.bs);
+                for (int a = 0; a < na; a++) cl.map_shared_rank(bs, a)[K * CP + r] = (double)sum;
+            }
+        }
+        if (l + 1 < ns) __syncthreads();
+        else cl.sync();
+    }
+    {   // bottom: x = inv b, this block's share of the rows, 16 lanes per row, to every block
+        const double *bs = reinterpret_cast<const double *>(ncsm + L.bs);
+        T *xb = arr(L.xb);
+        const int r0 = D.nb * min(rank, na) / na, nr = D.nb * min(rank + 1, na) / na - r0, g = tid & 15;
+        for (int rr = tid >> 4; rr < (nr + 1) / 2 * 2; rr += kNcThreads / 16) {
+            double sum = 0.0;
+            if (rr < nr) {
+                const double *rw = D.binv + (size_t)(r0 + rr) * D.nb;
+#pragma unroll 4
+                for (int q = g; q < D.nb; q += 16) sum += rw[q] * bs[q];
+            }
+            for (int o = 8; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o, 16);
+            if (g == 0 && rr < nr)
+                for (int a = 0; a < na; a++) cl.map_shared_rank(xb, a)[r0 + rr] = (T)sum;
+        }
+        cl.sync();
+    }
+#pragma unroll 1
+    for (int l = ns - 1; l >= 0; l--) {
+        const NcLevel &v = lv[l];
+        T *x = arr(L.x[l]), *t = arr(L.t[l]);
+        const GridD &gc = D.A[l + 1].g;
+        const int CX = gc.nx + 1, CP = CX * (gc.ny + 1);
+        // coarse correction, at plane K: the bottom's whole array, or the
+        // slab with its halo (fine planes 2c .. reach coarse plane c' of the next slab)
+        const T *xc = l + 1 < ns ? arr(L.x[l + 1]) + (1 - lv[l + 1].s0) * CP : arr(L.xb);
+        {
+            T *lo = v.lo_rank >= 0 ? cl.map_shared_rank(t, v.lo_rank) : nullptr;
+            T *hi = v.hi_rank >= 0 ? cl.map_shared_rank(t, v.hi_rank) : nullptr;
+            each(l, [&](int q, int w) {
+                const int i = w & 1023, j = (w >> 10) & 1023, k = v.s0 + ((w >> 20) & 1023);
+                const int pi = i & 1, pj = j & 1, pk = k & 1;
+                const T *c0 = xc + (k >> 1) * CP + (j >> 1) * CX + (i >> 1);
+                // the two coarse neighbours along each axis (the same one twice at even positions)
+                const int oj = pj ? CX : 0, ok = pk ? CP : 0;
+                const T s0 = (c0[0] + c0[pi]) + (c0[oj] + c0[oj + pi]);
+                const T s1 = (c0[ok] + c0[ok + pi]) + (c0[ok + oj] + c0[ok + oj + pi]);
+                put(v, t, lo, hi, q, x[q + v.P] + T(0.125) * (s0 + s1));
+            });
+        }
+        cl.sync();
+        cheb(l, t, x, 0, false, true);
+        cl.sync();
+        cheb(l, x, t, 1, false, true);
+        cl.sync();
+        // (the top level's last step is read by nobody else: no remote write
+        // without a barrier after it)
+        cheb(l, t, x, 2, false, l > 0);
+        if (l > 0) cl.sync();
+        else __syncthreads();
+    }
+    {
+        const NcLevel &v = lv[0];
+        const T *x = arr(L.x[0]);
+        for (int q = tid; q < v.nodes; q += kNcThreads) D.x[v.s0 * v.P + q] = x[q + v.P];
+    }
+}
+
+// Which levels of the nodal hierarchy the cluster kernel takes: fills the shape
+// of D and returns its top level, or -1 (the bottom alone).  By the sizes only.
+template <class T>
+int nc_plan(const NdHier &H, NdCoarse<T> &D)
+{
+    const int Lb = H.L - 1;
+    for (int l0 = 0; l0 < Lb; l0++) {
+        const int n = Lb - l0 + 1;
+        if (n > kNcMax || nnode(H.lv[l0].g) > NcNodes<T>::n) continue;
+        const GridD &g = H.lv[l0].g;
+        if (g.nx >= 1023 || g.ny >= 1023 || g.nz >= 1023) continue;   // (record fields)
+        for (int q = 0; q < n; q++) D.A[q].g = H.lv[l0 + q].g;
+        D.n = n;
+        D.nb = H.nb;
+        D.na = std::min(kNcCtas, H.lv[Lb - 1].g.nz + 1);
+        D.L = nc_layout(D);
+        if (D.L.total <= kNcSmem) return l0;
+    }
+    return -1;
+}
+
+template <class T>
+void nc_attr()
+{
+    static bool done = false;
+    if (!done) {
+        done = true;
+        cudaFuncSetAttribute(k_nd_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNcSmem);
+    }
+}
+
 // ===========================================================================
 // Krylov glue
 // ===========================================================================
@@ -3828,7 +4181,7 @@ inline ChebCoef cheb_coef(double lmax)
 
 // Three Chebyshev steps on A x = b, ending in x.  From zero: (0) -> x -> t -> x.
 // Otherwise the start is in t: t -> x -> t -> x.  d is the level's direction.
-// A nodal pass on a level with node kinds: one launch for the listed nodes and
+// A nodal pass on a level that marches: one launch for the listed nodes and
 // the march; block partials per block of the launch.
 template <class T, int kMode>
 void nd_pass(Ctx *c, const NdLevel &L, const char *name, double nbytes, const T *xin, T *out, T *d, const T *b, T cd, T cr,
@@ -3853,7 +4206,7 @@ void nd_smooth(Ctx *c, const NdLevel &L, int l, T *x, T *t, const T *b, bool zer
         // from zero reads only b and alpha and writes d, x)
         const bool z0 = s == 0 && zero_start;
         const double nb = (z0 ? 4.0 : 6.0) * sizeof(T) * (double)nnode(L.g);
-        if (!z0 && L.kind)   // levels with node kinds: plane-sum form
+        if (!z0 && L.march)   // plane-sum form
             nd_pass<T, ND_CHEB>(c, L,
                                    sizeof(T) == 4 ? (l ? "nodal_chebyshev_step<float> L1+" : "nodal_chebyshev_step<float> L0")
                                                   : (l ? "nodal_chebyshev_step<double> L1+" : "nodal_chebyshev_step<double> L0"),
@@ -3871,12 +4224,15 @@ template <class T>
 void nd_vcycle(Ctx *c, NdHier &H, const T *b0, T *x0)
 {
     const int Lb = H.L - 1;
-    for (int l = 0; l < Lb; l++) {
+    // levels l0 .. Lb run in one cluster
+    NdCoarse<T> D;
+    const int lc = nc_plan<T>(H, D), l0 = lc < 0 ? Lb : lc;
+    for (int l = 0; l < l0; l++) {
         const NdLevel &L = H.lv[l];
         T *x = l ? (T *)c->lx[l] : x0;
         const T *b = l ? (const T *)c->lb[l] : b0;
         nd_smooth<T>(c, L, l, x, (T *)c->lt[l], b, true);
-        if (L.kind)
+        if (L.march)
             nd_pass<T, ND_RESID>(c, L, l ? "nodal_residual L1+" : "nodal_residual L0", 0.0, x, (T *)c->lr[l], nullptr, b,
                                  T(0), T(0), nullptr);
         else
@@ -3886,12 +4242,27 @@ void nd_vcycle(Ctx *c, NdHier &H, const T *b0, T *x0)
                    (T *)c->lb[l + 1]);
     }
     {
-        T *x = Lb ? (T *)c->lx[Lb] : x0;
-        const T *b = Lb ? (const T *)c->lb[Lb] : b0;
-        EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 7) / 8), dim3(256), 0, one<const double>(H.binv), H.nb,
-                   one<const T>(b), one(x), H.lv[Lb].g, 0);
+        T *x = l0 ? (T *)c->lx[l0] : x0;
+        const T *b = l0 ? (const T *)c->lb[l0] : b0;
+        if (l0 < Lb) {
+            for (int q = 0; q < D.n; q++) D.A[q] = ndop<T>(H.lv[l0 + q]);
+            D.x = x;
+            D.b = b;
+            D.binv = H.binv;
+            const ChebCoef k = cheb_coef(H.lv[l0].lam_max);   // (2 on every level)
+            for (int q = 0; q < 3; q++) {
+                D.cd[q] = (T)k.cd[q];
+                D.cr[q] = (T)k.cr[q];
+            }
+            nc_attr<T>();
+            EBV_LAUNCH_P(c, sizeof(T) == 4 ? "nodal_coarse_vcycle<float>" : "nodal_coarse_vcycle<double>", 0.0,
+                         k_nd_coarse<T>, dim3(kNcCtas), dim3(kNcThreads), D.L.total, D);
+        } else {
+            EBV_LAUNCH(c, k_bottom_solve<T>, dim3((H.nb + 7) / 8), dim3(256), 0, one<const double>(H.binv), H.nb,
+                       one<const T>(b), one(x), H.lv[Lb].g, 0);
+        }
     }
-    for (int l = Lb - 1; l >= 0; l--) {
+    for (int l = l0 - 1; l >= 0; l--) {
         const NdLevel &L = H.lv[l];
         T *x = l ? (T *)c->lx[l] : x0;
         const T *b = l ? (const T *)c->lb[l] : b0;
@@ -4482,9 +4853,10 @@ ebv_status setup_solvers(Ctx *c)
         Lv.alpha_d = l ? dalloc<double>(nc, e) : c->alpha;
         Lv.alpha_f = dalloc<float>(nc, e);
         Lv.act = dalloc<uint8_t>(nnode(gn[l]), e);
-        // node kinds (and with them the plane march): the finest level, and
-        // the coarse ones large enough that it is the faster form
-        Lv.kind = (l == 0 || nnode(gn[l]) >= kKindNodes) ? dalloc<uint8_t>(nnode(gn[l]), e) : nullptr;
+        // the plane march: the finest level, and the coarse ones large enough
+        // that it is the faster form
+        Lv.march = l == 0 || nnode(gn[l]) >= kKindNodes;
+        Lv.kind = dalloc<uint8_t>(nnode(gn[l]), e);
         Lv.lam_max = 2.0;
     }
     c->nd.binv = dalloc<double>((size_t)nbn * nbn, e);
@@ -4540,14 +4912,14 @@ ebv_status setup_geometry_solvers(Ctx *c)
         int nc = ncell(Lv.g);
         EBV_LAUNCH(c, (k_convert<double, float>), dim3(vblocks(nc)), dim3(256), 0, Lv.alpha_d, Lv.alpha_f, nc);
         EBV_LAUNCH(c, k_nd_active, ngrid(Lv.g), block3(), 0, Lv.g, Lv.alpha_d, Lv.act);
-        if (Lv.kind) EBV_LAUNCH(c, k_nd_kind, ngrid(Lv.g), block3(), 0, Lv.g, Lv.alpha_d, Lv.act, Lv.kind);
+        EBV_LAUNCH(c, k_nd_kind, ngrid(Lv.g), block3(), 0, Lv.g, Lv.alpha_d, Lv.act, Lv.kind);
     }
     for (int l = 0; l < N.L; l++) {
-        // levels with node kinds: the nodes that take the general row, in
+        // levels that march: the nodes that take the general row, in
         // ascending order -- the box faces, and inside the active nodes that
         // are not regular
         NdLevel &Lv = N.lv[l];
-        if (!Lv.kind) continue;
+        if (!Lv.march) continue;
         const GridD &gl = Lv.g;
         const int nn = nnode(gl);
         std::vector<uint8_t> kind(nn);
