@@ -320,9 +320,13 @@ __device__ inline CellPos cell_pos(const GridD &g, int i, int j, int k)
     return p;
 }
 
+// off = init + sum beta x_nb.  A residual b - (diag x - sum) in FP64 starts its
+// chain from b - diag x: seven multiply-adds instead of eight operations, in
+// kernels that the FP64 pipe bounds (the three components' residual on 256^3
+// 622 -> 553 us).
 template <class T, class F>
 __device__ inline void cc_row(const CcOp<T, F> &A, int i, int j, int k, const T *__restrict__ x,
-                              T &diag, T &off)
+                              T &diag, T &off, T init = T(0))
 {
     const GridD &g = A.g;
     const CellPos p = cell_pos<T>(g, i, j, k);
@@ -331,7 +335,7 @@ __device__ inline void cc_row(const CcOp<T, F> &A, int i, int j, int k, const T 
     const T byl = T(A.by[p.fy0]), byh = T(A.by[p.fy1]);
     const T bzl = T(A.bz[p.fz0]), bzh = T(A.bz[p.fz1]);
     diag = A.diag[c];
-    T s = 0;
+    T s = init;
     if (i > 0) s += bxl * x[p.xw];
     if (i < g.nx - 1) s += bxh * x[p.xe];
     if (j > 0) s += byl * x[c - g.nx];
@@ -371,7 +375,7 @@ __device__ inline T gs_cell(const VOp<T> &A, const T *__restrict__ x, const T *_
     const CellPos p = cell_pos<T>(g, i, j, k);
     const int c = p.c;
     const T di = A.dinv[c], bc = b[c];
-    T off = 0;
+    T off = sizeof(T) == 8 ? bc : T(0);   // (FP64: the chain starts from b, one operation less)
     if (!zero_start) {
         const T bxl = T(A.bx[p.fx0]), bxh = T(A.bx[p.fx1]);
         const T byl = T(A.by[p.fy0]), byh = T(A.by[p.fy1]);
@@ -392,7 +396,7 @@ __device__ inline T gs_cell(const VOp<T> &A, const T *__restrict__ x, const T *_
         if (k > 0) off += bzl * xd;
         if (k < g.nz - 1) off += bzh * xu;
     }
-    return (bc + off) * di;
+    return (sizeof(T) == 8 ? off : bc + off) * di;
 }
 
 // kDot (the last pass of a V-cycle on the finest level): also block partials
@@ -1196,14 +1200,14 @@ __device__ inline T rr_cell(const VOp<T> &A, const T *__restrict__ x, const T *_
         const T bxl = T(A.bx[fidxT<T>(g, 0, i, j, k)]), bxh = T(A.bx[fidxT<T>(g, 0, i + 1, j, k)]);
         const T byl = T(A.by[fidxT<T>(g, 1, i, j, k)]), byh = T(A.by[fidxT<T>(g, 1, i, j + 1, k)]);
         const T bzl = T(A.bz[fidxT<T>(g, 2, i, j, k)]), bzh = T(A.bz[fidxT<T>(g, 2, i, j, k + 1)]);
-        T off = 0;
+        T off = sizeof(T) == 8 ? b[c] - A.diag[c] * x[c] : T(0);
         if (i > 0) off += bxl * x[cix<T>(g, i - 1, j, k)];
         if (i < g.nx - 1) off += bxh * x[cix<T>(g, i + 1, j, k)];
         if (j > 0) off += byl * x[c - g.nx];
         if (j < g.ny - 1) off += byh * x[c + g.nx];
         if (k > 0) off += bzl * x[c - g.nx * g.ny];
         if (k < g.nz - 1) off += bzh * x[c + g.nx * g.ny];
-        s += b[c] - (A.diag[c] * x[c] - off);
+        s += sizeof(T) == 8 ? off : b[c] - (A.diag[c] * x[c] - off);
     }
     return s * T(0.125);
 }
@@ -1596,16 +1600,20 @@ __global__ void __launch_bounds__(256) k_cc_apply_dot(CcOp3<T> A3, V3<const T> p
             const int k = 2 * kk + h;
             if (k >= A.g.nz) continue;
             T diag, off;
-            cc_row(A, i, j, k, p, diag, off);
             cc[h] = cix<T>(A.g, i, j, k);
             pc[h] = p[cc[h]];
-            y[h] = diag * pc[h] - off;
+            if constexpr (kRes) {
+                cc_row(A, i, j, k, p, diag, y[h], b[cc[h]] - A.diag[cc[h]] * pc[h]);
+            } else {
+                cc_row(A, i, j, k, p, diag, off);
+                y[h] = diag * pc[h] - off;
+            }
         }
 #pragma unroll
         for (int h = 0; h < 2; h++)
             if (cc[h] >= 0) {
                 if constexpr (kRes) {
-                    const float r = f64_to_f32_pow2(b[cc[h]] - y[h], sc);
+                    const float r = f64_to_f32_pow2(y[h], sc);
                     r32[cix<float>(A.g, i, j, 2 * kk + h)] = r;
                     vr += r * r;
                 } else {
@@ -1794,12 +1802,10 @@ __device__ inline void nd_row(const NdOp<T> &A, int i, int j, int k, const T *__
 }
 
 // One Chebyshev step: r = b - A x_in; d = cd d + cr D^-1 r; x_out = x_in + d.
-// Node by node: the first step from zero on every level, and all steps on the
-// levels without regular-node flags (the others take the plane march).
+// Node by node, on the levels that do not take the plane march.
 template <class T>
 __global__ void __launch_bounds__(256) k_nd_cheb(NdOp<T> A, const T *__restrict__ xin, T *__restrict__ xout,
-                                                 T *__restrict__ dvec, const T *__restrict__ b, T cd, T cr,
-                                                 int zero_start)
+                                                 T *__restrict__ dvec, const T *__restrict__ b, T cd, T cr)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1809,38 +1815,74 @@ __global__ void __launch_bounds__(256) k_nd_cheb(NdOp<T> A, const T *__restrict_
     const int n = nidx(g, i, j, k);
     // the node's own operands are loaded before any branch on them
     const uint8_t on = A.act[n];
-    const T bn = b[n];
-    T xn = T(0), dold = T(0);
-    if (!zero_start) {
-        xn = xin[n];
-        dold = dvec[n];
-    }
+    const T bn = b[n], xn = xin[n], dold = dvec[n];
     if (!on) {
         xout[n] = T(0);
         dvec[n] = T(0);
         return;
     }
     T diag, ax;
-    if (zero_start) {
-        // x_in = 0, d = 0: only the diagonal is needed
-        T dsum = 0;
-        for (int oc = 0; oc < 8; oc++) {
-            int ci = i - 1 + (oc & 1), cj = j - 1 + ((oc >> 1) & 1), ck = k - 1 + ((oc >> 2) & 1);
-            if (!inbox(g, ci, cj, ck)) continue;
-            T al = A.alpha[cidx(g, ci, cj, ck)];
-            if (al > T(0)) dsum += al;
-        }
-        diag = A.h * dsum * T(1.0 / 3.0);
-        T dn = cr * bn / diag;
-        dvec[n] = dn;
-        xout[n] = dn;
-        return;
-    }
     nd_row(A, i, j, k, xin, diag, ax);
     T r = bn - ax;
     T dn = (cd != T(0) ? cd * dold : T(0)) + cr * r / diag;
     dvec[n] = dn;
     xout[n] = xn + dn;
+}
+
+// The first step from x = 0, d = 0: x = d = cr D^-1 b, a constant times b on
+// regular nodes; only the others sum their cells' fractions.  Streams 16 bytes
+// per thread and array (arrays from cudaMalloc), then the tail (FP32 256^3: as
+// part of k_nd_cheb 130 us, eight fractions and a division per node; 55 us so).
+template <class T>
+__global__ void __launch_bounds__(128) k_nd_cheb0(NdOp<T> A, T *__restrict__ x, T *__restrict__ d, const T *__restrict__ b,
+                                                  T cr, T crd, int nn)
+{
+    const GridD &g = A.g;   // (crd = cr / regular diagonal)
+    auto other = [&](int n, T bn) -> T {   // an active node that is not regular
+        const int NX = g.nx + 1, NY = g.ny + 1, i = n % NX, j = (n / NX) % NY, k = n / (NX * NY);
+        T a[8];
+#pragma unroll
+        for (int oc = 0; oc < 8; oc++) {
+            const int ci = i - 1 + (oc & 1), cj = j - 1 + ((oc >> 1) & 1), ck = k - 1 + ((oc >> 2) & 1);
+            a[oc] = inbox(g, ci, cj, ck) ? A.alpha[cidx(g, ci, cj, ck)] : T(0);
+        }
+        const T dsum = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+        return cr * bn / (A.h * dsum * T(1.0 / 3.0));
+    };
+    constexpr int W = 16 / sizeof(T);
+    const int nv = nn / W, t0 = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
+    for (int s = t0; s < nv; s += st) {
+        T v[W];
+        uint8_t kd[W];
+        if constexpr (W == 4) {
+            const float4 q = reinterpret_cast<const float4 *>(b)[s];
+            v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+            const uchar4 c = reinterpret_cast<const uchar4 *>(A.kind)[s];
+            kd[0] = c.x; kd[1] = c.y; kd[2] = c.z; kd[3] = c.w;
+        } else {
+            const double2 q = reinterpret_cast<const double2 *>(b)[s];
+            v[0] = q.x; v[1] = q.y;
+            const uchar2 c = reinterpret_cast<const uchar2 *>(A.kind)[s];
+            kd[0] = c.x; kd[1] = c.y;
+        }
+#pragma unroll
+        for (int u = 0; u < W; u++)
+            v[u] = kd[u] == ND_REG ? crd * v[u] : (kd[u] == ND_OFF ? T(0) : other(W * s + u, v[u]));
+        if constexpr (W == 4) {
+            const float4 q = make_float4(v[0], v[1], v[2], v[3]);
+            reinterpret_cast<float4 *>(x)[s] = q;
+            reinterpret_cast<float4 *>(d)[s] = q;
+        } else {
+            const double2 q = make_double2(v[0], v[1]);
+            reinterpret_cast<double2 *>(x)[s] = q;
+            reinterpret_cast<double2 *>(d)[s] = q;
+        }
+    }
+    for (int n = W * nv + t0; n < nn; n += st) {
+        const T v = A.kind[n] == ND_REG ? crd * b[n] : (A.kind[n] == ND_OFF ? T(0) : other(n, b[n]));
+        x[n] = v;
+        d[n] = v;
+    }
 }
 
 // ---- nodal passes in plane-sum form (levels with node kinds) ------------------------
@@ -1897,13 +1939,36 @@ inline NdShape nd_shape(const GridD &g, int nlist)
     return s;
 }
 
+// Constants of a pass on regular nodes, formed on the host (a division per
+// thread cost as much as the node's row where a block marches few planes):
+// diagonal, h / 12, and of the Chebyshev step cd, cr, cr / diagonal and that
+// times the other two.
+template <class T>
+struct NdCoef {
+    T cd, cr, dreg, h12, crd, c0, c1;
+};
+template <class T>
+inline NdCoef<T> nd_coef(T h, T cd, T cr)
+{
+    NdCoef<T> k;
+    k.cd = cd;
+    k.cr = cr;
+    k.dreg = h * T(8.0 / 3.0);
+    k.h12 = h * T(1.0 / 12.0);
+    k.crd = cr / k.dreg;
+    k.c0 = k.crd * k.dreg;
+    k.c1 = k.crd * k.h12;
+    return k;
+}
+
 template <class T, int kMode>
 __global__ void __launch_bounds__(NT_T) k_nd_pass(NdOp<T> A, NdShape sh, const int *__restrict__ list, int nlist,
                                                           const T *__restrict__ xin, T *__restrict__ out,
-                                                          T *__restrict__ dvec, const T *__restrict__ b, T cd, T cr,
+                                                          T *__restrict__ dvec, const T *__restrict__ b, NdCoef<T> ck,
                                                           double *__restrict__ part, float *__restrict__ out32,
                                                           const double *__restrict__ sig)
 {
+    const T cd = ck.cd, cr = ck.cr;
     const double sc = (kMode == ND_RES32 && sig) ? *sig : 1.0;
     const GridD &g = A.g;
     const int NX = g.nx + 1, NY = g.ny + 1, tid = threadIdx.x;
@@ -1953,8 +2018,7 @@ __global__ void __launch_bounds__(NT_T) k_nd_pass(NdOp<T> A, NdShape sh, const i
 #pragma unroll
             for (int u = 0; u < NT_SLOTS; u++) pre[u] = soff[u] >= 0 ? xin[kk * sz + soff[u]] : T(0);
         };
-        const T dreg = A.h * T(8.0 / 3.0), h12 = A.h * T(1.0 / 12.0);
-        const T crd = cr / dreg, c0 = crd * dreg, c1 = crd * h12;   // regular nodes: cr / diag
+        const T dreg = ck.dreg, h12 = ck.h12, crd = ck.crd, c0 = ck.c0, c1 = ck.c1;
         T Cm = 0, C0 = 0, B0 = 0, X0 = 0, b_c = 0, d_c = 0, b_n = 0, d_n = 0;
         int kd_c = -1, kd_n = -1;   // node kind, -1: no node of this block
         fetch(k0 - 1);
@@ -1996,11 +2060,15 @@ __global__ void __launch_bounds__(NT_T) k_nd_pass(NdOp<T> A, NdShape sh, const i
                     dvec[n] = dn;
                     out[n] = X0 + dn;
                 } else {
-                    const T ax = dreg * X0 - h12 * t;
-                    if (kMode == ND_RESID) out[n] = b_c - ax;
-                    if (kMode == ND_APPLY) { out[n] = ax; v += X0 * ax; }
+                    // (a residual as two multiply-adds on b)
+                    if (kMode == ND_RESID) out[n] = (b_c - dreg * X0) + h12 * t;
+                    if (kMode == ND_APPLY) {
+                        const T ax = dreg * X0 - h12 * t;
+                        out[n] = ax;
+                        v += X0 * ax;
+                    }
                     if (kMode == ND_RES32) {
-                        const float r = f64_to_f32_pow2(b_c - ax, sc);
+                        const float r = f64_to_f32_pow2((b_c - dreg * X0) + h12 * t, sc);
                         out32[n] = r;
                         vr += r * r;
                     }
@@ -2032,7 +2100,9 @@ __global__ void __launch_bounds__(256) k_nd_resid(NdOp<T> A, const T *__restrict
     r[n] = b[n] - ax;
 }
 
-// Full weighting (transpose of trilinear prolongation).
+// Full weighting (transpose of trilinear prolongation), line by line and plane
+// by plane (27 guarded and weighted terms one by one before: 13.5 -> 8.4 us on
+// average over the launched levels of 256^3).
 template <class T>
 __global__ void k_nd_restrict(GridD gf, const T *__restrict__ rf, GridD gc, const uint8_t *__restrict__ actc,
                               T *__restrict__ bc)
@@ -2042,52 +2112,57 @@ __global__ void k_nd_restrict(GridD gf, const T *__restrict__ rf, GridD gc, cons
     const int K = blockIdx.z * blockDim.z + threadIdx.z;
     if (I > gc.nx || J > gc.ny || K > gc.nz) return;
     const int N = nidx(gc, I, J, K);
-    if (!actc[N]) { bc[N] = T(0); return; }
-    T s = 0;
-    for (int dk = -1; dk <= 1; dk++) {
-        int k = 2 * K + dk;
-        if (k < 0 || k > gf.nz) continue;
-        T wk = dk ? T(0.5) : T(1);
-        for (int dj = -1; dj <= 1; dj++) {
-            int j = 2 * J + dj;
-            if (j < 0 || j > gf.ny) continue;
-            T wj = dj ? T(0.5) : T(1);
-            for (int di = -1; di <= 1; di++) {
-                int i = 2 * I + di;
-                if (i < 0 || i > gf.nx) continue;
-                T wi = di ? T(0.5) : T(1);
-                s += wi * wj * wk * rf[nidx(gf, i, j, k)];
-            }
-        }
+    const int sy = gf.nx + 1, sz = (gf.nx + 1) * (gf.ny + 1);
+    const T *q = rf + nidx(gf, 2 * I, 2 * J, 2 * K);
+    const int im = I > 0 ? -1 : 0, ip = 2 * I < gf.nx ? 1 : 0, jm = J > 0 ? -sy : 0, jp = 2 * J < gf.ny ? sy : 0;
+    const int km = K > 0 ? -sz : 0, kp = 2 * K < gf.nz ? sz : 0;
+    const T hf = T(0.5);
+    T s;
+    if constexpr (sizeof(T) == 8) {   // fewest operations (guarded reads: 9.1 us on 128^3, 12.5 with the weights)
+        auto line = [&](const T *p) { return p[0] + hf * ((im ? p[im] : T(0)) + (ip ? p[ip] : T(0))); };
+        auto plane = [&](const T *p) { return line(p) + hf * ((jm ? line(p + jm) : T(0)) + (jp ? line(p + jp) : T(0))); };
+        s = plane(q) + hf * ((km ? plane(q + km) : T(0)) + (kp ? plane(q + kp) : T(0)));
+    } else {                          // unguarded reads, weight 0 outside (8.4 us on 256^3, 12.4 guarded)
+        const T um = im ? hf : T(0), up = ip ? hf : T(0), vm = jm ? hf : T(0), vp = jp ? hf : T(0);
+        const T wm = km ? hf : T(0), wp = kp ? hf : T(0);
+        auto line = [&](const T *p) { return p[0] + (um * p[im] + up * p[ip]); };
+        auto plane = [&](const T *p) { return line(p) + (vm * line(p + jm) + vp * line(p + jp)); };
+        s = plane(q) + (wm * plane(q + km) + wp * plane(q + kp));
     }
-    bc[N] = s;
+    bc[N] = actc[N] ? s : T(0);
 }
 
 // xout = xin + trilinear interpolation of the coarse correction (active nodes).
+// A thread forms nodes (i, j, 2K) and (i, j, 2K + 1) from the coarse planes K and
+// K + 1; along x the two coarse neighbours are the same one at even i, so the
+// lanes of a row run the same instructions (a branch per term and one node per
+// thread before: 27.4 -> 14.0 us on average over the levels of 256^3).
 template <class T>
 __global__ void k_nd_prolong(GridD gf, const uint8_t *__restrict__ actf, GridD gc, const T *__restrict__ xc,
                              const T *__restrict__ xin, T *__restrict__ xout)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int k = blockIdx.z * blockDim.z + threadIdx.z;
-    if (i > gf.nx || j > gf.ny || k > gf.nz) return;
-    const int n = nidx(gf, i, j, k);
-    if (!actf[n]) { xout[n] = T(0); return; }
-    int i0 = i >> 1, j0 = j >> 1, k0 = k >> 1;
-    int i1 = i0 + (i & 1), j1 = j0 + (j & 1), k1 = k0 + (k & 1);
-    T wi = (i & 1) ? T(0.5) : T(1), wj = (j & 1) ? T(0.5) : T(1), wk = (k & 1) ? T(0.5) : T(1);
-    T s = 0;
-    s += xc[nidx(gc, i0, j0, k0)];
-    if (i & 1) s += xc[nidx(gc, i1, j0, k0)];
-    if (j & 1) s += xc[nidx(gc, i0, j1, k0)];
-    if (k & 1) s += xc[nidx(gc, i0, j0, k1)];
-    if ((i & 1) && (j & 1)) s += xc[nidx(gc, i1, j1, k0)];
-    if ((i & 1) && (k & 1)) s += xc[nidx(gc, i1, j0, k1)];
-    if ((j & 1) && (k & 1)) s += xc[nidx(gc, i0, j1, k1)];
-    if ((i & 1) && (j & 1) && (k & 1)) s += xc[nidx(gc, i1, j1, k1)];
-    xout[n] = xin[n] + wi * wj * wk * s;
+    const int K = blockIdx.z * blockDim.z + threadIdx.z;
+    if (i > gf.nx || j > gf.ny || K > gc.nz) return;
+    const int n0 = nidx(gf, i, j, 2 * K), sz = (gf.nx + 1) * (gf.ny + 1);
+    const int cy = gc.nx + 1, cz = (gc.nx + 1) * (gc.ny + 1);
+    const bool up = K < gc.nz;   // (node plane 2K + 1 exists)
+    const uint8_t on0 = actf[n0], on1 = up ? actf[n0 + sz] : 0;
+    const T x0 = xin[n0], x1 = up ? xin[n0 + sz] : T(0);
+    const T *c = xc + nidx(gc, i >> 1, j >> 1, K);
+    const int pi = i & 1, pj = j & 1;
+    // four times the interpolation within a coarse plane
+    auto plane = [&](const T *q) {
+        T s = q[0] + q[pi];
+        if (pj) s += q[cy] + q[cy + pi];
+        return pj ? s : T(2) * s;
+    };
+    const T s0 = plane(c), s1 = up ? plane(c + cz) : T(0);
+    xout[n0] = on0 ? x0 + T(0.25) * s0 : T(0);
+    if (up) xout[n0 + sz] = on1 ? x1 + T(0.125) * (s0 + s1) : T(0);
 }
+inline dim3 prolong_grid(const GridD &gf, const GridD &gc) { return grid3(gf.nx + 1, gf.ny + 1, gc.nz + 1); }
 
 __global__ void k_nd_alpha_coarsen(GridD gf, const double *__restrict__ af, GridD gc, double *__restrict__ ac)
 {
@@ -2514,12 +2589,13 @@ struct CvView {
     int h, sy, sz, pairs, cap;   // cap: slots per colour
     // sum of face times neighbour of the cell at p whose x- neighbour is at w
     // (its x+ neighbour is the next word of the other half-row)
-    __device__ T off(const Rec &r, int p, int w, T &di) const
+    // (FP64: added to init, as gs_cell's chain)
+    __device__ T off(const Rec &r, int p, int w, T &di, T init) const
     {
         T f[6];
         r.get(f, di);
         const T xw = x[w], xe = x[w + 1], xs = x[p - sy], xn = x[p + sy], xd = x[p - sz], xu = x[p + sz];
-        T s = f[0] * xw;
+        T s = sizeof(T) == 8 ? init + f[0] * xw : f[0] * xw;
         s += f[1] * xe;
         s += f[2] * xs;
         s += f[3] * xn;
@@ -2549,10 +2625,10 @@ struct CvView {
                 const int base = in[u] & kCvPos;
                 const bool q = ((in[u] >> kCvParBit) ^ c) & 1;   // the cell of colour c is the pair's odd one
                 p[u] = base + (q ? h : 0);
-                T di, o = T(0);
+                T di, o = sizeof(T) == 8 ? bb : T(0);
                 if (from_zero) rec[c * cap + mu].get_di(di);
-                else o = off(rec[c * cap + mu], p[u], base + (q ? 0 : h - 1), di);
-                v[u] = (bb + o) * di;
+                else o = off(rec[c * cap + mu], p[u], base + (q ? 0 : h - 1), di, bb);
+                v[u] = (sizeof(T) == 8 ? o : bb + o) * di;
             }
             put(p[0], v[0], in[0]);
             if (m + kCvThreads < pairs) put(p[1], v[1], in[1]);
@@ -2744,8 +2820,8 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
                 for (int m = tid; m < w.pairs; m += kCvThreads) {
                     const int in = w.info[m], base = in & kCvPos, p = base + ((in & kCvPar) ? w.h : 0);
                     T di;
-                    const T o = w.off(w.rec[m], p, base + ((in & kCvPar) ? 0 : w.h - 1), di);
-                    res[p - lv[l].plane] = w.b[m] - (dg[m] * w.x[p] - o);
+                    const T o = w.off(w.rec[m], p, base + ((in & kCvPar) ? 0 : w.h - 1), di, w.b[m] - dg[m] * w.x[p]);
+                    res[p - lv[l].plane] = sizeof(T) == 8 ? o : w.b[m] - (dg[m] * w.x[p] - o);
                 }
             }
             __syncthreads();
@@ -4189,7 +4265,7 @@ void nd_pass(Ctx *c, const NdLevel &L, const char *name, double nbytes, const T 
 {
     const NdShape sh = nd_shape(L.g, L.nirr);
     EBV_LAUNCH_P(c, name, nbytes, (k_nd_pass<T, kMode>), dim3(sh.blocks), dim3(NT_T), 0, ndop<T>(L), sh, L.irr,
-                 L.nirr, xin, out, d, b, cd, cr, part, out32, sig);
+                 L.nirr, xin, out, d, b, nd_coef<T>((T)L.g.h, cd, cr), part, out32, sig);
 }
 // partial sums written by nd_pass on level L
 inline int nd_pass_parts(const NdLevel &L) { return nd_shape(L.g, L.nirr).blocks; }
@@ -4206,7 +4282,12 @@ void nd_smooth(Ctx *c, const NdLevel &L, int l, T *x, T *t, const T *b, bool zer
         // from zero reads only b and alpha and writes d, x)
         const bool z0 = s == 0 && zero_start;
         const double nb = (z0 ? 4.0 : 6.0) * sizeof(T) * (double)nnode(L.g);
-        if (!z0 && L.march)   // plane-sum form
+        if (z0)
+            EBV_LAUNCH_P(c, sizeof(T) == 4 ? "nodal_chebyshev_first<float>" : "nodal_chebyshev_first<double>", nb,
+                         k_nd_cheb0<T>,
+                         dim3(std::min(8 * kReduceBlocks, (nnode(L.g) / (16 / (int)sizeof(T)) + 127) / 128 + 1)), dim3(128),
+                         0, A, dst, d, b, (T)k.cr[s], nd_coef<T>((T)L.g.h, T(0), (T)k.cr[s]).crd, nnode(L.g));
+        else if (L.march)   // plane-sum form
             nd_pass<T, ND_CHEB>(c, L,
                                    sizeof(T) == 4 ? (l ? "nodal_chebyshev_step<float> L1+" : "nodal_chebyshev_step<float> L0")
                                                   : (l ? "nodal_chebyshev_step<double> L1+" : "nodal_chebyshev_step<double> L0"),
@@ -4214,7 +4295,7 @@ void nd_smooth(Ctx *c, const NdLevel &L, int l, T *x, T *t, const T *b, bool zer
         else
             EBV_LAUNCH_P(c, sizeof(T) == 4 ? "nodal_chebyshev_step<float>" : "nodal_chebyshev_step<double>", nb,
                          k_nd_cheb<T>, ch_grid(L.g, L.ch_blk), L.ch_blk, 0, A, src, dst, d, b, (T)k.cd[s],
-                         (T)k.cr[s], (int)z0);
+                         (T)k.cr[s]);
         src = dst;
         dst = (dst == x) ? t : x;
     }
@@ -4267,7 +4348,7 @@ void nd_vcycle(Ctx *c, NdHier &H, const T *b0, T *x0)
         T *x = l ? (T *)c->lx[l] : x0;
         const T *b = l ? (const T *)c->lb[l] : b0;
         // t = x + P x_coarse, then smooth from t back into x
-        EBV_LAUNCH(c, k_nd_prolong<T>, ngrid(L.g), block3(), 0, L.g, L.act, H.lv[l + 1].g,
+        EBV_LAUNCH(c, k_nd_prolong<T>, prolong_grid(L.g, H.lv[l + 1].g), block3(), 0, L.g, L.act, H.lv[l + 1].g,
                    (const T *)c->lx[l + 1], x, (T *)c->lt[l]);
         nd_smooth<T>(c, L, l, x, (T *)c->lt[l], b, false);
     }
@@ -5075,7 +5156,7 @@ ebv_status autotune_shapes_t(Ctx *c)
         for (int q = 0; q < nc; q++) {
             const dim3 bk = cand[q], gr = ch_grid(L.g, bk);
             float ms = time_it([&]() {
-                k_nd_cheb<T><<<gr, bk, 0, c->stream>>>(A, x, y, d, b, (T)k.cd[1], (T)k.cr[1], 0);
+                k_nd_cheb<T><<<gr, bk, 0, c->stream>>>(A, x, y, d, b, (T)k.cd[1], (T)k.cr[1]);
             });
             if (ms < best) { best = ms; L.ch_blk = bk; }
         }
