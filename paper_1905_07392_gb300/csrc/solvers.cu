@@ -182,6 +182,40 @@ __global__ void __cluster_dims__(kRedCtas, 1, 1) __launch_bounds__(kRedThreads)
     }
 }
 
+// k_reduce_final for at most kRedSmall partials: one small block per component.
+// The sum of few terms is latency -- of the shuffle steps, which every warp
+// takes through the FP64 pipe, and of the cluster's barriers (64^3, three
+// components: 3.2 us over a cluster, 1.8 us so).
+constexpr int kRedSmall = 1024, kRedSmallThreads = 128;
+__device__ inline double small_sum(const double *part, int n, int t, double *sm)
+{
+    // t: 0 .. kRedSmallThreads - 1; sm: one word per warp; valid in t = 0
+    double v = 0.0;
+    for (int s = t; s < n; s += kRedSmallThreads) v += part[s];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((t & 31) == 0) sm[t >> 5] = v;
+    __syncthreads();
+    return t == 0 ? (sm[0] + sm[1]) + (sm[2] + sm[3]) : 0.0;
+}
+__global__ void __launch_bounds__(kRedSmallThreads) k_reduce_small(const double *part, int n, double *out, double *scal,
+                                                                   int post, const int *act)
+{
+    __shared__ double sm[kRedSmallThreads / 32];
+    const int comp = blockIdx.y;
+    part += comp * kPartComp;
+    out += comp * kScalLen;
+    scal += comp * kScalLen;
+    const bool off = comp_off(act, comp);
+    // the quotient's other operand, loaded meanwhile
+    const double other = post == kRedAlpha ? scal[S_RZ] : (post == kRedBeta ? scal[S_RZOLD] : 0.0);
+    const double t = small_sum(part, n, threadIdx.x, sm);
+    if (threadIdx.x == 0 && !off) {
+        *out = t;
+        if (post == kRedAlpha) scal[S_ALPHA] = other / t;
+        if (post == kRedBeta) scal[S_BETA] = t / other;
+    }
+}
+
 __global__ void __launch_bounds__(256) k_dot(V3<const double> av, V3<const double> bv, int n,
                                              double *__restrict__ part)
 {
@@ -196,10 +230,16 @@ __global__ void __launch_bounds__(256) k_dot(V3<const double> av, V3<const doubl
 
 }  // namespace
 
+static void launch_reduce(Ctx *c, int nc, const double *part, int n, double *out, int post, const int *act)
+{
+    if (n <= kRedSmall)
+        EBV_LAUNCH(c, k_reduce_small, dim3(1, nc), dim3(kRedSmallThreads), 0, part, n, out, c->scal, post, act);
+    else
+        EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas, nc), dim3(kRedThreads), 0, part, n, out, c->scal, post, act);
+}
 ebv_status reduce_sum(Ctx *c, const double *part, int nblocks, double *out_dev)
 {
-    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas), dim3(kRedThreads), 0, part, nblocks, out_dev, c->scal,
-               (int)kRedSum, (const int *)nullptr);
+    launch_reduce(c, 1, part, nblocks, out_dev, kRedSum, nullptr);
     return EBV_OK;
 }
 // A sum of every component's partials into its scalar S; r.z and p.q of a CG
@@ -207,8 +247,7 @@ ebv_status reduce_sum(Ctx *c, const double *part, int nblocks, double *out_dev)
 static void reduce_comp(Ctx *c, int nc, int nblocks, int S, int post = kRedSum, const int *act = nullptr,
                         const double *part = nullptr)
 {
-    EBV_LAUNCH(c, k_reduce_final, dim3(kRedCtas, nc), dim3(kRedThreads), 0, part ? part : c->part, nblocks,
-               c->scal + S, c->scal, post, act);
+    launch_reduce(c, nc, part ? part : c->part, nblocks, c->scal + S, post, act);
 }
 
 namespace {
@@ -3362,14 +3401,13 @@ __global__ void k_solve_begin(int *ctl, int nc)
 __global__ void k_outer_check(double *scal0, int *ctl0, int nc, double tol, int maxit, int max_pass, int refine,
                               double inner_drop, cudaGraphConditionalHandle h, int use_h)
 {
-    if (threadIdx.x) return;
-    int any = 0;
-    for (int q = 0; q < nc; q++) {
-        double *scal = scal0 + q * kScalLen;
-        int *ctl = ctl0 + q * C_LEN;
-        if (!ctl[C_COND_OUT]) continue;   // (this component's solve has ended)
+    // a lane per component
+    int go = 0;
+    const int q = threadIdx.x;
+    double *scal = scal0 + q * kScalLen;
+    int *ctl = ctl0 + q * C_LEN;
+    if (q < nc && ctl[C_COND_OUT]) {   // (else this component's solve has ended)
         const double bb = scal[S_BB], rr = scal[S_RR];
-        int go = 0;
         if (ctl[C_ERR] == 0) {
             if (!isfinite(rr) || !isfinite(bb)) {
                 ctl[C_ERR] = E_NAN;
@@ -3391,10 +3429,12 @@ __global__ void k_outer_check(double *scal0, int *ctl0, int nc, double tol, int 
         ctl[C_NOUT]++;
         ctl[C_K] = 0;
         ctl[C_COND_OUT] = go;
-        any |= go;
     }
-    ctl0[J_NOUT]++;
-    set_cond(ctl0, J_OUT, any, h, use_h);
+    const int any = __any_sync(0xffffffffu, go);
+    if (q == 0) {
+        ctl0[J_NOUT]++;
+        set_cond(ctl0, J_OUT, any, h, use_h);
+    }
 }
 
 // After one CG iteration (S_RR = recursive residual norm^2).  FP64 path:
@@ -3429,39 +3469,29 @@ __device__ inline int inner_check(double *scal, int *ctl, double tol, int maxit,
 }
 
 // S_RR = the sum of the update's n block partials, then the same decision
-// (one launch instead of a reduction and a check), per component; the loop goes
-// on while one does.
-__global__ void __launch_bounds__(1024) k_reduce_inner_check(const double *part, int n, double *scal, int *ctl, int nc,
-                                                             double tol, int maxit, int refine,
-                                                             cudaGraphConditionalHandle h, int use_h)
+// (one launch instead of a reduction and a check), per component: 128 threads
+// sum, a lane of the first warp decides; the loop goes on while one component
+// does.  (With 1024 threads per component's sum and one thread for the three
+// decisions the FP64 shuffle steps and the chains of loads took 5.8 us for
+// three components at 64^3; 3.2 us so.)
+__global__ void __launch_bounds__(kMaxComp * kRedSmallThreads) k_reduce_inner_check(const double *part, int n, double *scal,
+                                                                                  int *ctl, int nc, double tol, int maxit,
+                                                                                  int refine,
+                                                                                  cudaGraphConditionalHandle h, int use_h)
 {
-    __shared__ double sm[kMaxComp][32];
-    double v[kMaxComp];
-    int on[kMaxComp];
-#pragma unroll
-    for (int q = 0; q < kMaxComp; q++) {
-        v[q] = 0.0;
-        on[q] = q < nc ? ctl[q * C_LEN + C_COND_IN] : 0;
-    }
-    for (int q = 0; q < nc; q++)
-        for (int s = threadIdx.x; s < n; s += 1024) v[q] += part[q * kPartComp + s];
-    // (as block_sum<1024>, the components' warp sums behind one barrier)
-    for (int q = 0; q < nc; q++) {
-        double w = v[q];
-        for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(0xffffffffu, w, o);
-        if ((threadIdx.x & 31) == 0) sm[q][threadIdx.x >> 5] = w;
-    }
+    __shared__ double sm[kMaxComp][kRedSmallThreads / 32], sum[kMaxComp];
+    const int q = threadIdx.x / kRedSmallThreads, t = threadIdx.x % kRedSmallThreads;
+    const double v = small_sum(part + q * kPartComp, n, t, sm[q]);
+    if (t == 0) sum[q] = v;
     __syncthreads();
     if (threadIdx.x >= 32) return;
-    int any = 0;
-    for (int q = 0; q < nc; q++) {
-        double w = sm[q][threadIdx.x];
-        for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(0xffffffffu, w, o);
-        if (threadIdx.x == 0 && on[q]) {
-            scal[q * kScalLen + S_RR] = w;
-            any |= inner_check(scal + q * kScalLen, ctl + q * C_LEN, tol, maxit, refine);
-        }
+    int go = 0;
+    if ((int)threadIdx.x < nc && ctl[threadIdx.x * C_LEN + C_COND_IN]) {
+        const int c = threadIdx.x;
+        scal[c * kScalLen + S_RR] = sum[c];
+        go = inner_check(scal + c * kScalLen, ctl + c * C_LEN, tol, maxit, refine);
     }
+    const int any = __any_sync(0xffffffffu, go);
     if (threadIdx.x == 0) {
         ctl[J_IT]++;
         set_cond(ctl, J_IN, any, h, use_h);
@@ -4555,7 +4585,7 @@ ebv_status pcg(Ctx *c, Problem &P, V3<const double> b, V3<double> x, int *iters,
             P.apply_dot(c, p, q, gin);
             reduce_comp(c, nc, P.apply_blocks(), S_PQ, kRedAlpha, in);
             EBV_LAUNCH(c, k_cg_update, gv, dim3(256), 0, x, r, p, q, c->scal, n, c->part, in);
-            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, vblocks(n), c->scal, c->ctl, nc, tol,
+            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(nc * kRedSmallThreads), 0, c->part, vblocks(n), c->scal, c->ctl, nc, tol,
                        maxit, 0, inner.h, inner.use_h);
         }
         inner_count = inner.body_launches();
@@ -4618,7 +4648,7 @@ ebv_status pcg_refine(Ctx *c, Problem &P, V3<const double> b, V3<double> x, int 
             P.apply_dot32(c, p, q, gin);
             reduce_comp(c, nc, P.apply_blocks32(), S_PQ, kRedAlpha, in);
             EBV_LAUNCH(c, k_cg_update32, g4, dim3(256), 0, r, q, c->scal, n, c->part, in);
-            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(1024), 0, c->part, v4blocks(n), c->scal, c->ctl, nc, tol,
+            EBV_LAUNCH(c, k_reduce_inner_check, dim3(1), dim3(nc * kRedSmallThreads), 0, c->part, v4blocks(n), c->scal, c->ctl, nc, tol,
                        maxit, 1, inner.h, inner.use_h);
         }
         inner_count = inner.body_launches();
