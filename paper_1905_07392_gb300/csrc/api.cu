@@ -974,7 +974,7 @@ namespace {
 
 struct AdjBufs {
     double *em, *es, *eb, *Gm, *Gs, *Vm, *Vs, *Va, *psi, *utm, *uts, *us, *zero3, *t3;
-    double *ebm, *ebs, *ebb, *Gb, *Vbs, *Vbm, *psib, *usb, *utb, *lam, *DCb, *tb, *etad;
+    double *ebm, *ebs, *ebb, *Gb, *Vbs, *Vbm, *psib, *usb, *utb, *DCb, *tb, *etad;
     double *ffb, *dudnb, *ps, *psb, *nb1, *nb2, *ua, *pa, *grads;
     // convective term: slopes and projected face velocities of both stages,
     // C of both stages and its average, their adjoints and work
@@ -991,7 +991,7 @@ ebv_status adj_buffers(Ctx *c, AdjBufs &B)
     size_t off = 0;
     std::vector<std::pair<double **, size_t>> parts;
     auto take = [&](double **dst, size_t n) { parts.push_back({dst, off}); off += n; };
-    for (double **d : {&B.em, &B.es, &B.eb, &B.ebm, &B.ebs, &B.ebb, &B.lam, &B.etad, &B.phib, &B.bbc}) take(d, N3);
+    for (double **d : {&B.em, &B.es, &B.eb, &B.ebm, &B.ebs, &B.ebb, &B.etad, &B.phib, &B.bbc}) take(d, N3);
     for (double **d : {&B.Gm, &B.Gs, &B.Gb, &B.Sm, &B.Ss, &B.Sb}) take(d, 9 * N3);
     for (double **d : {&B.Vm, &B.Vs, &B.Va, &B.psi, &B.utm, &B.uts, &B.us, &B.zero3, &B.t3, &B.Vbs, &B.Vbm, &B.psib,
                        &B.usb, &B.utb, &B.DCb, &B.tb, &B.ua, &B.Cm, &B.Cs, &B.Ca, &B.Cbm, &B.Cbs})

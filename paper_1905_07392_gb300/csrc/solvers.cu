@@ -2979,16 +2979,6 @@ int cv_plan(const CcHier &H, CoarseVC<T> &D)
     return -1;
 }
 
-template <class T>
-void cv_attr()
-{
-    static bool done = false;
-    if (!done) {
-        done = true;
-        cudaFuncSetAttribute(k_cc_coarse_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem);
-    }
-}
-
 // ---- the coarse end of the nodal V-cycle in one cluster --------------------------
 // Below a level of at most kNcNodes nodes a nodal V-cycle is ten launches per
 // level of two to four microseconds each.  One cluster of kNcCtas blocks runs
@@ -3330,16 +3320,6 @@ int nc_plan(const NdHier &H, NdCoarse<T> &D)
         if (D.L.total <= kNcSmem) return l0;
     }
     return -1;
-}
-
-template <class T>
-void nc_attr()
-{
-    static bool done = false;
-    if (!done) {
-        done = true;
-        cudaFuncSetAttribute(k_nd_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNcSmem);
-    }
 }
 
 // ===========================================================================
@@ -4250,7 +4230,6 @@ int cc_vcycle(Ctx *c, CcHier &H, int nc, const int *act, V3<const T> b0, V3<T> x
         D.part = l0 == 0 ? dot_part : nullptr;
         const size_t bytes = D.L.total;
         const char *nm = sizeof(T) == 4 ? "cc_coarse_vcycle<float>" : "cc_coarse_vcycle<double>";
-        cv_attr<T>();
         EBV_LAUNCH_P(c, nm, 0.0, k_cc_coarse_vcycle<T>, dim3(kCvCtas, nc), dim3(kCvThreads), bytes, D);
         if (l0 == 0) return dot_part ? kCvCtas : 0;
     } else {
@@ -4365,7 +4344,6 @@ void nd_vcycle(Ctx *c, NdHier &H, const T *b0, T *x0)
                 D.cd[q] = (T)k.cd[q];
                 D.cr[q] = (T)k.cr[q];
             }
-            nc_attr<T>();
             EBV_LAUNCH_P(c, sizeof(T) == 4 ? "nodal_coarse_vcycle<float>" : "nodal_coarse_vcycle<double>", 0.0,
                          k_nd_coarse<T>, dim3(kNcCtas), dim3(kNcThreads), D.L.total, D);
         } else {
@@ -4901,6 +4879,12 @@ ebv_status setup_solvers(Ctx *c)
 {
     const GridD &g = c->g;
     cudaError_t e = cudaSuccess;
+    // dynamic shared memory of the cluster kernels (per device: set for each context)
+    const cudaFuncAttribute smem_max = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_cc_coarse_vcycle<float>, smem_max, kCvSmem));
+    EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_cc_coarse_vcycle<double>, smem_max, kCvSmem));
+    EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_nd_coarse<float>, smem_max, kNcSmem));
+    EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_nd_coarse<double>, smem_max, kNcSmem));
     GridD gl[kMaxLevels];
     // cell-centred hierarchies (projection and viscous)
     int L = plan_levels(g, gl, false);
