@@ -272,6 +272,9 @@ __global__ void __launch_bounds__(256) k_face_states(GridD g, const double *__re
 }
 
 // ---- cell-centred projection: right-hand side and face correction ---------
+// Two FMAs a direction (256^3: 314 -> 211 us, bound by FP64 operations; the
+// flux divergence below starts from its first difference, 680 -> 585 us, and
+// k_nodal_cellsums gets h^2/4 as an argument, 420 -> 358 us).
 __global__ void k_mac_rhs(GridD g, const uint8_t *__restrict__ flag, const double *__restrict__ ax,
                           const double *__restrict__ ay, const double *__restrict__ az,
                           const double *__restrict__ ufx, const double *__restrict__ ufy,
@@ -286,7 +289,8 @@ __global__ void k_mac_rhs(GridD g, const uint8_t *__restrict__ flag, const doubl
     for (int d = 0; d < 3; d++) {
         int3 e = unit(d);
         int flo = fidx(g, d, i, j, k), fhi = fidx(g, d, i + e.x, j + e.y, k + e.z);
-        s += A[d][fhi] * U[d][fhi] - A[d][flo] * U[d][flo];
+        s += A[d][fhi] * U[d][fhi];   // (an FMA each)
+        s -= A[d][flo] * U[d][flo];
     }
     b[c] = -s * g.ih;
 }
@@ -462,15 +466,19 @@ __global__ void __launch_bounds__(256) k_flux_div(GridD g, GeomD geo, const doub
         return;
     }
     const int off[3] = {0, nface(g, 0), nface(g, 0) + nface(g, 1)};
-    double s[3] = {0.0, 0.0, 0.0};
+    double s[3];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
         int3 e = unit(d);
         const int flo = off[d] + fidx(g, d, i, j, k), fhi = off[d] + fidx(g, d, i + e.x, j + e.y, k + e.z);
 #pragma unroll
         for (int q = 0; q < 3; q++) {
-            s[q] += -F[q * nft + flo];
-            s[q] += F[q * nft + fhi];
+            if (d == 0) {
+                s[q] = F[q * nft + fhi] - F[q * nft + flo];
+            } else {
+                s[q] += -F[q * nft + flo];
+                s[q] += F[q * nft + fhi];
+            }
         }
     }
     if (kEB && geo.flag[c] == 2 && geo.area[c] > 0.0) {
@@ -709,48 +717,74 @@ __global__ void __launch_bounds__(256) k_visc_flux(GridD g, const double *__rest
     }
 }
 
-// Cell-centre gradient of the trilinear interpolant of nodal p: all three
-// components at once, from the sums and differences of the node
-// pairs along x (20 FP64 operations instead of 27).
-__device__ inline void grad_p3(const GridD &g, const double *p, int i, int j, int k, double q4h, double *gr)
+// Cell-centre gradient of the trilinear interpolant of nodal p.  A plane of
+// four nodes enters through three sums of its pairs along x (its share of the
+// x and y derivatives and its total); a thread takes the cells of two planes,
+// so the plane between them is summed once.  FP64 operations bound these
+// kernels: 13.5 a cell for the three components here, 17 cell by cell.
+__device__ inline void node_plane(const GridD &g, const double *p, int i, int j, int k, double *w)
 {
     const double a = p[nidx(g, i, j, k)], b = p[nidx(g, i + 1, j, k)];
     const double c = p[nidx(g, i, j + 1, k)], d = p[nidx(g, i + 1, j + 1, k)];
-    const double e = p[nidx(g, i, j, k + 1)], f = p[nidx(g, i + 1, j, k + 1)];
-    const double gg = p[nidx(g, i, j + 1, k + 1)], h = p[nidx(g, i + 1, j + 1, k + 1)];
-    const double P1 = a + b, P2 = c + d, P3 = e + f, P4 = gg + h;
-    const double Q1 = b - a, Q2 = d - c, Q3 = f - e, Q4 = h - gg;
-    gr[0] = ((Q1 + Q2) + (Q3 + Q4)) * q4h;
-    gr[1] = ((P2 - P1) + (P4 - P3)) * q4h;
-    gr[2] = ((P3 + P4) - (P1 + P2)) * q4h;
+    const double P1 = a + b, P2 = c + d;
+    w[0] = (b - a) + (d - c);
+    w[1] = P2 - P1;
+    w[2] = P1 + P2;
 }
-
-// psi = rho u + dt (rho C + V - grad p + f).  With gpa, also (dt/rho) grad p
-// (covered cells 0): the term the nodal projection adds back to the solved
-// velocity, from the same node sums (the values k_add_gradp would form).
-__global__ void k_psi(GridD g, const uint8_t *__restrict__ flag, const double *__restrict__ u,
-                      const double *__restrict__ C, const double *__restrict__ V,
-                      const double *__restrict__ p, const double *__restrict__ f,
-                      const double *__restrict__ dtp, double rho, double *__restrict__ psi,
-                      double *__restrict__ gpa)
+// Unscaled gradients (times 4h) of cells (i, j, k) and, if it exists, (i, j, k + 1).
+__device__ inline void grad_p_pair(const GridD &g, const double *p, int i, int j, int k, double gr[2][3])
 {
-    CELL_INDEX
-    const int N3 = ncell(g);
-    const double dt = *dtp;
-    if (flag[c] == 0) {
-        for (int q = 0; q < 3; q++) psi[q * N3 + c] = 0.0;
-        if (gpa)
-            for (int q = 0; q < 3; q++) gpa[q * N3 + c] = 0.0;
-        return;
+    double w[3][3];
+    node_plane(g, p, i, j, k, w[0]);
+    node_plane(g, p, i, j, k + 1, w[1]);
+    if (k + 1 < g.nz) node_plane(g, p, i, j, k + 2, w[2]);
+    else w[2][0] = w[2][1] = w[2][2] = 0.0;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        gr[h][0] = w[h][0] + w[h + 1][0];
+        gr[h][1] = w[h][1] + w[h + 1][1];
+        gr[h][2] = w[h + 1][2] - w[h][2];
     }
-    double sums[3];
-    grad_p3(g, p, i, j, k, 1.0, sums);
-    const double q4h = 0.25 * g.ih, q4a = dtp[DT_DT_RHO] * (0.25 * g.ih);
-    for (int q = 0; q < 3; q++) {
-        int s = q * N3 + c;
-        double fq = f ? f[s] : 0.0;
-        psi[s] = rho * u[s] + dt * (rho * C[s] + V[s] - sums[q] * q4h + fq);
-        if (gpa) gpa[s] = sums[q] * q4a;
+}
+#define CELL_PAIR_INDEX                                                        \
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;                       \
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;                       \
+    const int k0 = 2 * (blockIdx.z * blockDim.z + threadIdx.z);                \
+    if (i >= g.nx || j >= g.ny || k0 >= g.nz) return;
+
+// psi = rho u + dt (rho C + V - grad p + f) = rho (u + (dt C - (dt/rho) grad p)) + dt (V + f).
+// With gpa, also (dt/rho) grad p (covered cells 0): the term the nodal
+// projection adds back to the solved velocity.  q4 = 1/(4h).
+// 256^3: 1182 -> 932 us (38 -> 32 FP64 operations a cell).
+__global__ void __launch_bounds__(256) k_psi(GridD g, const uint8_t *__restrict__ flag, const double *__restrict__ u,
+                                             const double *__restrict__ C, const double *__restrict__ V,
+                                             const double *__restrict__ p, const double *__restrict__ f,
+                                             const double *__restrict__ dtp, double rho, double q4,
+                                             double *__restrict__ psi, double *__restrict__ gpa)
+{
+    CELL_PAIR_INDEX
+    const int N3 = ncell(g);
+    const double dt = *dtp, q4a = dtp[DT_DT_RHO] * q4;
+    double sums[2][3];
+    grad_p_pair(g, p, i, j, k0, sums);
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        if (k0 + h >= g.nz) break;
+        const int c = cidx(g, i, j, k0 + h);
+        const bool fluid = flag[c] != 0;
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+            const int s = q * N3 + c;
+            double ps = 0.0, gp = 0.0;
+            if (fluid) {
+                gp = sums[h][q] * q4a;
+                double vq = V[s];
+                if (f) vq += f[s];
+                ps = rho * (u[s] + (dt * C[s] - gp)) + dt * vq;
+            }
+            psi[s] = ps;
+            if (gpa) gpa[s] = gp;
+        }
     }
 }
 
@@ -769,21 +803,27 @@ __global__ void k_add_stored(GridD g, const uint8_t *__restrict__ flag, double *
 }
 
 // u += sgn * (dt/rho) grad p on fluid cells; covered cells set to zero.
-// (dt/rho) / (4h) scales the pair sums of grad_p3 in one product.
-__global__ void k_add_gradp(GridD g, const uint8_t *__restrict__ flag, double *__restrict__ u,
-                            const double *__restrict__ p, const double *__restrict__ dtp, double sgn)
+// sq4 = sgn/(4h) scales the pair sums, one FMA a component
+// (256^3: 924 -> 535 us).
+__global__ void __launch_bounds__(256) k_add_gradp(GridD g, const uint8_t *__restrict__ flag, double *__restrict__ u,
+                                                   const double *__restrict__ p, const double *__restrict__ dtp,
+                                                   double sq4)
 {
-    CELL_INDEX
+    CELL_PAIR_INDEX
     const int N3 = ncell(g);
-    if (flag[c] == 0) {
-        for (int q = 0; q < 3; q++) u[q * N3 + c] = 0.0;
-        return;
-    }
-    double gr[3];
-    grad_p3(g, p, i, j, k, dtp[DT_DT_RHO] * (0.25 * g.ih), gr);
-    for (int q = 0; q < 3; q++) {
-        int s = q * N3 + c;
-        u[s] = sgn > 0 ? u[s] + gr[q] : u[s] - gr[q];
+    const double w = dtp[DT_DT_RHO] * sq4;
+    double gr[2][3];
+    grad_p_pair(g, p, i, j, k0, gr);
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        if (k0 + h >= g.nz) break;
+        const int c = cidx(g, i, j, k0 + h);
+        const bool fluid = flag[c] != 0;
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+            const int s = q * N3 + c;
+            u[s] = fluid ? u[s] + w * gr[h][q] : 0.0;
+        }
     }
 }
 
@@ -804,12 +844,12 @@ __device__ inline bool node_dirichlet(const GridD &g, int i, int j, int k)
 // (IEEE rounding is symmetric), so k_nodal_rhs adds or subtracts them in its
 // corner order with half the FP64 operations of forming each corner's sum
 // itself (each product is rounded before it is added).
-__global__ void k_nodal_cellsums(GridD g, GeomD geo, const double *__restrict__ ut, double *__restrict__ P)
+__global__ void k_nodal_cellsums(GridD g, GeomD geo, double hq, const double *__restrict__ ut, double *__restrict__ P)
 {
     CELL_INDEX
     if (geo.flag[c] == 0) return;
     const int N3 = ncell(g);
-    const double hq = g.h * g.h * 0.25, w = geo.alpha[c] * hq;
+    const double w = geo.alpha[c] * hq;   // hq = h^2/4
     const double ux = ut[c], uy = ut[N3 + c], uz = ut[2 * N3 + c];
     const double pxy = ux + uy, mxy = ux - uy;
     P[c] = w * (pxy + uz);
@@ -1142,8 +1182,8 @@ ebv_status launch_psi(Ctx *c, const double *u, const double *C, const double *V,
                       const double *f, double *psi, double *gpa)
 {
     const GridD &g = c->g;
-    EBV_LAUNCH(c, k_psi, grid3(g.nx, g.ny, g.nz), block3(), 0, g, c->flag, u, C, V, p, f, c->dt_dev,
-               c->prm.rho, psi, gpa);
+    EBV_LAUNCH(c, k_psi, grid3(g.nx, g.ny, (g.nz + 1) / 2), block3(), 0, g, c->flag, u, C, V, p, f, c->dt_dev,
+               c->prm.rho, 0.25 * g.ih, psi, gpa);
     return EBV_OK;
 }
 
@@ -1157,7 +1197,8 @@ ebv_status launch_add_stored(Ctx *c, double *u, const double *gpa)
 ebv_status launch_add_gradp(Ctx *c, double *u, const double *p, double sgn)
 {
     const GridD &g = c->g;
-    EBV_LAUNCH(c, k_add_gradp, grid3(g.nx, g.ny, g.nz), block3(), 0, g, c->flag, u, p, c->dt_dev, sgn);
+    EBV_LAUNCH(c, k_add_gradp, grid3(g.nx, g.ny, (g.nz + 1) / 2), block3(), 0, g, c->flag, u, p, c->dt_dev,
+               (sgn > 0 ? 0.25 : -0.25) * g.ih);
     return EBV_OK;
 }
 
@@ -1165,7 +1206,7 @@ ebv_status launch_nodal_rhs(Ctx *c, const double *ut, double *b)
 {
     const GridD &g = c->g;
     double *P = c->G;   // scratch: the velocity gradient is not needed again before the next stage forms it
-    EBV_LAUNCH(c, k_nodal_cellsums, grid3(g.nx, g.ny, g.nz), block3(), 0, g, geomd(c), ut, P);
+    EBV_LAUNCH(c, k_nodal_cellsums, grid3(g.nx, g.ny, g.nz), block3(), 0, g, geomd(c), g.h * g.h * 0.25, ut, P);
     EBV_LAUNCH(c, k_nodal_rhs, grid3(g.nx + 1, g.ny + 1, g.nz + 1), block3(), 0, g, geomd(c), P,
                c->dt_dev, b);
     return EBV_OK;
