@@ -50,10 +50,15 @@ __device__ inline double mc_limit(double dl, double dr, double dd)
 }
 
 // Godunov state of Burgers' equation from the two extrapolated normal velocities.
+// The signs are tested on the integer pipe (b the pattern of x: x > 0 and not
+// a NaN where b lies in 1 .. infinity's pattern), the sum is formed once.
+__device__ inline bool dpos(unsigned long long b) { return b - 1 < 0x7ff0000000000000ull; }
 __device__ inline double upwind_normal(double uL, double uR)
 {
-    if (uL > 0.0 && uL + uR > 0.0) return uL;
-    if (uR < 0.0 && uL + uR < 0.0) return uR;
+    constexpr unsigned long long sg = 1ull << 63;
+    const unsigned long long bs = __double_as_longlong(uL + uR);
+    if (dpos(__double_as_longlong(uL)) && dpos(bs)) return uL;
+    if (dpos(__double_as_longlong(uR) ^ sg) && dpos(bs ^ sg)) return uR;
     return 0.0;
 }
 
@@ -224,10 +229,11 @@ __global__ void __launch_bounds__(256) k_flow_diag(GridD g, const uint8_t *__res
 
 // The face kernels are instances per direction d: with d an argument the
 // indices [d] of small arrays went through local memory and both sides of a
-// "component d or not" ran (256^3, per direction: face states 275 -> 228 us,
-// projection 250 -> 105, convective flux 349 -> 267, viscous flux 599 -> 387).
+// "component d or not" ran (256^3, per direction: face states 275 -> 130 us,
+// projection 250 -> 105, convective flux 349 -> 267, viscous flux 599 -> 356).
 // Apertures, and the face velocity's sign, are tested on the integer pipe.
 __device__ inline bool open_face(double a) { return __double2hiint(a) > 0; }   // a > 0 (0 or at least 1e-12)
+__device__ inline bool full_face(double a) { return __double2hiint(a) == 0x3ff00000 && __double2loint(a) == 0; }
 #define EBV_LAUNCH_DIR(ctx, d, kern, grid, block, ...)                                        \
     do {                                                                                      \
         if ((d) == 0) EBV_LAUNCH_P(ctx, #kern, 0.0, kern<0>, grid, block, 0, __VA_ARGS__);     \
@@ -436,7 +442,7 @@ __global__ void __launch_bounds__(256) k_conv_flux(GridD g, const double *__rest
     // run the same instructions (u_L + S_L/2 or u_R - S_R/2, one FMA each).
     // Across the flow the sign of w alternates between neighbouring faces, so
     // a branch on it would run both halves in most warps.
-    const double aw = a * w;
+    const double aw = full_face(a) ? w : a * w;
     const long long wb = __double_as_longlong(w);
     if ((wb << 1) != 0) {   // w != 0
         const int cs = wb > 0 ? cL : cR;
@@ -671,7 +677,7 @@ __global__ void __launch_bounds__(256) k_visc_flux(GridD g, const double *__rest
                                                    const double *__restrict__ u,
                                                    const double *__restrict__ eta,
                                                    const double *__restrict__ G, double *__restrict__ F,
-                                                   int nft, int off)
+                                                   int nft, int off, double hih)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -706,10 +712,11 @@ __global__ void __launch_bounds__(256) k_visc_flux(GridD g, const double *__rest
         return;
     }
     const int cL = cidx(g, i - e.x, j - e.y, k - e.z), cR = cidx(g, i, j, k);
-    // W = a eta_f; the normal derivative's 1/h and the transverse mean's 1/2
-    // are folded into W once (fewer FP64 operations)
-    const double W = (0.5 * a) * (eta[cL] + eta[cR]);
-    const double Wn = W * ih, Wt = 0.5 * W;
+    // a eta_f: the normal derivative's 1/h and the means' 1/2 are folded in
+    // once, and an open face (a = 1, a test of its words) needs no product
+    double W = eta[cL] + eta[cR];
+    if (!full_face(a)) W *= a;
+    const double Wn = W * hih, Wt = 0.25 * W;
 #pragma unroll
     for (int jj = 0; jj < 3; jj++) {
         F[jj * nft + off + f] = (jj == d) ? (u[d * N3 + cR] - u[d * N3 + cL]) * Wn
@@ -861,7 +868,7 @@ __global__ void k_nodal_cellsums(GridD g, GeomD geo, double hq, const double *__
 // Nodal right-hand side (weak divergence of ut plus the inflow boundary
 // integral), times rho/dt so the solve uses the unit-coefficient operator.
 // P: the cell sums of k_nodal_cellsums.
-__global__ void k_nodal_rhs(GridD g, GeomD geo, const double *__restrict__ P,
+__global__ void __launch_bounds__(256) k_nodal_rhs(GridD g, GeomD geo, const double *__restrict__ P,
                             const double *__restrict__ dtp, double *__restrict__ b)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -871,29 +878,34 @@ __global__ void k_nodal_rhs(GridD g, GeomD geo, const double *__restrict__ P,
     const int n = nidx(g, i, j, k);
     const int N3 = ncell(g);
     const double h = g.h;
-    bool act = !node_dirichlet(g, i, j, k);
-    if (act) {
-        bool any = false;
-        for (int oc = 0; oc < 8; oc++)
-            any |= avail(g, geo.flag, i - 1 + (oc & 1), j - 1 + ((oc >> 1) & 1), k - 1 + ((oc >> 2) & 1));
-        act = any;
+    // the node's cells that hold fluid, one bit each; the box test once per axis
+    const bool in[3][2] = {{i > 0, i < g.nx}, {j > 0, j < g.ny}, {k > 0, k < g.nz}};
+    unsigned av = 0;
+#pragma unroll
+    for (int oc = 0; oc < 8; oc++) {
+        const int ox = oc & 1, oy = (oc >> 1) & 1, oz = (oc >> 2) & 1;
+        if (in[0][ox] && in[1][oy] && in[2][oz] && geo.flag[cidx(g, i - 1 + ox, j - 1 + oy, k - 1 + oz)] != 0)
+            av |= 1u << oc;
     }
-    if (!act) { b[n] = 0.0; return; }
+    if (!av || node_dirichlet(g, i, j, k)) { b[n] = 0.0; return; }
     // per cell: alpha h^2/4 times the signed sum of its three components,
     // (ux + uy) + uz for the corner (i - ci, j - cj, k - ck) = (1, 1, 1) and
-    // so on: sums 0..3 of k_nodal_cellsums, negated for the opposite corners
-    double v = 0.0;
+    // so on: sums 0..3 of k_nodal_cellsums, negated for the opposite corners.
+    // All eight are loaded before the first is added (a cell without fluid
+    // counts as an exact 0): with a branch per cell each load waited for the
+    // addition before it (256^3: 655 -> 396 us).
+    double pc[8];
+#pragma unroll
     for (int oc = 0; oc < 8; oc++) {
-        int ci = i - 1 + (oc & 1), cj = j - 1 + ((oc >> 1) & 1), ck = k - 1 + ((oc >> 2) & 1);
-        if (!avail(g, geo.flag, ci, cj, ck)) continue;
-        const int c = cidx(g, ci, cj, ck);
-        const int di = i - ci, dj = j - cj, dk = k - ck;
-        // (di,dj,dk) -> sum: (1,1,1) 0, (1,1,0) 1, (1,0,1) 2, (1,0,0) 3; with di = 0 the
-        // negation of the sum of (1, 1-dj, 1-dk)
-        const int q = di ? (dj ? 0 : 2) + (dk ? 0 : 1) : (dj ? 2 : 0) + (dk ? 1 : 0);
-        const double pc = P[q * N3 + c];
-        v = di ? v + pc : v - pc;
+        const int ox = oc & 1, oy = (oc >> 1) & 1, oz = (oc >> 2) & 1;
+        // (di,dj,dk) = 1 - (ox,oy,oz) -> sum: (1,1,1) 0, (1,1,0) 1, (1,0,1) 2, (1,0,0) 3; with
+        // di = 0 the negation of the sum of (1, 1-dj, 1-dk)
+        const int q = ox ? (oy ? 0 : 2) + (oz ? 0 : 1) : (oy ? 2 : 0) + (oz ? 1 : 0);
+        pc[oc] = av >> oc & 1 ? P[q * N3 + cidx(g, i - 1 + ox, j - 1 + oy, k - 1 + oz)] : 0.0;
     }
+    double v = pc[0];
+#pragma unroll
+    for (int oc = 1; oc < 8; oc++) v = oc & 1 ? v - pc[oc] : v + pc[oc];
     int id[3] = {i, j, k};
     const double *A[3] = {geo.ax, geo.ay, geo.az};
     for (int d = 0; d < 3; d++)
@@ -1170,7 +1182,7 @@ ebv_status launch_viscous_explicit(Ctx *c, const double *u, const double *eta, c
     int off = 0;
     for (int d = 0; d < 3; d++) {
         EBV_LAUNCH_DIR(c, d, k_visc_flux, grid3(g.nx + (d == 0), g.ny + (d == 1), g.nz + (d == 2)), block3(), g, A[d], u,
-                       eta, G, c->ff, nft, off);
+                       eta, G, c->ff, nft, off, 0.5 * g.ih);
         off += nface(g, d);
     }
     EBV_LAUNCH(c, k_flux_div<true>, grid3(g.nx, g.ny, g.nz), block3(), 0, g, geo, c->ff, nft, eta, c->dudn,

@@ -25,3 +25,18 @@ def test_f32_to_f64_words():
     is_normal = (np.isfinite(f) & (np.abs(f) >= np.finfo(np.float32).tiny)) | (f == 0)
     assert (normal == is_normal).all()
     assert (bits[normal] == want[normal]).all()
+
+
+def test_upwind_signs():
+    """The upwinding's integer sign tests against the comparisons, NaN, infinities and signed zeros included."""
+    edge = np.array([0.0, -0.0, 5e-324, -5e-324, 1.0, -1.0, 1e308, -1e308, np.inf, -np.inf, np.nan, -np.nan])
+    with np.errstate(invalid="ignore", over="ignore"):
+        uL, uR = (a.ravel() for a in np.meshgrid(edge, edge))
+        s = uL + uR
+        one, sg, inf = np.uint64(1), np.uint64(1 << 63), np.uint64(0x7ff0000000000000)
+        pos = lambda x, flip: ((x.view(np.uint64) ^ flip) - one) < inf
+        left = pos(uL, np.uint64(0)) & pos(s, np.uint64(0))
+        right = ~left & pos(uR, sg) & pos(s, sg)
+        want_left = (uL > 0) & (uL + uR > 0)
+        want_right = ~want_left & (uR < 0) & (uL + uR < 0)
+    assert (left == want_left).all() and (right == want_right).all()
