@@ -296,7 +296,7 @@ void ebv_set_alloc_limit(long long bytes);
 void ebv_set_spin_limit(long long cycles);
 
 /* How FP32 multigrid levels whose x size is a multiple of 16 run a red-black
- * sweep: 0 as two colour passes, 1 (default) as whichever of the two colour
+ * sweep (the coarse levels that one launch per V-cycle holds take neither form): 0 as two colour passes, 1 (default) as whichever of the two colour
  * passes and the fused one-pass sweep was faster when the context's solvers
  * were set up (instances of an ebv_batch keep the colour passes: their steps
  * run side by side, where a lone kernel's time does not decide), 2 always as
