@@ -27,7 +27,8 @@ SHAPES = [(5, 3, 7),      # a single level, odd rows
           (20, 12, 28),   # odd half-rows on level 1
           (24, 20, 28),   # nx a multiple of 8 but not of 16
           (48, 16, 32),   # a multiple of 16, flat
-          (40, 24, 56)]   # a multiple of 8, odd bottom
+          (40, 24, 56),   # a multiple of 8, odd bottom
+          (2, 6, 3), (2, 2, 3)]   # too few cells to hold three components' vectors: solved one after another
 
 
 @pytest.mark.parametrize("precision", [0, 1])
