@@ -138,9 +138,15 @@ __device__ inline void store_dt(double *d, double dt, double rho, double h)
     d[DT_DTH2] = dt / (h * h);
 }
 
-// a > b for numbers that are not negative (or NaN, which compares greater),
-// on the integer pipe: an FP64 comparison takes an FP64-pipe slot.
-__device__ inline bool gt_nonneg(double a, double b) { return __double_as_longlong(a) > __double_as_longlong(b); }
+// a > b for b not negative and not a NaN, on the integer pipe (an FP64
+// comparison takes an FP64-pipe slot): the pattern of a lies above b's and not
+// above infinity's.  Like the comparison it is false for a NaN or negative a,
+// so a strain rate that is a NaN takes the laws' limits at rest.
+__device__ inline bool gt_nonneg(double a, double b)
+{
+    const unsigned long long ua = __double_as_longlong(a), ub = __double_as_longlong(b);
+    return ua - ub - 1 < 0x7ff0000000000000ull - ub;
+}
 
 // sr^(n_flow - 1).  CUDA's pow is over a hundred FP64-pipe operations per call
 // (three quarters of the viscosity kernel's time with a power law); flow
