@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <string>
 #include <vector>
 
@@ -78,7 +79,7 @@ struct ParamsD {
     int model;
     double delta_min;
     double inv_m;  // 1/m (the floor of the strain rate in the power laws)
-    double inv_tau0;  // 1/tau0, 0 without a yield stress
+    double inv_tau0;  // 1/tau0; 0 without a yield stress, or where that is no normal number
     int pow4;      // 4 (n_flow - 1) where that is a whole number from -4 to 4, else kPowAny
 };
 constexpr int kPowAny = 99;
@@ -460,7 +461,7 @@ inline ParamsD paramsd(const ebv_params &p)
     q.rho = p.rho; q.mu = p.mu; q.tau0 = p.tau0; q.m = p.m; q.n_flow = p.n_flow; q.eta0 = p.eta0;
     q.model = p.model; q.delta_min = p.delta_min;
     q.inv_m = 1.0 / p.m;
-    q.inv_tau0 = p.tau0 > 0.0 ? 1.0 / p.tau0 : 0.0;
+    q.inv_tau0 = std::isnormal(1.0 / p.tau0) ? 1.0 / p.tau0 : 0.0;
     const double q4 = 4.0 * (p.n_flow - 1.0);
     q.pow4 = q4 >= -4.0 && q4 <= 4.0 && q4 == (double)(int)q4 ? (int)q4 : kPowAny;
     return q;

@@ -223,8 +223,11 @@ __global__ void __launch_bounds__(256) k_flow_diag(GridD g, const uint8_t *__res
     lam[c] = gt_nonneg(sw, 0.0) ? (s - w2) / sw : 0.0;
     const double rsr = gt_nonneg(sh, 0.0) ? rsqrt(sh) : 0.0;
     const double sr = sh * rsr;
-    // (one rounding with the subtraction, in place of the division's)
-    sdev[c] = p.tau0 > 0.0 ? fma(eta_of(p, sr, rsr) * sr, p.inv_tau0, -1.0) : 0.0;
+    // (one rounding with the subtraction, in place of the division's; a tau0
+    // whose reciprocal is not a normal number divides)
+    const double tau = eta_of(p, sr, rsr) * sr;
+    if (p.inv_tau0 > 0.0) sdev[c] = fma(tau, p.inv_tau0, -1.0);
+    else sdev[c] = p.tau0 > 0.0 ? tau / p.tau0 - 1.0 : 0.0;
 }
 
 // The face kernels are instances per direction d: with d an argument the
