@@ -349,6 +349,7 @@ struct Ctx {
     enum { CV_X, CV_B, CV_T, CV_K, CV_KINDS };
     void *cvec[2][CV_KINDS][kMaxLevels] = {};
     bool joint = false;
+    int rb_res = 0;              // blocks of the fused sweep resident on this context's device
 
     // Solver loop control lives on the device: the convergence tests run in
     // one-thread kernels that write a condition word (read back by the host

@@ -3975,38 +3975,32 @@ bool rb_map(Ctx *c, const void *p, int kind, const GridD &g, CUtensorMap *out)
     return true;
 }
 
-template <bool kZero, bool kCorr, bool kDot>
-void rb_attr()
+// Shared-memory limit of the fused sweeps on the context's device (raised by
+// setup_solvers: the attribute belongs to the device, and a context on another
+// one, or a second thread, must not find it half set), and the blocks of one
+// that are resident on it at once.
+cudaError_t rb_setup(Ctx *c)
 {
-    static bool done = false;
-    if (!done) {
-        done = true;
-        cudaFuncSetAttribute(k_cc_rb_sweep<RbF, kZero, kCorr, kDot>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             RbSmem<RbF>::bytes);
-    }
-}
-
-// Blocks of the fused sweep resident on the device at once.
-int rb_resident()
-{
-    static int res = 0;
-    if (!res) {
-        rb_attr<false, false, false>();
-        int dev = 0, sms = 0, per = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cc_rb_sweep<RbF, false, false, false>, RB_THREADS,
-                                                      RbSmem<RbF>::bytes);
-        res = std::max(1, per) * std::max(1, sms);
-    }
-    return res;
+    const int sb = RbSmem<RbF>::bytes;
+    const cudaFuncAttribute smem_max = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_cc_rb_sweep<RbF, false, false, false>, smem_max, sb);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cc_rb_sweep<RbF, true, false, false>, smem_max, sb);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cc_rb_sweep<RbF, false, true, false>, smem_max, sb);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cc_rb_sweep<RbF, false, false, true>, smem_max, sb);
+    int dev = 0, sms = 0, per = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cc_rb_sweep<RbF, false, false, false>, RB_THREADS, sb);
+    c->rb_res = std::max(1, per) * std::max(1, sms);
+    return e;
 }
 
 // Planes per chunk of a block: the fewest waves of resident blocks times the
 // steps of one block (its planes and the two of the chunk's start).
-int rb_kz(const GridD &g, int nc = 1)
+int rb_kz(const Ctx *c, const GridD &g, int nc = 1)
 {
-    const long long nt = (long long)nc * rb_ntiles(g), res = rb_resident();
+    const long long nt = (long long)nc * rb_ntiles(g), res = c->rb_res;
     long long best = -1;
     int bkz = g.nz;
     for (int nc = 1; nc <= g.nz; nc++) {
@@ -4031,7 +4025,7 @@ void rb_launch(Ctx *c, const char *name, const GridD &g, const RbMaps &tm, V3<fl
     a.ctl = c->ctl;
     a.act = act;
     a.c0 = c0;
-    a.kz = kz > 0 ? kz : rb_kz(g, nc);
+    a.kz = kz > 0 ? kz : rb_kz(c, g, nc);
     a.nzb = (g.nz + a.kz - 1) / a.kz;
     a.spin = spin_limit();
     const dim3 gr((g.nx / 2 + RB_HW - 1) / RB_HW, (g.ny + RB_TY - 1) / RB_TY, a.nzb * nc);
@@ -4042,19 +4036,15 @@ void rb_launch(Ctx *c, const char *name, const GridD &g, const RbMaps &tm, V3<fl
     const int sb = RbSmem<RbF>::bytes;
     switch (mode) {
     case RB_ZERO:
-        rb_attr<true, false, false>();
         EBV_LAUNCH_P(c, name, nb, (k_cc_rb_sweep<RbF, true, false, false>), gr, dim3(RB_THREADS), sb, tm, a);
         break;
     case RB_CORR:
-        rb_attr<false, true, false>();
         EBV_LAUNCH_P(c, name, nb, (k_cc_rb_sweep<RbF, false, true, false>), gr, dim3(RB_THREADS), sb, tm, a);
         break;
     case RB_DOT:
-        rb_attr<false, false, true>();
         EBV_LAUNCH_P(c, name, nb, (k_cc_rb_sweep<RbF, false, false, true>), gr, dim3(RB_THREADS), sb, tm, a);
         break;
     default:
-        rb_attr<false, false, false>();
         EBV_LAUNCH_P(c, name, nb, (k_cc_rb_sweep<RbF, false, false, false>), gr, dim3(RB_THREADS), sb, tm, a);
     }
 }
@@ -4895,6 +4885,7 @@ ebv_status setup_solvers(Ctx *c)
     EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_cc_coarse_vcycle<double>, smem_max, kCvSmem));
     EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_nd_coarse<float>, smem_max, kNcSmem));
     EBV_CUDA_TRY(c, cudaFuncSetAttribute(k_nd_coarse<double>, smem_max, kNcSmem));
+    EBV_CUDA_TRY(c, rb_setup(c));
     GridD gl[kMaxLevels];
     // cell-centred hierarchies (projection and viscous)
     int L = plan_levels(g, gl, false);
@@ -5126,9 +5117,9 @@ ebv_status autotune_shapes_t(Ctx *c)
                 const long long nl = c->launches;
                 // planes per block: the model's choice, the most planes that
                 // still fill one wave, and half that (results do not depend on it)
-                const int nt = rb_ntiles(L.g), res = rb_resident(), nz = L.g.nz;
+                const int nt = rb_ntiles(L.g), res = c->rb_res, nz = L.g.nz;
                 const int wave = std::max(1, res / std::max(1, nt));   // chunks per wave
-                const int kzc[3] = {rb_kz(L.g), (nz + wave - 1) / wave, (nz + 2 * wave - 1) / (2 * wave)};
+                const int kzc[3] = {rb_kz(c, L.g), (nz + wave - 1) / wave, (nz + 2 * wave - 1) / (2 * wave)};
                 float best = 1e30f;
                 for (int kz : kzc) {
                     const float ms = time_it(
@@ -5283,19 +5274,18 @@ void set_inner_drop(double drop) { g_inner_drop = (drop > 0.0 && drop < 1.0) ? d
 bool tma_encode_4d(CUtensorMap *tm, CUtensorMapDataType type, void *base, const uint64_t dims[4],
                    const uint64_t strides[3], const uint32_t box[4])
 {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    // (one entry point per process, found by whichever thread comes first; the
+    // others wait for it)
+    static const EncodeTiledFn fn = []() -> EncodeTiledFn {
         void *f = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
                 cudaSuccess &&
             q == cudaDriverEntryPointSuccess && f)
-            fn = reinterpret_cast<EncodeTiledFn>(f);
-        else
-            cudaGetLastError();
-    }
+            return reinterpret_cast<EncodeTiledFn>(f);
+        cudaGetLastError();
+        return nullptr;
+    }();
     if (!fn || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
     const cuuint64_t d[4] = {dims[0], dims[1], dims[2], dims[3]};
     const cuuint64_t st[3] = {strides[0], strides[1], strides[2]};
