@@ -3582,22 +3582,36 @@ __global__ void k_cg_pupdate(V3<double> pv, V3<const double> zv, const double *_
 // Per-thread sums of the FP32 kernels stay FP32 (a few dozen terms), block and
 // final sums are FP64.
 
+// Below kWideDot elements a thread's elements would take four FP32 additions
+// where a thread per element takes none: there the FP32 products are summed in
+// FP64 (275 k elements 0.4 us of the FP64 pipe); from there on a thread of the
+// largest grid sums four or more of them either way.
+constexpr int kWideDot = 4 * 256 * kReduceBlocks;
 __global__ void __launch_bounds__(256) k_dot32(V3<const float> av, V3<const float> bv, int n, double *__restrict__ part)
 {
     const float *__restrict__ a = av.p[blockIdx.y], *__restrict__ b = bv.p[blockIdx.y];
     part += blockIdx.y * kPartComp;
     float v = 0.0f;
+    double dv = 0.0;
+    const bool wide = n < kWideDot;
     const int n4 = n >> 2, t0 = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
     const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
     for (int s = t0; s < n4; s += st) {
         const float4 u = a4[s], w = b4[s];
-        v += u.x * w.x;
-        v += u.y * w.y;
-        v += u.z * w.z;
-        v += u.w * w.w;
+        if (wide) {
+            dv += (f32_to_f64(u.x * w.x) + f32_to_f64(u.y * w.y)) + (f32_to_f64(u.z * w.z) + f32_to_f64(u.w * w.w));
+        } else {
+            v += u.x * w.x;
+            v += u.y * w.y;
+            v += u.z * w.z;
+            v += u.w * w.w;
+        }
     }
-    for (int s = 4 * n4 + t0; s < n; s += st) v += a[s] * b[s];
-    double dv = block_sum<256>((double)v);
+    for (int s = 4 * n4 + t0; s < n; s += st) {
+        if (wide) dv += f32_to_f64(a[s] * b[s]);
+        else v += a[s] * b[s];
+    }
+    dv = block_sum<256>(dv + (double)v);
     if (threadIdx.x == 0) part[blockIdx.x] = dv;
 }
 

@@ -1,0 +1,93 @@
+"""The width in which the solvers sum (no GPU): the text of a kernel is compiled as C++, its threads run
+one after another, and the partial sums are compared with the exact sum of what the kernel rounds --
+FP32 products, whose sums are FP64 wherever a thread per element would sum them so."""
+import ctypes
+import math
+import os
+import re
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1905_07392_gb300", "csrc")
+
+SHIM = r"""
+#include <cstdint>
+#include <cstring>
+#include <cstddef>
+#define __global__
+#define __device__
+#define __restrict__
+#define __launch_bounds__(...)
+struct Dim { int x, y, z; };
+static Dim blockIdx, blockDim, gridDim, threadIdx;
+struct float4 { float x, y, z, w; };
+template <class T> struct V3 { T *p[3]; };
+static const size_t kPartComp = (1 << 20) / 3;
+static unsigned __float_as_uint(float x) { unsigned u; memcpy(&u, &x, 4); return u; }
+static double __hiloint2double(int hi, int lo)
+{
+    uint64_t u = ((uint64_t)(uint32_t)hi << 32) | (uint32_t)lo;
+    double d;
+    memcpy(&d, &u, 8);
+    return d;
+}
+static double g_sum;   // of the block's threads, which run one after another
+template <int N> static double block_sum(double v) { g_sum = threadIdx.x ? g_sum + v : v; return g_sum; }
+"""
+
+
+def _source(name):
+    return open(os.path.join(CSRC, name)).read()
+
+
+def _function(text, head):
+    """The function whose declaration matches head, to its closing brace in the first column."""
+    m = re.search(head, text)
+    assert m, head
+    return text[m.start():text.index("\n}\n", m.start()) + 3]
+
+
+@pytest.fixture(scope="module")
+def kernels(tmp_path_factory):
+    d = tmp_path_factory.mktemp("kernels")
+    solvers, bits, head = _source("solvers.cu"), _source("fpbits.cuh"), _source("ebv_internal.cuh")
+    dot = re.sub(r"if \(threadIdx\.x == 0\) (part\[)", r"if (threadIdx.x == blockDim.x - 1) \1",
+                 _function(solvers, r"__global__ void __launch_bounds__\(256\) k_dot32\("))
+    src = SHIM
+    src += re.search(r"constexpr int kReduceBlocks = \d+;", head).group(0) + "\n"
+    src += "\n".join(re.findall(r"^constexpr int kWideDot = [^;]*;", solvers, flags=re.M)) + "\n"
+    src += _function(bits, r"__device__ inline double f32_to_f64\(") + dot + r"""
+extern "C" int blocks() { return kReduceBlocks; }
+extern "C" void dot(const float *a, const float *b, int n, int nb, double *part)
+{
+    V3<const float> av = {{a, a, a}}, bv = {{b, b, b}};
+    blockDim = {256, 1, 1};
+    gridDim = {nb, 1, 1};
+    for (int q = 0; q < nb; q++)
+        for (int t = 0; t < 256; t++) {
+            blockIdx = {q, 0, 0};
+            threadIdx = {t, 0, 0};
+            k_dot32(av, bv, n, part);
+        }
+}
+"""
+    cpp, lib = d / "k.cpp", d / "k.so"
+    cpp.write_text(src)
+    # (no contraction: a product that is added in FP64 is rounded to FP32 first)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-ffp-contract=off", "-fno-strict-aliasing", "-shared", "-fPIC", "-o", str(lib), str(cpp)], check=True)
+    return ctypes.CDLL(str(lib))
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 1023, 1024, 1025, 4913, 35937, 274625, 1245183])
+def test_small_dot_sums_in_fp64(kernels, n):
+    rng = np.random.Generator(np.random.PCG64(n))
+    a, b = (rng.standard_normal(n).astype(np.float32) for _ in range(2))
+    nb = min(kernels.blocks(), (n // 4 + 255) // 256 + 1)   # (v4blocks)
+    part = np.full(nb, np.nan)
+    ptr = lambda x, t: x.ctypes.data_as(ctypes.POINTER(t))
+    kernels.dot(ptr(a, ctypes.c_float), ptr(b, ctypes.c_float), n, nb, ptr(part, ctypes.c_double))
+    prod = (a * b).astype(np.float64)
+    # at most n FP64 roundings of partial sums no larger than sum |a b|
+    assert abs(math.fsum(part) - math.fsum(prod)) <= n * 2.0 ** -53 * math.fsum(abs(prod))
