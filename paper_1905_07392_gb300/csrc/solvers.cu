@@ -144,6 +144,11 @@ __device__ inline double block_sum3_t(T v)
     }
 }
 
+// A term of a dot product that is summed in FP64: the product rounded in its
+// operands' precision.
+__device__ inline double dot_term(float a, float b) { return f32_to_f64(a * b); }
+__device__ inline double dot_term(double a, double b) { return a * b; }
+
 // Sum of n block partials in a fixed order, over a cluster of kRedCtas
 // blocks: block q sums the slice [q n / kRedCtas, (q + 1) n / kRedCtas)
 // (strided over its threads, then its block sum) and stores that sum in
@@ -2932,8 +2937,8 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
 #pragma unroll 1
     for (int l = nl - 1; l >= 0; l--)
         if (l < nd || act) smooth(l, 1, l == nl - 1 ? xb : reinterpret_cast<const T *>(cvsm + lv[l + 1].x));
-    // the top level's x, and b.x over the block's cells (per thread and warp in T, across warps in FP64)
-    T dot = T(0);
+    // the top level's x, and b.x over the block's cells (FP32 products, FP64 sums: a block has few cells)
+    double dot = 0.0;
     {
         const GridD &g = D.A3[0].A.g;
         const CvView<T> w = view(0);
@@ -2945,12 +2950,12 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
             const T x0 = w.x[p], x1 = w.x[p + v.h];
             D.x.p[comp][cix<T>(g, 2 * t, j, k)] = x0;
             D.x.p[comp][cix<T>(g, 2 * t + 1, j, k)] = x1;
-            dot += w.b[c0 * w.cap + m] * x0 + w.b[(1 - c0) * w.cap + m] * x1;
+            if (D.part) dot += dot_term(w.b[c0 * w.cap + m], x0) + dot_term(w.b[(1 - c0) * w.cap + m], x1);
         }
     }
     if (D.part) {
         for (int o = 16; o > 0; o >>= 1) dot += __shfl_down_sync(0xffffffffu, dot, o);
-        if ((tid & 31) == 0) ps[tid >> 5] = (double)dot;
+        if ((tid & 31) == 0) ps[tid >> 5] = dot;
         __syncthreads();
         if (tid == 0) {
             double sum = 0.0;
@@ -3599,7 +3604,7 @@ __global__ void __launch_bounds__(256) k_dot32(V3<const float> av, V3<const floa
     for (int s = t0; s < n4; s += st) {
         const float4 u = a4[s], w = b4[s];
         if (wide) {
-            dv += (f32_to_f64(u.x * w.x) + f32_to_f64(u.y * w.y)) + (f32_to_f64(u.z * w.z) + f32_to_f64(u.w * w.w));
+            dv += (dot_term(u.x, w.x) + dot_term(u.y, w.y)) + (dot_term(u.z, w.z) + dot_term(u.w, w.w));
         } else {
             v += u.x * w.x;
             v += u.y * w.y;
@@ -3608,7 +3613,7 @@ __global__ void __launch_bounds__(256) k_dot32(V3<const float> av, V3<const floa
         }
     }
     for (int s = 4 * n4 + t0; s < n; s += st) {
-        if (wide) dv += f32_to_f64(a[s] * b[s]);
+        if (wide) dv += dot_term(a[s], b[s]);
         else v += a[s] * b[s];
     }
     dv = block_sum<256>(dv + (double)v);

@@ -58,7 +58,8 @@ def kernels(tmp_path_factory):
     src = SHIM
     src += re.search(r"constexpr int kReduceBlocks = \d+;", head).group(0) + "\n"
     src += "\n".join(re.findall(r"^constexpr int kWideDot = [^;]*;", solvers, flags=re.M)) + "\n"
-    src += _function(bits, r"__device__ inline double f32_to_f64\(") + dot + r"""
+    src += _function(bits, r"__device__ inline double f32_to_f64\(")
+    src += "\n".join(re.findall(r"^__device__ inline double dot_term\(.*$", solvers, flags=re.M)) + "\n" + dot + r"""
 extern "C" int blocks() { return kReduceBlocks; }
 extern "C" void dot(const float *a, const float *b, int n, int nb, double *part)
 {
@@ -91,3 +92,13 @@ def test_small_dot_sums_in_fp64(kernels, n):
     prod = (a * b).astype(np.float64)
     # at most n FP64 roundings of partial sums no larger than sum |a b|
     assert abs(math.fsum(part) - math.fsum(prod)) <= n * 2.0 ** -53 * math.fsum(abs(prod))
+
+
+def test_cluster_vcycle_sums_its_dot_in_fp64():
+    """r.z of a grid that the cluster kernel holds whole: each thread's sum, the warps' and the block's."""
+    text = _function(_source("solvers.cu"), r"__global__ void __cluster_dims__\(kCvCtas, 1, 1\)[^;{]*\bk_cc_coarse_vcycle\(")
+    assert re.findall(r"\b(\w+) dot = ", text) == ["double"]
+    adds = re.findall(r"\bdot \+= ([^;]*);", text)
+    assert adds == ["dot_term(w.b[c0 * w.cap + m], x0) + dot_term(w.b[(1 - c0) * w.cap + m], x1)",
+                    "__shfl_down_sync(0xffffffffu, dot, o)"]
+    assert re.search(r"\bps\[tid >> 5\] = dot;", text) and re.search(r"double \*bs = .*\*ps = reinterpret_cast<double \*>", text)
