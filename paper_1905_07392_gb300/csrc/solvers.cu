@@ -2026,9 +2026,10 @@ __global__ void __launch_bounds__(NT_T) k_nd_pass(NdOp<T> A, NdShape sh, const i
     const double sc = (kMode == ND_RES32 && sig) ? *sig : 1.0;
     const GridD &g = A.g;
     const int NX = g.nx + 1, NY = g.ny + 1, tid = threadIdx.x;
-    T v = 0;          // ND_APPLY: this thread's part of x.out
-    float vr = 0.0f;  // ND_RES32: its part of |r|^2, from the stored FP32 values
-    if ((int)blockIdx.x < sh.nlb) {
+    T v = 0;          // ND_APPLY: this thread's part of x.out; ND_RES32: of |r|^2 on the listed nodes
+    float vr = 0.0f;  // ND_RES32: its part of |r|^2 in the march, from the stored FP32 values too
+    const bool listed = (int)blockIdx.x < sh.nlb;
+    if (listed) {
         const int t = blockIdx.x * NT_T + tid;
         if (t < nlist) {
             const int n = list[t];
@@ -2047,7 +2048,7 @@ __global__ void __launch_bounds__(NT_T) k_nd_pass(NdOp<T> A, NdShape sh, const i
             if (kMode == ND_RES32) {
                 const float r = f64_to_f32_pow2(bn - ax, sc);
                 out32[n] = r;
-                vr = r * r;
+                v = T(r) * T(r);
             }
         }
     } else {
@@ -2133,7 +2134,7 @@ __global__ void __launch_bounds__(NT_T) k_nd_pass(NdOp<T> A, NdShape sh, const i
         }
     }
     if constexpr (kMode == ND_APPLY || kMode == ND_RES32) {
-        const double vs = kMode == ND_RES32 ? block_sum3_t<float>(vr) : block_sum3_t<T>(v);
+        const double vs = kMode == ND_RES32 && !listed ? block_sum3_t<float>(vr) : block_sum3_t<T>(v);
         if (tid == 0) part[blockIdx.x] = vs;
     }
 }

@@ -102,3 +102,14 @@ def test_cluster_vcycle_sums_its_dot_in_fp64():
     assert adds == ["dot_term(w.b[c0 * w.cap + m], x0) + dot_term(w.b[(1 - c0) * w.cap + m], x1)",
                     "__shfl_down_sync(0xffffffffu, dot, o)"]
     assert re.search(r"\bps\[tid >> 5\] = dot;", text) and re.search(r"double \*bs = .*\*ps = reinterpret_cast<double \*>", text)
+
+
+def test_listed_nodes_residual_norm_is_fp64():
+    """|r|^2 of the nodes that a nodal pass lists: FP64 squares of the stored FP32 residuals, FP64 sums
+    (k_nd_pass runs this mode with T = double; the march's own nodes are summed in FP32 within a warp)."""
+    solvers = _source("solvers.cu")
+    text = _function(solvers, r"__global__ void __launch_bounds__\(NT_T\) k_nd_pass\(")
+    lists = text[text.index("if (listed) {"):text.index("    } else {\n        __shared__ T sx")]
+    assert re.findall(r"\bvr? = T\(r\) \* T\(r\);", lists) == ["v = T(r) * T(r);"] and "vr" not in lists
+    assert "kMode == ND_RES32 && !listed ? block_sum3_t<float>(vr) : block_sum3_t<T>(v)" in text
+    assert re.findall(r"nd_pass<(\w+), ND_RES32>", solvers) == ["double"]
