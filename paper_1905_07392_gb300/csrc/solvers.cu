@@ -4675,10 +4675,12 @@ struct CcProblem : Problem {
                      ccop3<double>(*H, nc), p, q, c->part, gr.z, act);
     }
     // FP32 levels with nx a multiple of 8 large enough for two blocks per SM:
-    // the vectorised apply (its own partials; the choice follows the grid only)
+    // the vectorised apply.  Its partials sum eight FP32 terms a thread, the
+    // other's two, so the choice follows the grid of one component: a joint
+    // solve sums p.q as that component's own would
     bool vec32() const
     {
-        return gs4_ok(H->lv[0].g) && nc * nblocks3(apply4_grid(H->lv[0].g)) >= kVecMinBlocks;
+        return gs4_ok(H->lv[0].g) && nblocks3(apply4_grid(H->lv[0].g)) >= kVecMinBlocks;
     }
     int apply_blocks32() const override { return vec32() ? nblocks3(apply4_grid(H->lv[0].g)) : apply_blocks(); }
     void apply_dot32(Ctx *c, V3<const float> p, V3<float> q, const int *act) override

@@ -113,3 +113,12 @@ def test_listed_nodes_residual_norm_is_fp64():
     assert re.findall(r"\bvr? = T\(r\) \* T\(r\);", lists) == ["v = T(r) * T(r);"] and "vr" not in lists
     assert "kMode == ND_RES32 && !listed ? block_sum3_t<float>(vr) : block_sum3_t<T>(v)" in text
     assert re.findall(r"nd_pass<(\w+), ND_RES32>", solvers) == ["double"]
+
+
+def test_krylov_apply_is_chosen_by_one_components_grid():
+    """The vectorised FP32 apply sums p.q of eight cells a thread in FP32, the other one of two: a joint
+    solve takes the one that each component's own solve would take."""
+    text = _source("solvers.cu")
+    m = re.search(r"bool vec32\(\) const\s*\{(.*?)\n    \}", text, flags=re.S)
+    assert "nblocks3(apply4_grid(H->lv[0].g)) >= kVecMinBlocks" in m.group(1)
+    assert not re.search(r"\bnc\b", m.group(1))
