@@ -5012,15 +5012,10 @@ ebv_status setup_geometry_solvers(Ctx *c)
     CcLevel &M0 = c->mac.lv[0];
     EBV_LAUNCH(c, k_mac_coeffs, grid3(g.nx + 1, g.ny + 1, g.nz + 1), block3(), 0, g, c->flag, c->ax, c->ay, c->az,
                M0.extra_d, M0.bf_d[0], M0.bf_d[1], M0.bf_d[2]);
-    // both precisions of the projection hierarchy are kept
-    ebv_status s = cc_finish_hierarchy(c, c->mac, false);
+    // its levels and bottom inverse in the precision the solves use (the two
+    // share the blocks of the inverse diagonals, and the inverse)
+    ebv_status s = cc_finish_hierarchy(c, c->mac, c->prm.precision != EBV_FP64);
     if (s != EBV_OK) return s;
-    if (c->prm.precision != EBV_FP64) {
-        // FP32 levels derived from FP64 fine coefficients; the bottom inverse
-        // from the FP32 coarse operator
-        s = cc_finish_hierarchy(c, c->mac, true);
-        if (s != EBV_OK) return s;
-    }
     // nodal
     NdHier &N = c->nd;
     for (int l = 0; l < N.L; l++) {
