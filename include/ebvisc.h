@@ -296,13 +296,14 @@ void ebv_set_alloc_limit(long long bytes);
 void ebv_set_spin_limit(long long cycles);
 
 /* How FP32 multigrid levels whose x size is a multiple of 16 run a red-black
- * sweep (the coarse levels that one launch per V-cycle holds take neither form): 0 as two colour passes, 1 (default) as whichever of the two colour
+ * sweep (the coarse levels that one launch per V-cycle holds take neither
+ * form): 0 as two colour passes, 1 (default) as whichever of the two colour
  * passes and the fused one-pass sweep was faster when the context's solvers
  * were set up (instances of an ebv_batch keep the colour passes: their steps
  * run side by side, where a lone kernel's time does not decide), 2 always as
- * the fused sweep.  All give the same results bit
- * for bit; the switch exists to show that and to measure the difference.
- * Process-wide; read when a step is issued or captured. */
+ * the fused sweep.  All give the same results bit for bit; the switch exists
+ * to show that and to measure the difference.  Process-wide; read when a step
+ * is issued or captured. */
 void ebv_set_fused_sweep(int mode);
 
 /* EBV_FP32_REFINE / EBV_FP32_MIXED: the factor by which each FP32 correction

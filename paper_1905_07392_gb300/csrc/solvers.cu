@@ -2711,7 +2711,7 @@ __global__ void __cluster_dims__(kCvCtas, 1, 1) __launch_bounds__(kCvThreads, 1)
     __shared__ CvLevel lv[3];
     const int comp = blockIdx.y, tid = threadIdx.x, rank = (int)cl.block_rank(), na = D.na, split_z = D.split_z, nd = D.nd;
     const int npd = cv_np(D.A3[nd].A.g, split_z), nl = D.n - 1;   // nl smoothed levels
-    const bool act = rank < na, red = nl > nd;
+    const bool act = rank < na;
     const CvLayout &L = D.L;
     if (tid < nl) {
         const int l = tid;
@@ -4945,8 +4945,7 @@ ebv_status setup_solvers(Ctx *c)
             for (int d = 0; d < 3; d++) {
                 Lv.bf_d[d] = dalloc<double>(nface(gl[l], d), e);
                 Lv.bf_f[d] = dalloc<float>(nface(gl[l], d), e);
-                // one spare element: the coarse kernel stages BF16 arrays in 4-byte pairs
-                Lv.bf_h[d] = dalloc<__nv_bfloat16>(nface(gl[l], d) + 1, e);
+                Lv.bf_h[d] = dalloc<__nv_bfloat16>(nface(gl[l], d), e);
             }
             if (rb_fusable(gl[l]))
                 Lv.bxp = dalloc<RbF>((size_t)2 * rb_hxp(gl[l].nx) * gl[l].ny * gl[l].nz, e);
@@ -5062,10 +5061,10 @@ ebv_status setup_geometry_solvers(Ctx *c)
     return autotune_shapes(c);
 }
 
-// Launch-shape autotuner.  For every level it times each candidate block
-// shape of the colour pass (on the projection operator) and of the nodal
-// Chebyshev step, on zeroed scratch vectors in the precision the solves
-// use, and keeps the fastest; the viscous hierarchy shares the shapes of the
+// Launch-shape autotuner.  For every level that launches them it times each
+// candidate block shape of the colour pass (on the projection operator) and of
+// the node-by-node Chebyshev step, on zeroed scratch vectors in the precision
+// the solves use, and keeps the fastest; the viscous hierarchy shares the shapes of the
 // projection hierarchy (same level sizes).  The smoothers' results do not
 // depend on the shape: every update of a pass reads only values that the
 // pass does not write (the one pass that also sums r.z keeps the default
@@ -5093,8 +5092,13 @@ ebv_status autotune_shapes_t(Ctx *c)
         if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
         return ms;
     };
+    // (levels inside a cluster kernel launch neither; of these the ones that the
+    // fused sweep applies to are timed all the same, for ebv_sweep_timing)
+    CoarseVC<T> D;
+    const int lc = cv_plan<T>(c->mac, D), cl0 = lc < 0 ? c->mac.L - 1 : lc;
     for (int l = 0; l < c->mac.L; l++) {
         CcLevel &L = c->mac.lv[l];
+        if (l >= cl0 && !(sizeof(T) == 4 && rb_fusable(L.g) && gs4_ok(L.g))) continue;
         const VOp3<T> A = vop3<T>(c->mac, l, 1);
         const V3<T> xv = one(x);
         const V3<const T> bv = one<const T>(b), dv = one<const T>(d);
@@ -5181,8 +5185,11 @@ ebv_status autotune_shapes_t(Ctx *c)
         }
     }
     ChebCoef k = cheb_coef(2.0);
-    for (int l = 0; l < c->nd.L; l++) {
+    NdCoarse<T> DN;
+    const int ln = nc_plan<T>(c->nd, DN), nl0 = ln < 0 ? c->nd.L - 1 : ln;
+    for (int l = 0; l < nl0; l++) {
         NdLevel &L = c->nd.lv[l];
+        if (L.march) continue;   // (takes k_nd_pass)
         NdOp<T> A = ndop<T>(L);
         float best = 1e30f;
         for (int q = 0; q < nc; q++) {
