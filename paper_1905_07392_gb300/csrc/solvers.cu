@@ -144,6 +144,24 @@ __device__ inline double block_sum3_t(T v)
     }
 }
 
+// Block sum of FP32 partials of eight terms each, as wide as block_sum3_t's of
+// two: FP32 over groups of 8 lanes (64 terms, seven additions deep with the
+// thread's own), FP64 over the block's 32 groups.
+__device__ inline double block_sum8(float v)
+{
+    __shared__ double sm[32];
+    const int t = thread_linear();
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((t & 7) == 0) sm[t >> 3] = (double)v;
+    __syncthreads();
+    double r = 0.0;
+    if (t < 32) {
+        r = sm[t];
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+    }
+    return r;
+}
+
 // A term of a dot product that is summed in FP64: the product rounded in its
 // operands' precision.
 __device__ inline double dot_term(float a, float b) { return f32_to_f64(a * b); }
@@ -1683,9 +1701,9 @@ __global__ void __launch_bounds__(256) k_cc_apply_dot(CcOp3<T> A3, V3<const T> p
 // k_cc_apply_dot<float> for levels with nx a multiple of 8: a thread forms
 // q = A p at 4 consecutive cells of one half-row (half h = tx / nq) in each of
 // two planes, with 16-byte loads as in k_cc_gs4 (the x faces, rows of nx + 1,
-// as scalars), and adds p.q of its 8 cells to its block's partial.  Each q is
-// formed as in cc_row; the partial sums are grouped by this kernel's fixed
-// block shape (kApply4Blk).  (A cap of 48 registers, for five blocks per SM,
+// as scalars), and adds p.q of its 8 cells to its block's partial (block_sum8).
+// Each q is formed as in cc_row; the partial sums are grouped by this kernel's
+// fixed block shape (kApply4X x Y x Z).  (A cap of 48 registers, for five blocks per SM,
 // measures no faster than 64 registers and four blocks.)
 constexpr int kApply4X = 16, kApply4Y = 8, kApply4Z = 2;
 // The vectorised apply and restriction serve grids where they launch at least
@@ -1705,7 +1723,7 @@ __global__ void __launch_bounds__(256) k_cc_apply4(CcOp3<float> A3, V3<const flo
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int kk = cz.z * blockDim.z + threadIdx.z;
     const int sy = g.nx, sz = g.nx * g.ny;
-    float v = 0.f;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};   // per position: two terms, as a thread of k_cc_apply_dot
     if (tx < 2 * nq && j < g.ny) {
         const int h = tx / nq, t0 = 4 * (tx - h * nq);
 #pragma unroll
@@ -1743,12 +1761,12 @@ __global__ void __launch_bounds__(256) k_cc_apply4(CcOp3<float> A3, V3<const flo
                 if (k > 0) off += fz0[e] * xd[e];
                 if (k < g.nz - 1) off += fz1[e] * xu[e];
                 y[e] = dg[e] * pc[e] - off;
-                v += pc[e] * y[e];
+                v[e] += pc[e] * y[e];
             }
             *reinterpret_cast<float4 *>(q + c) = make_float4(y[0], y[1], y[2], y[3]);
         }
     }
-    const double vs = block_sum3_t<float>(v);
+    const double vs = block_sum8((v[0] + v[1]) + (v[2] + v[3]));
     if (thread_linear() == 0) part[cz.comp * kPartComp + cz.linear()] = vs;
 }
 inline dim3 apply4_grid(const GridD &g)
@@ -3617,7 +3635,8 @@ __global__ void __launch_bounds__(256) k_dot32(V3<const float> av, V3<const floa
         if (wide) dv += dot_term(a[s], b[s]);
         else v += a[s] * b[s];
     }
-    dv = block_sum<256>(dv + (double)v);
+    if (!wide) dv = (double)v;
+    dv = block_sum<256>(dv);
     if (threadIdx.x == 0) part[blockIdx.x] = dv;
 }
 
@@ -4675,12 +4694,12 @@ struct CcProblem : Problem {
                      ccop3<double>(*H, nc), p, q, c->part, gr.z, act);
     }
     // FP32 levels with nx a multiple of 8 large enough for two blocks per SM:
-    // the vectorised apply.  Its partials sum eight FP32 terms a thread, the
-    // other's two, so the choice follows the grid of one component: a joint
-    // solve sums p.q as that component's own would
+    // the vectorised apply.  By the operator, not by the components at hand
+    // (the viscous one has three, solved together or one after another), so a
+    // joint solve sums p.q as each component's own would
     bool vec32() const
     {
-        return gs4_ok(H->lv[0].g) && nblocks3(apply4_grid(H->lv[0].g)) >= kVecMinBlocks;
+        return gs4_ok(H->lv[0].g) && H->nvar * nblocks3(apply4_grid(H->lv[0].g)) >= kVecMinBlocks;
     }
     int apply_blocks32() const override { return vec32() ? nblocks3(apply4_grid(H->lv[0].g)) : apply_blocks(); }
     void apply_dot32(Ctx *c, V3<const float> p, V3<float> q, const int *act) override

@@ -122,3 +122,18 @@ def test_krylov_apply_is_chosen_by_one_components_grid():
     m = re.search(r"bool vec32\(\) const\s*\{(.*?)\n    \}", text, flags=re.S)
     assert "nblocks3(apply4_grid(H->lv[0].g)) >= kVecMinBlocks" in m.group(1)
     assert not re.search(r"\bnc\b", m.group(1))
+
+
+def test_vectorised_apply_sums_no_more_fp32_terms_than_the_other():
+    """p.q: a thread of k_cc_apply_dot adds two FP32 terms and its warp 32 of those sums, 64 terms and seven
+    additions deep (one fused with the first product).  A thread of k_cc_apply4 has eight: two to each of
+    four sums, those pairwise, and then no more than 8 lanes in FP32."""
+    text = _source("solvers.cu")
+    k = _function(text, r"__global__ void __launch_bounds__\(256\) k_cc_apply4\(")
+    assert "float v[4] = {0.f, 0.f, 0.f, 0.f};" in k and "v[e] += pc[e] * y[e];" in k
+    assert "block_sum8((v[0] + v[1]) + (v[2] + v[3]))" in k
+    b = _function(text, r"__device__ inline double block_sum8\(float v\)")
+    steps = re.findall(r"for \(int o = (\d+); o > 0; o >>= 1\) (\w+) \+= __shfl_down_sync", b)
+    assert steps == [("4", "v"), ("16", "r")] and "__shared__ double sm[32];" in b and "double r = 0.0;" in b
+    depth = 2 + 2 + int(steps[0][0]).bit_length()
+    assert 8 * 2 * int(steps[0][0]) <= 2 * 32 and depth <= 2 + 5
