@@ -34,7 +34,7 @@ static double __hiloint2double(int hi, int lo)
     return d;
 }
 static double g_sum;   // of the block's threads, which run one after another
-template <int N> static double block_sum(double v) { g_sum = threadIdx.x ? g_sum + v : v; return g_sum; }
+static double block_sum_flat(double v) { g_sum = threadIdx.x ? g_sum + v : v; return g_sum; }
 """
 
 
