@@ -4138,7 +4138,8 @@ int cc_smooth2(Ctx *c, const CcHier &H, int l, int nc, const int *act, V3<T> x, 
             // with r.z) was timed on its own against its colour passes
             const int mode = fused_sweep_mode();
             const int k1 = zero_start ? RB_ZERO : (corr ? RB_CORR : RB_PLAIN), k2 = dot_part ? RB_DOT : RB_PLAIN;
-            // (the pair runs x -> t -> x fused, or in place as passes: one form for both)
+            // (the pair runs x -> t -> x fused, or in place as passes: one form for
+            // both; timed with one component, for the joint solves too)
             const bool faster = L.rb_ms[k1][0] + L.rb_ms[k2][0] < L.rb_ms[k1][1] + L.rb_ms[k2][1];
             bool use = (mode == 2 || (mode == 1 && faster)) && rb_map(c, L.bxp, 4, g, &m1.fx) &&
                        rb_map(c, A.A.by, 2, g, &m1.fy) && rb_map(c, A.A.bz, 3, g, &m1.fz);
@@ -4582,6 +4583,8 @@ ebv_status finish_solve(Ctx *c, int nc, V3<double> x, int n, int *iters, double 
 // in every kernel; on smaller ones the condition word's load (half a
 // microsecond before each kernel's first) costs more than the redundant work,
 // which only rewrites scratch vectors.
+// (For one grid at a time: in a batch the redundant work takes SMs that other
+// instances wait for, which was not measured.)
 constexpr int kGateCells = 1 << 20;
 
 // Preconditioned CG in FP64, restarted from the true residual whenever the
